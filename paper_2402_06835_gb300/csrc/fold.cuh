@@ -18,12 +18,13 @@ template <typename T> struct __align__(4 * sizeof(T)) Node4 {
 
 // Node record of the exact path: the Node4 fields plus the differences to the
 // next epoch's depth, sigma and gain (NaN when the next epoch is missing or
-// invalid), so that an event is one record load and three FMAs.
+// invalid), so that an event is one record load and three FMAs.  pad holds the
+// largest gain an event on the interval can take (make_screen).
 template <typename T> struct __align__(8 * sizeof(T)) Node8 {
     T d, s, l, ig, dd, ds, dl, pad;
 };
 
-// Screening record of the FP64 path, one per (duration, epoch i): the FP32
+// Screening record, one per (duration, epoch i): the FP32
 // values and slopes of the interval [t0_i, t0_{i+1}], wsc = 2^-22 dt/gap (the
 // weight per unit of the 2^-22-slot position difference), and flags = 1 when
 // the interval is outside the screen's error model (epochs closer than dt/4,
@@ -36,18 +37,18 @@ struct __align__(32) ScreenRec {
 };
 
 // Byte layout of the exact path's per-(duration, epoch) arrays for n epochs:
-// Node8 records, then (FP64 only) screening records and pairs of fixed-point
-// epoch positions.
+// Node8 records, then (where the cells are screened) screening records and
+// pairs of fixed-point epoch positions.
 struct ExactLayout {
     size_t off_screen, off_vpos, total;
 };
-inline ExactLayout exact_layout(int64_t n, int n_D, bool fp64) {
+inline ExactLayout exact_layout(int64_t n, int n_D, bool fp64, bool screen = true) {
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     ExactLayout L;
     const size_t node = al((size_t)n * n_D * 8 * (fp64 ? 8 : 4));
     L.off_screen = node;
-    L.off_vpos = node + (fp64 ? al((size_t)n * n_D * sizeof(ScreenRec)) : 0);
-    L.total = L.off_vpos + (fp64 ? al((size_t)n * 16) : 0);
+    L.off_vpos = node + (screen ? al((size_t)n * n_D * sizeof(ScreenRec)) : 0);
+    L.total = L.off_vpos + (screen ? al((size_t)n * 16) : 0);
     return L;
 }
 
@@ -59,7 +60,7 @@ struct FoldSeg {
     int64_t n_bucket, bucket_off;
     int64_t n_slots, rec_off;
     int use_slots;
-    int screen;         // FP64 path: FP32 screening allowed for this curve
+    int screen;         // FP32 screening of the exact path allowed for this curve
     int64_t srec_off;   // FP64 path: first slot-indexed screening record
     int64_t gain_off;   // first entry of the curve's grouped gain table (either path)
     unsigned long long ulast;   // slot path: the last epoch's position, 24.40 slots
@@ -88,15 +89,12 @@ struct FoldScratch {
     void* nodes;            // exact-path records (exact_layout of all samples)
     int* bucket;            // bucket tables
     Node4<float>* rec;      // mixed slot records
-    float* lgm;             // mixed: the larger gain of each slot and the next (grouped)
+    float* lgm;             // gain tables (grouped): each curve's part for its own path
     ScreenRec* srec;        // FP64 slot-indexed screening records
     int* slot_of;           // FP64: slot of every sample
-    unsigned* reg;          // FP64: two words per curve (zeroed by the prep)
-    float* lint;            // FP64: largest gain of the interval at each slot
-    float* lm3;             //       and its maximum over the slot and both
-                            //       neighbours (grouped)
-    unsigned long long* peak;  // FP64: per curve, the key of its largest gain
-    PeriodConst* ptab;      // FP64: per period, its curve-independent constants
+    unsigned* reg;          // two words per curve (zeroed by the prep)
+    unsigned long long* peak;  // per curve, the key of its largest gain
+    PeriodConst* ptab;      // per period, its curve-independent constants
 };
 
 // Host side of the batch fold: per-curve layout and launches.

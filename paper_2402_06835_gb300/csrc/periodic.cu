@@ -788,7 +788,8 @@ struct ScreenGeom {
     int on;                            // screening allowed for this curve
     const unsigned long long* peak;    // key of the largest finite gain (k_gain_peak);
                                        // 0: none
-    const float* lm3;                  // grouped gain table (k_lmax3 of the interval gains)
+    const float* lm3;                  // grouped gain table (k_gain_table); nullptr: none
+    int f32;                           // the exact events are FP32 (mixed precision)
 };
 
 // Node sigma of one (duration, epoch) in FP64 (NaN when invalid).
@@ -824,7 +825,9 @@ __global__ void k_slot_offsets(const double* __restrict__ t0s, int64_t n_t0, dou
 
 // Screening record of epoch i of a curve with n epochs (gid indexes the
 // (duration, epoch) arrays; d is the duration), also placed at the epoch's
-// slot, and for the first duration row the pair of epoch positions.
+// slot, and for the first duration row the pair of epoch positions.  The
+// interval's largest gain goes to the pad of the epoch's node record (for
+// k_gain_table; k_nodes has run).
 template <typename T>
 __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
                                             const T* __restrict__ var,
@@ -833,7 +836,8 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
                                             int64_t i, int64_t n, int64_t d, double gap_max,
                                             double dt, ScreenRec* __restrict__ out,
                                             ScreenRec* __restrict__ sout,
-                                            float* __restrict__ lint, int64_t n_slots, const int* __restrict__ slot_of,
+                                            Node8<T>* __restrict__ nodes, int64_t n_slots,
+                                            const int* __restrict__ slot_of,
                                             ulonglong2* __restrict__ vpair) {
     // an interval needs both ends valid and a gap in (0, gap_max]
     bool v0 = i + 1 < n;
@@ -872,11 +876,12 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
             r.ds = 0.f;
         }
         // the exact event's gain fma(w, l1 - l0, l0) with w in [0, 1] (to a few
-        // units of FP64 rounding) is at most max(l0, l1) + 2^-50 (|l0| + |l1|);
-        // rounded up, and +inf when the interval is not screened
+        // units of its own rounding) is at most max(l0, l1) + 2^-50 (|l0| + |l1|)
+        // in FP64, 2^-20 (|l0| + |l1|) in FP32; rounded up, and +inf when the
+        // interval is not screened
+        const double slack = sizeof(T) == 8 ? 8.881784197001252e-16 : 9.5367431640625e-07;
         lmax = odd ? INFINITY
-                   : __double2float_ru(fmax(0.0, fmax(l0, l1)) +
-                                       8.881784197001252e-16 * (fabs(l0) + fabs(l1)));
+                   : __double2float_ru(fmax(0.0, fmax(l0, l1)) + slack * (fabs(l0) + fabs(l1)));
     } else {
         r.s = NAN;
         r.dd = 0.f;
@@ -886,10 +891,10 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
     }
     r.flags = flags;
     out[gid] = r;
-    const int sl = slot_of[i];
-    if (sl >= 0 && sl < n_slots) {
-        sout[d * n_slots + sl] = r;
-        lint[d * n_slots + sl] = lmax;
+    nodes[gid].pad = (T)lmax;
+    if (sout) {
+        const int sl = slot_of[i];
+        if (sl >= 0 && sl < n_slots) sout[d * n_slots + sl] = r;
     }
     if (d == 0) {
         auto pos = [&](int64_t k) -> unsigned long long {
@@ -912,28 +917,29 @@ __global__ void k_screen(const T* __restrict__ depth, const T* __restrict__ var,
                          const T* __restrict__ gain, const double* __restrict__ t0s,
                          int64_t n_t0, int n_D, double gap_max, double dt,
                          ScreenRec* __restrict__ rec, ScreenRec* __restrict__ srec,
-                         float* __restrict__ lint, int64_t n_slots,
+                         Node8<T>* __restrict__ nodes, int64_t n_slots,
                          const int* __restrict__ slot_of, ulonglong2* __restrict__ vpair) {
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (gid >= n_t0 * (int64_t)n_D) return;
     const int64_t d = gid / n_t0, i = gid - d * n_t0;
-    make_screen<T>(depth, var, gain, t0s, gid, i, n_t0, d, gap_max, dt, rec, srec, lint, n_slots,
-                   slot_of, vpair);
+    make_screen<T>(depth, var, gain, t0s, gid, i, n_t0, d, gap_max, dt, rec, srec, nodes,
+                   n_slots, slot_of, vpair);
 }
 
 // Entry o of a grouped gain table: the curve (segs: the batch's, else one
-// curve of n_slots1 slots), the source row's duration d and slot s.  Per
-// curve the table holds [groups][n_slots][W] entries from gain_off on; the
-// source rows are duration-major rows of n_slots from srec_off (FP64) or
-// rec_off (mixed).  Returns false for entries of no curve.
+// curve of n_slots1 slots), the duration d and slot s.  Per curve the table
+// holds [groups][n_slots][W] entries from gain_off on; the slot path's source
+// rows are duration-major rows of n_slots from rec_off.  Returns false for
+// entries of no curve of the path (screened, or else the slot path).
 struct GainSlot {
     int64_t src_off, n_slots;
-    int d, s;
+    int d, s, seg;
 };
 __device__ __forceinline__ bool gain_slot(const FoldSeg* __restrict__ segs, int n_seg,
-                                          int64_t n_slots1, int n_D, bool fp64, int64_t o,
+                                          int64_t n_slots1, int n_D, bool screened, int64_t o,
                                           GainSlot& gs) {
     int64_t out_off = 0;
+    gs.seg = 0;
     gs.src_off = 0;
     gs.n_slots = n_slots1;
     if (segs) {
@@ -945,9 +951,10 @@ __device__ __forceinline__ bool gain_slot(const FoldSeg* __restrict__ segs, int 
             if (segs[mid].gain_off <= o) lo = mid; else hi = mid;
         }
         const FoldSeg& f = segs[lo];
-        if (!(fp64 ? f.screen : f.use_slots)) return false;
+        if (!(screened ? f.screen : f.use_slots)) return false;
         out_off = f.gain_off;
-        gs.src_off = fp64 ? f.srec_off : f.rec_off;
+        gs.seg = lo;
+        gs.src_off = f.rec_off;
         gs.n_slots = f.n_slots;
     }
     const int W = gain_width(n_D);
@@ -960,23 +967,39 @@ __device__ __forceinline__ bool gain_slot(const FoldSeg* __restrict__ segs, int 
     return true;
 }
 
-// Grouped gain table of the FP64 screen: the maximum of lint over slots
-// s - 1, s and s + 1 of the row: the largest gain of an event whose walk
-// position lies in slot s (its interval starts at the epoch of slot s - 1, s
-// or s + 1, see the gain bound).
-__global__ void k_lmax3(const float* __restrict__ lint, const FoldSeg* __restrict__ segs,
-                        int n_seg, int64_t n_slots1, int n_D, int64_t n_out,
-                        float* __restrict__ lm3) {
+// Grouped gain table of the screen: per slot s the largest gain (the pad of the
+// node record) of the intervals that meet the positions [s - 1/4, s + 5/4), i.e. the largest gain
+// of an event whose walk position lies in slot s (the walk is within 1/4 slot
+// of the exact epoch, see the gain bound).  On a regular grid (epochs within
+// 2^-10 slot of their slots) these are the intervals that start at slots
+// s - 1, s and s + 1.  The bucket table gives the epoch at the slot; the range
+// is found from it by steps over the stored positions.
+template <typename T>
+__global__ void k_gain_table(const Node8<T>* __restrict__ nodes,
+                             const ulonglong2* __restrict__ vpair,
+                             const int* __restrict__ bucket, const FoldSeg* __restrict__ segs,
+                             int n_seg, int64_t n_t01, int64_t n_slots1, int64_t n_bucket1,
+                             int n_D, int64_t n_out, float* __restrict__ lm3) {
     const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (o >= n_out) return;
     GainSlot gs;
     if (!gain_slot(segs, n_seg, n_slots1, n_D, true, o, gs)) return;
     float m = 0.f;
     if (gs.d < n_D) {
-        const float* r = lint + gs.src_off + (int64_t)gs.d * gs.n_slots;
-        m = r[gs.s];
-        if (gs.s > 0) m = fmaxf(m, r[gs.s - 1]);
-        if (gs.s + 1 < gs.n_slots) m = fmaxf(m, r[gs.s + 1]);
+        const int64_t n_t0 = segs ? segs[gs.seg].n_t0 : n_t01;
+        const int64_t nb = segs ? segs[gs.seg].n_bucket : n_bucket1;
+        const int* bk = bucket + (segs ? segs[gs.seg].bucket_off : 0);
+        const ulonglong2* vp = vpair + (segs ? segs[gs.seg].s_off : 0);
+        const Node8<T>* row =
+            nodes + (segs ? segs[gs.seg].s_off * n_D : 0) + (int64_t)gs.d * n_t0;
+        const unsigned long long Q = 1ull << 38;                // 1/4 slot
+        const unsigned long long at = (unsigned long long)gs.s << 40;
+        const unsigned long long lo = at > Q ? at - Q : 0, hi = at + 5ull * Q;
+        int64_t i = (int64_t)bk[gs.s < nb ? gs.s : nb - 1] - 1;  // the epoch at or before slot s
+        if (i < 0) i = 0;
+        while (i > 0 && vp[i].x > lo) --i;
+        while (i + 1 < n_t0 && vp[i + 1].x <= lo) ++i;           // last epoch at or before lo
+        for (; i < n_t0 && (vp[i].x < hi); ++i) m = fmaxf(m, (float)row[i].pad);
     }
     lm3[o] = m;
 }
@@ -1040,6 +1063,9 @@ __device__ __forceinline__ ScreenPeriod screen_period_curve(const FoldGeom& g,
     if (sp.slots)
         sp.cv = fmaxf(sp.cv, (float)(2.02 * (1.1920928955078125e-07 + e_pos / SCALE + (double)off) +
                                      8.0 * 5.9604644775390625e-08));
+    // mixed precision: the exact event itself is computed in FP32 (node
+    // differences, weight and FMA: a few units of |x_i| + |x_{i+1}|)
+    if (sg.f32) sp.cv += 8.0f * 5.9604645e-08f;
     sp.hw = 0.5f - sp.dw;
     sp.wscale = (float)(4194304.0 * g.inv_dt);
     return sp;
@@ -1278,14 +1304,13 @@ __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom
     return acc.bound(sp.cv, bf);
 }
 
-// The gain bound of a cell on a regular grid, from 4 bytes per epoch.  By the
-// bound above, ln P <= S_L + 1/2, and every event's gain is at most the
-// larger gain of its interval's two nodes.  The walk's position u of epoch k
-// lies within half a slot of the exact epoch, and on a regular grid every
-// epoch is within 2^-10 slot of its slot, so the exact interval starts at
-// the epoch of slot floor(u) - 1, floor(u) or floor(u) + 1: lm3 at floor(u)
-// bounds the event's gain (0 for a dropped epoch, +inf on an interval outside
-// the screen's error model).  Extra walk positions past t_last (u < uend)
+// The gain bound of a cell, from 4 bytes per epoch.  By the bound above,
+// ln P <= S_L + 1/2, and every event's gain is at most the larger gain of its
+// interval's two nodes.  The walk's position u of epoch k lies within 1/4 slot
+// of the exact epoch (0.2 slot by the test below, plus the walk's own error,
+// below 2^-6), so the exact interval meets [floor(u) - 1/4, floor(u) + 5/4):
+// lm3 at floor(u) bounds the event's gain (0 for a dropped epoch, +inf on an
+// interval outside the screen's error model).  Extra walk positions past t_last (u < uend)
 // only add terms >= 0.  The FP32 sum of K terms >= 0 is rounded up by
 // (K + 16) 2^-23 of itself, and 1e-6 covers the exact path's own rounding.
 //
@@ -1295,9 +1320,7 @@ __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom
 // epoch k is at most 1 + k/2 units from the 64-bit walk.  F is chosen per
 // period so that no position the walk loads (up to end + 3 steps: four epochs
 // a round) exceeds 2^31 (the margin below allows twelve), and the walk is
-// used only when that error stays below half a slot for every epoch (the gain
-// bound tolerates the exact interval starting one slot either side of the
-// walk's slot).  The end is widened by the same error, so every epoch of the
+// used only when that error stays below 0.2 slot for every epoch.  The end is widened by the same error, so every epoch of the
 // 64-bit walk is counted; positions past it add terms >= 0 (the walk adds
 // four terms at a time; a position past the row is clamped to the padding
 // slot zs, whose term is 0).
@@ -1318,7 +1341,7 @@ __device__ __forceinline__ GainWalk32 gain_walk32(unsigned long long ustep,
     const double top = span + 12.0 * R + kmax + 8.0;         // slots a position can reach
     int F = 30 - ilogb(top);                                 // 2^F top < 2^31
     if (F > 24) F = 24;
-    if (F < 8 || (kmax + 2.0) * ldexp(1.0, -F) > 0.5) return w;
+    if (F < 8 || (kmax + 2.0) * ldexp(1.0, -F) > 0.2) return w;
     w.F = F;
     w.shift = 40 - F;
     w.step = (unsigned)((ustep + (1ull << (w.shift - 1))) >> w.shift);
@@ -1451,17 +1474,18 @@ __device__ __forceinline__ float gain_col(const float4& s, int i) {
 
 // Exact ln P of one cell computed by a whole warp (lanes over epochs); used
 // only to seed the pruning threshold.
+template <typename T>
 __device__ __forceinline__ double exact_cell_warp(const FoldGeom& g,
-                                                  const Node8<double>* __restrict__ nd,
+                                                  const Node8<T>* __restrict__ nd,
                                                   const CellCtx& c, int64_t j) {
     const int lane = threadIdx.x & 31;
     const double phi = cell_phi(c, j);
     const unsigned long long u0 = (unsigned long long)j * c.swp.u0;
     const int64_t kmax = cell_kmax(g, c, phi, u0);
-    ExactAcc<double> a1;
+    ExactAcc<T> a1;
     a1.init();
-    cell_pass1<double>(g, nd, c, phi, u0, kmax, lane, 32, a1);
-    double s_inv = a1.s_inv.s, s_d = a1.s_d.s, s_l = a1.s_l.s;
+    cell_pass1<T>(g, nd, c, phi, u0, kmax, lane, 32, a1);
+    T s_inv = a1.s_inv.s, s_d = a1.s_d.s, s_l = a1.s_l.s;
     int K = a1.K;
     for (int o = 16; o > 0; o >>= 1) {
         s_inv += __shfl_xor_sync(0xffffffffu, s_inv, o);
@@ -1470,13 +1494,13 @@ __device__ __forceinline__ double exact_cell_warp(const FoldGeom& g,
         K += __shfl_xor_sync(0xffffffffu, K, o);
     }
     if (K == 0) return -INFINITY;
-    const double s2 = 1.0 / s_inv;
-    ExactPen<double> a2;
+    const T s2 = T(1) / s_inv;
+    ExactPen<T> a2;
     a2.init(s2, s2 * s_d);
-    cell_pass2<double>(g, nd, c, phi, u0, kmax, lane, 32, a2);
-    double pen = a2.logsum() + a2.quad.s;
+    cell_pass2<T>(g, nd, c, phi, u0, kmax, lane, 32, a2);
+    T pen = (T)(a2.logsum() + (double)a2.quad.s);
     for (int o = 16; o > 0; o >>= 1) pen += __shfl_xor_sync(0xffffffffu, pen, o);
-    return s_l - 0.5 * pen;
+    return (double)s_l - 0.5 * (double)pen;
 }
 
 // Order-preserving unsigned key of a float (for a shared atomic max).
@@ -1495,18 +1519,19 @@ __device__ __forceinline__ float from_fkey(unsigned k) {
 // be zero on entry and stays zero when no gain is finite.  blockIdx.x is the
 // curve (s_off == nullptr: one curve of n_t0 epochs); the blocks along y
 // share a curve's entries.
-__global__ void k_gain_peak(const double* __restrict__ gain, const int64_t* __restrict__ s_off,
+template <typename T>
+__global__ void k_gain_peak(const T* __restrict__ gain, const int64_t* __restrict__ s_off,
                             int64_t n_t0, int n_D, unsigned long long* __restrict__ key) {
     const int g = blockIdx.x;
     const int64_t s0 = s_off ? s_off[g] : 0;
     const int64_t ng = s_off ? s_off[g + 1] - s0 : n_t0;
     const int64_t n = ng * n_D;
     if (n >= 0xffffffffLL) return;
-    const double* row = gain + s0 * n_D;
+    const T* row = gain + s0 * n_D;
     unsigned long long best = 0;
     for (int64_t e = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.y * blockDim.x) {
-        const double v = row[e];
+        const double v = (double)row[e];
         if (v > -INFINITY && v < INFINITY) {
             const unsigned long long k = ((unsigned long long)fkey((float)v) << 32) |
                                          (unsigned long long)(0xffffffffu - (unsigned)e);
@@ -1520,34 +1545,47 @@ __global__ void k_gain_peak(const double* __restrict__ gain, const int64_t* __re
     if ((threadIdx.x & 31) == 0 && best != 0) atomicMax(key + g, best);
 }
 
+// What the screens compare with: an FP32 value below every ln P that an
+// evaluated cell could lose by.  In FP64 the evaluated ln P rounded down; in
+// mixed precision the evaluated ln P carries FP32 rounding (the events', the
+// compensated sums', and up to 2^-21 per epoch from the logarithms), so the
+// screens, which bound the real ln P, leave 2e-4 relative and 5e-7 per epoch.
+template <typename T>
+__device__ __forceinline__ float screen_threshold(double lnp, float kmax) {
+    if (sizeof(T) == 8) return __double2float_rd(lnp);
+    const float l = (float)lnp;
+    return l - 2e-4f * (1.f + fabsf(l)) - 5e-7f * kmax;
+}
+
 // Exact evaluation of a queued cell by one thread; the thread's best is kept
 // in shared memory and the block's thresholds are raised.
+template <typename T>
 __device__ __forceinline__ void evaluate_queued(const FoldGeom& g,
-                                               const Node8<double>* __restrict__ nodes,
+                                               const Node8<T>* __restrict__ nodes,
                                                const CellCtx& c, int64_t n_phi, long long qcell,
                                                int qd, unsigned long long* sh_sbest,
                                                unsigned* sh_bfk, Best* tb) {
     const int64_t qj = qcell - (int64_t)qd * n_phi;
-    const Node8<double>* nd = nodes + (int64_t)qd * g.n_t0;
+    const Node8<T>* nd = nodes + (int64_t)qd * g.n_t0;
     const double phi = cell_phi(c, qj);
     const unsigned long long u0 = (unsigned long long)qj * c.swp.u0;
     const int64_t kmax = cell_kmax(g, c, phi, u0);
-    ExactAcc<double> a1;
+    ExactAcc<T> a1;
     a1.init();
-    cell_pass1<double>(g, nd, c, phi, u0, kmax, 0, 1, a1);
+    cell_pass1<T>(g, nd, c, phi, u0, kmax, 0, 1, a1);
     if (a1.K == 0 || a1.cannot_win(from_max_key(*sh_sbest))) return;
-    const double s2 = 1.0 / a1.s_inv.s;
-    const double Dl = s2 * a1.s_d.s;
-    ExactPen<double> a2;
+    const T s2 = T(1) / a1.s_inv.s;
+    const T Dl = s2 * a1.s_d.s;
+    ExactPen<T> a2;
     a2.init(s2, Dl);
-    cell_pass2<double>(g, nd, c, phi, u0, kmax, 0, 1, a2);
-    const double lnp = a1.s_l.s - 0.5 * (a2.logsum() + a2.quad.s);
+    cell_pass2<T>(g, nd, c, phi, u0, kmax, 0, 1, a2);
+    const double lnp = (double)a1.s_l.s - 0.5 * (a2.logsum() + (double)a2.quad.s);
     if (!(lnp == lnp)) return;   // NaN never selected
-    const Best cand{lnp, qcell, Dl, s2};
+    const Best cand{lnp, qcell, (double)Dl, (double)s2};
     if (better(cand, *tb)) *tb = cand;
     if (lnp > from_max_key(*sh_sbest)) {
         atomicMax(sh_sbest, max_key(lnp));
-        atomicMax(sh_bfk, fkey(__double2float_rd(lnp)));
+        atomicMax(sh_bfk, fkey(screen_threshold<T>(lnp, (float)(int)kmax)));
     }
 }
 
@@ -1609,9 +1647,16 @@ __device__ __forceinline__ void evaluate_queued_warp(const FoldGeom& g,
 // lower bound) are shared by the block through atomic maxima.
 // With TAB the period's curve-independent constants come from the table
 // entry pc (k_period_consts), else they are computed here.
-template <int MAXT = 256, bool TAB = false, bool GROUP = true>
+// T is the type of the exact events: double, or float for the mixed fold of
+// grids that are not regular (FP64 epochs, FP32 values and compensated sums;
+// every cell by the thread code, whose order of the sums defines the result).
+// Measured on a sector of barycentric times (19 440 epochs, 10 durations,
+// 20 000 periods): FP64 32.0 -> 11.3 ms when the gain bound came to irregular
+// grids; mixed 132.5 -> 10.3 ms (every cell's events took their epochs and
+// brackets in FP64 before, 64 cycles per warp instruction).
+template <typename T, int MAXT = 256, bool TAB = false, bool GROUP = true>
 __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const ScreenGeom& sg,
-                                                  const Node8<double>* __restrict__ nodes,
+                                                  const Node8<T>* __restrict__ nodes,
                                                   int n_D, double P, int64_t p,
                                                   double* __restrict__ Q_out,
                                                   double* __restrict__ T0_out,
@@ -1641,8 +1686,8 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
     if (threadIdx.x == 0) sh_sp = TAB ? screen_period(g, sg, P, *pc) : screen_period(g, sg, P, n_phi);
     __syncthreads();
     if (!sh_sp.on) {
-        fold_exact_one<double, 8, MAXT>(g, nodes, n_D, P, p, Q_out, T0_out, Didx_out, dep_out,
-                                  sig_out, lnp_out);
+        fold_exact_one<T, 8, MAXT>(g, nodes, n_D, P, p, Q_out, T0_out, Didx_out, dep_out,
+                                   sig_out, lnp_out);
         return;
     }
     sh_tb[threadIdx.x] = Best{-INFINITY, LLONG_MAX, NAN, NAN};
@@ -1658,6 +1703,18 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     // cells of 32 or more epochs are evaluated warp-cooperatively
     const bool coop = g.t_last - g.t_ref >= 32.0 * P;
+    // raise the thresholds to the warp's evaluation of a cell, less a margin
+    // that keeps the cell itself above them (it is evaluated again by the
+    // thread code, whose sums run in another order)
+    auto seed_with = [&](double lnp) {
+        if (lane == 0 && lnp == lnp && lnp > -INFINITY) {
+            const double margin = sizeof(T) == 8 ? 1e-9 : 1e-4;
+            const double seed = lnp - margin * (1.0 + fabs(lnp));
+            atomicMax(&sh_sbest, max_key(seed));
+            atomicMax(&sh_bfk,
+                      fkey(screen_threshold<T>(seed, (float)((g.t_last - g.t_ref) / P))));
+        }
+    };
     // Peak seed: the cell whose epochs pass through the epoch of the curve's
     // largest single-event gain (phase index nearest to it), evaluated
     // exactly by warp 0.  When one event dominates a short cell (a deep
@@ -1673,13 +1730,7 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
                 const double x = (g.t0s[e - pd * g.n_t0] - g.t_ref) / P;
                 int64_t pj = (int64_t)rint((x - floor(x)) * (double)n_phi);
                 if (pj >= n_phi || pj < 0) pj = 0;
-                const double lnp = exact_cell_warp(g, nodes + pd * g.n_t0, c, pj);
-                if (lane == 0 && lnp == lnp && lnp > -INFINITY) {
-                    // the same margin as the first-round seed below
-                    const double seed = lnp - 1e-9 * (1.0 + fabs(lnp));
-                    atomicMax(&sh_sbest, max_key(seed));
-                    atomicMax(&sh_bfk, fkey(__double2float_rd(seed)));
-                }
+                seed_with(exact_cell_warp<T>(g, nodes + pd * g.n_t0, c, pj));
             }
             __syncthreads();
         }
@@ -1691,11 +1742,10 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
     long long* qa = sh_qa[wid];
     int* qad = sh_qad[wid];
     int na = 0;
-    // Cascade on regular grids: after the warp's first round every cell is
-    // bounded from its gains alone (the gain bound, 4 bytes per epoch); the
+    // Cascade: after the warp's first round every cell is bounded from its gains alone (the gain bound, 4 bytes per epoch); the
     // cells that bound does not rule out are queued and screened in full 32
     // at a time, and the full screen's survivors are evaluated exactly.
-    const bool cascade = sp.slots && sg.lm3 != nullptr && sp.ustep < (1ull << 60) && sh_gw.ok;
+    const bool cascade = sg.lm3 != nullptr && sp.ustep < (1ull << 60) && sh_gw.ok;
     const unsigned ns1 = (unsigned)(sg.n_slots - 1);
     // append this lane's cell to a queue when keep (positions by ballot)
     auto push = [&](long long* qx, int* qy, int& n, bool keep, long long cl, int dl) {
@@ -1724,24 +1774,28 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
         }
         __syncwarp();
     };
-    // exact evaluation of the first 32 entries of the survivor queue
-    auto evaluate32 = [&]() {
-        if (coop) {
-            for (int q = 0; q < 32; ++q)
-                evaluate_queued_warp(g, nodes, c, n_phi, qc[q], qd[q], &sh_sbest, &sh_bfk,
-                                     &sh_tb[threadIdx.x]);
-        } else {
-            evaluate_queued(g, nodes, c, n_phi, qc[lane], qd[lane], &sh_sbest, &sh_bfk,
-                            &sh_tb[threadIdx.x]);
+    // exact evaluation of the first n <= 32 entries of the survivor queue
+    auto evaluate_first = [&](int n) {
+        if constexpr (sizeof(T) == 8) {
+            if (coop) {
+                for (int q = 0; q < n; ++q)
+                    evaluate_queued_warp(g, nodes, c, n_phi, qc[q], qd[q], &sh_sbest, &sh_bfk,
+                                         &sh_tb[threadIdx.x]);
+                return;
+            }
         }
+        if (lane < n)
+            evaluate_queued<T>(g, nodes, c, n_phi, qc[lane], qd[lane], &sh_sbest, &sh_bfk,
+                               &sh_tb[threadIdx.x]);
+    };
+    auto evaluate32 = [&]() {
+        evaluate_first(32);
         __syncwarp();
         pop32(qc, qd, nq);
     };
     // First-round seed: the warp evaluates its lane with the largest finite
     // bound (all lanes over its epochs), unless that bound is already below
-    // the threshold (the cell cannot raise it).  A 1e-9 margin keeps the
-    // seeding cell itself above the threshold: it is evaluated again by the
-    // thread code.
+    // the threshold (the cell cannot raise it).
     auto seed_warp = [&](float ub, int dl, int64_t jl) {
         float v = (ub < INFINITY) ? ub : -INFINITY;
         int src = lane;
@@ -1758,12 +1812,7 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
         if (v > -INFINITY && !(v < thr)) {
             const int pd = __shfl_sync(FULL, dl, src);
             const long long pj = __shfl_sync(FULL, (long long)jl, src);
-            const double lnp = exact_cell_warp(g, nodes + (int64_t)pd * g.n_t0, c, pj);
-            if (lane == 0 && lnp == lnp && lnp > -INFINITY) {
-                const double seed = lnp - 1e-9 * (1.0 + fabs(lnp));
-                atomicMax(&sh_sbest, max_key(seed));
-                atomicMax(&sh_bfk, fkey(__double2float_rd(seed)));
-            }
+            seed_with(exact_cell_warp<T>(g, nodes + (int64_t)pd * g.n_t0, c, pj));
             __syncwarp();
         }
     };
@@ -1865,14 +1914,7 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
     }
     if (na > 0) screen_queued(0, na);
     if (nq >= 32) evaluate32();
-    if (coop) {
-        for (int q = 0; q < nq; ++q)
-            evaluate_queued_warp(g, nodes, c, n_phi, qc[q], qd[q], &sh_sbest, &sh_bfk,
-                                 &sh_tb[threadIdx.x]);
-    } else if (lane < nq) {
-        evaluate_queued(g, nodes, c, n_phi, qc[lane], qd[lane], &sh_sbest, &sh_bfk,
-                        &sh_tb[threadIdx.x]);
-    }
+    evaluate_first(nq);
     __syncthreads();
     Best best = sh_tb[threadIdx.x];
     if (best.cell != LLONG_MAX) best.sigma = sqrt(best.sigma);   // held sigma^2
@@ -1896,19 +1938,19 @@ __device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const Scree
 #ifndef NU_SCREEN_GROUP_BLOCKS
 #define NU_SCREEN_GROUP_BLOCKS 12
 #endif
-template <int MAXT, bool GROUP>
+template <typename T, int MAXT, bool GROUP>
 __global__ void __launch_bounds__(MAXT, MAXT <= 64 ? (GROUP ? NU_SCREEN_GROUP_BLOCKS
                                                             : NU_SCREEN_SMALL_BLOCKS)
                                                    : NU_SCREEN_MIN_BLOCKS)
-k_fold_screened(FoldGeom g, ScreenGeom sg, const Node8<double>* __restrict__ nodes, int n_D,
+k_fold_screened(FoldGeom g, ScreenGeom sg, const Node8<T>* __restrict__ nodes, int n_D,
                 const double* __restrict__ periods, int64_t n_P, double* __restrict__ Q_out,
                 double* __restrict__ T0_out, int* __restrict__ Didx_out,
                 double* __restrict__ dep_out, double* __restrict__ sig_out,
                 double* __restrict__ lnp_out) {
     if ((int64_t)blockIdx.x >= n_P) return;
     const int64_t p = period_slot(blockIdx.x, periods, n_P);
-    fold_screened_one<MAXT, false, GROUP>(g, sg, nodes, n_D, periods[p], p, Q_out, T0_out,
-                                          Didx_out, dep_out, sig_out, lnp_out);
+    fold_screened_one<T, MAXT, false, GROUP>(g, sg, nodes, n_D, periods[p], p, Q_out, T0_out,
+                                             Didx_out, dep_out, sig_out, lnp_out);
 }
 
 // ---------------------------------------- slot path (mixed, regular grids)
@@ -2321,10 +2363,12 @@ k_fold_slots(const Node4<float>* __restrict__ rec, const float* __restrict__ lgm
 // ------------------------------------------------------------ batch path
 
 // Persistent fold over (curve, period) work items taken from a device
-// counter (no waits: a block takes items until none are left).  kind 0: the
-// exact FP64-epoch path with FP64 values; 1: exact path, FP32 values;
-// 2: slot path (mixed precision, regular grids).  Items of curves that do not
-// use this kernel's path are skipped.
+// counter (no waits: a block takes items until none are left).  kind 0 / 4:
+// the screened path with FP64 values (one duration / grouped gain walk);
+// 1 / 5: the same with FP32 values (mixed precision, grids that are not
+// regular); 2 / 3: slot path (mixed precision, regular grids; with / without
+// the cascade).  Items of curves that do not use this kernel's path are
+// skipped.
 // Resident blocks per SM the registers are sized for, by path and block size.
 // The FP64 batch kernel carries the work-item loop besides the screen: at 80
 // registers it spills, at 96 (10 x 64 threads) it does not; slots as the
@@ -2332,18 +2376,20 @@ k_fold_slots(const Node4<float>* __restrict__ rec, const float* __restrict__ lgm
 template <int KIND, int MAXT>
 struct BatchBlocks {
     static constexpr int value =
-        KIND == 0 || KIND == 4 ? (MAXT <= 64 ? 10 : (MAXT <= 128 ? 5 : NU_SCREEN_MIN_BLOCKS))
-                  : (KIND == 2 ? NU_SLOTS_CASC_MIN_BLOCKS * 256 / MAXT
-                               : KIND == 3 ? NU_SLOTS_MIN_BLOCKS * 256 / MAXT : 1);
+        KIND == 2 ? NU_SLOTS_CASC_MIN_BLOCKS * 256 / MAXT
+                  : (KIND == 3 ? NU_SLOTS_MIN_BLOCKS * 256 / MAXT
+                               : (MAXT <= 64 ? 10 : (MAXT <= 128 ? 5 : NU_SCREEN_MIN_BLOCKS)));
 };
+template <int KIND> struct BatchEvent { typedef double T; };
+template <> struct BatchEvent<1> { typedef float T; };
+template <> struct BatchEvent<5> { typedef float T; };
 
 template <int KIND, int MAXT>
 __global__ void __launch_bounds__(MAXT, BatchBlocks<KIND, MAXT>::value)
 k_fold_batch(const FoldSeg* __restrict__ segs, int n_seg, const double* __restrict__ t,
              const void* __restrict__ nodes, const ScreenRec* __restrict__ screen,
              const ulonglong2* __restrict__ vpair, const ScreenRec* __restrict__ srec,
-             const float* __restrict__ lm3, const float* __restrict__ lgm,
-             const unsigned* __restrict__ reg,
+             const float* __restrict__ lgm, const unsigned* __restrict__ reg,
              const unsigned long long* __restrict__ peak,
              const int* __restrict__ bucket,
              const Node4<float>* __restrict__ rec, int n_D, double dt, double gap_factor,
@@ -2374,19 +2420,14 @@ k_fold_batch(const FoldSeg* __restrict__ segs, int n_seg, const double* __restri
         } else {
             FoldGeom gg{t + fs.s_off, fs.n_t0, fs.t_ref, fs.t_last, dt, 1.0 / dt,
                         gap_factor * dt, bucket + fs.bucket_off, fs.n_bucket};
-            if (KIND == 0 || KIND == 4) {
-                const ScreenGeom sg{screen + fs.s_off * n_D, vpair + fs.s_off,
-                                    srec + fs.srec_off, fs.n_slots,
-                                    reg + 2 * g, fs.screen, peak + g, lm3 + fs.gain_off};
-                fold_screened_one<MAXT, true, KIND == 4>(gg, sg,
-                                              (const Node8<double>*)nodes + fs.s_off * n_D, n_D,
-                                              periods[p], o, Q_out, T0_out, Didx_out, dep_out,
-                                              sig_out, lnp_out, ptab + p);
-            }
-            else
-                fold_exact_one<float, 8, MAXT>(gg, (const Node8<float>*)nodes + fs.s_off * n_D, n_D,
-                                         periods[p], o, Q_out, T0_out, Didx_out, dep_out,
-                                         sig_out, lnp_out);
+            typedef typename BatchEvent<KIND>::T T;
+            const ScreenGeom sg{screen + fs.s_off * n_D, vpair + fs.s_off,
+                                sizeof(T) == 8 ? srec + fs.srec_off : nullptr, fs.n_slots,
+                                reg + 2 * g, fs.screen, peak + g, lgm + fs.gain_off,
+                                sizeof(T) == 4};
+            fold_screened_one<T, MAXT, true, KIND == 4 || KIND == 5>(
+                gg, sg, (const Node8<T>*)nodes + fs.s_off * n_D, n_D, periods[p], o, Q_out,
+                T0_out, Didx_out, dep_out, sig_out, lnp_out, ptab + p);
         }
     }
 }
@@ -2417,7 +2458,7 @@ __global__ void k_screen_batch(const T* __restrict__ depth, const T* __restrict_
                                const int64_t* __restrict__ s_off, int n_D, double gap_max,
                                double dt, ScreenRec* __restrict__ rec,
                                ulonglong2* __restrict__ vpair, ScreenRec* __restrict__ srec,
-                               float* __restrict__ lint,
+                               Node8<T>* __restrict__ nodes,
                                const int* __restrict__ slot_of) {
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (gid >= s_off[n_seg] * (int64_t)n_D) return;
@@ -2432,7 +2473,7 @@ __global__ void k_screen_batch(const T* __restrict__ depth, const T* __restrict_
     const int64_t w = gid - s0 * n_D;
     const int64_t d = w / ng, i = w - d * ng;
     make_screen<T>(depth, var, gain, t + s0, gid, i, ng, d, gap_max, dt, rec,
-                   srec + fs.srec_off, lint + fs.srec_off, fs.n_slots,
+                   srec ? srec + fs.srec_off : nullptr, nodes, fs.n_slots,
                    slot_of + s0, vpair + s0);
 }
 
@@ -2541,11 +2582,11 @@ void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double
         f.n_slots = f.n_bucket + 2;
         f.use_slots = (!fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span < 4.0e6 &&
                        !irregular[g]) ? 1 : 0;
-        f.screen = (fp64 && gap_factor < 2.0 && span < 8.0e6) ? 1 : 0;
+        f.screen = (!f.use_slots && gap_factor < 2.0 && span < 8.0e6) ? 1 : 0;
         f.srec_off = fb.n_srec_total;
-        fb.n_srec_total += f.screen ? f.n_slots * n_D : 0;
+        fb.n_srec_total += fp64 && f.screen ? f.n_slots * n_D : 0;
         f.gain_off = fb.n_gain_total;
-        fb.n_gain_total += (fp64 ? f.screen : f.use_slots) ? f.n_slots * gain_cols(n_D) : 0;
+        fb.n_gain_total += f.screen || f.use_slots ? f.n_slots * gain_cols(n_D) : 0;
         f.bucket_off = fb.n_bucket_total;
         fb.n_bucket_total += f.use_slots ? 0 : f.n_bucket;
         f.rec_off = fb.n_rec_total;
@@ -2567,52 +2608,52 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
     const int64_t ngrid = n_total * (int64_t)n_D;
     cudaError_t e = cudaSuccess;
     if (fb.any_exact) {
+        const ExactLayout L = exact_layout(n_total, n_D, fp64);
+        ScreenRec* screen = (ScreenRec*)((char*)fs.nodes + L.off_screen);
+        ulonglong2* vpair = (ulonglong2*)((char*)fs.nodes + L.off_vpos);
+        k_buckets_batch<<<div_up(fb.n_bucket_total, 256), 256, 0, st>>>(
+            t, segs_dev, n_seg, fb.n_bucket_total, dt, fs.bucket);
+        ++launched;
+        e = cudaMemsetAsync(fs.peak, 0, (size_t)n_seg * sizeof(unsigned long long), st);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(fs.reg, 0, (size_t)n_seg * 2 * sizeof(unsigned), st);
+        if (e != cudaSuccess) {
+            *n_launched = launched;
+            return e;
+        }
         if (fp64) {
-            const ExactLayout L = exact_layout(n_total, n_D, true);
             k_nodes_batch<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth, (const double*)var, (const double*)gain, t, segs_dev,
                 n_seg, s_off_dev, n_D, gap_factor * dt, (Node8<double>*)fs.nodes);
-            ++launched;
-            e = cudaMemsetAsync(fs.reg, 0, (size_t)n_seg * 2 * sizeof(unsigned), st);
-            if (e != cudaSuccess) {
-                *n_launched = launched;
-                return e;
-            }
             k_slot_offsets_batch<<<div_up(n_total, 256), 256, 0, st>>>(
                 t, segs_dev, n_seg, s_off_dev, 1.0 / dt, fs.slot_of, fs.reg);
             k_fill_screen<<<div_up(fb.n_srec_total + 1, 256), 256, 0, st>>>(
                 fs.srec, fb.n_srec_total);
-            launched += 2;
-            e = cudaMemsetAsync(fs.lint, 0, (size_t)(fb.n_srec_total + 1) * sizeof(float), st);
-            if (e != cudaSuccess) {
-                *n_launched = launched;
-                return e;
-            }
             k_screen_batch<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth, (const double*)var, (const double*)gain, t, segs_dev,
-                n_seg, s_off_dev, n_D, gap_factor * dt, dt,
-                (ScreenRec*)((char*)fs.nodes + L.off_screen),
-                (ulonglong2*)((char*)fs.nodes + L.off_vpos), fs.srec, fs.lint, fs.slot_of);
-            k_lmax3<<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
-                fs.lint, segs_dev, n_seg, 0, n_D, fb.n_gain_total, fs.lm3);
-            launched += 2;
-            e = cudaMemsetAsync(fs.peak, 0, (size_t)n_seg * sizeof(unsigned long long), st);
-            if (e != cudaSuccess) {
-                *n_launched = launched;
-                return e;
-            }
-            k_gain_peak<<<dim3(n_seg, 1), 256, 0, st>>>((const double*)gain, s_off_dev, 0, n_D,
-                                                       fs.peak);
-            ++launched;
+                n_seg, s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, fs.srec,
+                (Node8<double>*)fs.nodes, fs.slot_of);
+            k_gain_peak<double><<<dim3(n_seg, 1), 256, 0, st>>>((const double*)gain, s_off_dev,
+                                                               0, n_D, fs.peak);
+            k_gain_table<double><<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
+                (const Node8<double>*)fs.nodes, vpair, fs.bucket, segs_dev, n_seg, 0, 0, 0, n_D,
+                fb.n_gain_total, fs.lgm);
+            launched += 6;
         } else {
             k_nodes_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
                 s_off_dev, n_D, gap_factor * dt, (Node8<float>*)fs.nodes);
-            ++launched;
+            k_screen_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
+                (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
+                s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, nullptr,
+                (Node8<float>*)fs.nodes, nullptr);
+            k_gain_peak<float><<<dim3(n_seg, 1), 256, 0, st>>>((const float*)gain, s_off_dev, 0,
+                                                              n_D, fs.peak);
+            k_gain_table<float><<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
+                (const Node8<float>*)fs.nodes, vpair, fs.bucket, segs_dev, n_seg, 0, 0, 0, n_D,
+                fb.n_gain_total, fs.lgm);
+            launched += 4;
         }
-        k_buckets_batch<<<div_up(fb.n_bucket_total, 256), 256, 0, st>>>(
-            t, segs_dev, n_seg, fb.n_bucket_total, dt, fs.bucket);
-        ++launched;
     }
     if (fb.any_slots) {
         k_fill_nan<<<div_up(fb.n_rec_total, 256), 256, 0, st>>>(fs.rec, fb.n_rec_total);
@@ -2637,16 +2678,14 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       cudaStream_t st) {
     int launched = 0;
     const ExactLayout L = exact_layout(n_total, n_D, fp64);
-    const ScreenRec* screen =
-        fp64 ? (const ScreenRec*)((const char*)fs.nodes + L.off_screen) : nullptr;
-    const ulonglong2* vpair =
-        fp64 ? (const ulonglong2*)((const char*)fs.nodes + L.off_vpos) : nullptr;
+    const ScreenRec* screen = (const ScreenRec*)((const char*)fs.nodes + L.off_screen);
+    const ulonglong2* vpair = (const ulonglong2*)((const char*)fs.nodes + L.off_vpos);
     // the kernel instance whose shared arrays and register budget match the
     // block size (64, 128 or 256 threads)
 #define NU_FB(KIND_, MAXT_, CTR_)                                                          \
     k_fold_batch<KIND_, MAXT_><<<grid, MAXT_, 0, st>>>(                                  \
-        segs_dev, n_seg, t, fs.nodes, screen, vpair, fs.srec, fs.lm3, fs.lgm, fs.reg,      \
-        fs.peak, fs.bucket,                                                                \
+        segs_dev, n_seg, t, fs.nodes, screen, vpair, fs.srec, fs.lgm, fs.reg, fs.peak,     \
+         fs.bucket,                                                                \
         fs.rec, n_D, dt, gap_factor, periods, fs.ptab, n_P, CTR_, Q, T0, Didx, dep, sig, lnp)
 #define NU_FB_SIZE(KIND_, CTR_)                                                            \
     do {                                                                                   \
@@ -2655,16 +2694,14 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
         else NU_FB(KIND_, 256, CTR_);                                                      \
     } while (0)
     if (fb.any_exact) {
+        k_period_consts<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt, fs.ptab);
+        const bool group = gain_width(n_D) > 1;
         if (fp64) {
-            k_period_consts<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt, fs.ptab);
-            ++launched;
-            if (gain_width(n_D) > 1)
-                NU_FB_SIZE(4, counter);
-            else
-                NU_FB_SIZE(0, counter);
-        } else
-            NU_FB_SIZE(1, counter);
-        ++launched;
+            if (group) NU_FB_SIZE(4, counter); else NU_FB_SIZE(0, counter);
+        } else {
+            if (group) NU_FB_SIZE(5, counter); else NU_FB_SIZE(1, counter);
+        }
+        launched += 2;
     }
     if (fb.any_slots) {
         k_slot_periods<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt,
@@ -2693,27 +2730,36 @@ int launch_slots_test(const double* t, const int64_t* s_off_dev, int n_seg, int6
 // ------------------------------------------------ single-curve host side
 namespace nu {
 
-// Scratch layout of the single-curve fold.
+// Scratch layout of the single-curve fold.  In mixed precision the regular
+// and the irregular path are two uses of one region (which of them runs is
+// known after the slot test).  screen = false leaves out what the screen of
+// the mixed irregular path needs (the exact path evaluates every cell).
 struct SingleLayout {
     ExactLayout el;
-    size_t exact, bucket, slot_of, flag, rec, srec, lint, lm3, lgm, total;
+    size_t exact, bucket, slot_of, flag, rec, srec, lm3, lgm, total;
+    bool screen;
 };
 
-static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, bool fp64) {
+static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, bool fp64,
+                                  bool screen = true) {
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     SingleLayout L;
-    L.el = exact_layout(n_t0, n_D, fp64);
+    L.screen = fp64 || screen;
+    L.el = exact_layout(n_t0, n_D, fp64, L.screen);
     const int64_t n_slots = n_bucket + 2;          // slot records, NaN padded
-    L.exact = 0;
+    const size_t gain = al((size_t)n_slots * gain_cols(n_D) * sizeof(float));
+    L.flag = 0;
+    L.slot_of = 256;
+    L.exact = L.slot_of + al((size_t)n_t0 * sizeof(int));
+    // the mixed regular path
+    L.rec = L.exact;
+    L.lgm = L.rec + al((size_t)n_slots * n_D * sizeof(Node4<float>));
+    // the others
     L.bucket = L.exact + L.el.total;
-    L.slot_of = L.bucket + al((size_t)n_bucket * sizeof(int));
-    L.flag = L.slot_of + al((size_t)n_t0 * sizeof(int));
-    L.rec = L.flag + 256;
-    L.srec = L.rec + (fp64 ? 0 : al((size_t)n_slots * n_D * sizeof(Node4<float>)));
-    L.lint = L.srec + (fp64 ? al((size_t)n_slots * n_D * sizeof(ScreenRec)) : 0);
-    L.lm3 = L.lint + (fp64 ? al((size_t)n_slots * n_D * sizeof(float)) : 0);
-    L.lgm = L.lm3 + (fp64 ? al((size_t)n_slots * gain_cols(n_D) * sizeof(float)) : 0);
-    L.total = L.lgm + (fp64 ? 0 : al((size_t)n_slots * gain_cols(n_D) * sizeof(float)));
+    L.srec = L.bucket + al((size_t)n_bucket * sizeof(int));
+    L.lm3 = L.srec + (fp64 ? al((size_t)n_slots * n_D * sizeof(ScreenRec)) : 0);
+    L.total = L.lm3 + (L.screen ? gain : 0);
+    if (!fp64) L.total = std::max(L.total, L.lgm + gain);
     return L;
 }
 
@@ -2782,71 +2828,86 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
                                                         n_bucket, bucket);
         FoldGeom g{t0s_dev, n_t0, t_ref, t_last, phase_step, 1.0 / phase_step,
                    gap_factor * phase_step, bucket, n_bucket};
+        ScreenRec* nrec = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
+        ulonglong2* vpair = (ulonglong2*)(scratch + L.exact + L.el.off_vpos);
+        ScreenRec* srec = fp64 ? (ScreenRec*)(scratch + L.srec) : nullptr;
+        float* lm3 = (float*)(scratch + L.lm3);
+        unsigned* reg = (unsigned*)(flag + 1);
+        unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
+        const ScreenGeom sg{nrec, vpair, srec, n_slots, reg,
+                            (gap_factor < 2.0 && span_steps < 8.0e6) ? 1 : 0, peak, lm3,
+                            fp64 ? 0 : 1};
+        const int64_t nlm = n_slots * gain_cols(n_D);
+        const dim3 peak_grid(1, (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608));
+        e = cudaMemsetAsync(flag, 0, 256, st);
+        if (e != cudaSuccess) {
+            count_launches(launched);
+            return cuda_fail(e, (std::string(who) + ": memset").c_str());
+        }
+        // One block per period.  With many periods, 2-warp blocks: 14 fit
+        // on an SM (28 warps) and each period has 2 warps to seed; with
+        // few, 8-warp blocks keep the GPU full (C2, 20 000 periods: 16.5 ms
+        // at 256 threads, 14.0 at 128 (7 per SM), 13.6 at 64).
+        // (the grouped gain walk where the durations form groups)
+#define NU_FSC(T_, MAXT_)                                                                  \
+    do {                                                                                   \
+        if (gain_width(n_D) > 1)                                                           \
+            k_fold_screened<T_, MAXT_, true><<<(unsigned)n_P, MAXT_, 0, st>>>(             \
+                g, sg, (const Node8<T_>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,      \
+                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
+        else                                                                               \
+            k_fold_screened<T_, MAXT_, false><<<(unsigned)n_P, MAXT_, 0, st>>>(            \
+                g, sg, (const Node8<T_>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,      \
+                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
+    } while (0)
         if (fp64) {
-            ScreenRec* nrec = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
-            ulonglong2* vpair = (ulonglong2*)(scratch + L.exact + L.el.off_vpos);
-            ScreenRec* srec = (ScreenRec*)(scratch + L.srec);
-            float* lint = (float*)(scratch + L.lint);
-            float* lm3 = (float*)(scratch + L.lm3);
-            unsigned* reg = (unsigned*)(flag + 1);
-            unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
-            const ScreenGeom sg{nrec, vpair, srec, n_slots, reg,
-                                (gap_factor < 2.0 && span_steps < 8.0e6) ? 1 : 0, peak, lm3};
-            e = cudaMemsetAsync(flag, 0, 256, st);
-            if (e != cudaSuccess) {
-                count_launches(launched);
-                return cuda_fail(e, (std::string(who) + ": memset").c_str());
-            }
             k_slot_offsets<<<div_up(n_t0, 256), 256, 0, st>>>(t0s_dev, n_t0, 1.0 / phase_step,
                                                               n_slots, slot_of, reg);
             k_fill_screen<<<div_up(n_slots * n_D, 256), 256, 0, st>>>(srec, n_slots * n_D);
-            e = cudaMemsetAsync(lint, 0, (size_t)n_slots * n_D * sizeof(float), st);
-            if (e != cudaSuccess) {
-                count_launches(launched + 2);
-                return cuda_fail(e, (std::string(who) + ": memset").c_str());
-            }
             k_nodes<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
                 t0s_dev, n_t0, n_D, g.gap_max, (Node8<double>*)nodes);
             k_screen<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
-                t0s_dev, n_t0, n_D, g.gap_max, phase_step, nrec, srec, lint, n_slots, slot_of,
-                vpair);
-            const int64_t nlm = n_slots * gain_cols(n_D);
-            k_lmax3<<<div_up(nlm, 256), 256, 0, st>>>(lint, nullptr, 0, n_slots, n_D, nlm, lm3);
-            k_gain_peak<<<dim3(1, (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608)), 256, 0,
-                          st>>>((const double*)dlnl_dev, nullptr, n_t0, n_D, peak);
-            // One block per period.  With many periods, 2-warp blocks: 14 fit
-            // on an SM (28 warps) and each period has 2 warps to seed; with
-            // few, 8-warp blocks keep the GPU full (C2, 20 000 periods: 16.5 ms
-            // at 256 threads, 14.0 at 128 (7 per SM), 13.6 at 64).
-            // (the grouped gain walk where the durations form groups)
-#define NU_FSC(MAXT_)                                                                      \
-    do {                                                                                   \
-        if (gain_width(n_D) > 1)                                                           \
-            k_fold_screened<MAXT_, true><<<(unsigned)n_P, MAXT_, 0, st>>>(                 \
-                g, sg, (const Node8<double>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,  \
-                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
-        else                                                                               \
-            k_fold_screened<MAXT_, false><<<(unsigned)n_P, MAXT_, 0, st>>>(                \
-                g, sg, (const Node8<double>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,  \
-                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
-    } while (0)
+                t0s_dev, n_t0, n_D, g.gap_max, phase_step, nrec, srec, (Node8<double>*)nodes,
+                n_slots, slot_of, vpair);
+            k_gain_table<double><<<div_up(nlm, 256), 256, 0, st>>>(
+                (const Node8<double>*)nodes, vpair, bucket, nullptr, 0, n_t0, n_slots, n_bucket,
+                n_D, nlm, lm3);
+            k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)dlnl_dev, nullptr,
+                                                           n_t0, n_D, peak);
             if (n_P >= 8192)
-                NU_FSC(64);
+                NU_FSC(double, 64);
             else
-                NU_FSC(256);
-#undef NU_FSC
+                NU_FSC(double, 256);
             launched += 8;
         } else {
             k_nodes<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev,
                 t0s_dev, n_t0, n_D, g.gap_max, (Node8<float>*)nodes);
-            k_fold_exact<float, 8><<<(unsigned)n_P, 256, 0, st>>>(
-                g, (const Node8<float>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,
-                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
-            launched += 3;
+            if (L.screen && sg.on) {
+                k_screen<float><<<div_up(ngrid, 256), 256, 0, st>>>(
+                    (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev,
+                    t0s_dev, n_t0, n_D, g.gap_max, phase_step, nrec, nullptr,
+                    (Node8<float>*)nodes, n_slots, nullptr, vpair);
+                k_gain_table<float><<<div_up(nlm, 256), 256, 0, st>>>(
+                    (const Node8<float>*)nodes, vpair, bucket, nullptr, 0, n_t0, n_slots,
+                    n_bucket, n_D, nlm, lm3);
+                k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)dlnl_dev, nullptr,
+                                                              n_t0, n_D, peak);
+                if (n_P >= 8192)
+                    NU_FSC(float, 64);
+                else
+                    NU_FSC(float, 256);
+                launched += 6;
+            } else {
+                k_fold_exact<float, 8><<<(unsigned)n_P, 256, 0, st>>>(
+                    g, (const Node8<float>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,
+                    D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+                launched += 3;
+            }
         }
+#undef NU_FSC
     }
     count_launches(launched);
     e = cudaGetLastError();
@@ -3138,7 +3199,11 @@ extern "C" nu_status nu_periodic_search_noalloc(const double* t0s_dev, int64_t n
         return fail(NU_EINVAL, "nu_periodic_search_noalloc: phase grid too fine");
     const int64_t n_bucket = (int64_t)span_steps + 2;
     const bool fp64 = prec == NU_FP64;
-    const SingleLayout L = single_layout(n_t0, n_D, n_bucket, fp64);
+    // (the mixed path of irregular grids runs without its screen where only
+    // the screen's arrays exceed the limit)
+    SingleLayout L = single_layout(n_t0, n_D, n_bucket, fp64);
+    if (!fp64 && L.total > NU_NOALLOC_SCRATCH_BYTES)
+        L = single_layout(n_t0, n_D, n_bucket, fp64, false);
     if (L.total > NU_NOALLOC_SCRATCH_BYTES)
         return fail(NU_EINVAL,
                     "nu_periodic_search_noalloc: this grid needs %zu bytes of scratch, more "
