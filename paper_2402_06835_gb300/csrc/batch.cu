@@ -4,14 +4,14 @@
 // of one problem: the factor scans run over the chunks of all curves (a
 // chunk never crosses a curve), the linear search covers every curve's
 // (D, t0) grid with t0 = its samples, and the fold is a persistent kernel
-// that takes (curve, period) work items from a device counter, which
+// that takes (curve, period) work items from device counters, which
 // balances curves of different spans.  Host work (validation, layout, a
 // regularity test of each curve's cadence, uploads of the small tables)
 // happens before capture; the kernels are captured into one CUDA graph and
 // launched once.  The instantiated graph of a configuration is kept and, on
 // later calls, updated in place with the new call's parameters
 // (cudaGraphExecUpdate) instead of being instantiated again.  The launch
-// shapes of the fold (threads per block, resident blocks per SM) and of the
+// shapes of the fold (which items take a block, which a warp) and of the
 // linear search's window-start kernel (window starts per block, staged chunk)
 // are chosen by a small autotuner the first time a configuration is seen:
 // the candidates are timed on a slice of the batch and the fastest are
@@ -60,7 +60,7 @@ struct TuneKey {
     }
 };
 struct TuneVal {
-    int blocks_per_sm, threads;     // fold
+    int warps;                      // fold: one of FOLD_SHAPES (0: not tuned)
     WindowShape win;                // linear search
 };
 
@@ -72,12 +72,12 @@ std::map<TuneKey, TuneVal> g_tune;
 // out of the cache while it uses it, so two threads never launch one
 // executable graph at once.
 struct GraphKey {
-    int dev, nb, k, prec, n_D, n_lc, bps, threads, tlo, ch;
+    int dev, nb, k, prec, n_D, n_lc, warps, tlo, ch;
     int64_t N, n_P;
     bool operator<(const GraphKey& o) const {
-        return std::tie(dev, nb, k, prec, n_D, n_lc, bps, threads, tlo, ch, N, n_P) <
-               std::tie(o.dev, o.nb, o.k, o.prec, o.n_D, o.n_lc, o.bps, o.threads, o.tlo, o.ch,
-                        o.N, o.n_P);
+        return std::tie(dev, nb, k, prec, n_D, n_lc, warps, tlo, ch, N, n_P) <
+               std::tie(o.dev, o.nb, o.k, o.prec, o.n_D, o.n_lc, o.warps, o.tlo, o.ch, o.N,
+                        o.n_P);
     }
 };
 std::mutex g_graph_mu;
@@ -189,7 +189,6 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     const size_t o_ends = off;  off += al((size_t)n_lc * 2 * 8);
     const size_t o_irr = off;   off += al((size_t)n_lc * 4);
     const size_t o_Ds = off;    off += al((size_t)n_D * 8);
-    const size_t o_ctr = off;   off += 256;
     const size_t o_tune = off;  off += al(512 * 8);
     const bool win_lo = n_D <= 4096;            // window-start recursion of the box search
     const size_t o_wplan = off; off += win_lo ? al((size_t)n_lc * window_plan_ints(n_D) * 4) : 0;
@@ -264,34 +263,20 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     FoldBatch fbat;
     plan_fold_batch(plan.s_off, t_first, t_last, irregular, fp64, phase_step, gap_factor, n_D,
                     fbat);
-    size_t foff = 0;
-    const size_t f_segs = foff;  foff += al(fbat.segs.size() * sizeof(FoldSeg));
-    const size_t f_nodes = foff; foff += fbat.any_exact ? exact_layout(N, n_D, fp64).total : 0;
-    const size_t f_buck = foff;  foff += al((size_t)(fbat.n_bucket_total + 1) * 4);
-    const size_t f_rec = foff;   foff += al((size_t)(fbat.n_rec_total + 1) * sizeof(Node4<float>));
-    const size_t f_lgm = foff;   foff += al((size_t)(fbat.n_gain_total + 1) * sizeof(float));
-    const size_t f_srec = foff;  foff += al((size_t)(fbat.n_srec_total + 1) * sizeof(ScreenRec));
-    const size_t f_slot = foff;  foff += fp64 ? al((size_t)N * sizeof(int)) : 0;
-    const size_t f_reg = foff;   foff += al((size_t)n_lc * 2 * sizeof(unsigned));
-    const size_t f_peak = foff;  foff += al((size_t)n_lc * sizeof(unsigned long long));
-    const size_t f_ptab = foff;  foff += al((size_t)n_P * period_const_bytes());
+    const size_t f_segs = (fbat.segs.size() * sizeof(FoldSeg) + 255) / 256 * 256;
+    const size_t foff = f_segs + fold_scratch(fbat, N, n_lc, n_D, n_P, fp64, nullptr, nullptr);
     e = cudaMallocAsync((void**)&fold_mem, foff, st);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(fold_mem + f_segs, fbat.segs.data(), fbat.segs.size() * sizeof(FoldSeg),
+        e = cudaMemcpyAsync(fold_mem, fbat.segs.data(), fbat.segs.size() * sizeof(FoldSeg),
                             cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "nu_batch_search: fold setup");
     }
-    const FoldSeg* fsegs = (const FoldSeg*)(fold_mem + f_segs);
-    const FoldScratch fsc{fold_mem + f_nodes, (int*)(fold_mem + f_buck),
-                          (Node4<float>*)(fold_mem + f_rec), (float*)(fold_mem + f_lgm),
-                          (ScreenRec*)(fold_mem + f_srec),
-                          (int*)(fold_mem + f_slot), (unsigned*)(fold_mem + f_reg),
-                          (unsigned long long*)(fold_mem + f_peak),
-                          (PeriodConst*)(fold_mem + f_ptab)};
-    unsigned long long* ctr = (unsigned long long*)(mem + o_ctr);
+    const FoldSeg* fsegs = (const FoldSeg*)fold_mem;
+    FoldScratch fsc;
+    fold_scratch(fbat, N, n_lc, n_D, n_P, fp64, fold_mem + f_segs, &fsc);
     const double* Ds_dev = (const double*)(mem + o_Ds);
     int dev = 0, n_sm = 152;
     cudaGetDevice(&dev);
@@ -300,8 +285,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     cudaStream_t side = thread_side_stream();
     cudaError_t enq_err = cudaSuccess;      // first failed enqueue of a memset
     WindowShape win_shape = default_window_shape(N);
-    auto enqueue = [&](int grid, int threads, int64_t nP_run, int n_run,
-                       cudaStream_t st) -> int {
+    auto enqueue = [&](int warps, int64_t nP_run, int n_run, cudaStream_t st) -> int {
         int l = 0;
         k_init_dstat<<<div_up(n_lc, 128), 128, 0, st>>>(fb.dstat, s_off_dev, n_lc);
         ++l;
@@ -325,24 +309,22 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
                                                 fsc, st, &lp);
         l += lp;
         if (ep != cudaSuccess && enq_err == cudaSuccess) enq_err = ep;
-        const cudaError_t ec = cudaMemsetAsync(ctr, 0, 16, st);
-        if (ec != cudaSuccess && enq_err == cudaSuccess) enq_err = ec;
         l += launch_fold_batch(fbat, fsegs, n_run, N, fp64, t_dev, fsc, n_D,
-                               phase_step, gap_factor, periods_dev, nP_run, ctr, grid, threads,
+                               phase_step, gap_factor, periods_dev, nP_run, warps,
                                Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev,
-                               lnP_dev, st);
+                               lnP_dev, st, side, &enq_err);
         count_launches(l - lf);      // launch_factor counted its own
         return l;
     };
     // ------------------------------------------------------- autotuning
     const TuneKey key{nb, k, (int)prec, n_D};
-    TuneVal tv{0, 0, win_shape};
+    TuneVal tv{0, win_shape};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune.find(key);
         if (it != g_tune.end()) tv = it->second;
     }
-    if (tv.threads == 0) {
+    if (tv.warps == 0) {
         // time the fold on a slice (the first curves, periods spread over the
         // whole grid) for each shape; the slice holds several times more
         // (curve, period) items than the largest grid has blocks, so that it
@@ -353,28 +335,24 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
         k_sample_periods<<<2, 256, 0, st>>>(periods_dev, n_P, (int)nP_run, tune_periods);
         count_launches(1);
         ++launched;
-        // blocks per SM x threads; small blocks suit short curves, whose
-        // (curve, period) items hold few cells (each warp seeds its item)
-        const int cand[6][2] = {{2, 256}, {4, 256}, {4, 128}, {8, 128}, {8, 64}, {16, 64}};
         float best_ms = 1e30f;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
-        launched += enqueue(n_sm * 2, 256, nP_run, n_run, st);    // warm the caches
+        launched += enqueue(FOLD_SHAPES[0], nP_run, n_run, st);    // warm the caches
         if (enq_err != cudaSuccess) {
             cudaEventDestroy(e0);
             cudaEventDestroy(e1);
             cleanup();
             return cuda_fail(enq_err, "nu_batch_search: memset");
         }
-        for (int c = 0; c < 6; ++c) {
-            cudaMemsetAsync(ctr, 0, 16, st);
+        for (int c = 0; c < 5; ++c) {
             cudaEventRecord(e0, st);
             const int lt = launch_fold_batch(fbat, fsegs, n_run, N, fp64, t_dev, fsc,
                                              n_D, phase_step, gap_factor, tune_periods,
-                                             nP_run, ctr, n_sm * cand[c][0], cand[c][1], Q_dev,
+                                             nP_run, FOLD_SHAPES[c], Q_dev,
                                              T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev,
-                                             lnP_dev, st);
+                                             lnP_dev, st, side, &enq_err);
             count_launches(lt);
             launched += lt;
             cudaEventRecord(e1, st);
@@ -383,8 +361,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
             cudaEventElapsedTime(&ms, e0, e1);
             if (ms < best_ms) {
                 best_ms = ms;
-                tv.blocks_per_sm = cand[c][0];
-                tv.threads = cand[c][1];
+                tv.warps = FOLD_SHAPES[c];
             }
         }
         // the linear search's window-start kernel on the same curves: window
@@ -432,7 +409,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     // the executable graph of this configuration, when a previous call left
     // one, takes this call's parameters (buffers, outputs) by an update
     cudaGraph_t graph = nullptr;
-    const GraphKey gkey{dev, nb, k, (int)prec, n_D, n_lc, tv.blocks_per_sm, tv.threads,
+    const GraphKey gkey{dev, nb, k, (int)prec, n_D, n_lc, tv.warps,
                         win_shape.tlo, win_shape.ch, N, n_P};
     cudaGraphExec_t exec = take_graph(gkey);
     cudaStream_t cs = nullptr;
@@ -440,7 +417,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     int in_graph = 0;
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        in_graph = enqueue(n_sm * tv.blocks_per_sm, tv.threads, n_P, n_lc, cs);
+        in_graph = enqueue(tv.warps, n_P, n_lc, cs);
         e = cudaStreamEndCapture(cs, &graph);
         if (e == cudaSuccess && enq_err != cudaSuccess) e = enq_err;
     }

@@ -18,8 +18,7 @@ template <typename T> struct __align__(4 * sizeof(T)) Node4 {
 
 // Node record of the exact path: the Node4 fields plus the differences to the
 // next epoch's depth, sigma and gain (NaN when the next epoch is missing or
-// invalid), so that an event is one record load and three FMAs.  pad holds the
-// largest gain an event on the interval can take (make_screen).
+// invalid), so that an event is one record load and three FMAs. 
 template <typename T> struct __align__(8 * sizeof(T)) Node8 {
     T d, s, l, ig, dd, ds, dl, pad;
 };
@@ -62,24 +61,67 @@ struct FoldSeg {
     int use_slots;
     int screen;         // FP32 screening of the exact path allowed for this curve
     int64_t srec_off;   // FP64 path: first slot-indexed screening record
-    int64_t gain_off;   // first entry of the curve's grouped gain table (either path)
     unsigned long long ulast;   // slot path: the last epoch's position, 24.40 slots
+    int64_t tab_off;    // first entry of the curve's filter tables
+    int64_t g_off;      // first word of its G table
+    int64_t pair_off;   // first entry of its S and Q tables (durations in pairs)
+    unsigned long long uspan;   // screened curves: the last epoch's position, 24.40 slots
 };
 
-// Gain tables are grouped by duration: the gains of W consecutive durations
-// at one slot are adjacent, so that one vector load serves W cells of one
-// phase (their epochs are the same).  Per curve the table is [n_D / W groups
-// (rounded up)][n_slots][W] floats; columns past n_D hold 0.
-#ifndef NU_GAIN_W_MAX
-#define NU_GAIN_W_MAX 4
-#endif
-__host__ __device__ inline int gain_width(int n_D) {
-    return n_D >= 4 && NU_GAIN_W_MAX >= 4 ? 4 : (n_D >= 2 && NU_GAIN_W_MAX >= 2 ? 2 : 1);
+// ---- filter tables (see filter.cuh) and the lists of the cell kernels
+__host__ __device__ inline int64_t filter_slots(int64_t n_slots) { return (n_slots + 7) / 8 * 8; }
+// FP16 words of one G entry: 8, 4 or 2 durations per load
+__host__ __device__ inline int filter_words(int n_D) { return n_D >= 5 ? 4 : (n_D >= 3 ? 2 : 1); }
+__host__ __device__ inline int filter_groups(int n_D) {
+    const int w = 2 * filter_words(n_D);
+    return (n_D + w - 1) / w;
 }
-__host__ __device__ inline int gain_cols(int n_D) {
-    const int W = gain_width(n_D);
-    return (n_D + W - 1) / W * W;
+
+// Tables of all curves; rows of filter_slots(n_slots) per duration from
+// tab_off on (in rows' entries), G from g_off on (in words).
+struct FilterTab {
+    uint2* S;
+    float* gB;
+    float* L;
+    unsigned* Z;      // per slot (largest, smallest) Delta v as FP16 (source of Q)
+    uint2* Q;
+    unsigned* G;
+    unsigned* vmax;   // per (curve, duration): max 1/s^2 (float bits)
+};
+
+struct FilterLayout {
+    size_t S, gB, L, Z, Q, G, vmax, total;
+};
+inline FilterLayout filter_layout(int64_t entries, int64_t pairs, int64_t words, int64_t rows) {
+    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    FilterLayout F;
+    F.S = 0;
+    F.Q = F.S + al((size_t)pairs * 8);
+    F.gB = F.Q + al((size_t)pairs * 8);
+    F.L = F.gB + al((size_t)entries * 4);
+    F.Z = F.L + al((size_t)entries * 4);
+    F.G = F.Z + al((size_t)entries * 4);
+    F.vmax = F.G + al((size_t)words * 4);
+    F.total = F.vmax + al((size_t)rows * 4);
+    return F;
 }
+inline FilterTab filter_tab(char* p, const FilterLayout& F) {
+    return FilterTab{(uint2*)(p + F.S), (float*)(p + F.gB), (float*)(p + F.L),
+                     (unsigned*)(p + F.Z), (uint2*)(p + F.Q), (unsigned*)(p + F.G),
+                     (unsigned*)(p + F.vmax)};
+}
+
+struct FoldCand {
+    long long item;        // output index (curve * n_P + period); -1: none
+    unsigned j;            // phase
+    int d;                 // duration
+    double lnp, Dl, s2;    // written by k_cand_eval
+};
+struct SlotBest {          // slot path: the best cell of an item
+    float lnp, Dl, s2;
+    unsigned j;
+    int d;                 // -1: none, -2: invalid period
+};
 
 struct PeriodConst;
 size_t period_const_bytes();
@@ -89,22 +131,34 @@ struct FoldScratch {
     void* nodes;            // exact-path records (exact_layout of all samples)
     int* bucket;            // bucket tables
     Node4<float>* rec;      // mixed slot records
-    float* lgm;             // gain tables (grouped): each curve's part for its own path
     ScreenRec* srec;        // FP64 slot-indexed screening records
     int* slot_of;           // FP64: slot of every sample
     unsigned* reg;          // two words per curve (zeroed by the prep)
     unsigned long long* peak;  // per curve, the key of its largest gain
     PeriodConst* ptab;      // per period, its curve-independent constants
+    FilterTab tab;
+    FoldCand* cand;         // cells left for k_cand_eval (cap entries)
+    unsigned long long cap;
+    unsigned long long* n_cand;
+    unsigned* list;         // list of the block items and its counters (n_cand behind)
+    unsigned* n_list;
+    int2* range;            // per item: its candidates
+    struct ItemConst* items;   // per item: constants of the screen
+    SlotBest* sbest;        // per item of the slot path
 };
 
 // Host side of the batch fold: per-curve layout and launches.
 struct FoldBatch {
     std::vector<FoldSeg> segs;
     int64_t n_bucket_total = 0, n_rec_total = 0, n_srec_total = 0;
-    int64_t n_gain_total = 0;    // entries of the grouped gain tables (either path)
+    int64_t n_tab_total = 0;     // entries of the filter tables
+    int64_t n_pair_total = 0;    // of those with durations in pairs
+    int64_t n_g_total = 0;       // words of their G tables
     bool any_slots = false, any_exact = false;
-    bool slot_cascade = false;   // some curve's grid is large enough for the mixed cascade
 };
+// Bytes of the batch fold's scratch; with a base, *fs receives its pointers.
+size_t fold_scratch(const FoldBatch& fb, int64_t n_total, int n_lc, int n_D, int64_t n_P,
+                    bool fp64, char* base, FoldScratch* fs);
 
 void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double>& t_first,
                      const std::vector<double>& t_last, const std::vector<int>& irregular,
@@ -119,12 +173,18 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
                              const void* gain, int n_D, double dt, double gap_factor,
                              const FoldScratch& fs, cudaStream_t st, int* n_launched);
 
+// Shapes of the batch fold the autotuner tries: warps per (curve, period) item,
+// + 4: items of long cells take a block of eight.
+constexpr int FOLD_SHAPES[5] = {1, 2, 1 + 4, 2 + 4, 8};
+// Enqueues the fold of the first n_seg curves (warps: one of FOLD_SHAPES); side:
+// a stream of the caller's for the block items; returns the number of kernels launched, and the first error of an enqueued memset
+// in *err.
 int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       int64_t n_total, bool fp64, const double* t, const FoldScratch& fs,
                       int n_D, double dt, double gap_factor, const double* periods,
-                      int64_t n_P, unsigned long long* counter, int grid, int threads,
-                      double* Q, double* T0, int* Didx, double* dep, double* sig, double* lnp,
-                      cudaStream_t st);
+                      int64_t n_P, int warps, double* Q, double* T0, int* Didx, double* dep,
+                      double* sig, double* lnp, cudaStream_t st, cudaStream_t side,
+                      cudaError_t* err);
 
 int launch_slots_test(const double* t, const int64_t* s_off_dev, int n_seg, int64_t n_total,
                       double dt, int* irregular, cudaStream_t st);

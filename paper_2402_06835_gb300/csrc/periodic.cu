@@ -22,6 +22,8 @@
 #include <string>
 #include <vector>
 
+#include "factor_core.cuh"
+#include "filter.cuh"
 #include "fold.cuh"
 #include "nu_internal.cuh"
 
@@ -165,21 +167,30 @@ __global__ void k_fill_nan(Node4<float>* rec, int64_t n) {
     rec[i] = Node4<float>{NAN, NAN, NAN, 0.f};
 }
 
+// Compensated FP32 and plain FP64 sums.  The products that enter the sums are
+// written as the fused operations they are (add_prod, fma), so that every
+// kernel that evaluates a cell rounds alike.
 template <typename T> struct KSum {
     T s, c;
     __device__ __forceinline__ void init() { s = T(0); c = T(0); }
-    __device__ __forceinline__ void add(T x) {
-        const T y = x - c;
-        const T t = s + y;
-        c = (t - s) - y;
+    __device__ __forceinline__ void add_y(T y) {
+        const T t = __fadd_rn(s, y);
+        c = __fsub_rn(__fsub_rn(t, s), y);
         s = t;
     }
+    __device__ __forceinline__ void add(T x) { add_y(__fsub_rn(x, c)); }
+    __device__ __forceinline__ void add_prod(T a, T b) { add_y(__fmaf_rn(a, b, -c)); }
 };
 template <> struct KSum<double> {
     double s;
     __device__ __forceinline__ void init() { s = 0.0; }
-    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add(double x) { s = __dadd_rn(s, x); }
+    __device__ __forceinline__ void add_prod(double a, double b) { s = __fma_rn(a, b, s); }
 };
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
 struct Best {
     double lnp;
@@ -251,20 +262,6 @@ __device__ __forceinline__ bool cannot_win(double s_l, double s_inv, double s_d,
     return ub + 1e-6 * fmax(1.0, fabs(ub)) < best;
 }
 
-// FP32 form for the mixed kernel, with the tighter depth term
-// q / (2 (1 + x_max)), x_max = max_k sigma^2/s_k^2 = ivmax / S_inv <= 1
-// (sigma^2 + s_k^2 = s_k^2 (1 + x_k) <= s_k^2 (1 + x_max)).
-// The reciprocals are the hardware approximation (2^-21 relative, far inside
-// the margins).
-__device__ __forceinline__ bool cannot_win_f(float s_l, float s_inv, float s_d, float s_dd,
-                                             float ivmax, float best) {
-    const float r = rcp32(s_inv);
-    const float q = fmaxf(0.0f, s_dd - s_d * s_d * r - 1e-4f * s_dd);
-    const float x = fminf(1.0f, ivmax * r * 1.001f);
-    const float ub = s_l + 0.5f - 0.5f * q * rcp32(1.0f + x) * 0.9999f;
-    return ub + 1e-4f * fmaxf(1.0f, fabsf(ub)) < best;
-}
-
 __device__ __forceinline__ bool bad_period(double P, const FoldGeom& g) {
     // a period must be finite, > 0 and give at most 1e9 epochs and phases
     return !(P > 0.0) || !isfinite(P) || g.t_last - g.t_ref > 1.0e9 * P ||
@@ -312,18 +309,17 @@ template <typename T> __device__ __forceinline__ T rcp_t(T x);
 template <> __device__ __forceinline__ double rcp_t<double>(double x) { return rcp64(x); }
 template <> __device__ __forceinline__ float rcp_t<float>(float x) { return rcp32(x); }
 
-// One single event at epoch Tk: interpolated depth, variance and gain.
+// One single event at epoch Tk: interpolated depth, sigma and gain.
 template <typename T>
 __device__ __forceinline__ bool event_exact(const FoldGeom& g, const Node8<T>* __restrict__ nd,
-                                            double Tk, int64_t& i, T& dk, T& sk2, T& lk) {
+                                            double Tk, int64_t& i, T& dk, T& s, T& lk) {
     i = bracket_from(g, okey(Tk), i);
     const Node8<T> a = nd[i];
     const T w = (T)((Tk - g.t0s[i]) * (double)a.ig);   // NaN across a gap / at the end
-    const T s = fma(w, a.ds, a.s);
+    s = fma(w, a.ds, a.s);
     if (sizeof(T) == 8 ? nan64((double)s) : isnan(s)) return false;
     dk = fma(w, a.dd, a.d);
     lk = fma(w, a.dl, a.l);
-    sk2 = s * s;
     return true;
 }
 
@@ -359,9 +355,9 @@ struct ExactAcc {
         s_dd = T(0);
         K = 0;
     }
-    __device__ __forceinline__ void add(T dk, T sk2, T lk) {
-        const T iv = rcp_t<T>(sk2);
-        const T div = dk * iv;
+    __device__ __forceinline__ void add(T dk, T s, T lk) {
+        const T iv = rcp_t<T>(mul_rn(s, s));
+        const T div = mul_rn(dk, iv);
         s_inv.add(iv);
         s_d.add(div);
         s_dd = fma(div, dk, s_dd);
@@ -393,25 +389,28 @@ struct ExactPen {
         s2 = s2_;
         Dl = Dl_;
     }
-    __device__ __forceinline__ void add(T dk, T sk2) {
-        const T den = sk2 + s2;
-        const T iden = rcp_t<T>(den);
+    __device__ __forceinline__ void add(T dk, T s) {
+        const T sk2 = mul_rn(s, s);
+        const T iden = rcp_t<T>(add_rn(sk2, s2));
         const T r = dk - Dl;
-        quad.add(r * r * iden);
+        quad.add_prod(mul_rn(r, r), iden);
         if (sizeof(T) == 8) {
-            prod *= (double)(sk2 * iden);
+            prod *= (double)mul_rn(sk2, iden);
             if ((++cnt & 255) == 0) {
                 const int e = ((__double2hiint(prod) >> 20) & 0x7ff) - 1023;
                 prod = __hiloint2double(__double2hiint(prod) - (e << 20), __double2loint(prod));
                 expo += e;
             }
         } else {
-            lsum += lg2_32((float)(sk2 * iden));
+            lsum += lg2_32((float)mul_rn(sk2, iden));
         }
     }
-    __device__ __forceinline__ double logsum() const {
-        if (sizeof(T) == 8) return log(prod) + (double)expo * 0.69314718055994530942;
-        return (double)lsum * 0.69314718055994530942;
+    // both sums of the penalty
+    __device__ __forceinline__ double total() const {
+        if (sizeof(T) == 8)
+            return __dadd_rn(fma((double)expo, 0.69314718055994530942, log(prod)),
+                             (double)quad.s);
+        return fma((double)lsum, 0.69314718055994530942, (double)quad.s);
     }
 };
 
@@ -473,7 +472,6 @@ struct PeriodConst {
     int64_t n_phi;
     double R;                          // P / dt
     unsigned long long ustep, uph;     // screen steps (0 when R 2^40 >= 4e18)
-    float inv_ustep32;
     float c_inv_ustep32;
     SlotWalk swp, swk;
     double nphi_d, rphi;
@@ -488,10 +486,8 @@ __device__ __forceinline__ PeriodConst period_const(double P, double dt, double 
     if (pc.R * SCALE < 4.0e18) {
         pc.ustep = (unsigned long long)llrint(pc.R * SCALE);
         pc.uph = (unsigned long long)llrint(pc.R / (double)pc.n_phi * SCALE);
-        pc.inv_ustep32 = (float)(4294967296.0 / (double)pc.ustep);
     } else {
         pc.ustep = pc.uph = 0;
-        pc.inv_ustep32 = 0.f;
     }
     pc.swp = slot_walk(1.0 / (double)pc.n_phi, pc.R);
     pc.swk = slot_walk(0.0, pc.R);
@@ -501,15 +497,20 @@ __device__ __forceinline__ PeriodConst period_const(double P, double dt, double 
     return pc;
 }
 
-// cell_ctx from a table entry (the same values).
-__device__ __forceinline__ CellCtx cell_ctx(const FoldGeom& g, double P, const PeriodConst& pc) {
+// The position of a curve's last epoch for the exact paths' epoch counts.
+static inline unsigned long long exact_uspan(double t_ref, double t_last, double dt) {
+    const double u = (t_last - t_ref) * (1.0 / dt) * 1099511627776.0;
+    return u < 4.0e18 ? (unsigned long long)llrint(u) : 4000000000000000000ull;
+}
+// cell_ctx from a table entry and the curve's last position (the same values,
+// no FP64 arithmetic).
+__device__ __forceinline__ CellCtx cell_ctx(const FoldGeom& g, double P, const PeriodConst& pc,
+                                            unsigned long long uspan) {
     CellCtx c;
     c.P = P;
     c.swp = pc.swp;
     c.swk = pc.swk;
-    const double SCALE = 1099511627776.0;   // 2^40
-    const double ulast_d = (g.t_last - g.t_ref) * g.inv_dt * SCALE;
-    c.ulast = ulast_d < 4.0e18 ? (unsigned long long)llrint(ulast_d) : 4000000000000000000ull;
+    c.ulast = uspan;
     c.inv_ustep32 = pc.c_inv_ustep32;
     c.klast = okey(g.t_last);
     c.nphi_d = pc.nphi_d;
@@ -525,7 +526,7 @@ __global__ void k_period_consts(const double* __restrict__ periods, int64_t n_P,
     if (i >= n_P) return;
     const double P = periods[i];
     if (!(P > 0.0) || !isfinite(P) || P / dt > 1.0e9) {
-        out[i] = PeriodConst{1, 0.0, 0, 0, 0.f, 0.f, {0, 0}, {0, 0}, 1.0, 1.0};
+        out[i] = PeriodConst{1, 0.0, 0, 0, 0.f, {0, 0}, {0, 0}, 1.0, 1.0};
         return;
     }
     out[i] = period_const(P, dt, 1.0 / dt);
@@ -603,9 +604,9 @@ __device__ __forceinline__ void cell_pass1(const FoldGeom& g, const Node8<T>* __
     const double kds = (double)ks;
     for (int64_t k = k0; k < kmax; k += ks, u += us, kd += kds) {
         const double Tk = epoch_time(g, c, phi, kd);
-        T dk, sk2, lk;
+        T dk, sk, lk;
         int64_t i = guess_at(g, u);
-        if (event_exact<T>(g, nd, Tk, i, dk, sk2, lk)) a1.add(dk, sk2, lk);
+        if (event_exact<T>(g, nd, Tk, i, dk, sk, lk)) a1.add(dk, sk, lk);
     }
 }
 template <typename T>
@@ -618,9 +619,9 @@ __device__ __forceinline__ void cell_pass2(const FoldGeom& g, const Node8<T>* __
     const double kds = (double)ks;
     for (int64_t k = k0; k < kmax; k += ks, u += us, kd += kds) {
         const double Tk = epoch_time(g, c, phi, kd);
-        T dk, sk2, lk;
+        T dk, sk, lk;
         int64_t i = guess_at(g, u);
-        if (event_exact<T>(g, nd, Tk, i, dk, sk2, lk)) a2.add(dk, sk2);
+        if (event_exact<T>(g, nd, Tk, i, dk, sk, lk)) a2.add(dk, sk);
     }
 }
 
@@ -690,7 +691,7 @@ __device__ __forceinline__ void fold_exact_one(const FoldGeom& g, const Node8<T>
             ExactPen<T> a2;
             a2.init(qc.s2, qc.Dl);
             cell_pass2<T>(g, nd, c, qc.phi, qc.u0, qc.kmax, 0, 1, a2);
-            const double lnp = qc.s_l - 0.5 * (a2.logsum() + (double)a2.quad.s);
+            const double lnp = qc.s_l - 0.5 * a2.total();
             if (!(lnp == lnp)) continue;   // NaN never selected
             if (lnp > bl || (lnp == bl && qc.cell < bc)) {
                 bl = lnp;
@@ -718,7 +719,8 @@ __device__ __forceinline__ void fold_exact_one(const FoldGeom& g, const Node8<T>
 // ascending order, 13.8 ms descending).  Any order gives the same results.
 __device__ __forceinline__ int64_t period_slot(int64_t b, const double* __restrict__ periods,
                                               int64_t n_P) {
-    return periods[n_P - 1] < periods[0] ? n_P - 1 - b : b;
+    // (by integer keys: a NaN only changes the order)
+    return okey(periods[n_P - 1]) < okey(periods[0]) ? n_P - 1 - b : b;
 }
 
 template <typename T, int KC>
@@ -786,9 +788,6 @@ struct ScreenGeom {
     const unsigned* reg;               // [0]: an epoch is off the slot grid,
                                        // [1]: max |offset from its slot| (float bits)
     int on;                            // screening allowed for this curve
-    const unsigned long long* peak;    // key of the largest finite gain (k_gain_peak);
-                                       // 0: none
-    const float* lm3;                  // grouped gain table (k_gain_table); nullptr: none
     int f32;                           // the exact events are FP32 (mixed precision)
 };
 
@@ -825,9 +824,7 @@ __global__ void k_slot_offsets(const double* __restrict__ t0s, int64_t n_t0, dou
 
 // Screening record of epoch i of a curve with n epochs (gid indexes the
 // (duration, epoch) arrays; d is the duration), also placed at the epoch's
-// slot, and for the first duration row the pair of epoch positions.  The
-// interval's largest gain goes to the pad of the epoch's node record (for
-// k_gain_table; k_nodes has run).
+// slot, and for the first duration row the pair of epoch positions.
 template <typename T>
 __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
                                             const T* __restrict__ var,
@@ -836,8 +833,7 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
                                             int64_t i, int64_t n, int64_t d, double gap_max,
                                             double dt, ScreenRec* __restrict__ out,
                                             ScreenRec* __restrict__ sout,
-                                            Node8<T>* __restrict__ nodes, int64_t n_slots,
-                                            const int* __restrict__ slot_of,
+                                            int64_t n_slots, const int* __restrict__ slot_of,
                                             ulonglong2* __restrict__ vpair) {
     // an interval needs both ends valid and a gap in (0, gap_max]
     bool v0 = i + 1 < n;
@@ -848,7 +844,6 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
     }
     ScreenRec r;
     unsigned flags = 0u;
-    float lmax = 0.f;      // largest gain an event on the interval can take
     const double d0 = (double)depth[gid], l0 = (double)gain[gid];
     r.d = (float)d0;
     r.l = (float)l0;
@@ -875,13 +870,6 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
             r.s = INFINITY;
             r.ds = 0.f;
         }
-        // the exact event's gain fma(w, l1 - l0, l0) with w in [0, 1] (to a few
-        // units of its own rounding) is at most max(l0, l1) + 2^-50 (|l0| + |l1|)
-        // in FP64, 2^-20 (|l0| + |l1|) in FP32; rounded up, and +inf when the
-        // interval is not screened
-        const double slack = sizeof(T) == 8 ? 8.881784197001252e-16 : 9.5367431640625e-07;
-        lmax = odd ? INFINITY
-                   : __double2float_ru(fmax(0.0, fmax(l0, l1)) + slack * (fabs(l0) + fabs(l1)));
     } else {
         r.s = NAN;
         r.dd = 0.f;
@@ -891,7 +879,6 @@ __device__ __forceinline__ void make_screen(const T* __restrict__ depth,
     }
     r.flags = flags;
     out[gid] = r;
-    nodes[gid].pad = (T)lmax;
     if (sout) {
         const int sl = slot_of[i];
         if (sl >= 0 && sl < n_slots) sout[d * n_slots + sl] = r;
@@ -917,102 +904,23 @@ __global__ void k_screen(const T* __restrict__ depth, const T* __restrict__ var,
                          const T* __restrict__ gain, const double* __restrict__ t0s,
                          int64_t n_t0, int n_D, double gap_max, double dt,
                          ScreenRec* __restrict__ rec, ScreenRec* __restrict__ srec,
-                         Node8<T>* __restrict__ nodes, int64_t n_slots,
-                         const int* __restrict__ slot_of, ulonglong2* __restrict__ vpair) {
+                         int64_t n_slots, const int* __restrict__ slot_of,
+                         ulonglong2* __restrict__ vpair) {
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (gid >= n_t0 * (int64_t)n_D) return;
     const int64_t d = gid / n_t0, i = gid - d * n_t0;
-    make_screen<T>(depth, var, gain, t0s, gid, i, n_t0, d, gap_max, dt, rec, srec, nodes,
-                   n_slots, slot_of, vpair);
-}
-
-// Entry o of a grouped gain table: the curve (segs: the batch's, else one
-// curve of n_slots1 slots), the duration d and slot s.  Per curve the table
-// holds [groups][n_slots][W] entries from gain_off on; the slot path's source
-// rows are duration-major rows of n_slots from rec_off.  Returns false for
-// entries of no curve of the path (screened, or else the slot path).
-struct GainSlot {
-    int64_t src_off, n_slots;
-    int d, s, seg;
-};
-__device__ __forceinline__ bool gain_slot(const FoldSeg* __restrict__ segs, int n_seg,
-                                          int64_t n_slots1, int n_D, bool screened, int64_t o,
-                                          GainSlot& gs) {
-    int64_t out_off = 0;
-    gs.seg = 0;
-    gs.src_off = 0;
-    gs.n_slots = n_slots1;
-    if (segs) {
-        // the last curve whose table starts at or before o (curves without a
-        // table take no entries and share their successor's offset)
-        int lo = 0, hi = n_seg;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (segs[mid].gain_off <= o) lo = mid; else hi = mid;
-        }
-        const FoldSeg& f = segs[lo];
-        if (!(screened ? f.screen : f.use_slots)) return false;
-        out_off = f.gain_off;
-        gs.seg = lo;
-        gs.src_off = f.rec_off;
-        gs.n_slots = f.n_slots;
-    }
-    const int W = gain_width(n_D);
-    const int64_t local = o - out_off;
-    if (local < 0 || local >= gs.n_slots * gain_cols(n_D)) return false;
-    const int64_t g = local / (gs.n_slots * W);
-    const int64_t rem = local - g * gs.n_slots * W;
-    gs.s = (int)(rem / W);
-    gs.d = (int)(g * W + (rem - (int64_t)gs.s * W));
-    return true;
-}
-
-// Grouped gain table of the screen: per slot s the largest gain (the pad of the
-// node record) of the intervals that meet the positions [s - 1/4, s + 5/4), i.e. the largest gain
-// of an event whose walk position lies in slot s (the walk is within 1/4 slot
-// of the exact epoch, see the gain bound).  On a regular grid (epochs within
-// 2^-10 slot of their slots) these are the intervals that start at slots
-// s - 1, s and s + 1.  The bucket table gives the epoch at the slot; the range
-// is found from it by steps over the stored positions.
-template <typename T>
-__global__ void k_gain_table(const Node8<T>* __restrict__ nodes,
-                             const ulonglong2* __restrict__ vpair,
-                             const int* __restrict__ bucket, const FoldSeg* __restrict__ segs,
-                             int n_seg, int64_t n_t01, int64_t n_slots1, int64_t n_bucket1,
-                             int n_D, int64_t n_out, float* __restrict__ lm3) {
-    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (o >= n_out) return;
-    GainSlot gs;
-    if (!gain_slot(segs, n_seg, n_slots1, n_D, true, o, gs)) return;
-    float m = 0.f;
-    if (gs.d < n_D) {
-        const int64_t n_t0 = segs ? segs[gs.seg].n_t0 : n_t01;
-        const int64_t nb = segs ? segs[gs.seg].n_bucket : n_bucket1;
-        const int* bk = bucket + (segs ? segs[gs.seg].bucket_off : 0);
-        const ulonglong2* vp = vpair + (segs ? segs[gs.seg].s_off : 0);
-        const Node8<T>* row =
-            nodes + (segs ? segs[gs.seg].s_off * n_D : 0) + (int64_t)gs.d * n_t0;
-        const unsigned long long Q = 1ull << 38;                // 1/4 slot
-        const unsigned long long at = (unsigned long long)gs.s << 40;
-        const unsigned long long lo = at > Q ? at - Q : 0, hi = at + 5ull * Q;
-        int64_t i = (int64_t)bk[gs.s < nb ? gs.s : nb - 1] - 1;  // the epoch at or before slot s
-        if (i < 0) i = 0;
-        while (i > 0 && vp[i].x > lo) --i;
-        while (i + 1 < n_t0 && vp[i + 1].x <= lo) ++i;           // last epoch at or before lo
-        for (; i < n_t0 && (vp[i].x < hi); ++i) m = fmaxf(m, (float)row[i].pad);
-    }
-    lm3[o] = m;
+    make_screen<T>(depth, var, gain, t0s, gid, i, n_t0, d, gap_max, dt, rec, srec, n_slots,
+                   slot_of, vpair);
 }
 
 // Per-period constants of the screen.
 struct ScreenPeriod {
-    unsigned long long uph, ustep, ulast, delta;
-    unsigned long long uend;   // epochs walk while u < uend = ulast + delta
-    float inv_ustep32;
+    unsigned long long uph, ustep, delta;
+    unsigned long long uend;   // epochs walk while u < uend = (last epoch) + delta
     float wscale;   // 2^22 / dt (FP32): weight of an event in the band of an epoch
     float cv;       // error coefficient of an FP32 event value
-    float dw;       // half-width of the band around an epoch, as an interval weight
-    float hw;       // 1/2 - dw: an event is in a band when |w - 1/2| > hw
+    float hw;       // 1/2 - dw, dw the half-width of the band around an epoch as
+                    // an interval weight: an event is in a band when |w - 1/2| > hw
     bool on;
     bool slots;     // regular grid: events from the slot records
 };
@@ -1024,7 +932,7 @@ __device__ __forceinline__ ScreenPeriod screen_period_curve(const FoldGeom& g,
                                                             int64_t n_phi, double R,
                                                             double span, ScreenPeriod sp) {
     const double SCALE = 1099511627776.0;   // 2^40
-    sp.ulast = sg.vpair[g.n_t0 - 1].x;
+    const unsigned long long ulast = sg.vpair[g.n_t0 - 1].x;
     // position error of the walk against the FP64 epochs, in 2^-40 slots:
     // half a unit per phase and epoch step, the rounding of T, t0 and vpos
     const double kb = span / R + 2.0;
@@ -1034,7 +942,7 @@ __device__ __forceinline__ ScreenPeriod screen_period_curve(const FoldGeom& g,
     const double delta = 16.0 * e_pos + 1048576.0;          // + 2^-20 slot
     sp.on = delta < 1.6e10;                                  // below 2^-6 slot
     sp.delta = (unsigned long long)delta;
-    sp.uend = sp.ulast + sp.delta;
+    sp.uend = ulast + sp.delta;
     // regular grid: every epoch within 2^-10 slot of its own slot.  The error
     // terms below grow with the largest offset; a phase step taken as the
     // median spacing of FP64 times carries a relative rounding of about
@@ -1043,14 +951,15 @@ __device__ __forceinline__ ScreenPeriod screen_period_curve(const FoldGeom& g,
     const float off = sg.srec ? __uint_as_float(sg.reg[1]) : 1.f;
     sp.slots = sg.srec && sg.reg[0] == 0u && off <= 9.765625e-04f;
     double e_w;
+    float dw;
     if (sp.slots) {
         // the weight is the fraction of the slot: position error, the
         // epochs' offsets (3 x, both ends), 24-bit truncation
-        sp.dw = (float)(1.01 * (delta / SCALE + (double)off) + 2.4e-7);
+        dw = (float)(1.01 * (delta / SCALE + (double)off) + 2.4e-7);
         e_w = e_pos / SCALE + 3.0 * (double)off + 1.1920928955078125e-07;
     } else {
         // dt/gap <= 4 on a screened interval; 2^-22-slot truncation
-        sp.dw = (float)(4.04 * delta / SCALE + 2.0e-6);
+        dw = (float)(4.04 * delta / SCALE + 2.0e-6);
         e_w = 4.0 * e_pos / SCALE + 9.5367431640625e-07;
     }
     // (the weight of an event in the band of an epoch, computed in FP32 by
@@ -1066,33 +975,11 @@ __device__ __forceinline__ ScreenPeriod screen_period_curve(const FoldGeom& g,
     // mixed precision: the exact event itself is computed in FP32 (node
     // differences, weight and FMA: a few units of |x_i| + |x_{i+1}|)
     if (sg.f32) sp.cv += 8.0f * 5.9604645e-08f;
-    sp.hw = 0.5f - sp.dw;
+    sp.hw = 0.5f - dw;
     sp.wscale = (float)(4194304.0 * g.inv_dt);
     return sp;
 }
 
-__device__ __forceinline__ ScreenPeriod screen_period(const FoldGeom& g, const ScreenGeom& sg,
-                                                      double P, int64_t n_phi) {
-    ScreenPeriod sp;
-    const double SCALE = 1099511627776.0;   // 2^40
-    const double R = P * g.inv_dt;
-    const double span = (g.t_last - g.t_ref) * g.inv_dt;
-    sp.on = sg.on != 0 && R * SCALE < 4.0e18 && span < 8388608.0;
-    sp.slots = false;
-    sp.uph = sp.ustep = sp.ulast = sp.delta = sp.uend = 0;
-    sp.inv_ustep32 = 0.f;
-    sp.wscale = 0.f;
-    sp.cv = 0.f;
-    sp.dw = 0.f;
-    sp.hw = 0.5f;
-    if (!sp.on) return sp;
-    sp.ustep = (unsigned long long)llrint(R * SCALE);
-    sp.uph = (unsigned long long)llrint(R / (double)n_phi * SCALE);
-    sp.inv_ustep32 = (float)(4294967296.0 / (double)sp.ustep);
-    return screen_period_curve(g, sg, P, n_phi, R, span, sp);
-}
-
-// screen_period from a table entry (the same values).
 __device__ __forceinline__ ScreenPeriod screen_period(const FoldGeom& g, const ScreenGeom& sg,
                                                       double P, const PeriodConst& pc) {
     ScreenPeriod sp;
@@ -1101,16 +988,13 @@ __device__ __forceinline__ ScreenPeriod screen_period(const FoldGeom& g, const S
     const double span = (g.t_last - g.t_ref) * g.inv_dt;
     sp.on = sg.on != 0 && R * SCALE < 4.0e18 && span < 8388608.0;
     sp.slots = false;
-    sp.uph = sp.ustep = sp.ulast = sp.delta = sp.uend = 0;
-    sp.inv_ustep32 = 0.f;
+    sp.uph = sp.ustep = sp.delta = sp.uend = 0;
     sp.wscale = 0.f;
     sp.cv = 0.f;
-    sp.dw = 0.f;
     sp.hw = 0.5f;
     if (!sp.on) return sp;
     sp.ustep = pc.ustep;
     sp.uph = pc.uph;
-    sp.inv_ustep32 = pc.inv_ustep32;
     return screen_period_curve(g, sg, P, pc.n_phi, R, span, sp);
 }
 
@@ -1118,10 +1002,11 @@ __device__ __forceinline__ ScreenPeriod screen_period(const FoldGeom& g, const S
 // Integer-to-float conversions run on the FP64 pipe of this GPU, so the
 // screen counts events in a float and builds weights from bit patterns.
 struct ScreenAcc {
-    float sinv, sd, sdd, sdd2, sl, sabs, ivmax;
+    float sinv, sd, sdd, sdd2, sl, sabs, ivmax, ivmin;
     float K;                 // number of events (exact in FP32 below 2^24)
     __device__ __forceinline__ void init() {
         sinv = sd = sdd = sdd2 = sl = sabs = ivmax = 0.f;
+        ivmin = INFINITY;
         K = 0.f;
     }
     // event (depth dk, sigma s, gain lk) on an interval with depth and gain
@@ -1137,13 +1022,17 @@ struct ScreenAcc {
         sdd2 = fmaf(dd * dd, iv, sdd2);
         sabs += fmaf(2.f, fabsf(lk), fabsf(dl));
         ivmax = fmaxf(ivmax, iv);
+        ivmin = fminf(ivmin, iv);
         K += 1.f;
     }
     // Hardware reciprocal / reciprocal square root (relative error below
     // 2^-21, counted as 8u per use) with every term rounded the safe way.
     // The q term only lowers the bound, so the cheaper S_L + 1/2 + margins
     // is returned when it already falls below the threshold bf.
-    __device__ __forceinline__ float bound(float cv, float bf) const {
+    // *lb receives a lower bound on the cell's ln P (-inf when not computed):
+    // the log terms are at least ln(1 + x_max) / (2 x_max) (ln(1 + x) is
+    // concave and the x_k sum to 1), the depth terms at most q / (2 (1 + x_min)).
+    __device__ __forceinline__ float bound(float cv, float bf, float* lb) const {
         if (K == 0.f) return -INFINITY;
         const float U = 5.9604645e-8f;                        // 2^-24
         const float sk = (K + 2.f) * U;
@@ -1164,6 +1053,19 @@ struct ScreenAcc {
             if (a > e) q_lo = (a - e) * (a - e) * (1.f - 8.f * U);
         }
         const float x_hi = fminf(1.f, ivmax * r * (1.f + 4.f * gam + 2.f * sk + 24.f * U));
+        {
+            const float qch = fmaxf(qc + fmaf(4.f, K, 32.f) * U * sdd, 0.f);
+            const float x1 = qch * (1.f + 4.f * gam + 2.f * sk + 16.f * U);
+            const float y = fmaf(8.f, sdd, 2.f * sdd2) * (1.f + 2.f * gam + sk) * (1.f + 8.f * U);
+            const float a = x1 > 0.f ? x1 * rsqrt32(x1) * (1.f + 16.f * U) : 0.f;
+            const float e = y > 0.f ? 1.05f * cv * (y * rsqrt32(y)) * (1.f + 16.f * U) : 0.f;
+            const float q_hi = (a + e) * (a + e) * (1.f + 8.f * U);
+            const float x_lo = ivmin * r * (1.f - 4.f * gam - 2.f * sk - 24.f * U);
+            const float lg = 0.69314718f * lg2_32(1.f + x_hi) * rcp32(x_hi);
+            const float l = sl - e_l + 0.5f * lg - 0.5f * q_hi * rcp32(1.f + x_lo) -
+                            (sabs + q_hi + 1.f) * 4e-6f;
+            *lb = l == l ? l : -INFINITY;
+        }
         return sl + e_l + 0.5f - 0.5f * q_lo * rcp32(1.f + x_hi) * (1.f - 16.f * U) +
                8.f * U * (sabs + q_lo + 1.f);
     }
@@ -1198,12 +1100,14 @@ __device__ __forceinline__ int screen_exact_event(const FoldGeom& g,
 // Upper bound on ln P of cell (j, duration rows rd / rs) whose first
 // epoch is at u0 (see above): -inf when the cell has no event, +inf when an
 // event falls on an interval outside the screen's error model; any value
-// below bf when the cell is already known not to reach bf.
+// below bf when the cell is already known not to reach bf.  *lb: see
+// ScreenAcc::bound (left as it is when the cell is not bounded).
 __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom& sg,
                                              const ScreenRec* __restrict__ rd,
                                              const ScreenRec* __restrict__ rs,
                                              const ScreenPeriod& sp, const CellCtx& c,
-                                             int64_t j, unsigned long long u0, float bf) {
+                                             int64_t j, unsigned long long u0, float bf,
+                                             float* lb) {
     // epochs up to u < ulast + delta: those within delta of t_last (the last
     // epoch's position) fall in the band around it and take the exact event,
     // which drops T > t_last
@@ -1266,7 +1170,7 @@ __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom
             if (!visit(rb)) return INFINITY;
             u += sp.ustep;
         }
-        return acc.bound(sp.cv, bf);
+        return acc.bound(sp.cv, bf, lb);
     }
     const int64_t nb1 = g.n_bucket - 1;
     int bnext = g.bucket[min((int64_t)(u >> 40), nb1)];
@@ -1301,215 +1205,207 @@ __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom
         }
         acc.add(fmaf(w, r.dd, r.d), s, fmaf(w, r.dl, r.l), r.dd, r.dl);
     }
-    return acc.bound(sp.cv, bf);
+    return acc.bound(sp.cv, bf, lb);
 }
 
-// The gain bound of a cell, from 4 bytes per epoch.  By the bound above,
-// ln P <= S_L + 1/2, and every event's gain is at most the larger gain of its
-// interval's two nodes.  The walk's position u of epoch k lies within 1/4 slot
-// of the exact epoch (0.2 slot by the test below, plus the walk's own error,
-// below 2^-6), so the exact interval meets [floor(u) - 1/4, floor(u) + 5/4):
-// lm3 at floor(u) bounds the event's gain (0 for a dropped epoch, +inf on an
-// interval outside the screen's error model).  Extra walk positions past t_last (u < uend)
-// only add terms >= 0.  The FP32 sum of K terms >= 0 is rounded up by
-// (K + 16) 2^-23 of itself, and 1e-6 covers the exact path's own rounding.
+// ------------------------------------------------------- the cell kernels
+// Both paths fold one (curve, period) item by one warp, or by the eight warps
+// of a block where its cells are long: the filters (filter.cuh) over all cells, the FP32 screen (exact paths) or the first pass
+// (slot path) of the cells they leave, then the evaluation of the few cells
+// whose bound reaches the threshold.  The threshold is a lower bound of the
+// best ln P: every screened cell gives a lower bound beside its upper bound,
+// so no cell has to be evaluated to raise it.
 //
-// The walk runs in 32-bit fixed point (few instructions per epoch):
-// positions in units of 2^-F slot, started from the 64-bit position of a
-// cell's first epoch (truncated) and advanced by the rounded step, so that
-// epoch k is at most 1 + k/2 units from the 64-bit walk.  F is chosen per
-// period so that no position the walk loads (up to end + 3 steps: four epochs
-// a round) exceeds 2^31 (the margin below allows twelve), and the walk is
-// used only when that error stays below 0.2 slot for every epoch.  The end is widened by the same error, so every epoch of the
-// 64-bit walk is counted; positions past it add terms >= 0 (the walk adds
-// four terms at a time; a position past the row is clamped to the padding
-// slot zs, whose term is 0).
-struct GainWalk32 {
-    unsigned step, end;
-    int shift;            // 40 - F
-    int F;
-    int ok;
+// The exact evaluation is FP64 (64 cycles per warp instruction, whatever the
+// number of active lanes), and an item leaves one to a few cells: evaluating
+// them in place kept the FP64 pipe at 33 % on a sector's fold and at 74 % on
+// short curves.  The cells that are left go to a list instead, which k_cand_eval
+// evaluates with 32 cells of many items per warp and k_cand_best reduces, one
+// thread per item.  An item that has more cells than its queues hold, or finds
+// the list full, evaluates in place.
+// What the screen needs of one (curve, period) item besides the period table:
+// FP64 arithmetic done by k_item_consts for 32 items per warp instruction.
+struct ItemConst {
+    unsigned long long uend, delta;   // ScreenPeriod
+    float cv, hw;
+    float K;                          // span / P
+    int flags;                        // 1: bad period, 2: screened, 4: slot records,
+                                      // 8: cells of 32 or more epochs
 };
-__device__ __forceinline__ GainWalk32 gain_walk32(unsigned long long ustep,
-                                                  unsigned long long uend) {
-    GainWalk32 w{0u, 0u, 0, 0, 0};
-    const double S40 = 9.094947017729282e-13;               // 2^-40
-    const double R = (double)ustep * S40;                    // slots per period
-    if (!(R > 0.0)) return w;
-    const double span = (double)uend * S40;
-    const double kmax = span / R + 2.0;                      // epochs walked, at most
-    const double top = span + 12.0 * R + kmax + 8.0;         // slots a position can reach
-    int F = 30 - ilogb(top);                                 // 2^F top < 2^31
-    if (F > 24) F = 24;
-    if (F < 8 || (kmax + 2.0) * ldexp(1.0, -F) > 0.2) return w;
-    w.F = F;
-    w.shift = 40 - F;
-    w.step = (unsigned)((ustep + (1ull << (w.shift - 1))) >> w.shift);
-    w.end = (unsigned)((uend >> w.shift) + 2ull + (unsigned long long)(kmax + 2.0));
-    w.ok = w.step > 0u;
-    return w;
-}
 
-// The gain tables are grouped by duration (gain_width): the W cells of one
-// phase and W consecutive durations share their epochs, so a lane walks them
-// together with one W-wide load per epoch.  row points at the group's first
-// slot; the sums of the W columns go to s (the unused ones stay 0) and the
-// number of terms, the same for every column, is returned.
-template <int W>
-struct GainVec;
-template <>
-struct GainVec<1> {
-    typedef float T;
-    __device__ static __forceinline__ T zero() { return 0.f; }
-    __device__ static __forceinline__ void add(float4& s, T a, T b, T c, T e) {
-        s.x += (a + c) + (b + e);
-    }
+// The items whose cells have heavy_k or more epochs: a block's eight warps fold
+// each of them (their walks are long, and one warp would still be at it when
+// the rest of a small grid is done: the first period of the sector grid, 0.2 d,
+// ran 5.1 ms in one warp beside 2.6 ms for all others).  The others take one or
+// two warps each, blocks of neighbouring periods together: neighbouring periods
+// read the same table entries at nearly the same time, which the L1 serves
+// (warps that took their items one by one from a counter: 3.8 ms on the
+// sector's FP64 fold against 3.4 ms).
+struct FoldLists {
+    unsigned* block;       // item indices, appended by the preparation kernels
+    unsigned* n;           // [0] their number, [1] taken
+    float heavy_k;
 };
-template <>
-struct GainVec<2> {
-    typedef float2 T;
-    __device__ static __forceinline__ T zero() { return make_float2(0.f, 0.f); }
-    __device__ static __forceinline__ void add(float4& s, T a, T b, T c, T e) {
-        s.x += (a.x + c.x) + (b.x + e.x);
-        s.y += (a.y + c.y) + (b.y + e.y);
-    }
-};
-template <>
-struct GainVec<4> {
-    typedef float4 T;
-    __device__ static __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-    __device__ static __forceinline__ void add(float4& s, T a, T b, T c, T e) {
-        s.x += (a.x + c.x) + (b.x + e.x);
-        s.y += (a.y + c.y) + (b.y + e.y);
-        s.z += (a.z + c.z) + (b.z + e.z);
-        s.w += (a.w + c.w) + (b.w + e.w);
-    }
-};
-// (NU_GAIN_UNROLL4 epochs a round for 4-wide groups, four for the others)
-#ifndef NU_GAIN_UNROLL4
-#define NU_GAIN_UNROLL4 4
-#endif
-template <int W>
-__device__ __forceinline__ float gain_walk_w(const float* __restrict__ row, unsigned zs,
-                                             unsigned u, const GainWalk32& w, float4& s) {
-    typedef typename GainVec<W>::T V;
-    const V* __restrict__ r = reinterpret_cast<const V*>(row);
-    const unsigned st = w.step;
-    float K = 0.f;
-    if (W == 4 && NU_GAIN_UNROLL4 == 2) {
-        // two epochs a round, the second clamped past the end (a zero term)
-        for (; u < w.end; u += 2u * st) {
-            const V a = r[min(u >> w.F, zs)];
-            const V b = r[min((u + st) >> w.F, zs)];
-            const V z = GainVec<W>::zero();
-            GainVec<W>::add(s, a, b, z, z);
-            K += 2.f;
-        }
-        return K;
-    }
-    for (; u < w.end; u += 4u * st) {
-        const V a = r[min(u >> w.F, zs)];
-        const V b = r[min((u + st) >> w.F, zs)];
-        const V c = r[min((u + 2u * st) >> w.F, zs)];
-        const V e = r[min((u + 3u * st) >> w.F, zs)];
-        GainVec<W>::add(s, a, b, c, e);
-        K += 4.f;
-    }
-    return K;
-}
-__device__ __forceinline__ float gain_walk(const float* __restrict__ row, int W, unsigned zs,
-                                           unsigned u, const GainWalk32& w, float4& s) {
-    s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (W == 4) return gain_walk_w<4>(row, zs, u, w, s);
-    if (W == 2) return gain_walk_w<2>(row, zs, u, w, s);
-    return gain_walk_w<1>(row, zs, u, w, s);
-}
-// The same walk on the 64-bit positions (2^-40 slot) that define the mixed
-// fold's events: each epoch's slot is exactly its event's, so the table needs
-// no neighbours.  Positions past uend add terms >= 0 (clamped to zs);
-// ustep < 2^60 and u < 2^62 keep u + 3 ustep from wrapping.
-template <int W>
-__device__ __forceinline__ float gain_walk64_w(const float* __restrict__ row, unsigned zs,
-                                               unsigned long long u, unsigned long long ustep,
-                                               unsigned long long uend, float4& s) {
-    typedef typename GainVec<W>::T V;
-    const V* __restrict__ r = reinterpret_cast<const V*>(row);
-    float K = 0.f;
-    for (; u < uend; u += 4ull * ustep) {
-        const V a = r[min((unsigned)(u >> 40), zs)];
-        const V b = r[min((unsigned)((u + ustep) >> 40), zs)];
-        const V c = r[min((unsigned)((u + 2ull * ustep) >> 40), zs)];
-        const V e = r[min((unsigned)((u + 3ull * ustep) >> 40), zs)];
-        GainVec<W>::add(s, a, b, c, e);
-        K += 4.f;
-    }
-    return K;
-}
-__device__ __forceinline__ float gain_walk64(const float* __restrict__ row, int W, unsigned zs,
-                                             unsigned long long u, unsigned long long ustep,
-                                             unsigned long long uend, float4& s) {
-    s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (W == 4) return gain_walk64_w<4>(row, zs, u, ustep, uend, s);
-    if (W == 2) return gain_walk64_w<2>(row, zs, u, ustep, uend, s);
-    return gain_walk64_w<1>(row, zs, u, ustep, uend, s);
-}
-__device__ __forceinline__ float gain_col(const float4& s, int i) {
-    return i == 0 ? s.x : (i == 1 ? s.y : (i == 2 ? s.z : s.w));
-}
-
-// The mixed fold's cascade runs on periods with at least NU_CASCADE_ROUNDS
-// rounds of cells per warp.
-#ifndef NU_CASCADE_ROUNDS
-#define NU_CASCADE_ROUNDS 32
-#endif
-
-// A warp whose gain bounds pass at least NU_GAIN_PASS_MAX of its 32 cells
-// screens its next NU_GAIN_DIRECT_ROUNDS rounds in full without them.
-#ifndef NU_GAIN_PASS_MAX
-#define NU_GAIN_PASS_MAX 28
-#endif
-#ifndef NU_GAIN_DIRECT_ROUNDS
-#define NU_GAIN_DIRECT_ROUNDS 16
-#endif
-
-// Exact ln P of one cell computed by a whole warp (lanes over epochs); used
-// only to seed the pruning threshold.
-template <typename T>
-__device__ __forceinline__ double exact_cell_warp(const FoldGeom& g,
-                                                  const Node8<T>* __restrict__ nd,
-                                                  const CellCtx& c, int64_t j) {
+__device__ __forceinline__ void list_item(const FoldLists& l, bool heavy, unsigned o) {
     const int lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(0xffffffffu, heavy);
+    if (!m) return;
+    unsigned at = 0u;
+    if (lane == __ffs(m) - 1) at = atomicAdd(l.n, (unsigned)__popc(m));
+    at = __shfl_sync(0xffffffffu, at, __ffs(m) - 1);
+    if (heavy) l.block[at + __popc(m & ((1u << lane) - 1u))] = o;
+}
+
+struct FoldJob {
+    const FoldSeg* segs;   // the batch's curves, or nullptr: the one curve
+    FoldSeg one;
+    int n_seg, n_D;
+    double dt, inv_dt, gap_max;
+    const double* t;
+    const void* nodes;
+    const ScreenRec* screen;
+    const ulonglong2* vpair;
+    const ScreenRec* srec;
+    const unsigned* reg;
+    const unsigned long long* peak;
+    const int* bucket;
+    const Node4<float>* rec;
+    FilterTab tab;
+    const double* periods;
+    const PeriodConst* ptab;     // nullptr: computed per item
+    const SlotPeriod* stab;
+    ItemConst* items;            // nullptr: computed by the item
+    int64_t n_P;
+    double *Q, *T0;
+    int* Didx;
+    double *dep, *sig, *lnp;
+    FoldCand* cand;              // nullptr: evaluate in place
+    unsigned long long* n_cand;
+    unsigned long long cap;
+    int2* range;                 // per item: first candidate, count (-1: written)
+    SlotBest* sbest;             // nullptr: the item writes its result
+    FoldLists list;              // block == nullptr: none
+    unsigned* counters;          // the list's and (behind) the candidates', 32 bytes
+};
+
+__device__ __forceinline__ FoldGeom job_geom(const FoldJob& J, const FoldSeg& fs) {
+    return FoldGeom{J.t + fs.s_off, fs.n_t0, fs.t_ref, fs.t_last, J.dt, J.inv_dt,
+                    J.gap_max, J.bucket + fs.bucket_off, fs.n_bucket};
+}
+__device__ __forceinline__ ScreenGeom job_screen(const FoldJob& J, const FoldSeg& fs,
+                                                 int64_t seg, bool f32) {
+    return ScreenGeom{J.screen + fs.s_off * J.n_D, J.vpair + fs.s_off,
+                      J.srec ? J.srec + fs.srec_off : nullptr, fs.n_slots, J.reg + 2 * seg,
+                      fs.screen, f32 ? 1 : 0};
+}
+__device__ __forceinline__ ItemConst item_const(const FoldGeom& g, const ScreenGeom& sg, double P,
+                                                const PeriodConst& pc) {
+    ItemConst ic{0ull, 0ull, 0.f, 0.f, 0.f, 0};
+    if (bad_period(P, g)) {
+        ic.flags = 1;
+        return ic;
+    }
+    const ScreenPeriod sp = screen_period(g, sg, P, pc);
+    ic.uend = sp.uend;
+    ic.delta = sp.delta;
+    ic.cv = sp.cv;
+    ic.hw = sp.hw;
+    ic.K = (float)(unsigned)(sp.uend >> 32) / (float)max((unsigned)(sp.ustep >> 32), 1u);
+    ic.flags = (sp.on ? 2 : 0) | (sp.slots ? 4 : 0) |
+               (g.t_last - g.t_ref >= 32.0 * P ? 8 : 0);
+    return ic;
+}
+__device__ __forceinline__ bool item_heavy(const FoldJob& J, const ItemConst& ic) {
+    return J.list.block && (!(ic.K < J.list.heavy_k) || !(ic.flags & 2));
+}
+// One thread per item: its constants, and its place in the list.
+__global__ void k_item_consts(const __grid_constant__ FoldJob J, int f32) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    bool in = i < (int64_t)J.n_seg * J.n_P, heavy = false;
+    int64_t o = 0;
+    if (in) {
+        const int64_t seg = J.n_seg == 1 ? 0 : i / J.n_P;
+        const int64_t p = period_slot(i - seg * J.n_P, J.periods, J.n_P);
+        o = seg * J.n_P + p;
+        const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+        if (fs.use_slots) {
+            in = false;
+        } else {
+            const ItemConst ic = item_const(job_geom(J, fs), job_screen(J, fs, seg, f32 != 0),
+                                            J.periods[p], J.ptab[p]);
+            J.items[o] = ic;
+            heavy = item_heavy(J, ic);
+        }
+    }
+    if (J.list.block) list_item(J.list, in && heavy, (unsigned)o);
+}
+
+// What the screens compare with: an FP32 value below every ln P that an
+// evaluated cell could lose by.  In FP64 the bound itself (its margins are far
+// above FP64 rounding); in mixed precision the evaluated ln P carries FP32
+// rounding (the events', the compensated sums', and up to 2^-21 per epoch
+// from the logarithms), so the screens, which bound the real ln P, leave 2e-4
+// relative and 5e-7 per epoch.
+template <typename T>
+__device__ __forceinline__ float screen_threshold(float lb, float K) {
+    return sizeof(T) == 8 ? lb : lb - 2e-4f * (1.f + fabsf(lb)) - 5e-7f * K;
+}
+
+// Exact evaluation of a cell by one thread (the order of the sums over the
+// epochs defines the result).
+template <typename T>
+__device__ __forceinline__ bool evaluate_cell(const FoldGeom& g, const Node8<T>* __restrict__ nd,
+                                              const CellCtx& c, int64_t j, double& lnp, T& Dl,
+                                              T& s2) {
     const double phi = cell_phi(c, j);
     const unsigned long long u0 = (unsigned long long)j * c.swp.u0;
     const int64_t kmax = cell_kmax(g, c, phi, u0);
     ExactAcc<T> a1;
     a1.init();
-    cell_pass1<T>(g, nd, c, phi, u0, kmax, lane, 32, a1);
-    T s_inv = a1.s_inv.s, s_d = a1.s_d.s, s_l = a1.s_l.s;
-    int K = a1.K;
-    for (int o = 16; o > 0; o >>= 1) {
-        s_inv += __shfl_xor_sync(0xffffffffu, s_inv, o);
-        s_d += __shfl_xor_sync(0xffffffffu, s_d, o);
-        s_l += __shfl_xor_sync(0xffffffffu, s_l, o);
-        K += __shfl_xor_sync(0xffffffffu, K, o);
-    }
-    if (K == 0) return -INFINITY;
-    const T s2 = T(1) / s_inv;
+    cell_pass1<T>(g, nd, c, phi, u0, kmax, 0, 1, a1);
+    if (a1.K == 0) return false;
+    s2 = T(1) / a1.s_inv.s;
+    Dl = s2 * a1.s_d.s;
     ExactPen<T> a2;
-    a2.init(s2, s2 * s_d);
-    cell_pass2<T>(g, nd, c, phi, u0, kmax, lane, 32, a2);
-    T pen = (T)(a2.logsum() + (double)a2.quad.s);
-    for (int o = 16; o > 0; o >>= 1) pen += __shfl_xor_sync(0xffffffffu, pen, o);
-    return (double)s_l - 0.5 * (double)pen;
+    a2.init(s2, Dl);
+    cell_pass2<T>(g, nd, c, phi, u0, kmax, 0, 1, a2);
+    lnp = (double)a1.s_l.s - 0.5 * a2.total();
+    return lnp == lnp;                       // NaN never selected
 }
 
-// Order-preserving unsigned key of a float (for a shared atomic max).
-__device__ __forceinline__ unsigned fkey(float x) {
-    const unsigned b = __float_as_uint(x);
-    return (b >> 31) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float from_fkey(unsigned k) {
-    return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k);
+// The same by a whole warp (lanes over epochs, fixed reduction order), called
+// by all lanes with the same cell: the FP64 evaluation of every cell of a
+// period whose cells have 32 or more epochs.
+__device__ __forceinline__ bool evaluate_cell_warp(const FoldGeom& g,
+                                                   const Node8<double>* __restrict__ nd,
+                                                   const CellCtx& c, int64_t j, double& lnp,
+                                                   double& Dl, double& s2) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const double phi = cell_phi(c, j);
+    const unsigned long long u0 = (unsigned long long)j * c.swp.u0;
+    const int64_t kmax = cell_kmax(g, c, phi, u0);
+    ExactAcc<double> a1;
+    a1.init();
+    cell_pass1<double>(g, nd, c, phi, u0, kmax, lane, 32, a1);
+    double s_inv = a1.s_inv.s, s_d = a1.s_d.s, s_l = a1.s_l.s;
+    int K = a1.K;
+    for (int o = 16; o > 0; o >>= 1) {
+        s_inv += __shfl_xor_sync(FULL, s_inv, o);
+        s_d += __shfl_xor_sync(FULL, s_d, o);
+        s_l += __shfl_xor_sync(FULL, s_l, o);
+        K += __shfl_xor_sync(FULL, K, o);
+    }
+    if (K == 0) return false;
+    s2 = 1.0 / s_inv;
+    Dl = s2 * s_d;
+    ExactPen<double> a2;
+    a2.init(s2, Dl);
+    cell_pass2<double>(g, nd, c, phi, u0, kmax, lane, 32, a2);
+    double pen = a2.total();
+    for (int o = 16; o > 0; o >>= 1) pen += __shfl_xor_sync(FULL, pen, o);
+    lnp = s_l - 0.5 * pen;
+    return lnp == lnp;
 }
 
 // A large finite single-event gain of each curve, for the peak seed: key[g]
@@ -1545,412 +1441,478 @@ __global__ void k_gain_peak(const T* __restrict__ gain, const int64_t* __restric
     if ((threadIdx.x & 31) == 0 && best != 0) atomicMax(key + g, best);
 }
 
-// What the screens compare with: an FP32 value below every ln P that an
-// evaluated cell could lose by.  In FP64 the evaluated ln P rounded down; in
-// mixed precision the evaluated ln P carries FP32 rounding (the events', the
-// compensated sums', and up to 2^-21 per epoch from the logarithms), so the
-// screens, which bound the real ln P, leave 2e-4 relative and 5e-7 per epoch.
-template <typename T>
-__device__ __forceinline__ float screen_threshold(double lnp, float kmax) {
-    if (sizeof(T) == 8) return __double2float_rd(lnp);
-    const float l = (float)lnp;
-    return l - 2e-4f * (1.f + fabsf(l)) - 5e-7f * kmax;
+// The phases about an epoch at walk position u: the cells of one period that
+// pass closest to it (the peak seed's).  Lane l < 8 gets phase l - 4 about the
+// nearest.
+__device__ __forceinline__ unsigned seed_phase(unsigned long long u, unsigned long long ustep,
+                                               unsigned long long uph, int64_t n_phi, int l) {
+    const unsigned long long r = u % ustep;
+    int64_t j = (int64_t)(uph ? (r + (uph >> 1)) / uph : 0ull) + l - 4;
+    j = j < 0 ? j + n_phi : (j >= n_phi ? j - n_phi : j);
+    return (unsigned)(j < 0 ? 0 : (j >= n_phi ? n_phi - 1 : j));
 }
 
-// Exact evaluation of a queued cell by one thread; the thread's best is kept
-// in shared memory and the block's thresholds are raised.
+// the warps of an item: one, or the block's
+template <int NW>
+__device__ __forceinline__ void item_sync() {
+    if (NW == 1) __syncwarp(); else __syncthreads();
+}
+#ifndef NU_FOLD_WARPS
+#define NU_FOLD_WARPS 32           // resident warps per SM (64 registers)
+#endif
+#ifndef NU_WARP_ITEMS_FROM
+#define NU_WARP_ITEMS_FROM 6000    // periods from which two warps fold one (single curve)
+#endif
+#ifndef NU_ONE_WARP_FROM
+#define NU_ONE_WARP_FROM 40000     // and one warp
+#endif
+#ifndef NU_HEAVY_K
+#define NU_HEAVY_K 22.f            // epochs per cell of an item that takes a block then
+#endif
+// Work item i of the job in the order of the fold (short periods first).
+__device__ __forceinline__ bool ordered_item(const FoldJob& J, int64_t i, int64_t& item) {
+    if (i >= (int64_t)J.n_seg * J.n_P) return false;
+    const int64_t seg = J.n_seg == 1 ? 0 : i / J.n_P;
+    item = seg * J.n_P + period_slot(i - seg * J.n_P, J.periods, J.n_P);
+    return true;
+}
+// The k-th item of a block of the eight-warp kernels (*sh is the block's);
+// false when no work is left.
+__device__ __forceinline__ bool next_item(const FoldJob& J, int k_th, unsigned* sh,
+                                          int64_t& item) {
+    __syncthreads();
+    if (J.list.block == nullptr)
+        return ordered_item(J, blockIdx.x + (int64_t)k_th * gridDim.x, item);
+    if (threadIdx.x == 0) *sh = atomicAdd(J.list.n + 1, 1u);
+    __syncthreads();
+    const unsigned k = *sh;
+    if (k >= J.list.n[0]) return false;
+    item = J.list.block[k];
+    return true;
+}
+// The item of a warp of the other kernels (blocks of 4 / NW items).
+template <int NW>
+__device__ __forceinline__ bool warp_item(const FoldJob& J, int64_t& item) {
+    return ordered_item(J, NW == 1 ? (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5) : blockIdx.x,
+                        item);
+}
+__host__ __device__ constexpr int fold_threads(int nw) { return nw == 1 ? 128 : 32 * nw; }
+
+// Per-warp shared state of the exact paths: survivors of the screen (their
+// cells and bounds).
+struct CellQueues {
+    FilterQueues f;
+    uint2 b[64];
+    float bu[64];
+    int nb;
+};
+struct CellItem {          // per-item shared state of the exact paths
+    FilterCtx x;
+    ScreenPeriod sp;
+    CellCtx cc;
+    FoldGeom g;
+    ScreenGeom sg;
+    int64_t item;
+    int coop;              // cells evaluated by the warp's lanes
+    int inl;               // some cell was evaluated in place
+    unsigned cnt;
+    long long start;
+};
+
+// The screen of the exact paths (filter.cuh) and what follows it.
 template <typename T>
-__device__ __forceinline__ void evaluate_queued(const FoldGeom& g,
-                                               const Node8<T>* __restrict__ nodes,
-                                               const CellCtx& c, int64_t n_phi, long long qcell,
-                                               int qd, unsigned long long* sh_sbest,
-                                               unsigned* sh_bfk, Best* tb) {
-    const int64_t qj = qcell - (int64_t)qd * n_phi;
-    const Node8<T>* nd = nodes + (int64_t)qd * g.n_t0;
-    const double phi = cell_phi(c, qj);
-    const unsigned long long u0 = (unsigned long long)qj * c.swp.u0;
-    const int64_t kmax = cell_kmax(g, c, phi, u0);
-    ExactAcc<T> a1;
-    a1.init();
-    cell_pass1<T>(g, nd, c, phi, u0, kmax, 0, 1, a1);
-    if (a1.K == 0 || a1.cannot_win(from_max_key(*sh_sbest))) return;
-    const T s2 = T(1) / a1.s_inv.s;
-    const T Dl = s2 * a1.s_d.s;
-    ExactPen<T> a2;
-    a2.init(s2, Dl);
-    cell_pass2<T>(g, nd, c, phi, u0, kmax, 0, 1, a2);
-    const double lnp = (double)a1.s_l.s - 0.5 * (a2.logsum() + (double)a2.quad.s);
-    if (!(lnp == lnp)) return;   // NaN never selected
-    const Best cand{lnp, qcell, (double)Dl, (double)s2};
-    if (better(cand, *tb)) *tb = cand;
-    if (lnp > from_max_key(*sh_sbest)) {
-        atomicMax(sh_sbest, max_key(lnp));
-        atomicMax(sh_bfk, fkey(screen_threshold<T>(lnp, (float)(int)kmax)));
+struct CellScreen {
+    CellItem& it;
+    CellQueues& q;
+    const Node8<T>* nodes;
+    Best& tb;              // the warp's best cell evaluated in place (shared)
+
+    // drop the survivors that the threshold has overtaken
+    __device__ __noinline__ void compact() {
+        const int lane = threadIdx.x & 31;
+        const float t = filter_thr(it.x);
+        const int nb = q.nb;
+        int n = 0;
+        for (int h = 0; h < nb; h += 32) {
+            const bool in = h + lane < nb;
+            const uint2 cl = in ? q.b[h + lane] : make_uint2(0u, 0u);
+            const float ub = in ? q.bu[h + lane] : 0.f;
+            const bool keep = in && !(ub < t);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int pos = n + __popc(m & ((1u << lane) - 1u));
+                q.b[pos] = cl;
+                q.bu[pos] = ub;
+            }
+            n += __popc(m);
+            __syncwarp();
+        }
+        if (lane == 0) q.nb = n;
+        __syncwarp();
     }
+
+    // evaluation in place of the first n <= 32 survivors
+    __device__ __noinline__ void evaluate(int n) {
+        const unsigned FULL = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        const FoldGeom& g = it.g;
+        const CellCtx& c = it.cc;
+        const int64_t n_phi = it.x.fp.n_phi;
+        Best best{-INFINITY, LLONG_MAX, NAN, NAN};
+        auto take = [&](const uint2& cl, double lnp, double Dl, double s2) {
+            const Best cand{lnp, (long long)cl.y * n_phi + cl.x, Dl, s2};
+            if (better(cand, best)) best = cand;
+        };
+        bool done = false;
+        if constexpr (sizeof(T) == 8) {
+            if (it.coop) {
+                for (int e = 0; e < n; ++e) {
+                    const uint2 cl = q.b[e];
+                    double lnp, Dl, s2;
+                    if (evaluate_cell_warp(g, nodes + (int64_t)cl.y * g.n_t0, c, cl.x, lnp, Dl,
+                                           s2))
+                        take(cl, lnp, Dl, s2);
+                }
+                done = true;
+            }
+        }
+        if (!done && lane < n) {
+            const uint2 cl = q.b[lane];
+            double lnp;
+            T Dl, s2;
+            if (evaluate_cell<T>(g, nodes + (int64_t)cl.y * g.n_t0, c, cl.x, lnp, Dl, s2))
+                take(cl, lnp, (double)Dl, (double)s2);
+        }
+        for (int s = 16; s > 0; s >>= 1) {
+            const Best b{__shfl_xor_sync(FULL, best.lnp, s), __shfl_xor_sync(FULL, best.cell, s),
+                         __shfl_xor_sync(FULL, best.depth, s),
+                         __shfl_xor_sync(FULL, best.sigma, s)};
+            if (better(b, best)) best = b;
+        }
+        if (lane == 0) {
+            it.inl = 1;
+            if (better(best, tb)) tb = best;
+            if (best.cell != LLONG_MAX)
+                filter_raise(it.x, fkey(screen_threshold<T>(__double2float_rd(best.lnp),
+                                                            it.x.fp.K)));
+        }
+        __syncwarp();
+    }
+
+    __device__ __noinline__ void push(bool keep, const uint2& cl, float ub) {
+        const int lane = threadIdx.x & 31;
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        const int nb = q.nb;
+        if (keep) {
+            const int pos = nb + __popc(m & ((1u << lane) - 1u));
+            q.b[pos] = cl;
+            q.bu[pos] = ub;
+        }
+        __syncwarp();
+        if (lane == 0) q.nb = nb + __popc(m);
+        __syncwarp();
+        if (q.nb < 32) return;
+        compact();
+        const int n = q.nb;
+        if (n < 32) return;
+        evaluate(32);
+        const float u2 = lane < n - 32 ? q.bu[32 + lane] : 0.f;
+        filter_shift_queue(q.b, n, 32);
+        if (lane < n - 32) q.bu[lane] = u2;
+        if (lane == 0) q.nb = n - 32;
+        __syncwarp();
+    }
+
+    // full screen of the queue's first cnt cells
+    __device__ __noinline__ void operator()(int cnt) {
+        const int lane = threadIdx.x & 31;
+        float ub = -INFINITY, lb = -INFINITY;
+        uint2 cl = make_uint2(0u, 0u);
+        const ScreenGeom& sg = it.sg;
+        if (lane < cnt) {
+            cl = q.f.cell[lane];
+            ub = screen_cell(it.g, sg, sg.rec + (int64_t)cl.y * it.g.n_t0,
+                             sg.srec ? sg.srec + (int64_t)cl.y * sg.n_slots : nullptr, it.sp,
+                             it.cc, (int64_t)cl.x, (unsigned long long)cl.x * it.sp.uph,
+                             filter_thr(it.x), &lb);
+        }
+        const unsigned k =
+            __reduce_max_sync(0xffffffffu, fkey(screen_threshold<T>(lb, it.x.fp.K)));
+        if (lane == 0) filter_raise(it.x, k);
+        __syncwarp();
+        // a cell without events (bound -inf) is never the argmax; NaN survives
+        push(lane < cnt && !(ub == -INFINITY) && !(ub < filter_thr(it.x)), cl, ub);
+    }
+};
+
+// Shared state of an item, by one warp (an invalid period is written here).
+__device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs, int64_t seg,
+                                             int64_t p, int64_t o, bool f32, CellItem& it) {
+    if ((threadIdx.x & 31) != 0) return;
+    const double P = J.periods[p];
+    const FoldGeom g = job_geom(J, fs);
+    const ScreenGeom sg = job_screen(J, fs, seg, f32);
+    PeriodConst tmp;
+    const PeriodConst* pc = J.ptab ? J.ptab + p : &tmp;
+    ItemConst ic;
+    if (J.items) {
+        ic = J.items[o];
+    } else {
+        tmp = bad_period(P, g) ? PeriodConst{1, 0.0, 0, 0, 0.f, {0, 0}, {0, 0}, 1.0, 1.0}
+                               : period_const(P, J.dt, J.inv_dt);
+        ic = item_const(g, sg, P, *pc);
+    }
+    it.item = o;
+    if (ic.flags & 1) {
+        write_bad(o, J.Q, J.T0, J.Didx, J.dep, J.sig, J.lnp);
+        if (J.range) J.range[o] = make_int2(0, -1);
+        it.item = -1;
+        return;
+    }
+    it.g = g;
+    it.sg = sg;
+    it.cc = cell_ctx(g, P, *pc, fs.uspan);
+    const bool on = ic.flags & 2;
+    ScreenPeriod& sp = it.sp;
+    sp.uph = on ? pc->uph : 0ull;
+    sp.ustep = on ? pc->ustep : 0ull;
+    sp.delta = ic.delta;
+    sp.uend = ic.uend;
+    sp.wscale = (float)(4194304.0 * J.inv_dt);
+    sp.cv = ic.cv;
+    sp.hw = ic.hw;
+    sp.on = on;
+    sp.slots = ic.flags & 4;
+    FilterPeriod f;
+    f.ustep = sp.ustep;
+    f.uph = sp.uph;
+    f.uend = sp.uend;
+    f.n_phi = pc->n_phi;
+    f.K = ic.K + 2.f;
+    f.mode = on ? filter_mode(J.tab.S != nullptr && sp.delta <= 8ull * FILTER_MARGIN, sp.ustep,
+                              ic.K, f.n_phi * J.n_D)
+                : FILTER_NONE;
+    it.x.fp = f;
+    it.x.f = filter_view(J.tab, fs);
+    it.x.n_D = J.n_D;
+    it.x.bfk = fkey(-INFINITY);
+    // FP64 sums of long cells by the warp's lanes (one fixed order for every
+    // cell of the period)
+    it.coop = !f32 && on && (ic.flags & 8);
+    it.inl = 0;
+    it.cnt = 0u;
 }
 
-// The same evaluation by a whole warp (lanes over epochs, fixed reduction
-// order); called by all lanes with the same cell.  Used for every evaluation
-// of a period whose cells have 32 or more epochs, where one cell per lane
-// would leave most lanes idle whenever fewer than 32 cells are queued.
-__device__ __forceinline__ void evaluate_queued_warp(const FoldGeom& g,
-                                                    const Node8<double>* __restrict__ nodes,
-                                                    const CellCtx& c, int64_t n_phi,
-                                                    long long qcell, int qd,
-                                                    unsigned long long* sh_sbest,
-                                                    unsigned* sh_bfk, Best* tb) {
+// One item of the exact paths by the nw warps that share it (w: this one).
+template <typename T, int nw>
+__device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int w, CellItem& it,
+                                                CellQueues& q, Best* tbs) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int64_t qj = qcell - (int64_t)qd * n_phi;
-    const Node8<double>* nd = nodes + (int64_t)qd * g.n_t0;
-    const double phi = cell_phi(c, qj);
-    const unsigned long long u0 = (unsigned long long)qj * c.swp.u0;
-    const int64_t kmax = cell_kmax(g, c, phi, u0);
-    ExactAcc<double> a1;
-    a1.init();
-    cell_pass1<double>(g, nd, c, phi, u0, kmax, lane, 32, a1);
-    double s_inv = a1.s_inv.s, s_d = a1.s_d.s, s_l = a1.s_l.s, s_dd = a1.s_dd;
-    int K = a1.K;
-    for (int o = 16; o > 0; o >>= 1) {
-        s_inv += __shfl_xor_sync(FULL, s_inv, o);
-        s_d += __shfl_xor_sync(FULL, s_d, o);
-        s_l += __shfl_xor_sync(FULL, s_l, o);
-        s_dd += __shfl_xor_sync(FULL, s_dd, o);
-        K += __shfl_xor_sync(FULL, K, o);
+    const int64_t seg = J.n_seg == 1 ? 0 : o / J.n_P;
+    const int64_t p = o - seg * J.n_P;
+    const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+    if (fs.use_slots) return;
+    if (nw < 8 && J.items && item_heavy(J, J.items[o])) return;
+    const int n_D = J.n_D;
+    if (lane == 0) {
+        q.f.ni = q.f.nq = q.f.nc = q.nb = 0;
+        tbs[w] = Best{-INFINITY, LLONG_MAX, NAN, NAN};
     }
-    const double best_now = __shfl_sync(FULL, from_max_key(*sh_sbest), 0);
-    if (K == 0 || cannot_win(s_l, s_inv, s_d, s_dd, best_now)) return;
-    const double s2 = 1.0 / s_inv;
-    const double Dl = s2 * s_d;
-    ExactPen<double> a2;
-    a2.init(s2, Dl);
-    cell_pass2<double>(g, nd, c, phi, u0, kmax, lane, 32, a2);
-    double pen = a2.logsum() + a2.quad.s;
-    for (int o = 16; o > 0; o >>= 1) pen += __shfl_xor_sync(FULL, pen, o);
-    const double lnp = s_l - 0.5 * pen;
-    if (lane != 0 || !(lnp == lnp)) return;      // NaN never selected
-    const Best cand{lnp, qcell, Dl, s2};
-    if (better(cand, *tb)) *tb = cand;
-    if (lnp > from_max_key(*sh_sbest)) {
-        atomicMax(sh_sbest, max_key(lnp));
-        atomicMax(sh_bfk, fkey(__double2float_rd(lnp)));
+    if (w == 0) cell_item_setup(J, fs, seg, p, o, sizeof(T) == 4, it);
+    item_sync<nw>();
+    if (it.item < 0) return;
+    CellScreen<T> screen{it, q, (const Node8<T>*)J.nodes + fs.s_off * n_D, tbs[w]};
+    if (it.x.fp.mode != FILTER_NONE) {
+        // peak seed: the cells about the curve's largest single-event gain
+        const unsigned long long pk = J.peak[seg];
+        if (pk != 0 && w == 0) {
+            const unsigned e = 0xffffffffu - (unsigned)(pk & 0xffffffffu);
+            const unsigned pd = e / (unsigned)fs.n_t0;
+            const unsigned long long u = it.sg.vpair[e - pd * (unsigned)fs.n_t0].x;
+            if (lane < 8)
+                q.f.cell[lane] = make_uint2(
+                    seed_phase(u, it.x.fp.ustep, it.x.fp.uph, it.x.fp.n_phi, lane), pd);
+            __syncwarp();
+            screen(8);
+            __syncwarp();
+        }
+        item_sync<nw>();
+        filter_cells(it.x, w, nw, q.f, screen);
+    } else {
+        // every cell: to the screen, or (no screen) to the evaluation
+        const int64_t n_phi = it.x.fp.n_phi, n_cells = n_phi * n_D;
+        for (int64_t base = (int64_t)w * 32; base < n_cells; base += nw * 32) {
+            const int64_t cell = base + lane;
+            const bool in = cell < n_cells;
+            const unsigned d = in ? (unsigned)(cell / n_phi) : 0u;
+            const uint2 cl = make_uint2(in ? (unsigned)(cell - (int64_t)d * n_phi) : 0u, d);
+            if (it.sp.on) {
+                q.f.cell[lane] = cl;
+                __syncwarp();
+                screen((int)min((int64_t)32, n_cells - base));
+                __syncwarp();
+            } else {
+                screen.push(in, cl, INFINITY);
+            }
+        }
+    }
+    item_sync<nw>();
+    screen.compact();
+    const int nb = q.nb;
+    // hand the survivors on, unless some were evaluated here or the list is full
+    if (J.cand != nullptr && it.inl == 0) {
+        unsigned at = 0u;
+        if (lane == 0) at = atomicAdd(&it.cnt, (unsigned)nb);
+        item_sync<nw>();
+        if (w == 0 && lane == 0) {
+            const unsigned n = it.cnt;
+            long long start = n ? (long long)atomicAdd(J.n_cand, (unsigned long long)n) : 0;
+            if (n && (unsigned long long)start + n > J.cap) {
+                for (unsigned long long i = start; i < J.cap && i < start + n; ++i)
+                    J.cand[i].item = -1;
+                start = -1;
+            } else {
+                J.range[o] = make_int2((int)start, (int)n);
+            }
+            it.start = start;
+        }
+        item_sync<nw>();
+        if (it.start >= 0) {
+            at = __shfl_sync(FULL, at, 0);
+            if (lane < nb) {
+                FoldCand& cd = J.cand[it.start + at + lane];
+                cd.item = o;
+                cd.j = q.b[lane].x;
+                cd.d = (int)q.b[lane].y;
+            }
+            return;
+        }
+    }
+    if (nb > 0) screen.evaluate(nb);
+    item_sync<nw>();
+    if (w == 0 && lane == 0) {
+        Best tb = tbs[0];
+        for (int i = 1; i < nw; ++i)
+            if (better(tbs[i], tb)) tb = tbs[i];
+        if (tb.cell != LLONG_MAX) tb.sigma = sqrt(tb.sigma);   // held sigma^2
+        write_best(tb, o, it.x.fp.n_phi, it.g.t_ref, J.periods[p], J.Q, J.T0, J.Didx, J.dep,
+                   J.sig, J.lnp);
+        if (J.range) J.range[o] = make_int2(0, -1);
     }
 }
 
-// One period of the FP64 path with the screen.  Each warp screens its own
-// cells (the block's cells in strides of blockDim) and queues the survivors
-// in its own shared queue; a full queue (32 cells) is evaluated exactly, one
-// cell per lane, by that warp alone, so the screen needs no block barriers.
-// Warp 0 first evaluates the cell through the curve's largest single-event
-// gain, and in its first round each warp evaluates its best-bounded cell with
-// all its lanes when that bound is above the threshold.  The thresholds (best ln P, and its FP32
-// lower bound) are shared by the block through atomic maxima.
-// With TAB the period's curve-independent constants come from the table
-// entry pc (k_period_consts), else they are computed here.
-// T is the type of the exact events: double, or float for the mixed fold of
-// grids that are not regular (FP64 epochs, FP32 values and compensated sums;
-// every cell by the thread code, whose order of the sums defines the result).
-// Measured on a sector of barycentric times (19 440 epochs, 10 durations,
-// 20 000 periods): FP64 32.0 -> 11.3 ms when the gain bound came to irregular
-// grids; mixed 132.5 -> 10.3 ms (every cell's events took their epochs and
-// brackets in FP64 before, 64 cycles per warp instruction).
-template <typename T, int MAXT = 256, bool TAB = false, bool GROUP = true>
-__device__ __forceinline__ void fold_screened_one(const FoldGeom& g, const ScreenGeom& sg,
-                                                  const Node8<T>* __restrict__ nodes,
-                                                  int n_D, double P, int64_t p,
-                                                  double* __restrict__ Q_out,
-                                                  double* __restrict__ T0_out,
-                                                  int* __restrict__ Didx_out,
-                                                  double* __restrict__ dep_out,
-                                                  double* __restrict__ sig_out,
-                                                  double* __restrict__ lnp_out,
-                                                  const PeriodConst* __restrict__ pc = nullptr) {
-    __shared__ long long sh_qc[MAXT / 32][64];      // per-warp survivor queues
-    __shared__ int sh_qd[MAXT / 32][64];
-    __shared__ long long sh_qa[MAXT / 32][160];     // per-warp cells for the full screen
-    __shared__ int sh_qad[MAXT / 32][160];
-    __shared__ unsigned long long sh_sbest; // best ln P evaluated (max key)
-    __shared__ unsigned sh_bfk;             // its FP32 lower bound (float key)
-    __shared__ Best sh_tb[MAXT];            // each thread's best evaluated cell (kept
-                                            // out of registers during the screen)
-    if (bad_period(P, g)) {
-        if (threadIdx.x == 0) write_bad(p, Q_out, T0_out, Didx_out, dep_out, sig_out, lnp_out);
-        return;
+// Exact paths (FP64 epochs; T: the type of the events).
+template <typename T, int NW>
+__global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
+k_fold_cells(const __grid_constant__ FoldJob J) {
+    constexpr int W = fold_threads(NW) / 32;
+    __shared__ CellQueues sh_q[W];
+    __shared__ CellItem sh_i[W / NW];
+    __shared__ Best sh_tb[W];
+    const int wid = threadIdx.x >> 5;
+    int64_t item = 0;
+    if (NW == 8) {
+        __shared__ unsigned sh_k;
+        for (int k = 0; next_item(J, k, &sh_k, item); ++k)
+            fold_cells_item<T, NW>(J, item, wid, sh_i[0], sh_q[wid], sh_tb);
+    } else if (warp_item<NW>(J, item)) {
+        fold_cells_item<T, NW>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid],
+                               sh_tb + wid / NW * NW);
     }
-    // the period's constants live in shared memory: registers are kept for
-    // the screen loop (most of these are read only on rare paths)
-    __shared__ ScreenPeriod sh_sp;
-    __shared__ CellCtx sh_cc;
-    __shared__ GainWalk32 sh_gw;
-    const int64_t n_phi = TAB ? pc->n_phi : (int64_t)ceil(P / g.dt);
-    if (threadIdx.x == 0) sh_sp = TAB ? screen_period(g, sg, P, *pc) : screen_period(g, sg, P, n_phi);
-    __syncthreads();
-    if (!sh_sp.on) {
-        fold_exact_one<T, 8, MAXT>(g, nodes, n_D, P, p, Q_out, T0_out, Didx_out, dep_out,
-                                   sig_out, lnp_out);
-        return;
-    }
-    sh_tb[threadIdx.x] = Best{-INFINITY, LLONG_MAX, NAN, NAN};
-    if (threadIdx.x == 0) {
-        sh_gw = gain_walk32(sh_sp.ustep, sh_sp.uend);
-        sh_cc = TAB ? cell_ctx(g, P, *pc) : cell_ctx(g, P, n_phi);
-        sh_sbest = max_key(-INFINITY);
-        sh_bfk = fkey(-INFINITY);
-    }
-    __syncthreads();
-    const ScreenPeriod& sp = sh_sp;
-    const CellCtx& c = sh_cc;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    // cells of 32 or more epochs are evaluated warp-cooperatively
-    const bool coop = g.t_last - g.t_ref >= 32.0 * P;
-    // raise the thresholds to the warp's evaluation of a cell, less a margin
-    // that keeps the cell itself above them (it is evaluated again by the
-    // thread code, whose sums run in another order)
-    auto seed_with = [&](double lnp) {
-        if (lane == 0 && lnp == lnp && lnp > -INFINITY) {
-            const double margin = sizeof(T) == 8 ? 1e-9 : 1e-4;
-            const double seed = lnp - margin * (1.0 + fabs(lnp));
-            atomicMax(&sh_sbest, max_key(seed));
-            atomicMax(&sh_bfk,
-                      fkey(screen_threshold<T>(seed, (float)((g.t_last - g.t_ref) / P))));
-        }
-    };
-    // Peak seed: the cell whose epochs pass through the epoch of the curve's
-    // largest single-event gain (phase index nearest to it), evaluated
-    // exactly by warp 0.  When one event dominates a short cell (a deep
-    // transit), every cell that catches it would otherwise pass the screen
-    // until the threshold has risen.  Long cells are left to the first-round
-    // seeds: there one event weighs less, and the seed costs a long walk.
-    if (sg.peak && !coop) {
-        const unsigned long long pk = *sg.peak;
-        if (pk != 0) {
-            if (wid == 0) {
-                const int64_t e = (int64_t)(0xffffffffu - (unsigned)(pk & 0xffffffffu));
-                const int64_t pd = e / g.n_t0;
-                const double x = (g.t0s[e - pd * g.n_t0] - g.t_ref) / P;
-                int64_t pj = (int64_t)rint((x - floor(x)) * (double)n_phi);
-                if (pj >= n_phi || pj < 0) pj = 0;
-                seed_with(exact_cell_warp<T>(g, nodes + pd * g.n_t0, c, pj));
-            }
-            __syncthreads();
-        }
-    }
+}
+
+// Exact evaluation of the listed cells, one per lane (or one per warp, see
+// evaluate_cell_warp).
+template <typename T>
+__global__ void __launch_bounds__(64) k_cand_eval(const __grid_constant__ FoldJob J) {
     const unsigned FULL = 0xffffffffu;
-    long long* qc = sh_qc[wid];
-    int* qd = sh_qd[wid];
-    int nq = 0;                              // warp-uniform queue lengths
-    long long* qa = sh_qa[wid];
-    int* qad = sh_qad[wid];
-    int na = 0;
-    // Cascade: after the warp's first round every cell is bounded from its gains alone (the gain bound, 4 bytes per epoch); the
-    // cells that bound does not rule out are queued and screened in full 32
-    // at a time, and the full screen's survivors are evaluated exactly.
-    const bool cascade = sg.lm3 != nullptr && sp.ustep < (1ull << 60) && sh_gw.ok;
-    const unsigned ns1 = (unsigned)(sg.n_slots - 1);
-    // append this lane's cell to a queue when keep (positions by ballot)
-    auto push = [&](long long* qx, int* qy, int& n, bool keep, long long cl, int dl) {
-        const unsigned m = __ballot_sync(FULL, keep);
-        if (keep) {
-            const int pos = n + __popc(m & ((1u << lane) - 1u));
-            qx[pos] = cl;
-            qy[pos] = dl;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long n = min(*J.n_cand, J.cap);
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long base = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) -
+                                   lane;
+         base < n; base += stride) {
+        FoldCand cd;
+        cd.item = -1;
+        cd.j = 0u;
+        cd.d = 0;
+        if (base + lane < n) {
+            const FoldCand* s = J.cand + base + lane;
+            cd.item = s->item;
+            cd.j = s->j;
+            cd.d = s->d;
         }
-        n += __popc(m);
-        __syncwarp();
-    };
-    // drop the first 32 entries of a queue
-    auto pop32 = [&](long long* qx, int* qy, int& n) {
-        n -= 32;
-        long long c2 = 0;
-        int d2 = 0;
-        if (lane < n) {
-            c2 = qx[32 + lane];
-            d2 = qy[32 + lane];
+        const bool in = cd.item >= 0;
+        const long long item = in ? cd.item : 0;
+        const int64_t seg = J.n_seg == 1 ? 0 : item / J.n_P;
+        const int64_t p = item - seg * J.n_P;
+        const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+        const FoldGeom g = job_geom(J, fs);
+        const double P = J.periods[p];
+        const bool coop = sizeof(T) == 8 && in && g.t_last - g.t_ref >= 32.0 * P;
+        double lnp = NAN, Dl = NAN, s2 = NAN;
+        if (in && !coop) {
+            const CellCtx c = cell_ctx(g, P, J.ptab[p], fs.uspan);
+            const Node8<T>* nd =
+                (const Node8<T>*)J.nodes + fs.s_off * J.n_D + (int64_t)cd.d * g.n_t0;
+            T D, s;
+            if (!evaluate_cell<T>(g, nd, c, (int64_t)cd.j, lnp, D, s)) lnp = NAN;
+            Dl = (double)D;
+            s2 = (double)s;
         }
-        __syncwarp();
-        if (lane < n) {
-            qx[lane] = c2;
-            qy[lane] = d2;
-        }
-        __syncwarp();
-    };
-    // exact evaluation of the first n <= 32 entries of the survivor queue
-    auto evaluate_first = [&](int n) {
         if constexpr (sizeof(T) == 8) {
-            if (coop) {
-                for (int q = 0; q < n; ++q)
-                    evaluate_queued_warp(g, nodes, c, n_phi, qc[q], qd[q], &sh_sbest, &sh_bfk,
-                                         &sh_tb[threadIdx.x]);
-                return;
+            for (unsigned m = __ballot_sync(FULL, coop); m; m &= m - 1u) {
+                const int src = __ffs(m) - 1;
+                const long long it2 = __shfl_sync(FULL, cd.item, src);
+                const unsigned j2 = __shfl_sync(FULL, cd.j, src);
+                const int d2 = __shfl_sync(FULL, cd.d, src);
+                const int64_t seg2 = J.n_seg == 1 ? 0 : it2 / J.n_P;
+                const int64_t p2 = it2 - seg2 * J.n_P;
+                const FoldSeg& f2 = J.segs ? J.segs[seg2] : J.one;
+                const FoldGeom g2 = job_geom(J, f2);
+                const CellCtx c2 = cell_ctx(g2, J.periods[p2], J.ptab[p2], f2.uspan);
+                double l, D, s;
+                const bool ok = evaluate_cell_warp(
+                    g2, (const Node8<double>*)J.nodes + f2.s_off * J.n_D + (int64_t)d2 * g2.n_t0,
+                    c2, (int64_t)j2, l, D, s);
+                if (lane == src) {
+                    lnp = ok ? l : NAN;
+                    Dl = D;
+                    s2 = s;
+                }
             }
         }
-        if (lane < n)
-            evaluate_queued<T>(g, nodes, c, n_phi, qc[lane], qd[lane], &sh_sbest, &sh_bfk,
-                               &sh_tb[threadIdx.x]);
-    };
-    auto evaluate32 = [&]() {
-        evaluate_first(32);
-        __syncwarp();
-        pop32(qc, qd, nq);
-    };
-    // First-round seed: the warp evaluates its lane with the largest finite
-    // bound (all lanes over its epochs), unless that bound is already below
-    // the threshold (the cell cannot raise it).
-    auto seed_warp = [&](float ub, int dl, int64_t jl) {
-        float v = (ub < INFINITY) ? ub : -INFINITY;
-        int src = lane;
-        for (int o = 16; o > 0; o >>= 1) {
-            const float v2 = __shfl_xor_sync(FULL, v, o);
-            const int s2 = __shfl_xor_sync(FULL, src, o);
-            if (v2 > v || (v2 == v && s2 < src)) {
-                v = v2;
-                src = s2;
-            }
-        }
-        // (the threshold is broadcast so that the branch is warp-uniform)
-        const float thr = __shfl_sync(FULL, from_fkey(sh_bfk), 0);
-        if (v > -INFINITY && !(v < thr)) {
-            const int pd = __shfl_sync(FULL, dl, src);
-            const long long pj = __shfl_sync(FULL, (long long)jl, src);
-            seed_with(exact_cell_warp<T>(g, nodes + (int64_t)pd * g.n_t0, c, pj));
-            __syncwarp();
-        }
-    };
-    // Cells are taken W durations at a time (one gain group, one phase per
-    // lane; W = 1 without the cascade).  Without the cascade, the warp's
-    // first round and its direct rounds every cell goes on; otherwise those
-    // whose gain bound reaches the threshold.  Cells that go on are screened
-    // in full from queue A, 32 at a time (the warp's first such screen seeds
-    // the threshold), and the screen's survivors are evaluated exactly from
-    // the survivor queue.
-    bool seed = true;
-    // full screen of queue A's entries h .. h + cnt - 1 (one per lane)
-    auto screen_queued = [&](int h, int cnt) {
-        float ub = -INFINITY;
-        long long cl = 0;
-        int dl = 0;
-        int64_t jl = 0;
-        if (lane < cnt) {
-            cl = qa[h + lane];
-            dl = qad[h + lane];
-            jl = cl - (int64_t)dl * n_phi;
-            ub = screen_cell(g, sg, sg.rec + (int64_t)dl * g.n_t0,
-                             sg.srec ? sg.srec + (int64_t)dl * sg.n_slots : nullptr, sp, c, jl,
-                             (unsigned long long)jl * sp.uph, from_fkey(sh_bfk));
-        }
-        if (seed) {
-            seed = false;
-            seed_warp(ub, dl, jl);
-        }
-        // a cell without events (bound -inf) is never the argmax; NaN
-        // survives.  The FP32 threshold is at most every evaluated ln P.
-        push(qc, qd, nq, lane < cnt && !(ub == -INFINITY) && !(ub < from_fkey(sh_bfk)), cl,
-             dl);
-    };
-    // (GROUP = false compiles the one-duration walk alone: the wider walks'
-    // registers would otherwise weigh on the grids of one duration)
-    const int W = cascade && GROUP ? gain_width(n_D) : 1;
-    const int64_t n_gc = (int64_t)((n_D + W - 1) / W) * n_phi;
-    const int dr = NU_GAIN_DIRECT_ROUNDS / W > 0 ? NU_GAIN_DIRECT_ROUNDS / W : 1;
-    const unsigned zs = ns1 - 1u;
-    int gi = (int)(threadIdx.x / n_phi);
-    int64_t j = (int64_t)threadIdx.x - (int64_t)gi * n_phi;
-    bool first = true;
-    int direct = 0;                          // rounds left without the gain bound
-    for (int64_t base = (int64_t)wid * 32; base < n_gc; base += blockDim.x, j += blockDim.x) {
-        while (j >= n_phi) {
-            j -= n_phi;
-            ++gi;
-        }
-        const int d0 = gi * W;
-        const int nv = base + lane < n_gc ? min(W, n_D - d0) : 0;   // this lane's cells
-        unsigned pass = 0u;
-        if (!cascade || first || direct > 0) {
-            if (cascade && !first) --direct;
-            first = false;
-            pass = (1u << nv) - 1u;
-        } else {
-            if (nv > 0) {
-                float4 sk;
-                const float K = gain_walk(sg.lm3 + (int64_t)gi * sg.n_slots * W, W, zs,
-                                          (unsigned)(((unsigned long long)j * sp.uph) >>
-                                                     sh_gw.shift),
-                                          sh_gw, sk);
-                const float f = fmaf(K + 16.f, 1.1920929e-7f, 1.f);
-                const float thr = from_fkey(sh_bfk);
-                for (int i = 0; i < nv; ++i)
-                    if (!(gain_col(sk, i) * f + 0.5f + 1e-6f < thr)) pass |= 1u << i;
-            }
-            // where the gain bound rules out almost nothing (cells of many
-            // epochs, whose bound needs the depth terms) the warp screens its
-            // next rounds in full directly
-            const int np = __reduce_add_sync(FULL, (unsigned)__popc(pass));
-            const int nt = __reduce_add_sync(FULL, (unsigned)nv);
-            if (nt > 0 && np * 32 >= NU_GAIN_PASS_MAX * nt) direct = dr;
-        }
-        for (int i = 0; i < W; ++i)
-            push(qa, qad, na, (pass >> i) & 1u, (long long)(d0 + i) * n_phi + j, d0 + i);
-        // queue A holds at most 31 + 32 W entries here
-        int h = 0;
-        for (; na - h >= 32; h += 32) {
-            screen_queued(h, 32);
-            if (nq >= 32) evaluate32();
-        }
-        if (h > 0) {
-            na -= h;
-            long long c2 = 0;
-            int d2 = 0;
-            if (lane < na) {
-                c2 = qa[h + lane];
-                d2 = qad[h + lane];
-            }
-            __syncwarp();
-            if (lane < na) {
-                qa[lane] = c2;
-                qad[lane] = d2;
-            }
-            __syncwarp();
+        if (in) {
+            FoldCand* s = J.cand + base + lane;
+            s->lnp = lnp;
+            s->Dl = Dl;
+            s->s2 = s2;
         }
     }
-    if (na > 0) screen_queued(0, na);
-    if (nq >= 32) evaluate32();
-    evaluate_first(nq);
-    __syncthreads();
-    Best best = sh_tb[threadIdx.x];
-    if (best.cell != LLONG_MAX) best.sigma = sqrt(best.sigma);   // held sigma^2
-    const Best b = block_argmax<MAXT>(best);
-    if (threadIdx.x == 0)
-        write_best(b, p, n_phi, g.t_ref, P, Q_out, T0_out, Didx_out, dep_out, sig_out, lnp_out);
 }
 
-// resident blocks per SM the register allocation is sized for
-#ifndef NU_SCREEN_MIN_BLOCKS
-#define NU_SCREEN_MIN_BLOCKS 3
-#endif
-
-// 256-thread blocks: 3 per SM (about 80 registers); 64-thread blocks:
-// NU_SCREEN_SMALL_BLOCKS per SM (the shared arrays are sized for 2 warps),
-// NU_SCREEN_GROUP_BLOCKS with the grouped gain walk, whose registers need 80
-// (C2 fold 8.52 ms at 12 blocks, 8.74 ms at 14 with 72 registers).
-#ifndef NU_SCREEN_SMALL_BLOCKS
-#define NU_SCREEN_SMALL_BLOCKS 14
-#endif
-#ifndef NU_SCREEN_GROUP_BLOCKS
-#define NU_SCREEN_GROUP_BLOCKS 12
-#endif
-template <typename T, int MAXT, bool GROUP>
-__global__ void __launch_bounds__(MAXT, MAXT <= 64 ? (GROUP ? NU_SCREEN_GROUP_BLOCKS
-                                                            : NU_SCREEN_SMALL_BLOCKS)
-                                                   : NU_SCREEN_MIN_BLOCKS)
-k_fold_screened(FoldGeom g, ScreenGeom sg, const Node8<T>* __restrict__ nodes, int n_D,
-                const double* __restrict__ periods, int64_t n_P, double* __restrict__ Q_out,
-                double* __restrict__ T0_out, int* __restrict__ Didx_out,
-                double* __restrict__ dep_out, double* __restrict__ sig_out,
-                double* __restrict__ lnp_out) {
-    if ((int64_t)blockIdx.x >= n_P) return;
-    const int64_t p = period_slot(blockIdx.x, periods, n_P);
-    fold_screened_one<T, MAXT, false, GROUP>(g, sg, nodes, n_D, periods[p], p, Q_out, T0_out,
-                                             Didx_out, dep_out, sig_out, lnp_out);
+// The best of each item's evaluated cells, one thread per item.
+__global__ void k_cand_best(const __grid_constant__ FoldJob J) {
+    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (o >= (int64_t)J.n_seg * J.n_P) return;
+    const int64_t seg = J.n_seg == 1 ? 0 : o / J.n_P;
+    const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+    const double P = J.periods[o - seg * J.n_P];
+    if (fs.use_slots) return;
+    const int2 r = J.range[o];
+    if (r.y < 0) return;
+    const int64_t n_phi = J.ptab[o - seg * J.n_P].n_phi;
+    Best b{-INFINITY, LLONG_MAX, NAN, NAN};
+    for (int i = 0; i < r.y; ++i) {
+        const FoldCand& cd = J.cand[(unsigned)r.x + i];
+        const double lnp = cd.lnp;
+        if (!(lnp == lnp)) continue;
+        const Best x{lnp, (long long)cd.d * n_phi + cd.j, cd.Dl, cd.s2};
+        if (better(x, b)) b = x;
+    }
+    if (b.cell != LLONG_MAX) b.sigma = sqrt(b.sigma);
+    write_best(b, o, n_phi, fs.t_ref, P, J.Q, J.T0, J.Didx, J.dep, J.sig, J.lnp);
 }
 
 // ---------------------------------------- slot path (mixed, regular grids)
@@ -1967,16 +1929,16 @@ __device__ __forceinline__ SlotEvent slot_event(const Node4<float>* __restrict__
     const Node4<float> a = rd[s];
     const Node4<float> b = rd[s + 1];
     SlotEvent e;
-    e.s = a.s + w * (b.s - a.s);
-    e.d = a.d + w * (b.d - a.d);
-    e.l = a.l + w * (b.l - a.l);
+    e.s = __fmaf_rn(w, b.s - a.s, a.s);
+    e.d = __fmaf_rn(w, b.d - a.d, a.d);
+    e.l = __fmaf_rn(w, b.l - a.l, a.l);
     return e;
 }
 
 struct SlotPass1 {
     KSum<float> s_inv, s_d, s_l;
     float s_dd;            // sum Delta_k^2 / s_k^2 (bound only)
-    float ivmax;           // max 1/s_k^2 (bound only)
+    float ivmax, ivmin;    // max and min 1/s_k^2 (bounds only)
     int K;
     __device__ __forceinline__ void init() {
         s_inv.init();
@@ -1984,16 +1946,35 @@ struct SlotPass1 {
         s_l.init();
         s_dd = 0.f;
         ivmax = 0.f;
+        ivmin = INFINITY;
         K = 0;
+    }
+    // The bounds of ScreenAcc::bound on the sums; x_max, x_min = max and min
+    // 1/s_k^2 over S_inv.  The reciprocals are the hardware approximation
+    // (2^-21 relative, far inside the margins).
+    __device__ __forceinline__ float upper() const {
+        const float r = rcp32(s_inv.s);
+        const float q = fmaxf(0.0f, s_dd - s_d.s * s_d.s * r - 1e-4f * s_dd);
+        const float x = fminf(1.0f, ivmax * r * 1.001f);
+        return s_l.s + 0.5f - 0.5f * q * rcp32(1.0f + x) * 0.9999f;
+    }
+    __device__ __forceinline__ float lower() const {
+        const float r = rcp32(s_inv.s);
+        const float q = fmaxf(0.0f, s_dd - s_d.s * s_d.s * r + 1e-4f * s_dd);
+        const float xh = fminf(1.0f, ivmax * r * 1.001f), xl = ivmin * r * 0.999f;
+        const float lb = s_l.s + 0.34657f * lg2_32(1.0f + xh) * rcp32(xh) -
+                         0.5f * q * rcp32(1.0f + xl) * 1.0001f - 1e-4f;
+        return lb == lb ? lb : -INFINITY;
     }
     __device__ __forceinline__ void add(const SlotEvent& e) {
         if (isnan(e.s)) return;
-        const float iv = rcp32(e.s * e.s);
-        const float div = e.d * iv;
+        const float iv = rcp32(__fmul_rn(e.s, e.s));
+        const float div = __fmul_rn(e.d, iv);
         s_inv.add(iv);
         s_d.add(div);
         s_dd = fmaf(div, e.d, s_dd);
         ivmax = fmaxf(ivmax, iv);
+        ivmin = fminf(ivmin, iv);
         s_l.add(e.l);
         ++K;
     }
@@ -2011,44 +1992,30 @@ struct SlotPass2 {
     }
     __device__ __forceinline__ void add(float dk, float sg) {
         if (isnan(sg)) return;
-        const float sk2 = sg * sg;
-        const float iden = rcp32(sk2 + s2);
+        const float sk2 = __fmul_rn(sg, sg);
+        const float iden = rcp32(__fadd_rn(sk2, s2));
         const float r = dk - Dl;
-        quad.add(r * r * iden);
-        lsum += lg2_32(sk2 * iden);
+        quad.add_prod(__fmul_rn(r, r), iden);
+        lsum += lg2_32(__fmul_rn(sk2, iden));
     }
 };
+
+__device__ __forceinline__ void write_slot_best(const SlotBest& sb, int64_t o, int64_t n_phi,
+                                                double t_ref, double P, const FoldJob& J) {
+    Best b{-INFINITY, LLONG_MAX, NAN, NAN};
+    if (sb.d >= 0)
+        b = Best{(double)sb.lnp, (long long)sb.d * n_phi + sb.j, (double)sb.Dl,
+                 sqrt((double)sb.s2)};
+    write_best(b, o, n_phi, t_ref, P, J.Q, J.T0, J.Didx, J.dep, J.sig, J.lnp);
+}
 
 // A cell of the slot path that passed the bound, queued for its second pass.
 struct SCell {
     unsigned long long u0;
-    long long cell;
-    float s_l, s2, Dl;
-    int d, kmax, pad;
+    unsigned j;
+    int d, kmax;
+    float s_l, s2, Dl, ub;
 };
-
-// Gain table of the slot path.  An event at walk position u interpolates the
-// records of slots floor(u) and floor(u) + 1, so its gain is at most the
-// pair gain of floor(u): the larger gain of the two records when both are
-// valid (0 otherwise, a dropped event), rounded up (to cover the FP32
-// rounding of the interpolation).  The gain walk reads it at the 64-bit
-// positions that define the events (gain_walk64).  Grouped by duration
-// (gain_slot).
-__global__ void k_slot_gain(const Node4<float>* __restrict__ rec,
-                            const FoldSeg* __restrict__ segs, int n_seg, int64_t n_slots1,
-                            int n_D, int64_t n_out, float* __restrict__ lgm) {
-    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (o >= n_out) return;
-    GainSlot gs;
-    if (!gain_slot(segs, n_seg, n_slots1, n_D, false, o, gs)) return;
-    float m = 0.f;
-    if (gs.d < n_D && gs.s + 1 < gs.n_slots) {
-        const Node4<float>* r = rec + gs.src_off + (int64_t)gs.d * gs.n_slots;
-        const Node4<float> a = r[gs.s], b = r[gs.s + 1];
-        if (!isnan(a.s) && !isnan(b.s)) m = __fmul_ru(fmaxf(0.f, fmaxf(a.l, b.l)), 1.0000005f);
-    }
-    lgm[o] = m;
-}
 
 // Epochs walk the slot grid in 24.40 fixed point: u = (T - t_ref)/dt =
 // (j/n_phi + k) P/dt.  The interval is (slot, slot+1) and the weight is the
@@ -2056,77 +2023,37 @@ __global__ void k_slot_gain(const Node4<float>* __restrict__ rec,
 // interpolation between the bracketing epochs up to their offsets from the
 // slot centres (checked to be below 1e-3 slot).
 //
-// Cascade per warp (no block barriers until the final argmax):
-//   1. gain bound of each cell from lgm (4 bytes per epoch): with the bound
-//      of cannot_win, ln P <= S_L + 1/2, and S_L is at most the sum of the
-//      epochs' lgm; cells below the threshold stop here.  A lane bounds the
-//      cells of one phase and one group of durations (gain_width) in one
-//      walk;
-//   2. queued, 32 at a time: the first pass (FP32 sums) and the bound of
-//      cannot_win_f;
-//   3. queued, 32 at a time: the second pass, whose ln P raises the threshold.
-// A warp's first round skips step 1.  Warps whose gain bounds pass almost
-// every cell (cells of many epochs) skip it for their next rounds, and
-// periods with few cells per warp (short curves) skip the cascade
-// throughout, running the first pass directly: their threshold does not rise
-// in time for the bound to pay.
-// CASC = false compiles the fold without the cascade (its registers spill
-// the plain path's), for grids too small for it (the host decides).
-// (Evaluating the best-bounded cell of the first round at once, as a seed
-// of the threshold, did not pay either.)
-template <int KC, int MAXT = 256, bool CASC = true>
-__device__ __forceinline__ void fold_slots_one(const Node4<float>* __restrict__ rec,
-                                               const float* __restrict__ lgm,
-                                               int64_t n_slots, int n_D, double dt,
-                                               double t_ref, double t_last, double P, int64_t p,
-                                               const SlotPeriod* __restrict__ spp,
-                                               unsigned long long ulast_in,
-                                               double* __restrict__ Q_out,
-                                               double* __restrict__ T0_out,
-                                               int* __restrict__ Didx_out,
-                                               double* __restrict__ dep_out,
-                                               double* __restrict__ sig_out,
-                                               double* __restrict__ lnp_out) {
-    __shared__ SCell sh_q[MAXT / 32][64];
-    __shared__ long long sh_qa[MAXT / 32][CASC ? 160 : 1];   // cells for the first pass
-    __shared__ int sh_qad[MAXT / 32][CASC ? 160 : 1];
-    __shared__ unsigned int sh_best;
-    // the period's constants from the batch's table (spp) or computed here;
-    // the curve's last epoch position from the batch (ulast_in) or here
-    const SlotPeriod spc = spp ? *spp : slot_period(P, dt);
-    if (spc.bad || t_last - t_ref > 1.0e9 * P) {
-        if (threadIdx.x == 0) write_bad(p, Q_out, T0_out, Didx_out, dep_out, sig_out, lnp_out);
-        return;
-    }
-    const unsigned FULL = 0xffffffffu;
-    const int64_t n_phi = spc.n_phi;
-    const int64_t n_cells = n_phi * n_D;
-    const unsigned long long ulast = spp ? ulast_in : slot_ulast(t_ref, t_last, dt);
-    const unsigned long long ustep = spc.ustep, uph = spc.uph;
-    float bl = -INFINITY, bD = NAN, bs2 = NAN;
-    long long bc = LLONG_MAX;
-    if (threadIdx.x == 0) sh_best = 0u;     // key below every finite float
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    SCell* q = sh_q[wid];
-    int nq = 0;                              // warp-uniform queue lengths
-    long long* qa = sh_qa[wid];
-    int* qad = sh_qad[wid];
-    int na = 0;
-    const unsigned ns1 = (unsigned)(n_slots - 1);
-    // the gain walk adds 4 positions past ulast at most: ustep < 2^60 keeps
-    // them from wrapping (ulast < 2^62).  The cascade needs the threshold to
-    // rise before it pays: periods of fewer than NU_CASCADE_ROUNDS rounds of
-    // cells per warp (short light curves) run the first pass on every cell.
-    const bool cascade = CASC && lgm != nullptr && ustep < (1ull << 60) &&
-                         n_cells >= (int64_t)NU_CASCADE_ROUNDS * blockDim.x;
-    auto best_now = [&]() {
-        const unsigned int kb = sh_best;
-        return fmaxf(bl, kb ? __uint_as_float((kb >> 31) ? (kb & 0x7fffffffu) : ~kb)
-                            : -INFINITY);
-    };
+// Per item: the filters, whose tables hold the events of this walk; the first
+// pass (FP32 compensated sums) of the cells they leave, with the bound of
+// cannot_win_f and a lower bound that raises the threshold; and the second
+// pass of the cells whose bound still reaches it, at the end or when 32 are
+// queued.
+struct SlotItem {
+    FilterCtx x;
+    int bad;
+    SlotBest wb[8];
+};
+struct SlotQueues {
+    FilterQueues f;
+    SCell c[64];
+    int n;
+    float bl[32], bD[32], bs2[32];     // each lane's best cell
+    unsigned bj[32];
+    int bd[32];                        // -1: none
+};
+
+struct SlotScreen {
+    SlotItem& it;
+    SlotQueues& q;
+    const Node4<float>* rec;
+    int64_t n_slots;
+    unsigned long long ulast;
+
     // second pass of queued cell e, by one lane
-    auto pass2 = [&](const SCell& e) {
+    __device__ __forceinline__ void pass2(const SCell& e) {
+        if (e.ub + 1e-4f * fmaxf(1.f, fabsf(e.ub)) < filter_thr(it.x)) return;   // overtaken
+        const int lane = threadIdx.x & 31;
+        const unsigned long long ustep = it.x.fp.ustep;
         const Node4<float>* rd = rec + (int64_t)e.d * n_slots;
         SlotPass2 p2;
         p2.init(e.s2, e.Dl);
@@ -2135,302 +2062,231 @@ __device__ __forceinline__ void fold_slots_one(const Node4<float>* __restrict__ 
             const SlotEvent ev = slot_event(rd, u);
             p2.add(ev.d, ev.s);
         }
-        const float lnp = e.s_l - 0.5f * (p2.lsum * 0.693147180559945f + p2.quad.s);
+        const float lnp = e.s_l - 0.5f * __fmaf_rn(p2.lsum, 0.693147180559945f, p2.quad.s);
         if (!(lnp == lnp)) return;
-        if (lnp > bl || (lnp == bl && e.cell < bc)) {
-            bl = lnp;
-            bc = e.cell;
-            bD = p2.Dl;
-            bs2 = p2.s2;
+        const int bd = q.bd[lane];
+        const float bl = q.bl[lane];
+        if (bd < 0 || lnp > bl ||
+            (lnp == bl && (e.d < bd || (e.d == bd && e.j < q.bj[lane])))) {
+            q.bl[lane] = lnp;
+            q.bD[lane] = p2.Dl;
+            q.bs2[lane] = p2.s2;
+            q.bj[lane] = e.j;
+            q.bd[lane] = e.d;
         }
-        const unsigned int b32 = __float_as_uint(lnp);
-        atomicMax(&sh_best, (b32 >> 31) ? ~b32 : (b32 | 0x80000000u));
-    };
-    // first pass and bound of cell (dl, jl); *ub receives the bound (-inf:
-    // no event) and e the queue entry; returns whether the cell is kept
-    auto pass1 = [&](int dl, int64_t jl, long long cl, SCell& e, float* ub) -> bool {
-        *ub = -INFINITY;
-        const unsigned long long u0 = (unsigned long long)jl * uph;
-        if (u0 > ulast) return false;
-        // epochs with u <= ulast, counted as they are walked
-        const Node4<float>* rd = rec + (int64_t)dl * n_slots;
-        SlotPass1 p1;
-        p1.init();
-        int kmax = 0;
-        // two epochs' record loads in flight
-#pragma unroll 2
-        for (unsigned long long u = u0; u <= ulast; u += ustep, ++kmax) p1.add(slot_event(rd, u));
-        if (p1.K == 0) return false;
-        *ub = p1.s_l.s + 0.5f;
-        if (cannot_win_f(p1.s_l.s, p1.s_inv.s, p1.s_d.s, p1.s_dd, p1.ivmax, best_now()))
-            return false;
-        const float s2 = 1.0f / p1.s_inv.s;
-        e = SCell{u0, cl, p1.s_l.s, s2, s2 * p1.s_d.s, dl, kmax, 0};
-        return true;
-    };
-    auto push_b = [&](bool keep, const SCell& e) {
-        const unsigned m = __ballot_sync(FULL, keep);
-        if (keep) q[nq + __popc(m & ((1u << lane) - 1u))] = e;
-        nq += __popc(m);
+        filter_raise(it.x, fkey(screen_threshold<float>(lnp, it.x.fp.K)));
+    }
+    __device__ __noinline__ void flush(int cnt) {
+        const int lane = threadIdx.x & 31;
+        if (lane < cnt) pass2(q.c[lane]);
         __syncwarp();
-    };
-    auto flush_b = [&]() {
-        pass2(q[lane]);
-        __syncwarp();
-        nq -= 32;
-        SCell e2;
-        if (lane < nq) e2 = q[32 + lane];
-        __syncwarp();
-        if (lane < nq) q[lane] = e2;
-        __syncwarp();
-    };
-    // first passes of the first cnt entries of queue A, one per lane; the
-    // survivors join queue B, which is flushed at once when it holds 32 (so
-    // it never holds more than 63 entries)
-    auto flush_a = [&](int h, int cnt) {
+    }
+
+    // first pass and bounds of the queue's first cnt cells
+    __device__ __noinline__ void operator()(int cnt) {
+        const unsigned FULL = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        const unsigned long long ustep = it.x.fp.ustep;
         SCell e;
-        float ub;
         bool keep = false;
+        float lb = -INFINITY;
         if (lane < cnt) {
-            const long long cl = qa[h + lane];
-            const int dl = qad[h + lane];
-            keep = pass1(dl, cl - (int64_t)dl * n_phi, cl, e, &ub);
-        }
-        push_b(keep, e);
-        if (nq >= 32) flush_b();
-    };
-    if (cascade) {
-        // cells W durations at a time (one gain group, one phase per lane),
-        // as in the FP64 fold: the first and the direct rounds pass every
-        // cell to queue A, the others those whose gain bound reaches the
-        // threshold (with the margins of cannot_win_f on top of the rounding
-        // of the sum)
-        const int W = gain_width(n_D);
-        const int64_t n_gc = (int64_t)((n_D + W - 1) / W) * n_phi;
-        const int dr = NU_GAIN_DIRECT_ROUNDS / W > 0 ? NU_GAIN_DIRECT_ROUNDS / W : 1;
-        const unsigned zs = ns1 - 1u;
-        int gi = (int)(threadIdx.x / n_phi);
-        int64_t j = (int64_t)threadIdx.x - (int64_t)gi * n_phi;
-        bool first = true;
-        int direct = 0;                      // rounds left without the gain bound
-        for (int64_t base = (int64_t)wid * 32; base < n_gc; base += blockDim.x,
-                     j += blockDim.x) {
-            while (j >= n_phi) {
-                j -= n_phi;
-                ++gi;
-            }
-            const int d0 = gi * W;
-            const int nv = base + lane < n_gc ? min(W, n_D - d0) : 0;   // this lane's cells
-            unsigned pass = 0u;
-            if (first || direct > 0) {
-                if (!first) --direct;
-                first = false;
-                pass = (1u << nv) - 1u;
-            } else {
-                if (nv > 0) {
-                    float4 sk;
-                    const float K = gain_walk64(lgm + (int64_t)gi * n_slots * W, W, zs,
-                                                (unsigned long long)j * uph, ustep, ulast + 1,
-                                                sk);
-                    const float f = fmaf(K + 16.f, 1.1920929e-7f, 1.f);
-                    const float thr = best_now();
-                    if (K > 0.f)
-                        for (int i = 0; i < nv; ++i) {
-                            const float gb = gain_col(sk, i) * f + 0.5f;
-                            if (!(gb + 1e-4f * fmaxf(1.f, fabsf(gb)) < thr)) pass |= 1u << i;
-                        }
-                }
-                const int np = __reduce_add_sync(FULL, (unsigned)__popc(pass));
-                const int nt = __reduce_add_sync(FULL, (unsigned)nv);
-                if (nt > 0 && np * 32 >= NU_GAIN_PASS_MAX * nt) direct = dr;
-            }
-            for (int i = 0; i < W; ++i) {
-                const bool keep = (pass >> i) & 1u;
-                const unsigned m = __ballot_sync(FULL, keep);
-                if (keep) {
-                    const int pos = na + __popc(m & ((1u << lane) - 1u));
-                    qa[pos] = (long long)(d0 + i) * n_phi + j;
-                    qad[pos] = d0 + i;
-                }
-                na += __popc(m);
-                __syncwarp();
-            }
-            // queue A holds at most 31 + 32 W entries here
-            int h = 0;
-            for (; na - h >= 32; h += 32) flush_a(h, 32);
-            if (h > 0) {
-                na -= h;
-                long long c2 = 0;
-                int d2 = 0;
-                if (lane < na) {
-                    c2 = qa[h + lane];
-                    d2 = qad[h + lane];
-                }
-                __syncwarp();
-                if (lane < na) {
-                    qa[lane] = c2;
-                    qad[lane] = d2;
-                }
-                __syncwarp();
+            const uint2 cl = q.f.cell[lane];
+            const unsigned long long u0 = (unsigned long long)cl.x * it.x.fp.uph;
+            const Node4<float>* rd = rec + (int64_t)cl.y * n_slots;
+            SlotPass1 p1;
+            p1.init();
+            int kmax = 0;
+            // two epochs' record loads in flight
+#pragma unroll 2
+            for (unsigned long long u = u0; u <= ulast; u += ustep, ++kmax)
+                p1.add(slot_event(rd, u));
+            if (p1.K > 0) {
+                lb = p1.lower();
+                e.ub = p1.upper();
+                keep = !(e.ub + 1e-4f * fmaxf(1.f, fabsf(e.ub)) < filter_thr(it.x));
+                e.s2 = 1.0f / p1.s_inv.s;
+                e.Dl = e.s2 * p1.s_d.s;
+                e.s_l = p1.s_l.s;
+                e.u0 = u0;
+                e.j = cl.x;
+                e.d = (int)cl.y;
+                e.kmax = kmax;
             }
         }
-        if (na > 0) flush_a(0, na);
+        const unsigned k = __reduce_max_sync(FULL, fkey(screen_threshold<float>(lb, it.x.fp.K)));
+        if (lane == 0) filter_raise(it.x, k);
+        const unsigned m = __ballot_sync(FULL, keep);
+        int n = q.n;
+        if (keep) q.c[n + __popc(m & ((1u << lane) - 1u))] = e;
+        n += __popc(m);
+        __syncwarp();
+        if (n >= 32) {
+            flush(32);
+            n -= 32;
+            SCell e2;
+            if (lane < n) e2 = q.c[32 + lane];
+            __syncwarp();
+            if (lane < n) q.c[lane] = e2;
+            __syncwarp();
+        }
+        if (lane == 0) q.n = n;
+        __syncwarp();
+    }
+};
+
+__device__ __forceinline__ float slot_K(const FoldSeg& fs, const SlotPeriod& sp) {
+    return (float)(unsigned)(fs.ulast >> 32) / (float)max((unsigned)(sp.ustep >> 32), 1u);
+}
+// The slot path's list, as k_item_consts.
+__global__ void k_slot_items(const __grid_constant__ FoldJob J) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    bool in = i < (int64_t)J.n_seg * J.n_P, heavy = false;
+    int64_t o = 0;
+    if (in) {
+        const int64_t seg = J.n_seg == 1 ? 0 : i / J.n_P;
+        const int64_t p = period_slot(i - seg * J.n_P, J.periods, J.n_P);
+        o = seg * J.n_P + p;
+        const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+        if (!fs.use_slots) {
+            in = false;
+        } else {
+            heavy = !(slot_K(fs, J.stab[p]) < J.list.heavy_k);
+        }
+    }
+    list_item(J.list, in && heavy, (unsigned)o);
+}
+
+// One item of the slot path by the nw warps that share it.
+template <int nw>
+__device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int w, SlotItem& it,
+                                                SlotQueues& q) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t seg = J.n_seg == 1 ? 0 : o / J.n_P;
+    const int64_t p = o - seg * J.n_P;
+    const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+    if (!fs.use_slots) return;
+    if (nw < 8 && J.list.block && !(slot_K(fs, J.stab[p]) < J.list.heavy_k)) return;
+    const int n_D = J.n_D;
+    if (lane == 0) q.f.ni = q.f.nq = q.f.nc = q.n = 0;
+    q.bd[lane] = -1;
+    q.bl[lane] = -INFINITY;
+    if (w == 0 && lane == 0) {
+        const double P = J.periods[p];
+        const SlotPeriod sp = J.stab ? J.stab[p] : slot_period(P, J.dt);
+        it.bad = sp.bad || fs.t_last - fs.t_ref > 1.0e9 * P;
+        FilterPeriod f;
+        f.ustep = sp.ustep;
+        f.uph = sp.uph;
+        f.uend = fs.ulast + 1ull;
+        f.n_phi = sp.n_phi;
+        const float K = slot_K(fs, sp);
+        f.K = K + 2.f;
+        f.mode = filter_mode(J.tab.S != nullptr, sp.ustep, K, f.n_phi * n_D);
+        it.x.fp = f;
+        it.x.f = filter_view(J.tab, fs);
+        it.x.n_D = n_D;
+        it.x.bfk = fkey(-INFINITY);
+    }
+    item_sync<nw>();
+    if (it.bad) {
+        if (w == 0 && lane == 0) {
+            write_bad(o, J.Q, J.T0, J.Didx, J.dep, J.sig, J.lnp);
+            if (J.sbest) J.sbest[o].d = -2;
+        }
+        return;
+    }
+    SlotScreen screen{it, q, J.rec + fs.rec_off, fs.n_slots, fs.ulast};
+    if (it.x.fp.mode != FILTER_NONE) {
+        const unsigned long long pk = J.peak[seg];
+        if (pk != 0 && w == 0) {
+            const unsigned e = 0xffffffffu - (unsigned)(pk & 0xffffffffu);
+            const unsigned pd = e / (unsigned)fs.n_t0;
+            const double x = (J.t[fs.s_off + (e - pd * (unsigned)fs.n_t0)] - fs.t_ref) * J.inv_dt;
+            const unsigned long long u = (unsigned long long)llrint(fmax(x, 0.0)) << 40;
+            if (lane < 8)
+                q.f.cell[lane] = make_uint2(
+                    seed_phase(u, it.x.fp.ustep, it.x.fp.uph, it.x.fp.n_phi, lane), pd);
+            __syncwarp();
+            screen(8);
+            __syncwarp();
+        }
+        item_sync<nw>();
+        filter_cells(it.x, w, nw, q.f, screen);
     } else {
-        int d = (int)(threadIdx.x / n_phi);
-        int64_t j = (int64_t)threadIdx.x - (int64_t)d * n_phi;
-        for (int64_t base = (int64_t)wid * 32; base < n_cells; base += blockDim.x,
-                     j += blockDim.x) {
-            while (j >= n_phi) {
-                j -= n_phi;
-                ++d;
-            }
-            const int64_t cell = base + lane;
-            SCell e;
-            float ub = -INFINITY;
-            const bool keep = cell < n_cells && pass1(d, j, cell, e, &ub);
-            push_b(keep, e);
-            if (nq >= 32) flush_b();
+        const int64_t n_phi = it.x.fp.n_phi, n_cells = n_phi * n_D;
+        for (int64_t base = (int64_t)w * 32; base < n_cells; base += nw * 32) {
+            const int64_t cell = min(base + lane, n_cells - 1);
+            const unsigned d = (unsigned)(cell / n_phi);
+            q.f.cell[lane] = make_uint2((unsigned)(cell - (int64_t)d * n_phi), d);
+            __syncwarp();
+            screen((int)min((int64_t)32, n_cells - base));
+            __syncwarp();
         }
     }
-    if (nq >= 32) flush_b();
-    if (lane < nq) pass2(q[lane]);
-    // block argmax in FP32 (larger ln P, ties to the smaller cell): warp
-    // shuffles, then the warps' winners through shared memory; FP64 only for
-    // the one result (the FP64 pipe is 1/64 of the FP32 one on this part)
-    for (int o = 16; o > 0; o >>= 1) {
-        const float l2 = __shfl_xor_sync(FULL, bl, o);
-        const long long c2 = __shfl_xor_sync(FULL, bc, o);
-        const float D2 = __shfl_xor_sync(FULL, bD, o);
-        const float s2 = __shfl_xor_sync(FULL, bs2, o);
-        if (l2 > bl || (l2 == bl && c2 < bc)) {
-            bl = l2;
-            bc = c2;
-            bD = D2;
-            bs2 = s2;
-        }
+    item_sync<nw>();
+    screen.flush(q.n);
+    // argmax in FP32 (larger ln P, ties to the smaller cell)
+    SlotBest sb{q.bl[lane], q.bD[lane], q.bs2[lane], q.bj[lane], q.bd[lane]};
+    auto over = [](const SlotBest& a, const SlotBest& b) {   // a beats b
+        if (a.d < 0) return false;
+        if (b.d < 0 || a.lnp > b.lnp) return true;
+        return a.lnp == b.lnp && (a.d < b.d || (a.d == b.d && a.j < b.j));
+    };
+    for (int s = 16; s > 0; s >>= 1) {
+        const SlotBest b{__shfl_xor_sync(FULL, sb.lnp, s), __shfl_xor_sync(FULL, sb.Dl, s),
+                         __shfl_xor_sync(FULL, sb.s2, s), __shfl_xor_sync(FULL, sb.j, s),
+                         __shfl_xor_sync(FULL, sb.d, s)};
+        if (over(b, sb)) sb = b;
     }
-    __shared__ float sh_bl[MAXT / 32], sh_bD[MAXT / 32], sh_bs2[MAXT / 32];
-    __shared__ long long sh_bc[MAXT / 32];
-    if (lane == 0) {
-        sh_bl[wid] = bl;
-        sh_bc[wid] = bc;
-        sh_bD[wid] = bD;
-        sh_bs2[wid] = bs2;
+    if (nw > 1) {
+        if (lane == 0) it.wb[w] = sb;
+        __syncthreads();
+        if (w == 0 && lane == 0)
+            for (int i = 1; i < nw; ++i)
+                if (over(it.wb[i], sb)) sb = it.wb[i];
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            if (sh_bl[w] > bl || (sh_bl[w] == bl && sh_bc[w] < bc)) {
-                bl = sh_bl[w];
-                bc = sh_bc[w];
-                bD = sh_bD[w];
-                bs2 = sh_bs2[w];
-            }
-        Best b{-INFINITY, LLONG_MAX, NAN, NAN};
-        if (bc != LLONG_MAX) b = Best{(double)bl, bc, (double)bD, sqrt((double)bs2)};
-        write_best(b, p, n_phi, t_ref, P, Q_out, T0_out, Didx_out, dep_out, sig_out, lnp_out);
+    if (w == 0 && lane == 0) {
+        if (J.sbest)
+            J.sbest[o] = sb;                  // k_slot_best writes the outputs
+        else
+            write_slot_best(sb, o, it.x.fp.n_phi, fs.t_ref, J.periods[p], J);
     }
 }
 
-#ifndef NU_SLOTS_SMALL
-#define NU_SLOTS_SMALL 128         // block size of the mixed fold on large grids
-#endif
-#ifndef NU_SLOTS_SMALL_FROM
-#define NU_SLOTS_SMALL_FROM 8192   // periods from which it is used
-#endif
-#ifndef NU_SLOTS_MIN_BLOCKS
-#define NU_SLOTS_MIN_BLOCKS 4
-#endif
-#ifndef NU_SLOTS_CASC_MIN_BLOCKS
-#define NU_SLOTS_CASC_MIN_BLOCKS 4
-#endif
+template <int NW>
+__global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
+k_fold_slot_cells(const __grid_constant__ FoldJob J) {
+    constexpr int W = fold_threads(NW) / 32;
+    __shared__ SlotQueues sh_q[W];
+    __shared__ SlotItem sh_i[W / NW];
+    const int wid = threadIdx.x >> 5;
+    int64_t item = 0;
+    if (NW == 8) {
+        __shared__ unsigned sh_k;
+        for (int k = 0; next_item(J, k, &sh_k, item); ++k)
+            fold_slots_item<NW>(J, item, wid, sh_i[0], sh_q[wid]);
+    } else if (warp_item<NW>(J, item)) {
+        fold_slots_item<NW>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid]);
+    }
+}
 
-template <int KC, int MAXT, bool CASC>
-__global__ void __launch_bounds__(MAXT, (CASC ? NU_SLOTS_CASC_MIN_BLOCKS : NU_SLOTS_MIN_BLOCKS) * 256 / MAXT)
-k_fold_slots(const Node4<float>* __restrict__ rec, const float* __restrict__ lgm,
-             int64_t n_slots, int n_D, double dt, double t_ref, double t_last,
-             const double* __restrict__ periods, int64_t n_P, double* __restrict__ Q_out,
-             double* __restrict__ T0_out, int* __restrict__ Didx_out,
-             double* __restrict__ dep_out, double* __restrict__ sig_out,
-             double* __restrict__ lnp_out) {
-    if ((int64_t)blockIdx.x >= n_P) return;
-    const int64_t p = period_slot(blockIdx.x, periods, n_P);
-    fold_slots_one<KC, MAXT, CASC>(rec, lgm, n_slots, n_D, dt, t_ref, t_last, periods[p], p,
-                                   nullptr, 0ull,
-                                   Q_out, T0_out, Didx_out, dep_out, sig_out, lnp_out);
+// Outputs of the slot path, one thread per item: the FP64 divisions and roots
+// of 32 items in one warp instruction.
+__global__ void k_slot_best(const __grid_constant__ FoldJob J) {
+    const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (o >= (int64_t)J.n_seg * J.n_P) return;
+    const int64_t seg = J.n_seg == 1 ? 0 : o / J.n_P;
+    const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
+    if (!fs.use_slots) return;
+    const SlotBest sb = J.sbest[o];
+    if (sb.d == -2) return;
+    const int64_t p = o - seg * J.n_P;
+    write_slot_best(sb, o, J.stab[p].n_phi, fs.t_ref, J.periods[p], J);
 }
 
 // ------------------------------------------------------------ batch path
-
-// Persistent fold over (curve, period) work items taken from a device
-// counter (no waits: a block takes items until none are left).  kind 0 / 4:
-// the screened path with FP64 values (one duration / grouped gain walk);
-// 1 / 5: the same with FP32 values (mixed precision, grids that are not
-// regular); 2 / 3: slot path (mixed precision, regular grids; with / without
-// the cascade).  Items of curves that do not use this kernel's path are
-// skipped.
-// Resident blocks per SM the registers are sized for, by path and block size.
-// The FP64 batch kernel carries the work-item loop besides the screen: at 80
-// registers it spills, at 96 (10 x 64 threads) it does not; slots as the
-// single-curve kernel (64 registers at any size).
-template <int KIND, int MAXT>
-struct BatchBlocks {
-    static constexpr int value =
-        KIND == 2 ? NU_SLOTS_CASC_MIN_BLOCKS * 256 / MAXT
-                  : (KIND == 3 ? NU_SLOTS_MIN_BLOCKS * 256 / MAXT
-                               : (MAXT <= 64 ? 10 : (MAXT <= 128 ? 5 : NU_SCREEN_MIN_BLOCKS)));
-};
-template <int KIND> struct BatchEvent { typedef double T; };
-template <> struct BatchEvent<1> { typedef float T; };
-template <> struct BatchEvent<5> { typedef float T; };
-
-template <int KIND, int MAXT>
-__global__ void __launch_bounds__(MAXT, BatchBlocks<KIND, MAXT>::value)
-k_fold_batch(const FoldSeg* __restrict__ segs, int n_seg, const double* __restrict__ t,
-             const void* __restrict__ nodes, const ScreenRec* __restrict__ screen,
-             const ulonglong2* __restrict__ vpair, const ScreenRec* __restrict__ srec,
-             const float* __restrict__ lgm, const unsigned* __restrict__ reg,
-             const unsigned long long* __restrict__ peak,
-             const int* __restrict__ bucket,
-             const Node4<float>* __restrict__ rec, int n_D, double dt, double gap_factor,
-             const double* __restrict__ periods, const PeriodConst* __restrict__ ptab,
-             int64_t n_P, unsigned long long* counter,
-             double* __restrict__ Q_out, double* __restrict__ T0_out,
-             int* __restrict__ Didx_out, double* __restrict__ dep_out,
-             double* __restrict__ sig_out, double* __restrict__ lnp_out) {
-    __shared__ unsigned long long item_sh;
-    const unsigned long long total = (unsigned long long)n_seg * (unsigned long long)n_P;
-    while (true) {
-        __syncthreads();
-        if (threadIdx.x == 0) item_sh = atomicAdd(counter, 1ull);
-        __syncthreads();
-        const unsigned long long item = item_sh;
-        if (item >= total) break;
-        const int g = (int)(item / (unsigned long long)n_P);
-        const int64_t p = period_slot((int64_t)(item % (unsigned long long)n_P), periods, n_P);
-        const FoldSeg fs = segs[g];
-        if ((KIND == 2 || KIND == 3) != (fs.use_slots != 0)) continue;
-        const int64_t o = (int64_t)g * n_P + p;
-        if (KIND == 2 || KIND == 3) {
-            // (the slot path's period table shares the FP64 path's buffer)
-            fold_slots_one<8, MAXT, KIND == 2>(
-                rec + fs.rec_off, lgm + fs.gain_off, fs.n_slots, n_D, dt, fs.t_ref, fs.t_last,
-                periods[p], o, reinterpret_cast<const SlotPeriod*>(ptab) + p, fs.ulast, Q_out,
-                T0_out, Didx_out, dep_out, sig_out, lnp_out);
-        } else {
-            FoldGeom gg{t + fs.s_off, fs.n_t0, fs.t_ref, fs.t_last, dt, 1.0 / dt,
-                        gap_factor * dt, bucket + fs.bucket_off, fs.n_bucket};
-            typedef typename BatchEvent<KIND>::T T;
-            const ScreenGeom sg{screen + fs.s_off * n_D, vpair + fs.s_off,
-                                sizeof(T) == 8 ? srec + fs.srec_off : nullptr, fs.n_slots,
-                                reg + 2 * g, fs.screen, peak + g, lgm + fs.gain_off,
-                                sizeof(T) == 4};
-            fold_screened_one<T, MAXT, true, KIND == 4 || KIND == 5>(
-                gg, sg, (const Node8<T>*)nodes + fs.s_off * n_D, n_D, periods[p], o, Q_out,
-                T0_out, Didx_out, dep_out, sig_out, lnp_out, ptab + p);
-        }
-    }
-}
 
 // Per-curve node records (exact path) and bucket tables; slot tables.
 template <typename T>
@@ -2458,7 +2314,6 @@ __global__ void k_screen_batch(const T* __restrict__ depth, const T* __restrict_
                                const int64_t* __restrict__ s_off, int n_D, double gap_max,
                                double dt, ScreenRec* __restrict__ rec,
                                ulonglong2* __restrict__ vpair, ScreenRec* __restrict__ srec,
-                               Node8<T>* __restrict__ nodes,
                                const int* __restrict__ slot_of) {
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (gid >= s_off[n_seg] * (int64_t)n_D) return;
@@ -2473,7 +2328,7 @@ __global__ void k_screen_batch(const T* __restrict__ depth, const T* __restrict_
     const int64_t w = gid - s0 * n_D;
     const int64_t d = w / ng, i = w - d * ng;
     make_screen<T>(depth, var, gain, t + s0, gid, i, ng, d, gap_max, dt, rec,
-                   srec ? srec + fs.srec_off : nullptr, nodes, fs.n_slots,
+                   srec ? srec + fs.srec_off : nullptr, fs.n_slots,
                    slot_of + s0, vpair + s0);
 }
 
@@ -2577,6 +2432,7 @@ void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double
         f.t_ref = t_first[g];
         f.t_last = t_last[g];
         f.ulast = slot_ulast(f.t_ref, f.t_last, dt);
+        f.uspan = exact_uspan(f.t_ref, f.t_last, dt);
         const double span = (t_last[g] - t_first[g]) / dt;
         f.n_bucket = (int64_t)span + 2;
         f.n_slots = f.n_bucket + 2;
@@ -2585,17 +2441,78 @@ void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double
         f.screen = (!f.use_slots && gap_factor < 2.0 && span < 8.0e6) ? 1 : 0;
         f.srec_off = fb.n_srec_total;
         fb.n_srec_total += fp64 && f.screen ? f.n_slots * n_D : 0;
-        f.gain_off = fb.n_gain_total;
-        fb.n_gain_total += f.screen || f.use_slots ? f.n_slots * gain_cols(n_D) : 0;
+        f.tab_off = fb.n_tab_total;
+        f.g_off = fb.n_g_total;
+        if (f.screen || f.use_slots) {
+            const int64_t ns = filter_slots(f.n_slots);
+            f.pair_off = fb.n_pair_total;
+            fb.n_pair_total += ns * ((n_D + 1) / 2 * 2);
+            fb.n_tab_total += ns * n_D;
+            fb.n_g_total += ns * filter_groups(n_D) * filter_words(n_D);
+        }
         f.bucket_off = fb.n_bucket_total;
         fb.n_bucket_total += f.use_slots ? 0 : f.n_bucket;
         f.rec_off = fb.n_rec_total;
         fb.n_rec_total += f.use_slots ? f.n_slots * n_D : 0;
         fb.any_slots = fb.any_slots || f.use_slots;
-        if (f.use_slots && f.n_slots * (int64_t)n_D >= (int64_t)NU_CASCADE_ROUNDS * 128)
-            fb.slot_cascade = true;
         fb.any_exact = fb.any_exact || !f.use_slots;
     }
+}
+
+size_t fold_scratch(const FoldBatch& fb, int64_t n_total, int n_lc, int n_D, int64_t n_P,
+                    bool fp64, char* base, FoldScratch* fs) {
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        char* p = base ? base + off : nullptr;
+        off += (bytes + 255) / 256 * 256;
+        return p;
+    };
+    const int64_t items = (int64_t)n_lc * n_P;
+    FoldScratch f;
+    f.nodes = take(fb.any_exact ? exact_layout(n_total, n_D, fp64).total : 0);
+    f.bucket = (int*)take((size_t)(fb.n_bucket_total + 1) * 4);
+    f.rec = (Node4<float>*)take((size_t)(fb.n_rec_total + 1) * sizeof(Node4<float>));
+    f.srec = (ScreenRec*)take((size_t)(fb.n_srec_total + 1) * sizeof(ScreenRec));
+    f.slot_of = (int*)take(fp64 ? (size_t)n_total * sizeof(int) : 0);
+    f.reg = (unsigned*)take((size_t)n_lc * 2 * sizeof(unsigned));
+    f.peak = (unsigned long long*)take((size_t)n_lc * sizeof(unsigned long long));
+    f.ptab = (PeriodConst*)take((size_t)n_P * period_const_bytes());
+    const FilterLayout F = filter_layout(fb.n_tab_total, fb.n_pair_total, fb.n_g_total,
+                                          (int64_t)n_lc * n_D);
+    char* tab = take(F.total);
+    f.tab = base ? filter_tab(tab, F) : FilterTab{};
+    // one item leaves a few cells; an item that finds the list full evaluates
+    // its own
+    f.cap = fb.any_exact ? (unsigned long long)std::min<int64_t>(4 * items + 4096, 1ll << 30) : 0;
+    f.cand = (FoldCand*)take((size_t)f.cap * sizeof(FoldCand));
+    f.n_list = (unsigned*)take(32);
+    f.n_cand = (unsigned long long*)(f.n_list + 4);
+    f.list = (unsigned*)take((size_t)items * sizeof(unsigned));
+    f.range = (int2*)take(fb.any_exact ? (size_t)items * sizeof(int2) : 0);
+    f.items = (ItemConst*)take(fb.any_exact ? (size_t)items * sizeof(ItemConst) : 0);
+    f.sbest = (SlotBest*)take(fb.any_slots ? (size_t)items * sizeof(SlotBest) : 0);
+    if (fs) *fs = f;
+    return off;
+}
+
+// The filter tables of every curve (the records they are built from are
+// there).  Returns the first error of the memset.
+static cudaError_t launch_filter_tables(const FoldSeg* segs, const FoldSeg& one, int n_seg,
+                                        int n_D, int64_t n_entries, int64_t n_t0,
+                                        const ScreenRec* screen, const ulonglong2* vpair,
+                                        const int* bucket, const Node4<float>* rec,
+                                        const FilterTab& tab, cudaStream_t st, int* launched) {
+    if (n_entries == 0) return cudaSuccess;
+    const int64_t rows = (int64_t)n_seg * n_D;
+    const cudaError_t e = cudaMemsetAsync(tab.vmax, 0, (size_t)rows * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    const unsigned gy = (unsigned)std::min<int64_t>(std::max<int64_t>(n_t0 / 2048, 1), 64);
+    k_filter_vmax<<<dim3((unsigned)rows, gy), 256, 0, st>>>(screen, rec, segs, one, n_D, tab.vmax);
+    k_filter_slots<<<div_up(n_entries, 128), 128, 0, st>>>(screen, vpair, bucket, rec, segs, one,
+                                                           n_seg, n_D, n_entries, tab);
+    k_filter_groups<<<div_up(n_entries, 256), 256, 0, st>>>(segs, one, n_seg, n_D, n_entries, tab);
+    *launched += 3;
+    return cudaSuccess;
 }
 
 cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
@@ -2606,21 +2523,18 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
     int launched = 0;
     *n_launched = 0;
     const int64_t ngrid = n_total * (int64_t)n_D;
-    cudaError_t e = cudaSuccess;
+    const ExactLayout L = exact_layout(n_total, n_D, fp64);
+    ScreenRec* screen = (ScreenRec*)((char*)fs.nodes + L.off_screen);
+    ulonglong2* vpair = (ulonglong2*)((char*)fs.nodes + L.off_vpos);
+    cudaError_t e = cudaMemsetAsync(fs.peak, 0, (size_t)n_seg * sizeof(unsigned long long), st);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(fs.reg, 0, (size_t)n_seg * 2 * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    const dim3 peak_grid(n_seg, 1);
     if (fb.any_exact) {
-        const ExactLayout L = exact_layout(n_total, n_D, fp64);
-        ScreenRec* screen = (ScreenRec*)((char*)fs.nodes + L.off_screen);
-        ulonglong2* vpair = (ulonglong2*)((char*)fs.nodes + L.off_vpos);
         k_buckets_batch<<<div_up(fb.n_bucket_total, 256), 256, 0, st>>>(
             t, segs_dev, n_seg, fb.n_bucket_total, dt, fs.bucket);
         ++launched;
-        e = cudaMemsetAsync(fs.peak, 0, (size_t)n_seg * sizeof(unsigned long long), st);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(fs.reg, 0, (size_t)n_seg * 2 * sizeof(unsigned), st);
-        if (e != cudaSuccess) {
-            *n_launched = launched;
-            return e;
-        }
         if (fp64) {
             k_nodes_batch<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth, (const double*)var, (const double*)gain, t, segs_dev,
@@ -2631,28 +2545,16 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
                 fs.srec, fb.n_srec_total);
             k_screen_batch<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth, (const double*)var, (const double*)gain, t, segs_dev,
-                n_seg, s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, fs.srec,
-                (Node8<double>*)fs.nodes, fs.slot_of);
-            k_gain_peak<double><<<dim3(n_seg, 1), 256, 0, st>>>((const double*)gain, s_off_dev,
-                                                               0, n_D, fs.peak);
-            k_gain_table<double><<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
-                (const Node8<double>*)fs.nodes, vpair, fs.bucket, segs_dev, n_seg, 0, 0, 0, n_D,
-                fb.n_gain_total, fs.lgm);
-            launched += 6;
+                n_seg, s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, fs.srec, fs.slot_of);
+            launched += 4;
         } else {
             k_nodes_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
                 s_off_dev, n_D, gap_factor * dt, (Node8<float>*)fs.nodes);
             k_screen_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
-                s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, nullptr,
-                (Node8<float>*)fs.nodes, nullptr);
-            k_gain_peak<float><<<dim3(n_seg, 1), 256, 0, st>>>((const float*)gain, s_off_dev, 0,
-                                                              n_D, fs.peak);
-            k_gain_table<float><<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
-                (const Node8<float>*)fs.nodes, vpair, fs.bucket, segs_dev, n_seg, 0, 0, 0, n_D,
-                fb.n_gain_total, fs.lgm);
-            launched += 4;
+                s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, nullptr, nullptr);
+            launched += 2;
         }
     }
     if (fb.any_slots) {
@@ -2660,61 +2562,148 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
         k_slot_fill_batch<<<div_up(ngrid, 256), 256, 0, st>>>(
             (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
             s_off_dev, n_D, 1.0 / dt, fs.rec);
-        k_slot_gain<<<div_up(fb.n_gain_total + 1, 256), 256, 0, st>>>(
-            fs.rec, segs_dev, n_seg, 0, n_D, fb.n_gain_total, fs.lgm);
-        launched += 3;
+        launched += 2;
     }
+    if (fp64)
+        k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)gain, s_off_dev, 0, n_D,
+                                                       fs.peak);
+    else
+        k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)gain, s_off_dev, 0, n_D,
+                                                      fs.peak);
+    ++launched;
+    e = launch_filter_tables(segs_dev, FoldSeg{}, n_seg, n_D, fb.n_tab_total, n_total / n_seg,
+                             screen, vpair, fs.bucket, fs.rec, fs.tab, st, &launched);
     *n_launched = launched;
-    return cudaSuccess;
+    return e;
 }
 
-// The persistent fold kernels; counter[0..1] must be zero.  blocks_per_sm
-// and threads come from the autotuner.
+// The cell kernels of one job: the exact paths' items, then the slot path's.
+// nw = 1 or 2 warps per item; with a list, its items run in eight-warp blocks on
+// the side stream meanwhile.  nw = 8: every item in such a block.
+static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int nw,
+                        cudaStream_t st, cudaStream_t side, cudaError_t* err) {
+    const int64_t items = (int64_t)J.n_seg * J.n_P;
+    int launched = 0;
+    int dev = 0, n_sm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    auto check = [&](cudaError_t e) {
+        if (e != cudaSuccess && *err == cudaSuccess) *err = e;
+    };
+    if (nw == 2 && items > 0x7fffffffLL) nw = 1;          // the grid's limit
+    const int g8 = (int)std::min<int64_t>(items, (int64_t)n_sm * (NU_FOLD_WARPS / 8));
+#define NU_CELLS(NW_, GRID_, ST_)                                                          \
+    do {                                                                                   \
+        if (path == 1) k_fold_slot_cells<NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J);    \
+        else if (fp64) k_fold_cells<double, NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J); \
+        else k_fold_cells<float, NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J);            \
+        ++launched;                                                                        \
+    } while (0)
+    for (int path = 0; path < 2; ++path) {
+        if (!(path == 0 ? exact : slots)) continue;
+        // the list's counters and, behind them, the candidates'
+        if (J.cand || J.list.block) check(cudaMemsetAsync(J.counters, 0, 32, st));
+        if (path == 0 && J.items) {
+            k_item_consts<<<div_up(items, 128), 128, 0, st>>>(J, fp64 ? 0 : 1);
+            ++launched;
+        }
+        if (path == 1 && J.list.block) {
+            k_slot_items<<<div_up(items, 128), 128, 0, st>>>(J);
+            ++launched;
+        }
+        if (nw == 8) {
+            NU_CELLS(8, g8, st);
+        } else {
+            cudaEvent_t fork = nullptr, join = nullptr;
+            bool forked = false;
+            if (J.list.block) {
+                forked = side && side != st &&
+                         cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
+                         cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess &&
+                         cudaEventRecord(fork, st) == cudaSuccess &&
+                         cudaStreamWaitEvent(side, fork, 0) == cudaSuccess;
+                const cudaStream_t hs = forked ? side : st;
+                NU_CELLS(8, g8, hs);
+                if (forked) check(cudaEventRecord(join, side));
+            }
+            if (nw == 2) NU_CELLS(2, (unsigned)items, st);
+            else NU_CELLS(1, div_up(items, 4), st);
+            if (forked) check(cudaStreamWaitEvent(st, join, 0));
+            if (fork) cudaEventDestroy(fork);
+            if (join) cudaEventDestroy(join);
+        }
+        if (path == 0 && J.cand) {
+            // a warp per 32 cells, enough warps that each takes few rounds
+            const int eg = (int)std::min<int64_t>(div_up(items, 16), n_sm * 16);
+            if (fp64) k_cand_eval<double><<<eg, 64, 0, st>>>(J);
+            else k_cand_eval<float><<<eg, 64, 0, st>>>(J);
+            k_cand_best<<<div_up(items, 128), 128, 0, st>>>(J);
+            launched += 2;
+        }
+        if (path == 1 && J.sbest) {
+            k_slot_best<<<div_up(items, 128), 128, 0, st>>>(J);
+            ++launched;
+        }
+    }
+#undef NU_CELLS
+    return launched;
+}
+
 int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       int64_t n_total, bool fp64, const double* t, const FoldScratch& fs,
                       int n_D, double dt, double gap_factor, const double* periods,
-                      int64_t n_P, unsigned long long* counter, int grid, int threads,
-                      double* Q, double* T0, int* Didx, double* dep, double* sig, double* lnp,
-                      cudaStream_t st) {
+                      int64_t n_P, int warps, double* Q, double* T0, int* Didx, double* dep,
+                      double* sig, double* lnp, cudaStream_t st, cudaStream_t side,
+                      cudaError_t* err) {
     int launched = 0;
     const ExactLayout L = exact_layout(n_total, n_D, fp64);
-    const ScreenRec* screen = (const ScreenRec*)((const char*)fs.nodes + L.off_screen);
-    const ulonglong2* vpair = (const ulonglong2*)((const char*)fs.nodes + L.off_vpos);
-    // the kernel instance whose shared arrays and register budget match the
-    // block size (64, 128 or 256 threads)
-#define NU_FB(KIND_, MAXT_, CTR_)                                                          \
-    k_fold_batch<KIND_, MAXT_><<<grid, MAXT_, 0, st>>>(                                  \
-        segs_dev, n_seg, t, fs.nodes, screen, vpair, fs.srec, fs.lgm, fs.reg, fs.peak,     \
-         fs.bucket,                                                                \
-        fs.rec, n_D, dt, gap_factor, periods, fs.ptab, n_P, CTR_, Q, T0, Didx, dep, sig, lnp)
-#define NU_FB_SIZE(KIND_, CTR_)                                                            \
-    do {                                                                                   \
-        if (threads <= 64) NU_FB(KIND_, 64, CTR_);                                         \
-        else if (threads <= 128) NU_FB(KIND_, 128, CTR_);                                  \
-        else NU_FB(KIND_, 256, CTR_);                                                      \
-    } while (0)
+    FoldJob J{};
+    J.segs = segs_dev;
+    J.n_seg = n_seg;
+    J.n_D = n_D;
+    J.dt = dt;
+    J.inv_dt = 1.0 / dt;
+    J.gap_max = gap_factor * dt;
+    J.t = t;
+    J.nodes = fs.nodes;
+    J.screen = (const ScreenRec*)((const char*)fs.nodes + L.off_screen);
+    J.vpair = (const ulonglong2*)((const char*)fs.nodes + L.off_vpos);
+    J.srec = fp64 ? fs.srec : nullptr;
+    J.reg = fs.reg;
+    J.peak = fs.peak;
+    J.bucket = fs.bucket;
+    J.rec = fs.rec;
+    J.tab = fs.tab;
+    J.periods = periods;
+    J.ptab = fs.ptab;
+    J.stab = reinterpret_cast<const SlotPeriod*>(fs.ptab);
+    J.n_P = n_P;
+    J.Q = Q;
+    J.T0 = T0;
+    J.Didx = Didx;
+    J.dep = dep;
+    J.sig = sig;
+    J.lnp = lnp;
+    J.cand = fs.cand;
+    J.n_cand = fs.n_cand;
+    J.cap = fs.cap;
+    J.range = fs.range;
+    J.items = fs.items;
+    J.sbest = fs.sbest;
+    J.counters = fs.n_list;
+    const int nw = warps == 8 ? 8 : warps & 3;
+    if ((warps & 4) && nw != 8 && (int64_t)n_seg * n_P < 0xffffffffLL)    // (32-bit list)
+        J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
+    // (the two paths' period tables share a buffer)
     if (fb.any_exact) {
         k_period_consts<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt, fs.ptab);
-        const bool group = gain_width(n_D) > 1;
-        if (fp64) {
-            if (group) NU_FB_SIZE(4, counter); else NU_FB_SIZE(0, counter);
-        } else {
-            if (group) NU_FB_SIZE(5, counter); else NU_FB_SIZE(1, counter);
-        }
-        launched += 2;
+        launched += 1 + launch_cells(J, fp64, true, false, nw, st, side, err);
     }
     if (fb.any_slots) {
         k_slot_periods<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt,
                                                          reinterpret_cast<SlotPeriod*>(fs.ptab));
-        ++launched;
-        if (fb.slot_cascade)
-            NU_FB_SIZE(2, counter + 1);
-        else
-            NU_FB_SIZE(3, counter + 1);
-        ++launched;
+        launched += 1 + launch_cells(J, fp64, false, true, nw, st, side, err);
     }
-#undef NU_FB_SIZE
-#undef NU_FB
     return launched;
 }
 
@@ -2732,34 +2721,45 @@ namespace nu {
 
 // Scratch layout of the single-curve fold.  In mixed precision the regular
 // and the irregular path are two uses of one region (which of them runs is
-// known after the slot test).  screen = false leaves out what the screen of
-// the mixed irregular path needs (the exact path evaluates every cell).
+// known after the slot test).  level 2: everything; 1: without the filter
+// tables, the period table and the lists (every cell is screened, survivors
+// are evaluated in place); 0: also without what the screen of the mixed
+// irregular path needs (every cell is evaluated).
 struct SingleLayout {
     ExactLayout el;
-    size_t exact, bucket, slot_of, flag, rec, srec, lm3, lgm, total;
-    bool screen;
+    FilterLayout fl;
+    size_t exact, bucket, slot_of, flag, rec, srec, tab, ptab, cand, range, items, list, sbest, total;
+    unsigned long long cap;
+    int level;
 };
 
-static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, bool fp64,
-                                  bool screen = true) {
+static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, int64_t n_P, bool fp64,
+                                  int level = 2) {
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
     SingleLayout L;
-    L.screen = fp64 || screen;
-    L.el = exact_layout(n_t0, n_D, fp64, L.screen);
+    L.level = level;
+    L.el = exact_layout(n_t0, n_D, fp64, fp64 || level > 0);
     const int64_t n_slots = n_bucket + 2;          // slot records, NaN padded
-    const size_t gain = al((size_t)n_slots * gain_cols(n_D) * sizeof(float));
     L.flag = 0;
     L.slot_of = 256;
     L.exact = L.slot_of + al((size_t)n_t0 * sizeof(int));
-    // the mixed regular path
-    L.rec = L.exact;
-    L.lgm = L.rec + al((size_t)n_slots * n_D * sizeof(Node4<float>));
-    // the others
-    L.bucket = L.exact + L.el.total;
+    L.rec = L.exact;                               // the mixed regular path's
+    L.bucket = L.exact + L.el.total;               // the others'
     L.srec = L.bucket + al((size_t)n_bucket * sizeof(int));
-    L.lm3 = L.srec + (fp64 ? al((size_t)n_slots * n_D * sizeof(ScreenRec)) : 0);
-    L.total = L.lm3 + (L.screen ? gain : 0);
-    if (!fp64) L.total = std::max(L.total, L.lgm + gain);
+    size_t end = L.srec + (fp64 ? al((size_t)n_slots * n_D * sizeof(ScreenRec)) : 0);
+    if (!fp64) end = std::max(end, L.rec + al((size_t)n_slots * n_D * sizeof(Node4<float>)));
+    const int64_t ns = filter_slots(n_slots);
+    L.fl = filter_layout(ns * n_D, ns * ((n_D + 1) / 2 * 2),
+                         ns * filter_groups(n_D) * filter_words(n_D), n_D);
+    L.cap = (unsigned long long)std::min<int64_t>(8 * n_P + 4096, 1ll << 30);
+    L.tab = end;
+    L.ptab = L.tab + L.fl.total;
+    L.cand = L.ptab + al((size_t)n_P * period_const_bytes());
+    L.range = L.cand + al((size_t)L.cap * sizeof(FoldCand));
+    L.items = L.range + al((size_t)n_P * sizeof(int2));
+    L.list = L.items + al((size_t)n_P * sizeof(ItemConst));
+    L.sbest = L.list + al((size_t)n_P * sizeof(unsigned));
+    L.total = level == 2 ? L.sbest + (fp64 ? 0 : al((size_t)n_P * sizeof(SlotBest))) : end;
     return L;
 }
 
@@ -2776,141 +2776,161 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
     const double span_steps = (t_last - t_ref) / phase_step;
     const int64_t ngrid = n_t0 * (int64_t)n_D;
     const int64_t n_slots = n_bucket + 2;
-    void* nodes = scratch + L.exact;
-    int* bucket = (int*)(scratch + L.bucket);
     int* slot_of = (int*)(scratch + L.slot_of);
     int* flag = (int*)(scratch + L.flag);
-    Node4<float>* rec = (Node4<float>*)(scratch + L.rec);
     int launched = 0;
-    cudaError_t e = cudaSuccess;
+    // one block of flags: [0] slot test, [1..2] regular-grid test, then the
+    // peak key and the candidate counter
+    cudaError_t e = cudaMemsetAsync(flag, 0, 256, st);
     // the slot path needs a regular grid and a gap rule that only joins
     // neighbouring slots (1 < gap_factor < 2)
     bool use_slots = !fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span_steps < 4.0e6;
     if (use_slots) {
         int irregular = 0;
-        e = cudaMemsetAsync(flag, 0, sizeof(int), st);
         k_slots<<<div_up(n_t0, 256), 256, 0, st>>>(t0s_dev, n_t0, t_ref, 1.0 / phase_step,
                                                   slot_of, flag);
         ++launched;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&irregular, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) {
-            count_launches(launched);
-            return cuda_fail(e, (std::string(who) + ": slot test").c_str());
-        }
         use_slots = irregular == 0;
+    }
+    if (e != cudaSuccess) {
+        count_launches(launched);
+        return cuda_fail(e, (std::string(who) + ": slot test").c_str());
+    }
+    FoldJob J{};
+    J.n_seg = 1;
+    J.n_D = n_D;
+    J.dt = phase_step;
+    J.inv_dt = 1.0 / phase_step;
+    J.gap_max = gap_factor * phase_step;
+    J.t = t0s_dev;
+    J.nodes = scratch + L.exact;
+    J.screen = (const ScreenRec*)(scratch + L.exact + L.el.off_screen);
+    J.vpair = (const ulonglong2*)(scratch + L.exact + L.el.off_vpos);
+    J.srec = fp64 ? (const ScreenRec*)(scratch + L.srec) : nullptr;
+    J.reg = (const unsigned*)(flag + 1);
+    J.peak = (const unsigned long long*)(scratch + L.flag + 16);
+    J.bucket = (const int*)(scratch + L.bucket);
+    J.rec = (const Node4<float>*)(scratch + L.rec);
+    J.periods = periods_dev;
+    J.n_P = n_P;
+    J.Q = Q_dev;
+    J.T0 = T0_dev;
+    J.Didx = D_idx_dev;
+    J.dep = depth_out_dev;
+    J.sig = sigma_out_dev;
+    J.lnp = lnP_dev;
+    FoldSeg& one = J.one;
+    one.n_t0 = n_t0;
+    one.t_ref = t_ref;
+    one.t_last = t_last;
+    one.n_bucket = n_bucket;
+    one.n_slots = n_slots;
+    one.use_slots = use_slots ? 1 : 0;
+    one.screen = !use_slots && gap_factor < 2.0 && span_steps < 8.0e6 && (fp64 || L.level > 0);
+    if (use_slots) one.ulast = slot_ulast(t_ref, t_last, phase_step);
+    else one.uspan = exact_uspan(t_ref, t_last, phase_step);
+    if (L.level == 2) {
+        J.tab = filter_tab(scratch + L.tab, L.fl);
+        J.ptab = (const PeriodConst*)(scratch + L.ptab);
+        J.stab = (const SlotPeriod*)(scratch + L.ptab);
+        J.cand = (FoldCand*)(scratch + L.cand);
+        J.counters = (unsigned*)(scratch + L.flag + 64);
+        J.n_cand = (unsigned long long*)(J.counters + 4);
+        J.cap = L.cap;
+        J.range = (int2*)(scratch + L.range);
+        J.items = (ItemConst*)(scratch + L.items);
+        J.sbest = fp64 ? nullptr : (SlotBest*)(scratch + L.sbest);
     }
     if (use_slots) {
         const int64_t nrec = n_slots * n_D;
+        Node4<float>* rec = (Node4<float>*)(scratch + L.rec);
         k_fill_nan<<<div_up(nrec, 256), 256, 0, st>>>(rec, nrec);
         k_slot_fill<<<div_up(ngrid, 256), 256, 0, st>>>(
             (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, slot_of,
             n_t0, n_D, n_slots, rec);
-        float* lgm = (float*)(scratch + L.lgm);
-        const int64_t nlg = n_slots * gain_cols(n_D);
-        k_slot_gain<<<div_up(nlg, 256), 256, 0, st>>>(rec, nullptr, 0, n_slots, n_D, nlg, lgm);
-        // the cascade's instance where a period can hold enough cells for it
-        const bool casc = nrec >= (int64_t)NU_CASCADE_ROUNDS * 128;
-#define NU_FS(MAXT_, CASC_)                                                                \
-    k_fold_slots<8, MAXT_, CASC_><<<(unsigned)n_P, MAXT_, 0, st>>>(                        \
-        rec, lgm, n_slots, n_D, phase_step, t_ref, t_last, periods_dev, n_P, Q_dev, T0_dev, \
-        D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev)
-        if (n_P >= NU_SLOTS_SMALL_FROM) {
-            if (casc) NU_FS(NU_SLOTS_SMALL, true); else NU_FS(NU_SLOTS_SMALL, false);
-        } else {
-            if (casc) NU_FS(256, true); else NU_FS(256, false);
+        launched += 2;
+        if (J.stab) {
+            k_slot_periods<<<div_up(n_P, 256), 256, 0, st>>>(periods_dev, n_P, phase_step,
+                                                             (SlotPeriod*)(scratch + L.ptab));
+            ++launched;
         }
-#undef NU_FS
-        launched += 4;
     } else {
         k_buckets<<<div_up(n_bucket, 256), 256, 0, st>>>(t0s_dev, n_t0, t_ref, phase_step,
-                                                        n_bucket, bucket);
-        FoldGeom g{t0s_dev, n_t0, t_ref, t_last, phase_step, 1.0 / phase_step,
-                   gap_factor * phase_step, bucket, n_bucket};
-        ScreenRec* nrec = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
+                                                        n_bucket, (int*)(scratch + L.bucket));
+        const double gap_max = gap_factor * phase_step;
+        ScreenRec* screen = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
         ulonglong2* vpair = (ulonglong2*)(scratch + L.exact + L.el.off_vpos);
-        ScreenRec* srec = fp64 ? (ScreenRec*)(scratch + L.srec) : nullptr;
-        float* lm3 = (float*)(scratch + L.lm3);
-        unsigned* reg = (unsigned*)(flag + 1);
-        unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
-        const ScreenGeom sg{nrec, vpair, srec, n_slots, reg,
-                            (gap_factor < 2.0 && span_steps < 8.0e6) ? 1 : 0, peak, lm3,
-                            fp64 ? 0 : 1};
-        const int64_t nlm = n_slots * gain_cols(n_D);
-        const dim3 peak_grid(1, (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608));
-        e = cudaMemsetAsync(flag, 0, 256, st);
-        if (e != cudaSuccess) {
-            count_launches(launched);
-            return cuda_fail(e, (std::string(who) + ": memset").c_str());
-        }
-        // One block per period.  With many periods, 2-warp blocks: 14 fit
-        // on an SM (28 warps) and each period has 2 warps to seed; with
-        // few, 8-warp blocks keep the GPU full (C2, 20 000 periods: 16.5 ms
-        // at 256 threads, 14.0 at 128 (7 per SM), 13.6 at 64).
-        // (the grouped gain walk where the durations form groups)
-#define NU_FSC(T_, MAXT_)                                                                  \
-    do {                                                                                   \
-        if (gain_width(n_D) > 1)                                                           \
-            k_fold_screened<T_, MAXT_, true><<<(unsigned)n_P, MAXT_, 0, st>>>(             \
-                g, sg, (const Node8<T_>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,      \
-                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
-        else                                                                               \
-            k_fold_screened<T_, MAXT_, false><<<(unsigned)n_P, MAXT_, 0, st>>>(            \
-                g, sg, (const Node8<T_>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,      \
-                D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);                         \
-    } while (0)
-        if (fp64) {
-            k_slot_offsets<<<div_up(n_t0, 256), 256, 0, st>>>(t0s_dev, n_t0, 1.0 / phase_step,
-                                                              n_slots, slot_of, reg);
-            k_fill_screen<<<div_up(n_slots * n_D, 256), 256, 0, st>>>(srec, n_slots * n_D);
+        if (fp64)
             k_nodes<double><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
-                t0s_dev, n_t0, n_D, g.gap_max, (Node8<double>*)nodes);
-            k_screen<double><<<div_up(ngrid, 256), 256, 0, st>>>(
-                (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
-                t0s_dev, n_t0, n_D, g.gap_max, phase_step, nrec, srec, (Node8<double>*)nodes,
-                n_slots, slot_of, vpair);
-            k_gain_table<double><<<div_up(nlm, 256), 256, 0, st>>>(
-                (const Node8<double>*)nodes, vpair, bucket, nullptr, 0, n_t0, n_slots, n_bucket,
-                n_D, nlm, lm3);
-            k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)dlnl_dev, nullptr,
-                                                           n_t0, n_D, peak);
-            if (n_P >= 8192)
-                NU_FSC(double, 64);
-            else
-                NU_FSC(double, 256);
-            launched += 8;
-        } else {
+                t0s_dev, n_t0, n_D, gap_max, (Node8<double>*)(scratch + L.exact));
+        else
             k_nodes<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev,
-                t0s_dev, n_t0, n_D, g.gap_max, (Node8<float>*)nodes);
-            if (L.screen && sg.on) {
-                k_screen<float><<<div_up(ngrid, 256), 256, 0, st>>>(
-                    (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev,
-                    t0s_dev, n_t0, n_D, g.gap_max, phase_step, nrec, nullptr,
-                    (Node8<float>*)nodes, n_slots, nullptr, vpair);
-                k_gain_table<float><<<div_up(nlm, 256), 256, 0, st>>>(
-                    (const Node8<float>*)nodes, vpair, bucket, nullptr, 0, n_t0, n_slots,
-                    n_bucket, n_D, nlm, lm3);
-                k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)dlnl_dev, nullptr,
-                                                              n_t0, n_D, peak);
-                if (n_P >= 8192)
-                    NU_FSC(float, 64);
-                else
-                    NU_FSC(float, 256);
-                launched += 6;
-            } else {
+                t0s_dev, n_t0, n_D, gap_max, (Node8<float>*)(scratch + L.exact));
+        launched += 2;
+        if (!one.screen) {
+            // gap rules and spans the screen does not cover: every cell
+            const FoldGeom g{t0s_dev, n_t0, t_ref, t_last, phase_step, 1.0 / phase_step, gap_max,
+                             (const int*)(scratch + L.bucket), n_bucket};
+            if (fp64)
+                k_fold_exact<double, 8><<<(unsigned)n_P, 256, 0, st>>>(
+                    g, (const Node8<double>*)(scratch + L.exact), n_D, periods_dev, n_P, Q_dev,
+                    T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+            else
                 k_fold_exact<float, 8><<<(unsigned)n_P, 256, 0, st>>>(
-                    g, (const Node8<float>*)nodes, n_D, periods_dev, n_P, Q_dev, T0_dev,
-                    D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
-                launched += 3;
-            }
+                    g, (const Node8<float>*)(scratch + L.exact), n_D, periods_dev, n_P, Q_dev,
+                    T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+            count_launches(launched + 1);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_fail(e, (std::string(who) + ": launch").c_str());
+            return NU_OK;
         }
-#undef NU_FSC
+        if (fp64) {
+            ScreenRec* srec = (ScreenRec*)(scratch + L.srec);
+            k_slot_offsets<<<div_up(n_t0, 256), 256, 0, st>>>(
+                t0s_dev, n_t0, 1.0 / phase_step, n_slots, slot_of, (unsigned*)(flag + 1));
+            k_fill_screen<<<div_up(n_slots * n_D, 256), 256, 0, st>>>(srec, n_slots * n_D);
+            k_screen<double><<<div_up(ngrid, 256), 256, 0, st>>>(
+                (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
+                t0s_dev, n_t0, n_D, gap_max, phase_step, screen, srec, n_slots, slot_of, vpair);
+            launched += 3;
+        } else {
+            k_screen<float><<<div_up(ngrid, 256), 256, 0, st>>>(
+                (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, t0s_dev,
+                n_t0, n_D, gap_max, phase_step, screen, nullptr, n_slots, nullptr, vpair);
+            ++launched;
+        }
+        if (J.ptab) {
+            k_period_consts<<<div_up(n_P, 256), 256, 0, st>>>(periods_dev, n_P, phase_step,
+                                                              (PeriodConst*)(scratch + L.ptab));
+            ++launched;
+        }
     }
+    const dim3 peak_grid(1, (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608));
+    unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
+    if (fp64)
+        k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)dlnl_dev, nullptr, n_t0,
+                                                       n_D, peak);
+    else
+        k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)dlnl_dev, nullptr, n_t0, n_D,
+                                                      peak);
+    ++launched;
+    if (J.tab.S)
+        e = launch_filter_tables(nullptr, one, 1, n_D, filter_slots(n_slots) * n_D, n_t0, J.screen,
+                                 J.vpair, J.bucket, J.rec, J.tab, st, &launched);
+    // Warps per period: eight where the periods are few, one or two (and eight
+    // for the long ones) where they alone fill the GPU.  Sector grid, FP64, at
+    // 2 500 periods 1.7 ms with eight, 2.0 with one.
+    const int nw = n_P >= NU_ONE_WARP_FROM ? 1 : (n_P >= NU_WARP_ITEMS_FROM ? 2 : 8);
+    if (J.items && nw != 8)
+        J.list = FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K};
+    launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, thread_side_stream(), &e);
     count_launches(launched);
-    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, (std::string(who) + ": launch").c_str());
     return NU_OK;
 }
@@ -2987,7 +3007,7 @@ extern "C" nu_status nu_periodic_search(const double* t0s_dev, int64_t n_t0,
     if (span_steps > 1.0e9) return fail(NU_EINVAL, "nu_periodic_search: phase grid too fine");
     const int64_t n_bucket = (int64_t)span_steps + 2;
     const bool fp64 = prec == NU_FP64;
-    const SingleLayout L = single_layout(n_t0, n_D, n_bucket, fp64);
+    const SingleLayout L = single_layout(n_t0, n_D, n_bucket, n_P, fp64);
     pool_keep_memory();
     char* scratch = nullptr;
     e = cudaMallocAsync((void**)&scratch, L.total, st);
@@ -3199,11 +3219,11 @@ extern "C" nu_status nu_periodic_search_noalloc(const double* t0s_dev, int64_t n
         return fail(NU_EINVAL, "nu_periodic_search_noalloc: phase grid too fine");
     const int64_t n_bucket = (int64_t)span_steps + 2;
     const bool fp64 = prec == NU_FP64;
-    // (the mixed path of irregular grids runs without its screen where only
-    // the screen's arrays exceed the limit)
-    SingleLayout L = single_layout(n_t0, n_D, n_bucket, fp64);
-    if (!fp64 && L.total > NU_NOALLOC_SCRATCH_BYTES)
-        L = single_layout(n_t0, n_D, n_bucket, fp64, false);
+    // (near the limit without the filters, and the mixed path of irregular
+    // grids without its screen)
+    SingleLayout L = single_layout(n_t0, n_D, n_bucket, n_P, fp64);
+    for (int level = 1; level >= (fp64 ? 1 : 0) && L.total > NU_NOALLOC_SCRATCH_BYTES; --level)
+        L = single_layout(n_t0, n_D, n_bucket, n_P, fp64, level);
     if (L.total > NU_NOALLOC_SCRATCH_BYTES)
         return fail(NU_EINVAL,
                     "nu_periodic_search_noalloc: this grid needs %zu bytes of scratch, more "
