@@ -175,8 +175,8 @@ nu_status nu_linear_search(const nu_factor* f, const double* t0s_dev, int64_t n_
  * ln L_k; the cell maximising ln P (first in duration-major, then phase order)
  * is Eq. phi0's argmax.
  *
- *   phase_step    > 0, or 0 for the median spacing of t0s (computed on the
- *                 host from a copy of t0s; this synchronises the stream)
+ *   phase_step    > 0, or 0 for the median spacing of t0s (this
+ *                 synchronises the stream)
  *   gap_factor    > 0 (1.5 is the default reading)
  *   outputs (n_P each): Q = Delta/sigma, T0 = t0s[0] + phi0*P, D_idx (int32,
  *   -1 when no cell has an epoch), depth Delta, sigma, lnP.  A period with no
@@ -322,8 +322,7 @@ uint64_t nu_periodic_search_noalloc_limit(void);
  *   k             1 or 2: X = [1] or [1, t] per curve
  *   Ds_host (n_D), periods_dev (n_P): shared grids
  *   phase_step    > 0 (shared by all curves), or 0 for the median sample
- *                 spacing of the first curve (computed on the host from a
- *                 copy of that curve's times)
+ *                 spacing of the first curve
  *   outputs, [n_lc][n_P] each: Q, T0, D_idx, depth, sigma, lnP (as in
  *   nu_periodic_search); status_host (n_lc) per-curve factor status.
  * Synchronises the stream before returning (the statuses are host data).

@@ -154,18 +154,10 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     cudaStream_t st = (cudaStream_t)stream;
     if (phase_step == 0.0) {
         // default phase step: the median sample spacing of the first curve
-        // (a host copy of its times; this synchronises the stream)
-        const int64_t n0 = offsets_host[1];
-        std::vector<double> h(n0);
-        cudaError_t ec = cudaMemcpyAsync(h.data(), t_dev, n0 * sizeof(double),
-                                         cudaMemcpyDeviceToHost, st);
-        if (ec == cudaSuccess) ec = cudaStreamSynchronize(st);
-        if (ec != cudaSuccess) return cuda_fail(ec, "nu_batch_search: copy of curve 0");
-        std::vector<double> d(n0 - 1);
-        for (int64_t i = 0; i + 1 < n0; ++i) d[i] = h[i + 1] - h[i];
-        std::sort(d.begin(), d.end());
-        const size_t m = d.size();
-        phase_step = (m % 2) ? d[m / 2] : 0.5 * (d[m / 2 - 1] + d[m / 2]);
+        // (this synchronises the stream)
+        double t0, t1;
+        const cudaError_t ec = median_spacing(t_dev, offsets_host[1], st, &phase_step, &t0, &t1);
+        if (ec != cudaSuccess) return cuda_fail(ec, "nu_batch_search: median spacing of curve 0");
         if (!(phase_step > 0.0) || !std::isfinite(phase_step))
             return fail(NU_EINVAL, "nu_batch_search: curve 0 gives no positive median spacing");
     }

@@ -473,33 +473,41 @@ __device__ __forceinline__ float filter_bound(float sd, float v, float g, float 
     return fmaf(g, 1.f + c, 0.500001f) + eff * sd * sd * r * 1.00001f;
 }
 
-// Gain sums of eight phases of a group of 2 NW durations (the rest of a stays 0).
+// Gain sums of two groups of eight phases, each of 2 NW durations (rows r0, r1,
+// walks from u0, u1; the rest of a stays 0).  Two epochs of both a round, four
+// loads in flight: the walks are short (two to five epochs), so that a round
+// is mostly the latency of its loads.  Positions past the end, of either walk,
+// add terms >= 0 (the empty last entry, or an event the cell does not have).
 template <int NW> struct FilterWords;
 template <> struct FilterWords<1> { typedef unsigned T; };
 template <> struct FilterWords<2> { typedef uint2 T; };
 template <> struct FilterWords<4> { typedef uint4 T; };
 template <int NW>
-__device__ __forceinline__ void filter_gain(const unsigned* __restrict__ Gg, int ns,
-                                            unsigned long long u,
-                                            const FilterPeriod& fp, __half2 (&a)[4]) {
+__device__ __forceinline__ void filter_gain(const unsigned* __restrict__ g0,
+                                            const unsigned* __restrict__ g1, unsigned ns,
+                                            unsigned long long u0, unsigned long long u1,
+                                            unsigned long long ustep, unsigned long long uend,
+                                            __half2 (&a)[4], __half2 (&b)[4]) {
     typedef typename FilterWords<NW>::T V;
-    const V* __restrict__ r = reinterpret_cast<const V*>(Gg);
-    const unsigned n8 = (unsigned)ns >> 3, last = (unsigned)ns - 1u;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = __half2half2(__float2half(0.f));
+    const V* __restrict__ r0 = reinterpret_cast<const V*>(g0);
+    const V* __restrict__ r1 = reinterpret_cast<const V*>(g1);
+    const unsigned n8 = ns >> 3, last = ns - 1u;
     auto at = [&](unsigned long long x) {
         const unsigned s = min((unsigned)(x >> 40), last);
-        return r[(s & 7u) * n8 + (s >> 3)];
+        return (s & 7u) * n8 + (s >> 3);
     };
-    auto add = [&](const V& v) {
+    auto add = [&](__half2 (&c)[4], const V& v) {
         const unsigned* w = reinterpret_cast<const unsigned*>(&v);
 #pragma unroll
-        for (int i = 0; i < NW; ++i) a[i] = __hadd2(a[i], *reinterpret_cast<const __half2*>(w + i));
+        for (int i = 0; i < NW; ++i) c[i] = __hadd2(c[i], *reinterpret_cast<const __half2*>(w + i));
     };
-    for (; u < fp.uend; u += 2ull * fp.ustep) {
-        const V x = at(u), y = at(u + fp.ustep);
-        add(x);
-        add(y);
+    for (; min(u0, u1) < uend; u0 += 2ull * ustep, u1 += 2ull * ustep) {
+        const V x0 = r0[at(u0)], x1 = r1[at(u1)];
+        const V y0 = r0[at(u0 + ustep)], y1 = r1[at(u1 + ustep)];
+        add(a, x0);
+        add(b, x1);
+        add(a, y0);
+        add(b, y1);
     }
 }
 
@@ -578,6 +586,45 @@ __device__ __forceinline__ int filter_shift(int mode) {
 }
 __device__ __forceinline__ float filter_slack(const FilterPeriod& fp) {
     return (fp.K + 8.f) * 1.1920929e-7f;
+}
+
+// Gain sums of the groups (q0, g0) and (q1, g1): eight durations' FP16 numbers
+// each.
+struct FilterGains {
+    __half2 a[4], b[4];
+};
+__device__ __forceinline__ void filter_gains(const FilterCtx& x, unsigned q0, int g0, unsigned q1,
+                                             int g1, FilterGains& s) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s.a[i] = s.b[i] = __half2half2(__float2half(0.f));
+    const int NW = filter_words(x.n_D);
+    const unsigned ns = (unsigned)x.f.ns;
+    const unsigned long long uph8 = x.fp.uph << 3;
+    const unsigned long long u0 = q0 * uph8, u1 = q1 * uph8;
+    const unsigned* r0 = x.f.G + (int64_t)g0 * (int)ns * NW;
+    const unsigned* r1 = x.f.G + (int64_t)g1 * (int)ns * NW;
+    if (NW == 4) filter_gain<4>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
+    else if (NW == 2) filter_gain<2>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
+    else filter_gain<1>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
+}
+// Which of them reach the threshold: bit i is duration i of the first group,
+// bit 16 + i of the second.
+__device__ __noinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q0, int g0,
+                                                  unsigned q1, int g1) {
+    FilterGains s;
+    filter_gains(x, q0, g0, q1, g1, s);
+    // FP16 sums of K terms: 2^-11 of the sum per addition; a sum of 0, no event,
+    // is below the smallest FP16 number
+    const float inv_ch = 0.999999f - (x.fp.K + 4.f) * 5.4e-4f;
+    const float t = fmaxf((filter_thr(x) - 0.500002f) * inv_ch, 5.9604645e-08f);
+    const __half2 t2 = __half2half2(__float2half_rd(t));
+    unsigned pass = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const unsigned m = __hge2_mask(s.a[i], t2), n = __hge2_mask(s.b[i], t2);
+        pass |= ((m & 1u) | ((m >> 15) & 2u) | ((n & 1u) << 16) | ((n & 0x10000u) << 1)) << (2 * i);
+    }
+    return pass;
 }
 
 // Bounds of four phases (Q) or one phase (S) of four durations from d0 (the
@@ -815,7 +862,9 @@ __device__ __noinline__ void filter_take(FilterCtx& x, FilterQueues& q, unsigned
         return;
     }
     const int total = __reduce_add_sync(FULL, __popc(pass));
-    if (q.ni + total <= FILTER_ITEMS + 32) {
+    const int n0 = q.ni;
+    __syncwarp();                          // (read by all before any lane adds)
+    if (n0 + total <= FILTER_ITEMS + 32) {
         int pos = pass ? atomicAdd(&q.ni, __popc(pass)) : 0;
         for (; pass; pass &= pass - 1u)
             q.item[pos++] = make_uint2(g, (unsigned)(d0 + __ffs(pass) - 1));
@@ -855,6 +904,56 @@ __device__ __noinline__ void filter_seed(FilterCtx& x, FilterQueues& q, float b,
     filter_rest(q, screen);
 }
 
+// The groups of one mode, in the order the warps take them.
+struct FilterGroups {
+    unsigned nq, n_it, stride;
+    int W;                 // durations of a group
+    __device__ __forceinline__ void advance(unsigned& q, int& g) const {
+        q += stride;
+        while (q >= nq) {
+            q -= nq;
+            ++g;
+        }
+    }
+};
+// Seed from a warp's first round: the largest bound of its lanes' first groups.
+template <class Screen>
+__device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool act, unsigned qi,
+                                          int gi, Screen& screen) {
+    float b = 0.f;
+    int bd = 0;
+    const int n_D = x.n_D;
+    if (x.fp.mode == FILTER_GAIN) {
+        const int d0 = gi * 2 * filter_words(n_D);
+        if (act) {
+            FilterGains s;
+            filter_gains(x, qi, gi, qi, gi, s);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float lo = __low2float(s.a[i]), hi = __high2float(s.a[i]);
+                if (lo > b && lo < INFINITY) { b = lo; bd = 2 * i; }
+                if (hi > b && hi < INFINITY) { b = hi; bd = 2 * i + 1; }
+            }
+        }
+        bd += d0;
+    } else {
+        const int d0 = gi * 4;
+        if (act) {
+            const float4 u = filter_sums(x, ((unsigned long long)qi << filter_shift(x.fp.mode)) *
+                                                x.fp.uph, d0);
+            const float ub[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (d0 + i < n_D && ub[i] > b && ub[i] < INFINITY) {
+                    b = ub[i];
+                    bd = i;
+                }
+        }
+        bd += d0;
+    }
+    filter_seed(x, q, b, qi, bd, screen);
+}
+
 // Runs the filters over every cell of a period.  The item's warps (wid of
 // nw) share the work.  Cells below the threshold are dropped, the others go
 // through the screen.
@@ -863,93 +962,56 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
                                              Screen& screen) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const FilterPeriod fp = x.fp;
-    const FilterView f = x.f;
-    const int n_D = x.n_D, mode = fp.mode;
+    const int n_D = x.n_D, mode = x.fp.mode;
     const int sh = filter_shift(mode);
-    const int NW = filter_words(n_D);             // gain groups of 2 NW durations
-    constexpr int WS = 4;                         // durations per lane of the other filters
-    const int W = mode == FILTER_GAIN ? 2 * NW : WS;
-    const unsigned nq = (unsigned)((fp.n_phi + (1 << sh) - 1) >> sh);
-    const unsigned n_it = nq * (unsigned)((n_D + W - 1) / W);
-    int gi = (int)((unsigned)(wid * 32 + lane) / nq);
-    unsigned qi = (unsigned)(wid * 32 + lane) - (unsigned)gi * nq;
-    const unsigned stride = (unsigned)nw * 32u;
-    // FP16 sums of K terms: 2^-11 of the sum per addition
-    const float inv_ch = 0.999999f / (1.f + (fp.K + 4.f) * 5.4e-4f);
-    bool first = true;
-    for (unsigned base = (unsigned)wid * 32u; base < n_it; base += stride, qi += stride) {
-        while (qi >= nq) {
-            qi -= nq;
-            ++gi;
+    FilterGroups g;
+    g.W = mode == FILTER_GAIN ? 2 * filter_words(n_D) : 4;
+    g.nq = (unsigned)((x.fp.n_phi + (1 << sh) - 1) >> sh);
+    g.n_it = g.nq * (unsigned)((n_D + g.W - 1) / g.W);
+    g.stride = (unsigned)nw * 32u;
+    unsigned i = (unsigned)(wid * 32 + lane);            // this lane's group
+    int gi = (int)(i / g.nq);
+    unsigned qi = i - (unsigned)gi * g.nq;
+    if ((unsigned)wid * 32u < g.n_it) filter_first(x, q, i < g.n_it, qi, gi, screen);
+    auto mask = [&](unsigned pass, int d0) {             // durations past the last
+        return d0 + g.W > n_D ? (d0 < n_D ? pass & ((1u << (n_D - d0)) - 1u) : 0u) : pass;
+    };
+    if (mode == FILTER_GAIN) {
+        for (unsigned base = (unsigned)wid * 32u; base < g.n_it;
+             base += 2u * g.stride, i += 2u * g.stride) {
+            unsigned q1 = qi;
+            int g1 = gi;
+            g.advance(q1, g1);
+            const bool in0 = i < g.n_it, in1 = in0 && i + g.stride < g.n_it;
+            unsigned pass = 0u;
+            if (in0) pass = filter_gain_pass(x, qi, gi, in1 ? q1 : qi, in1 ? g1 : gi);
+            const int d0 = gi * g.W, d1 = g1 * g.W;
+            const unsigned p0 = mask(pass & 0xffffu, d0), p1 = in1 ? mask(pass >> 16, d1) : 0u;
+            if (__any_sync(FULL, (p0 | p1) != 0u)) {
+                filter_take(x, q, p0, qi, d0, screen);
+                filter_take(x, q, p1, q1, d1, screen);
+            }
+            qi = q1;
+            gi = g1;
+            g.advance(qi, gi);
         }
-        const bool act = base + lane < n_it;
-        const int d0 = gi * W;
-        const unsigned long long u = ((unsigned long long)qi << sh) * fp.uph;
-        unsigned pass = 0u;
-        if (mode == FILTER_GAIN) {
-            __half2 a[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = __half2half2(__float2half(0.f));
-            if (act) {
-                const unsigned* row = f.G + (int64_t)gi * f.ns * NW;
-                if (NW == 4) filter_gain<4>(row, f.ns, u, fp, a);
-                else if (NW == 2) filter_gain<2>(row, f.ns, u, fp, a);
-                else filter_gain<1>(row, f.ns, u, fp, a);
+    } else {
+        for (unsigned base = (unsigned)wid * 32u; base < g.n_it;
+             base += g.stride, i += g.stride) {
+            const int d0 = gi * 4;
+            unsigned pass = 0u;
+            if (i < g.n_it) {
+                const float4 u = filter_sums(x, ((unsigned long long)qi << sh) * x.fp.uph, d0);
+                const float t = filter_thr(x);
+                pass = (!(u.x < t) && u.x != -INFINITY ? 1u : 0u) |
+                       (!(u.y < t) && u.y != -INFINITY ? 2u : 0u) |
+                       (!(u.z < t) && u.z != -INFINITY ? 4u : 0u) |
+                       (!(u.w < t) && u.w != -INFINITY ? 8u : 0u);
+                pass = mask(pass, d0);
             }
-            if (first) {
-                first = false;
-                float b = 0.f;
-                int bd = 0;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float lo = __low2float(a[i]), hi = __high2float(a[i]);
-                    if (lo > b && lo < INFINITY) { b = lo; bd = 2 * i; }
-                    if (hi > b && hi < INFINITY) { b = hi; bd = 2 * i + 1; }
-                }
-                filter_seed(x, q, b, qi, d0 + bd, screen);
-            }
-            // (a sum of 0, no event, is below the smallest FP16 number)
-            const float t = fmaxf((filter_thr(x) - 0.500002f) * inv_ch, 5.9604645e-08f);
-            const __half2 t2 = __half2half2(__float2half_rd(t));
-            unsigned mk[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) mk[i] = __hge2_mask(a[i], t2);
-            if (mk[0] | mk[1] | mk[2] | mk[3]) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    pass |= ((mk[i] & 1u) | ((mk[i] >> 15) & 2u)) << (2 * i);
-            }
-        } else {
-            float ub[WS];
-#pragma unroll
-            for (int i = 0; i < WS; ++i) ub[i] = -INFINITY;
-            if (act) {
-                const float4 b4 = filter_sums(x, u, d0);
-                ub[0] = b4.x;
-                ub[1] = b4.y;
-                ub[2] = b4.z;
-                ub[3] = b4.w;
-            }
-            if (first) {
-                first = false;
-                float b = 0.f;
-                int bd = 0;
-#pragma unroll
-                for (int i = 0; i < WS; ++i)
-                    if (d0 + i < n_D && ub[i] > b && ub[i] < INFINITY) {
-                        b = ub[i];
-                        bd = i;
-                    }
-                filter_seed(x, q, b, qi, d0 + bd, screen);
-            }
-            const float t = filter_thr(x);
-#pragma unroll
-            for (int i = 0; i < WS; ++i)
-                if (!(ub[i] < t) && ub[i] != -INFINITY) pass |= 1u << i;
+            if (__any_sync(FULL, pass != 0u)) filter_take(x, q, pass, qi, d0, screen);
+            g.advance(qi, gi);
         }
-        if (d0 + W > n_D) pass &= d0 < n_D ? (1u << (n_D - d0)) - 1u : 0u;
-        if (__any_sync(FULL, pass != 0u)) filter_take(x, q, pass, qi, d0, screen);
     }
     if (mode != FILTER_CELL) filter_drain(x, q, true, screen);
     filter_rest(q, screen);

@@ -1,0 +1,141 @@
+// Median spacing of a sorted grid of epochs, and the grid's ends, on the device.
+//
+// The default phase step is the median of t[i+1] - t[i].  Copying the epochs to
+// the host and sorting the differences there cost 1.1 ms for 19 440 epochs, a
+// third of the fold that follows.  Here one block selects the middle element
+// (or the two middle ones) by radix, eight bits of an order-preserving key per
+// pass, and 32 bytes come back.
+#include <vector>
+
+#include "nu_internal.cuh"
+
+namespace nu {
+
+__device__ __forceinline__ unsigned long long diff_key(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double key_diff(unsigned long long k) {
+    const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
+    return __longlong_as_double((long long)b);
+}
+
+// The differences' keys once: an FP64 subtraction holds its pipe for 64 cycles
+// per warp, and the selection reads every difference up to nine times.
+__global__ void k_diff_keys(const double* __restrict__ t, int64_t m,
+                            unsigned long long* __restrict__ key) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i < m) key[i] = diff_key(t[i + 1] - t[i]);
+}
+
+// Short grids: the keys stay in the selecting block's shared memory, computed by
+// that block (48 FP64 subtractions a warp at most).
+constexpr int64_t MEDIAN_SHARED = 5120;
+
+// out = {element (m - 1) / 2, element m / 2 of the sorted differences, t[0], t[m]}.
+// keys: those of k_diff_keys, or nullptr: in shared memory (m <= MEDIAN_SHARED).
+__global__ void __launch_bounds__(1024)
+k_median(const double* __restrict__ t, int64_t m, const unsigned long long* __restrict__ keys,
+         double* __restrict__ out) {
+    __shared__ unsigned hist[256];
+    __shared__ unsigned long long sh_key[MEDIAN_SHARED];
+    __shared__ unsigned long long sh_prefix, sh_next;
+    __shared__ unsigned sh_rank, sh_left;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long* key = keys ? keys : sh_key;
+    if (!keys)
+        for (int64_t i = threadIdx.x; i < m; i += blockDim.x) sh_key[i] = diff_key(t[i + 1] - t[i]);
+    if (threadIdx.x == 0) {
+        sh_prefix = 0ull;
+        sh_rank = (unsigned)((m - 1) / 2);      // (m < 2^31)
+        sh_next = ~0ull;
+    }
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        if (threadIdx.x < 256) hist[threadIdx.x] = 0u;
+        __syncthreads();
+        const unsigned long long prefix = sh_prefix;
+        for (int64_t base = 0; base < m; base += blockDim.x) {
+            const int64_t i = base + threadIdx.x;
+            const unsigned long long k = i < m ? key[i] : 0ull;
+            // (shift + 8 = 64: every key has the empty prefix)
+            const bool in = i < m && (shift == 56 || (k >> (shift + 8)) == prefix);
+            const unsigned bin = in ? (unsigned)(k >> shift) & 255u : 256u;
+            // most spacings are the cadence: one atomic per distinct bin and warp
+            const unsigned same = __match_any_sync(FULL, bin);
+            if (in && lane == __ffs(same) - 1) atomicAdd(&hist[bin], (unsigned)__popc(same));
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            // the bin of the rank: eight bins a lane, prefix sums over the lanes
+            unsigned h[8], sum = 0u;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                h[b] = hist[8 * lane + b];
+                sum += h[b];
+            }
+            unsigned before = sum;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(FULL, before, o);
+                if (lane >= o) before += v;
+            }
+            before -= sum;
+            const unsigned r = sh_rank;
+            __syncwarp();
+            if (r >= before && r < before + sum) {          // (one lane)
+                int b = 0;
+                while (r >= before + h[b]) before += h[b++];
+                sh_rank = r - before;
+                sh_prefix = (prefix << 8) | (unsigned)(8 * lane + b);
+                sh_left = h[b];
+            }
+        }
+        __syncthreads();
+    }
+    const unsigned long long lo = sh_prefix;
+    // the next element: the same value when more of it are left, else the
+    // smallest larger one
+    const bool again = sh_rank + 1u < sh_left || (m & 1);
+    if (!again) {
+        unsigned long long best = ~0ull;
+        for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
+            const unsigned long long k = key[i];
+            if (k > lo && k < best) best = k;
+        }
+        if (best != ~0ull) atomicMin(&sh_next, best);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        out[0] = key_diff(lo);
+        out[1] = again ? out[0] : key_diff(sh_next);
+        out[2] = t[0];
+        out[3] = t[m];
+    }
+}
+
+cudaError_t median_spacing(const double* t_dev, int64_t n, cudaStream_t st, double* step,
+                           double* t_first, double* t_last) {
+    const int64_t m = n - 1;
+    char* mem = nullptr;
+    pool_keep_memory();
+    const bool shared = m <= MEDIAN_SHARED;
+    cudaError_t e = cudaMallocAsync((void**)&mem, (shared ? 0 : (size_t)m * 8) + 256, st);
+    if (e != cudaSuccess) return e;
+    unsigned long long* key = shared ? nullptr : (unsigned long long*)(mem + 256);
+    if (!shared) k_diff_keys<<<div_up(m, 256), 256, 0, st>>>(t_dev, m, key);
+    k_median<<<1, 1024, 0, st>>>(t_dev, m, key, (double*)mem);
+    count_launches(shared ? 1 : 2);
+    double h[4];
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h, mem, sizeof(h), cudaMemcpyDeviceToHost, st);
+    const cudaError_t f = cudaFreeAsync(mem, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    *step = (m % 2) ? h[1] : 0.5 * (h[0] + h[1]);
+    *t_first = h[2];
+    *t_last = h[3];
+    return f;
+}
+
+}  // namespace nu

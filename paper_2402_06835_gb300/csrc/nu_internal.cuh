@@ -45,6 +45,11 @@ struct Blocks {
 // repeated calls reuse memory without new device allocations.
 void pool_keep_memory();
 
+// Median spacing of the n >= 2 epochs t (the two middle ones' mean when their
+// number is even) and the first and last epoch.  Synchronises the stream.
+cudaError_t median_spacing(const double* t_dev, int64_t n, cudaStream_t st, double* step,
+                           double* t_first, double* t_last);
+
 // Number of kernels this library has launched (nu_launch_count).
 void count_launches(int k);
 

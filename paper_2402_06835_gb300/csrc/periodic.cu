@@ -2076,7 +2076,9 @@ struct SlotScreen {
         }
         filter_raise(it.x, fkey(screen_threshold<float>(lnp, it.x.fp.K)));
     }
-    __device__ __noinline__ void flush(int cnt) {
+    // (inlined: the lanes leave pass2 one by one, and a caller's shuffle after a
+    // call that returns like that has been seen to miss the late ones)
+    __device__ __forceinline__ void flush(int cnt) {
         const int lane = threadIdx.x & 31;
         if (lane < cnt) pass2(q.c[lane]);
         __syncwarp();
@@ -2227,18 +2229,26 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
     }
     item_sync<nw>();
     screen.flush(q.n);
-    // argmax in FP32 (larger ln P, ties to the smaller cell)
-    SlotBest sb{q.bl[lane], q.bD[lane], q.bs2[lane], q.bj[lane], q.bd[lane]};
+    // argmax in FP32 (larger ln P, ties to the smaller cell): the largest ln P,
+    // then the smallest duration and phase among its lanes
     auto over = [](const SlotBest& a, const SlotBest& b) {   // a beats b
         if (a.d < 0) return false;
         if (b.d < 0 || a.lnp > b.lnp) return true;
         return a.lnp == b.lnp && (a.d < b.d || (a.d == b.d && a.j < b.j));
     };
-    for (int s = 16; s > 0; s >>= 1) {
-        const SlotBest b{__shfl_xor_sync(FULL, sb.lnp, s), __shfl_xor_sync(FULL, sb.Dl, s),
-                         __shfl_xor_sync(FULL, sb.s2, s), __shfl_xor_sync(FULL, sb.j, s),
-                         __shfl_xor_sync(FULL, sb.d, s)};
-        if (over(b, sb)) sb = b;
+    __syncwarp();
+    const int bd = q.bd[lane];
+    const unsigned key = bd >= 0 ? fkey(q.bl[lane] + 0.f) : 0u;   // (-0 ties with 0)
+    const unsigned top = __reduce_max_sync(FULL, key);
+    const bool lead = bd >= 0 && key == top;
+    const unsigned d0 = __reduce_min_sync(FULL, lead ? (unsigned)bd : ~0u);
+    const bool lead_d = lead && (unsigned)bd == d0;
+    const unsigned j0 = __reduce_min_sync(FULL, lead_d ? q.bj[lane] : ~0u);
+    const unsigned m = __ballot_sync(FULL, lead_d && q.bj[lane] == j0);
+    SlotBest sb{-INFINITY, NAN, NAN, 0u, -1};
+    if (m) {
+        const int l = __ffs(m) - 1;
+        sb = SlotBest{q.bl[l], q.bD[l], q.bs2[l], q.bj[l], q.bd[l]};
     }
     if (nw > 1) {
         if (lane == 0) it.wb[w] = sb;
@@ -2974,22 +2984,13 @@ extern "C" nu_status nu_periodic_search(const double* t0s_dev, int64_t n_t0,
     if (s != NU_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
-    // grid end points (host copies; the step, when not given, is the median
-    // spacing of the epochs)
+    // grid end points (the step, when not given, is the median spacing of the
+    // epochs)
     double ends[2];
     double t_ref, t_last;
     if (!(phase_step > 0.0)) {
-        std::vector<double> h(n_t0);
-        e = cudaMemcpyAsync(h.data(), t0s_dev, n_t0 * sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "nu_periodic_search: copy t0s");
-        std::vector<double> d(n_t0 - 1);
-        for (int64_t i = 0; i + 1 < n_t0; ++i) d[i] = h[i + 1] - h[i];
-        std::sort(d.begin(), d.end());
-        const size_t m = d.size();
-        phase_step = (m % 2) ? d[m / 2] : 0.5 * (d[m / 2 - 1] + d[m / 2]);
-        t_ref = h[0];
-        t_last = h[n_t0 - 1];
+        e = median_spacing(t0s_dev, n_t0, st, &phase_step, &t_ref, &t_last);
+        if (e != cudaSuccess) return cuda_fail(e, "nu_periodic_search: median spacing");
     } else {
         e = cudaMemcpyAsync(&ends[0], t0s_dev, sizeof(double), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess)

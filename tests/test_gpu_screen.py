@@ -77,6 +77,34 @@ def test_mixed_irregular_screen_equals_every_cell(kind, consistent):
         np.testing.assert_array_equal(got[k], every[k], err_msg=k)
 
 
+@pytest.mark.parametrize("kind, precision, n, n_D", [
+    ("regular", "fp64", 15500, 14), ("drift", "fp64", 15500, 14), ("jitter", "fp64", 15500, 14),
+    ("regular", "mixed", 33000, 13), ("drift", "mixed", 33000, 13),
+    ("regular", "fp64", 70000, 3), ("regular", "mixed", 130000, 3),
+    ("regular", "fp64", 190000, 1), ("drift", "mixed", 350000, 1)])
+def test_filters_equal_every_cell_screened(kind, precision, n, n_D):
+    """The filters over groups of cells drop nothing that could win: on grids
+    whose filter tables (and only those) exceed the fixed scratch, the
+    allocation-free entry point screens every cell.  Periods from 1.3 to 600
+    epochs per cell, each filter's range and its limits."""
+    t, depth, var, dlnl, dt = _grid(n, n_D, 5 + n_D, kind)
+    span = t[-1] - t[0]
+    rng = np.random.default_rng(1)
+    K = np.concatenate([np.exp(rng.uniform(np.log(1.3), np.log(30.0), 90)),
+                        [5.4, 5.6, 21.9, 22.1, 50.0, 150.0, 600.0]])
+    periods = np.concatenate([span / K, [200 * dt, 1000.5 * dt]])
+    every = _fold(api.nu_periodic_search_noalloc, t, depth, var, dlnl, periods, precision, dt)
+    got = _fold(api.nu_periodic_search, t, depth, var, dlnl, periods, precision, dt)
+    for k in KEYS:
+        np.testing.assert_array_equal(got[k], every[k], err_msg=k)
+    # and with two warps or one per period instead of a block
+    for copies in (70, 410):
+        got = _fold(api.nu_periodic_search, t, depth, var, dlnl, np.tile(periods, copies),
+                    precision, dt)
+        for k in KEYS:
+            np.testing.assert_array_equal(got[k], np.tile(every[k], copies), err_msg=k)
+
+
 @pytest.mark.parametrize("kind, precision", [("regular", "fp64"), ("drift", "fp64"),
                                              ("jitter", "fp64"), ("drift", "mixed"),
                                              ("jitter", "mixed")])
