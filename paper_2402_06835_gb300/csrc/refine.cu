@@ -21,13 +21,13 @@
 // (k_refine_blocks), so a zero-input stretch costs one J x J step per block
 // plus single samples at its ends.
 //
-// One warp takes one candidate (k_refine).  GB300 issues one FP64 warp
+// One to eight warps take one candidate (k_refine).  GB300 issues one FP64 warp
 // instruction per 64 cycles per sub-partition, so a candidate's cost is the
-// length of its longest serial chain; the lanes split the samples into RS
-// block-aligned segments and the solve into three phases: each lane's
-// zero-state response of its segment to the template, a short serial pass
-// over the segments' maps (Pseg, k_refine_segs) for the states entering them,
-// and each lane's segment again from its true incoming state.  FP64
+// length of its longest serial chain; the lanes split the samples into
+// block-aligned segments (32 per warp) and the solve into three phases: each
+// lane's zero-state response of its segment to the template, a short serial
+// pass over the segments' maps (Pseg, k_refine_segs) for the states entering
+// them, and each lane's segment again from its true incoming state.  FP64
 // throughout.
 #include <cmath>
 
@@ -38,7 +38,7 @@
 namespace nu {
 
 constexpr int RB = 32;   // samples per tabulated block
-constexpr int RS = 32;   // segments per candidate (one per lane)
+constexpr int RS = 32;   // segments per warp of a candidate (one per lane)
 
 __device__ __forceinline__ int64_t rf_lower_bound(const double* __restrict__ t, int64_t n,
                                                   double x) {
@@ -54,6 +54,9 @@ __device__ __forceinline__ int64_t rf_lower_bound(const double* __restrict__ t, 
 // [b RB, (b+1) RB): with s the state entering sample b RB and zero input,
 // the state leaving the block is Phi_b s and the block's sum of e_i^2 / D_i
 // is s^T M_b s.  Only blocks whose transitions all exist ((b+1) RB <= n-1).
+// A lane per column of Phi: a block's chain is 32 dependent samples of FP64
+// work, and a lane for a whole block left 5 thread blocks on the GPU (83 us at
+// 19 440 samples).
 template <int NB>
 __global__ void __launch_bounds__(128)
 k_refine_blocks(const double* __restrict__ F, const double* __restrict__ kg,
@@ -61,54 +64,48 @@ k_refine_blocks(const double* __restrict__ F, const double* __restrict__ kg,
                 double* __restrict__ Mq) {
     constexpr int J = Dims<NB>::J;
     constexpr int JJ = Dims<NB>::JJ;
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= n_blk) return;
-    double Ph[J][J], M[JJ];
+    // J lanes per block (8 or 32 / J rounded down: J = 6 uses 30 lanes of a warp)
+    constexpr int PER = 32 / J;
+    const int lane = threadIdx.x & 31, c = lane % J, base = lane - c;
+    const int64_t b = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * PER +
+                      lane / J;
+    const bool on = lane < PER * J && b < n_blk;
+    // column c of Phi and of M (rows <= c)
+    double col[J], M[J];
 #pragma unroll
-    for (int r = 0; r < J; ++r)
-#pragma unroll
-        for (int c = 0; c < J; ++c) Ph[r][c] = r == c ? 1.0 : 0.0;
-#pragma unroll
-    for (int a = 0; a < JJ; ++a) M[a] = 0.0;
-    const int64_t i0 = b * RB;
+    for (int r = 0; r < J; ++r) {
+        col[r] = r == c ? 1.0 : 0.0;
+        M[r] = 0.0;
+    }
+    const int64_t i0 = on ? b * RB : 0;
     for (int64_t i = i0; i < i0 + RB; ++i) {
         // g^T = h^T Phi: the innovation of sample i is -g^T s
-        double g[J];
+        double g = col[0];
 #pragma unroll
-        for (int c = 0; c < J; ++c) {
-            double v = Ph[0][c];
-#pragma unroll
-            for (int q = 1; q < NB; ++q) v += Ph[2 * q][c];
-            g[c] = v;
-        }
+        for (int q = 1; q < NB; ++q) g += col[2 * q];
         const double iD = invD[i];
+        const double gi = g * iD;
 #pragma unroll
         for (int r = 0; r < J; ++r) {
-            const double gr = g[r] * iD;
-#pragma unroll
-            for (int c = r; c < J; ++c) M[pk(r, c, J)] = fma(gr, g[c], M[pk(r, c, J)]);
+            const double gr = __shfl_sync(0xffffffffu, gi, (base + r) & 31);
+            M[r] = fma(gr, g, M[r]);
         }
         // Phi <- F_{i+1} (Phi - kg_i g^T)
         const double* kgi = kg + i * J;
         const double* f = F + (i + 1) * NB * 4;
+        double tmp[J];
 #pragma unroll
-        for (int c = 0; c < J; ++c) {
-            double col[J], out[J];
-#pragma unroll
-            for (int r = 0; r < J; ++r) col[r] = fma(-kgi[r], g[c], Ph[r][c]);
-            apply_F<NB>(f, col, out);
-#pragma unroll
-            for (int r = 0; r < J; ++r) Ph[r][c] = out[r];
-        }
+        for (int r = 0; r < J; ++r) tmp[r] = fma(-kgi[r], g, col[r]);
+        apply_F<NB>(f, tmp, col);
     }
+    if (!on) return;
     double* po = Phi + b * J * J;
-#pragma unroll
-    for (int r = 0; r < J; ++r)
-#pragma unroll
-        for (int c = 0; c < J; ++c) po[r * J + c] = Ph[r][c];
     double* mo = Mq + b * JJ;
 #pragma unroll
-    for (int a = 0; a < JJ; ++a) mo[a] = M[a];
+    for (int r = 0; r < J; ++r) {
+        po[r * J + c] = col[r];
+        if (r <= c) mo[pk(r, c, J)] = M[r];
+    }
 }
 
 // One sample of the forward solve with input x: e = x - h^T s, adds e^2/D_i,
@@ -255,10 +252,10 @@ __device__ __forceinline__ bool rf_segment(const double* __restrict__ t, int64_t
 template <int NB>
 __global__ void __launch_bounds__(128)
 k_refine_segs(const double* __restrict__ Phi, int64_t n_blk, int64_t nbs,
-              double* __restrict__ Pseg) {
+              int n_segs, double* __restrict__ Pseg) {
     constexpr int J = Dims<NB>::J;
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= RS * J) return;
+    if (gid >= n_segs * J) return;
     const int g = gid / J, col = gid - g * J;
     double v[J];
 #pragma unroll
@@ -282,15 +279,21 @@ k_refine_segs(const double* __restrict__ Phi, int64_t n_blk, int64_t nbs,
     for (int r = 0; r < J; ++r) Pseg[(int64_t)g * J * J + r * J + col] = v[r];
 }
 
-// One warp per candidate; lane g owns segment g (nbs blocks of RB samples).
-// (a) each lane: the zero-state response of its segment to the template,
+// W warps per candidate; thread g of them owns segment g of 32 W (nbs blocks of
+// RB samples each).
+// (a) each thread: the zero-state response of its segment to the template,
 //     beta_g, at the segment's end;
-// (b) lane 0: the states entering the segments, S_{g+1} = Pseg_g S_g + beta_g;
-// (c) each lane between the first and the last segment with a template
+// (b) the states entering the segments, S_{g+1} = Pseg_g S_g + beta_g, by J
+//     lanes of the first warp, a row each;
+// (c) each thread between the first and the last segment with a template
 //     sample: its segment again from S_g, accumulating e^2/D, num and bt; the
 //     last one closes with the future information G after its last window.
-template <int NB, int TMPL>
-__global__ void __launch_bounds__(128)
+// A candidate's time is the serial FP64 chain of its longest segment walk (64
+// cycles per instruction), so while the candidates leave sub-partitions idle,
+// more warps share one.  64 candidates on 19 440 samples: 1.00 ms with one warp
+// each, 0.47 ms with eight (J lanes per block in k_refine_blocks included).
+template <int NB, int TMPL, int W>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
 k_refine(const double* __restrict__ t, int64_t n, int k, FactorView<double> fv,
          const double* __restrict__ Phi, const double* __restrict__ Mq, int64_t n_blk,
          const double* __restrict__ Pseg, int64_t nbs, const double* __restrict__ Ps,
@@ -301,23 +304,34 @@ k_refine(const double* __restrict__ t, int64_t n, int k, FactorView<double> fv,
     constexpr int J = Dims<NB>::J;
     constexpr int JJ = Dims<NB>::JJ;
     constexpr unsigned FULL = 0xffffffffu;
-    __shared__ double sh_b[4][RS][J];        // beta_g, then S_g
-    __shared__ int sh_any[4][RS];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t cid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (cid >= n_cand) return;                                  // whole warps
-    if (lane == 0) {
+    constexpr int NC = W == 1 ? 4 : 1;       // candidates per block
+    constexpr int NS = 32 * W;               // segments
+    __shared__ double sh_b[NC][NS][J];       // beta_g, then S_g
+    __shared__ unsigned sh_any[NC][W];       // segments with a template sample, per warp
+    __shared__ int sh_bad[NC];
+    __shared__ double sh_sum[W][2 + NU_MAX_K];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int w = W == 1 ? wid : 0, v = W == 1 ? 0 : wid;    // candidate, warp of it
+    const int seg = 32 * v + lane;
+    auto sync = [&]() {
+        if (W == 1) __syncwarp(); else __syncthreads();
+    };
+    const int64_t cid = W == 1 ? (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5
+                               : (int64_t)blockIdx.x;
+    if (cid >= n_cand) return;                                  // whole candidates
+    if (seg == 0) {
         out_depth[cid] = NAN;
         out_var[cid] = NAN;
         out_dlnl[cid] = NAN;
         out_snr[cid] = NAN;
+        sh_bad[w] = 0;
     }
     const int jd = Didx[cid];
     if (jd < 0 || jd >= n_D) return;
     const double P = Ps[cid], T0 = T0s[cid], D = Ds[jd];
     if (!isfinite(P) || !isfinite(T0) || !(D > 0.0) || !(2.0 * D <= P)) return;
     const double half = D * 0.5;
-    const int64_t seg_lo0 = (int64_t)lane * nbs * RB;
+    const int64_t seg_lo0 = (int64_t)seg * nbs * RB;
     const int64_t seg_lo = seg_lo0 < n ? seg_lo0 : n;
     const int64_t seg_hi = seg_lo0 + nbs * RB < n ? seg_lo0 + nbs * RB : n;
     bool bad = false;
@@ -335,62 +349,71 @@ k_refine(const double* __restrict__ t, int64_t n, int k, FactorView<double> fv,
                                                  bad);
     if (any && seg_hi < n) rf_zero_walk<NB, false>(fv, n, Phi, Mq, n_blk, cur, seg_hi, s, c2);
 #pragma unroll
-    for (int q = 0; q < J; ++q) sh_b[w][lane][q] = any ? s[q] : 0.0;
-    sh_any[w][lane] = any ? 1 : 0;
-    if (__any_sync(FULL, bad)) return;
-    __syncwarp();
+    for (int q = 0; q < J; ++q) sh_b[w][seg][q] = any ? s[q] : 0.0;
     const unsigned have = __ballot_sync(FULL, any);
-    if (have == 0u) return;                                     // no sample in any window
-    const int first = __ffs(have) - 1, last = 31 - __clz(have);
+    if (lane == 0) sh_any[w][v] = have;
+    sync();
+    if (bad) sh_bad[w] = 1;
+    sync();
+    if (sh_bad[w]) return;
+    int first = NS, last = -1;
+    for (int i = 0; i < W; ++i) {
+        const unsigned m = sh_any[w][i];
+        if (m == 0u) continue;
+        if (first == NS) first = 32 * i + __ffs(m) - 1;
+        last = 32 * i + 31 - __clz(m);
+    }
+    if (last < 0) return;                                       // no sample in any window
 
     // (b)
-    if (lane == 0) {
-        double x[J];
-#pragma unroll
-        for (int q = 0; q < J; ++q) x[q] = 0.0;
+    if (v == 0) {
+        const int r = lane < J ? lane : 0;
+        double x = 0.0;                                         // row r of the state
         for (int g = first; g <= last; ++g) {
-            double beta[J];
+            const double beta = sh_b[w][g][r];
+            const double* pg = Pseg + ((int64_t)g * J + r) * J;
+            double a = beta;
 #pragma unroll
-            for (int q = 0; q < J; ++q) {
-                beta[q] = sh_b[w][g][q];
-                sh_b[w][g][q] = x[q];                           // S_g
-            }
-            const double* pg = Pseg + (int64_t)g * J * J;
-            double o[J];
-#pragma unroll
-            for (int r = 0; r < J; ++r) {
-                double a = beta[r];
-#pragma unroll
-                for (int q = 0; q < J; ++q) a = fma(pg[r * J + q], x[q], a);
-                o[r] = a;
-            }
-#pragma unroll
-            for (int q = 0; q < J; ++q) x[q] = o[q];
+            for (int q = 0; q < J; ++q) a = fma(pg[q], __shfl_sync(FULL, x, q), a);
+            if (lane < J) sh_b[w][g][r] = x;                    // S_g
+            x = a;
         }
     }
-    __syncwarp();
+    sync();
 
     // (c)
     c2 = 0.0;
-    if (lane >= first && lane <= last) {
+    if (seg >= first && seg <= last) {
 #pragma unroll
-        for (int q = 0; q < J; ++q) s[q] = sh_b[w][lane][q];
+        for (int q = 0; q < J; ++q) s[q] = sh_b[w][seg][q];
         rf_segment<NB, TMPL, true>(t, n, k, fv, Phi, Mq, n_blk, seg_lo, seg_hi, P, T0, D, half,
-                                   ta, s, lane == first, c2, num, bt, cur, bad);
-        if (lane == last) {
+                                   ta, s, seg == first, c2, num, bt, cur, bad);
+        if (seg == last) {
             if (cur < n) c2 += rf_quad<J>(fv.G + cur * JJ, s);   // zero input to the end
         } else {
             rf_zero_walk<NB, true>(fv, n, Phi, Mq, n_blk, cur, seg_hi, s, c2);
         }
     }
-    if (__any_sync(FULL, bad)) return;
+    __syncwarp();
     for (int o = 16; o > 0; o >>= 1) {
         c2 += __shfl_xor_sync(FULL, c2, o);
         num += __shfl_xor_sync(FULL, num, o);
 #pragma unroll
         for (int q = 0; q < NU_MAX_K; ++q) bt[q] += __shfl_xor_sync(FULL, bt[q], o);
     }
-    if (lane != 0) return;
+    if (bad) sh_bad[w] = 1;
+    if (W > 1 && lane == 0) {
+        sh_sum[v][0] = c2;
+        sh_sum[v][1] = num;
+        for (int q = 0; q < NU_MAX_K; ++q) sh_sum[v][2 + q] = bt[q];
+    }
+    sync();
+    if (sh_bad[w] || seg != 0) return;
+    for (int i = 1; i < W; ++i) {
+        c2 += sh_sum[i][0];
+        num += sh_sum[i][1];
+        for (int q = 0; q < NU_MAX_K; ++q) bt[q] += sh_sum[i][2 + q];
+    }
     double bb = 0.0;
     for (int q = 0; q < k; ++q) bb = fma(bt[q], bt[q], bb);
     const double sch = c2 - bb;
@@ -403,6 +426,11 @@ k_refine(const double* __restrict__ t, int64_t n, int k, FactorView<double> fv,
     out_snr[cid] = dep / sqrt(var);
 }
 
+// Warps per candidate: as many as leave every warp an FP64 pipe of its own
+// (608 sub-partitions: 76 x 8, 304 x 2); beyond, more warps only take turns and
+// add segments to walk.
+static int refine_warps(int64_t n_cand) { return n_cand <= 76 ? 8 : (n_cand <= 304 ? 2 : 1); }
+
 template <int NB>
 static void launch_refine(const nu_factor* f, const double* Phi, const double* Mq,
                           int64_t n_blk, double* Pseg, const double* P, const double* T0,
@@ -410,27 +438,29 @@ static void launch_refine(const nu_factor* f, const double* Phi, const double* M
                           const TmplArgs& ta, double* d, double* v, double* l, double* snr,
                           cudaStream_t st) {
     const FactorView<double> fv{f->F, f->kg, f->invD, f->G, f->z0, f->Zt};
-    const int th = 128;
-    // segments of nbs blocks cover every sample: RS * nbs * RB >= n
+    const int W = refine_warps(n_cand);
+    // segments of nbs blocks cover every sample: n_segs * nbs * RB >= n
+    const int n_segs = RS * W;
     const int64_t blocks_all = (f->n + RB - 1) / RB;
-    const int64_t nbs = (blocks_all + RS - 1) / RS;
+    const int64_t nbs = (blocks_all + n_segs - 1) / n_segs;
+    constexpr int PER = 32 / (2 * NB);                   // blocks per warp
     if (n_blk > 0)
-        k_refine_blocks<NB><<<div_up(n_blk, th), th, 0, st>>>(f->F, f->kg, f->invD, n_blk,
-                                                             (double*)Phi, (double*)Mq);
-    k_refine_segs<NB><<<div_up(RS * 2 * NB, th), th, 0, st>>>(Phi, n_blk, nbs, Pseg);
-    const int grid = div_up(n_cand * 32, th);
-    if (tmpl == NU_BOX)
-        k_refine<NB, NU_BOX><<<grid, th, 0, st>>>(f->t, f->n, f->k, fv, Phi, Mq, n_blk, Pseg,
-                                                 nbs, P, T0, Didx, n_cand, Ds, n_D, ta, d, v, l,
-                                                 snr);
-    else if (tmpl == NU_TRAPEZOID)
-        k_refine<NB, NU_TRAPEZOID><<<grid, th, 0, st>>>(f->t, f->n, f->k, fv, Phi, Mq, n_blk,
-                                                       Pseg, nbs, P, T0, Didx, n_cand, Ds, n_D,
-                                                       ta, d, v, l, snr);
-    else
-        k_refine<NB, NU_LIMB_QUAD><<<grid, th, 0, st>>>(f->t, f->n, f->k, fv, Phi, Mq, n_blk,
-                                                       Pseg, nbs, P, T0, Didx, n_cand, Ds, n_D,
-                                                       ta, d, v, l, snr);
+        k_refine_blocks<NB><<<div_up(n_blk, PER), 32, 0, st>>>(f->F, f->kg, f->invD, n_blk,
+                                                               (double*)Phi, (double*)Mq);
+    k_refine_segs<NB><<<div_up(n_segs * 2 * NB, 32), 32, 0, st>>>(Phi, n_blk, nbs, n_segs, Pseg);
+#define NU_REFINE(T_, W_)                                                                  \
+    k_refine<NB, T_, W_><<<W_ == 1 ? div_up(n_cand, 4) : (int)n_cand, W_ == 1 ? 128 : 32 * W_, \
+                           0, st>>>(f->t, f->n, f->k, fv, Phi, Mq, n_blk, Pseg, nbs, P, T0, \
+                                    Didx, n_cand, Ds, n_D, ta, d, v, l, snr)
+#define NU_REFINE_W(T_)                                                                    \
+    do {                                                                                   \
+        if (W == 8) NU_REFINE(T_, 8); else if (W == 2) NU_REFINE(T_, 2); else NU_REFINE(T_, 1); \
+    } while (0)
+    if (tmpl == NU_BOX) NU_REFINE_W(NU_BOX);
+    else if (tmpl == NU_TRAPEZOID) NU_REFINE_W(NU_TRAPEZOID);
+    else NU_REFINE_W(NU_LIMB_QUAD);
+#undef NU_REFINE_W
+#undef NU_REFINE
 }
 
 }  // namespace nu
@@ -461,7 +491,7 @@ extern "C" nu_status nu_periodic_refine(const nu_factor* f, const double* P_dev,
     cudaStream_t st = (cudaStream_t)stream;
     const int J = 2 * f->nb, JJ = J * (J + 1) / 2;
     const int64_t n_blk = (f->n - 1) / RB;
-    const size_t bytes = (n_D + n_blk * (int64_t)(J * J + JJ) + RS * J * J) * sizeof(double);
+    const size_t bytes = (n_D + n_blk * (int64_t)(J * J + JJ) + RS * refine_warps(n_cand) * J * J) * sizeof(double);
     pool_keep_memory();
     double* mem = nullptr;
     cudaError_t e = cudaMallocAsync(&mem, bytes, st);
