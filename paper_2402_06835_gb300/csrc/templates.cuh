@@ -30,8 +30,17 @@ __device__ __forceinline__ double template_value(double t, double t0, double hal
     if (TMPL == NU_BOX) return -1.0;
     if (TMPL == NU_TRAPEZOID) {
         const double ramp = __dmul_rn(a.p0, D);
-        const double dd = __ddiv_rn(__dsub_rn(half, fabs(__dsub_rn(t, t0))), ramp);
-        return -fmin(fmax(dd, 0.0), 1.0);
+        const double x = __dsub_rn(half, fabs(__dsub_rn(t, t0)));
+        // Neighbouring lanes hold neighbouring epochs, so most steps of a warp
+        // lie on the plateau for all its lanes: the division (a dozen FP64
+        // instructions of 64 cycles each) is left to the ramps, and the
+        // comparisons are on the bits (x >= ramp, positive and finite: the
+        // quotient rounds to 1 or more; x <= 0: it is clamped to 0).  19 440
+        // epochs x 10 durations of 20 min to 3 h, FP64: 608 -> 473 us.
+        const long long xb = __double_as_longlong(x), rb = __double_as_longlong(ramp);
+        if (xb >= rb && rb > 0 && rb < 0x7ff0000000000000ll) return -1.0;
+        if (xb <= 0) return 0.0;
+        return -fmin(__ddiv_rn(x, ramp), 1.0);
     }
     const double r = __ddiv_rn(__dmul_rn(2.0, __dsub_rn(t, t0)), D);
     const double mu = __dsqrt_rn(__dsub_rn(1.0, __dmul_rn(r, r)));
