@@ -1457,6 +1457,24 @@ template <typename T> struct FoldPrep {
     unsigned long long* peak;
     unsigned end[PREP_N];
 };
+// The same on the slot path: blocks [0, b_rec) clear the slot records, [b_rec,
+// b_peak) find the largest gain, the rest fill the period table.
+__global__ void __launch_bounds__(256)
+k_slot_prep(Node4<float>* __restrict__ rec, int64_t n_rec, unsigned b_rec,
+            const float* __restrict__ gain, int64_t n, unsigned b_peak,
+            unsigned long long* __restrict__ peak, const double* __restrict__ periods,
+            int64_t n_P, double dt, SlotPeriod* __restrict__ stab) {
+    const unsigned b = blockIdx.x;
+    if (b < b_rec) {
+        const int64_t i = b * (int64_t)blockDim.x + threadIdx.x;
+        if (i < n_rec) rec[i] = Node4<float>{NAN, NAN, NAN, 0.f};
+    } else if (b < b_peak) {
+        gain_peak<float>(gain, n, b - b_rec, b_peak - b_rec, peak);
+    } else {
+        const int64_t i = (b - b_peak) * (int64_t)blockDim.x + threadIdx.x;
+        if (i < n_P) stab[i] = slot_period(periods[i], dt);
+    }
+}
 template <typename T>
 __global__ void __launch_bounds__(256) k_fold_prep(const __grid_constant__ FoldPrep<T> A) {
     int job = 0;
@@ -2559,7 +2577,7 @@ static cudaError_t launch_filter_tables(const FoldSeg* segs, const FoldSeg& one,
     const int64_t rows = (int64_t)n_seg * n_D;
     const cudaError_t e = cudaMemsetAsync(tab.vmax, 0, (size_t)rows * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
-    const unsigned gy = (unsigned)std::min<int64_t>(std::max<int64_t>(n_t0 / 2048, 1), 64);
+    const unsigned gy = (unsigned)std::min<int64_t>(std::max<int64_t>(n_t0 / 512, 1), 64);
     k_filter_vmax<<<dim3((unsigned)rows, gy), 256, 0, st>>>(screen, rec, segs, one, n_D, tab.vmax);
     k_filter_slots<<<div_up(n_entries, 128), 128, 0, st>>>(screen, vpair, bucket, rec, segs, one,
                                                            n_seg, n_D, n_entries, tab);
@@ -2835,6 +2853,8 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
     // one block of flags: [0] slot test, [1..2] regular-grid test, then the
     // peak key and the candidate counter
     cudaError_t e = cudaMemsetAsync(flag, 0, 256, st);
+    const unsigned peak_grid = (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608);
+    unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
     // the slot path needs a regular grid and a gap rule that only joins
     // neighbouring slots (1 < gap_factor < 2)
     bool use_slots = !fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span_steps < 4.0e6;
@@ -2842,7 +2862,20 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
         int irregular = 0;
         k_slots<<<div_up(n_t0, 256), 256, 0, st>>>(t0s_dev, n_t0, t_ref, 1.0 / phase_step,
                                                   slot_of, flag);
-        ++launched;
+        // The tables of that path are filled before the test is read, so that
+        // the host's next launch is the fold's (an irregular curve overwrites
+        // them: 10 us on the GPU, hidden in part by the wait).
+        const int64_t nrec = n_slots * n_D;
+        Node4<float>* rec = (Node4<float>*)(scratch + L.rec);
+        const unsigned b_rec = (unsigned)div_up(nrec, 256), b_peak = b_rec + peak_grid;
+        const unsigned b_all = b_peak + (L.level == 2 ? (unsigned)div_up(n_P, 256) : 0u);
+        k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, b_rec, (const float*)dlnl_dev, ngrid,
+                                           b_peak, peak, periods_dev, n_P, phase_step,
+                                           (SlotPeriod*)(scratch + L.ptab));
+        k_slot_fill<<<div_up(ngrid, 256), 256, 0, st>>>(
+            (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, slot_of,
+            n_t0, n_D, n_slots, rec);
+        launched += 3;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&irregular, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -2885,10 +2918,29 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
     one.screen = !use_slots && gap_factor < 2.0 && span_steps < 8.0e6 && (fp64 || L.level > 0);
     if (use_slots) one.ulast = slot_ulast(t_ref, t_last, phase_step);
     else one.uspan = exact_uspan(t_ref, t_last, phase_step);
+    // Warps per period: eight where the periods are few for their size, two (and
+    // eight for the long ones) from where they fill the GPU, one from 40 000.
+    // FP64: 4 000 periods of 2 000 epochs x 4 durations 0.49 ms with eight, 0.31
+    // with two, 0.34 with one; 1 200 of 8 000 x 4 0.40 / 0.49 / 0.66; 2 500 of
+    // 19 440 x 10 1.7 with eight, 2.0 with one.
+    const double item_steps = span_steps * n_D;
+    const int nw = n_P >= NU_ONE_WARP_FROM
+                       ? 1
+                       : (n_P >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + item_steps / 32.0)
+                              ? 2 : 8);
+    // Small calls: screening every cell costs less than the filters' tables and
+    // rounds, and a few survivors per block less than the launches that pack
+    // them.  Mixed / FP64, us with filters -> without: 4 000 epochs x 4 durations
+    // x 1 200 periods (19 M steps) 309 / 365 -> 208 / 276, 1 100 x 12 x 300 (4 M)
+    // 239 / 285 -> 158 / 174; 2 000 x 12 x 1 200 (29 M) 269 / 325 -> 272 / 352; one
+    // duration, 8 000 x 4 000 (32 M) 432 / 472 -> 299 / 429.
+    const bool small = item_steps * (double)n_P < (n_D == 1 ? 4.0e7 : 2.4e7);
     if (L.level == 2) {
-        J.tab = filter_tab(scratch + L.tab, L.fl);
         J.ptab = (const PeriodConst*)(scratch + L.ptab);
         J.stab = (const SlotPeriod*)(scratch + L.ptab);
+        if (!small) J.tab = filter_tab(scratch + L.tab, L.fl);
+    }
+    if (L.level == 2 && !(small && (nw == 8 || use_slots))) {
         J.cand = (FoldCand*)(scratch + L.cand);
         J.counters = (unsigned*)(scratch + L.flag + 64);
         J.n_cand = (unsigned long long*)(J.counters + 4);
@@ -2897,24 +2949,7 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
         J.items = (ItemConst*)(scratch + L.items);
         J.sbest = fp64 ? nullptr : (SlotBest*)(scratch + L.sbest);
     }
-    const dim3 peak_grid(1, (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608));
-    unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
-    if (use_slots) {
-        const int64_t nrec = n_slots * n_D;
-        Node4<float>* rec = (Node4<float>*)(scratch + L.rec);
-        k_fill_nan<<<div_up(nrec, 256), 256, 0, st>>>(rec, nrec);
-        k_slot_fill<<<div_up(ngrid, 256), 256, 0, st>>>(
-            (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, slot_of,
-            n_t0, n_D, n_slots, rec);
-        k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)dlnl_dev, nullptr, n_t0, n_D,
-                                                      peak);
-        launched += 3;
-        if (J.stab) {
-            k_slot_periods<<<div_up(n_P, 256), 256, 0, st>>>(periods_dev, n_P, phase_step,
-                                                             (SlotPeriod*)(scratch + L.ptab));
-            ++launched;
-        }
-    } else {
+    if (!use_slots) {
         const double gap_max = gap_factor * phase_step;
         ScreenRec* screen = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
         ulonglong2* vpair = (ulonglong2*)(scratch + L.exact + L.el.off_vpos);
@@ -2927,7 +2962,7 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
                           slot_of, (unsigned*)(flag + 1), srec, periods_dev, n_P,
                           J.ptab ? (PeriodConst*)(scratch + L.ptab) : nullptr, peak, {}};
             const unsigned blocks[PREP_N] = {
-                (unsigned)div_up(n_bucket, 256), one.screen ? peak_grid.y : 0u,
+                (unsigned)div_up(n_bucket, 256), one.screen ? peak_grid : 0u,
                 one.screen && J.ptab ? (unsigned)div_up(n_P, 256) : 0u,
                 one.screen && srec ? (unsigned)div_up(n_t0, 256) : 0u,
                 one.screen && srec ? (unsigned)div_up(n_slots * n_D, 256) : 0u,
@@ -2969,10 +3004,6 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
     if (J.tab.S)
         e = launch_filter_tables(nullptr, one, 1, n_D, filter_slots(n_slots) * n_D, n_t0, J.screen,
                                  J.vpair, J.bucket, J.rec, J.tab, st, &launched);
-    // Warps per period: eight where the periods are few, one or two (and eight
-    // for the long ones) where they alone fill the GPU.  Sector grid, FP64, at
-    // 2 500 periods 1.7 ms with eight, 2.0 with one.
-    const int nw = n_P >= NU_ONE_WARP_FROM ? 1 : (n_P >= NU_WARP_ITEMS_FROM ? 2 : 8);
     if (J.items && nw != 8)
         J.list = FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K};
     launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, thread_side_stream(), &e);
