@@ -267,7 +267,7 @@ def pipeline_entry(name, pipe, stages, world, ncu=None, clock_mhz=None):
             "fold_visits_per_s": visits / (float(sm[2]) / 1e3),
             "roofline": fold_roofline(len(lc.t), n_D, pipe.n_periods, float(sm[2]), visits,
                                       8 if fp64 else 4,
-                                      "k_fold_screened" if fp64 else "k_fold_slots",
+                                      "k_fold_cells" if fp64 else "k_fold_slot_cells",
                                       ncu, clock_mhz)}
 
 

@@ -3,9 +3,9 @@
 // The curves are packed back to back.  Every stage treats them as segments
 // of one problem: the factor scans run over the chunks of all curves (a
 // chunk never crosses a curve), the linear search covers every curve's
-// (D, t0) grid with t0 = its samples, and the fold is a persistent kernel
-// that takes (curve, period) work items from device counters, which
-// balances curves of different spans.  Host work (validation, layout, a
+// (D, t0) grid with t0 = its samples, and the fold runs over (curve, period)
+// items, the long ones by blocks and the others by warps, with one list of the
+// cells left for exact evaluation.  Host work (validation, layout, a
 // regularity test of each curve's cadence, uploads of the small tables)
 // happens before capture; the kernels are captured into one CUDA graph and
 // launched once.  The instantiated graph of a configuration is kept and, on

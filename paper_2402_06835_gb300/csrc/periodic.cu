@@ -1,7 +1,6 @@
 // nu_periodic_search: Sect. 2.3-2.4 on the products of the linear search.
 //
-// For each trial period P (one thread block), every (duration d, phase j)
-// cell gathers its single events at epochs T_k = T_ref + (j/n_phi + k) P,
+// For each trial period P every (duration d, phase j) cell gathers its single events at epochs T_k = T_ref + (j/n_phi + k) P,
 // linearly interpolated in time between the bracketing grid epochs, and
 // combines them with Eq. result using the biased estimates of
 // Eq. sigma_delta:
@@ -527,9 +526,8 @@ __global__ void k_period_consts(const double* __restrict__ periods, int64_t n_P,
 }
 
 // Per-period constants of the slot path: phases, and the epoch and phase
-// steps in 24.40 fixed point.  The single-curve fold computes them per block;
-// the batch reads them from a table filled by the same function
-// (k_slot_periods), so both fold a curve identically.  bad marks a period
+// steps in 24.40 fixed point, in a table (k_slot_prep, k_slot_periods) or, where
+// there is no room for one, per item by the same function.  bad marks a period
 // that is not folded for any curve (the curve's own limit, a span of more
 // than 1e9 periods, is tested per curve).
 struct SlotPeriod {
@@ -1198,8 +1196,9 @@ __device__ __forceinline__ float screen_cell(const FoldGeom& g, const ScreenGeom
 }
 
 // ------------------------------------------------------- the cell kernels
-// Both paths fold one (curve, period) item by one warp, or by the eight warps
-// of a block where its cells are long: the filters (filter.cuh) over all cells, the FP32 screen (exact paths) or the first pass
+// Both paths fold one (curve, period) item by one or two warps, or by the eight
+// warps of a block where its cells are long or the items few: the filters
+// (filter.cuh) over all cells, the FP32 screen (exact paths) or the first pass
 // (slot path) of the cells they leave, then the evaluation of the few cells
 // whose bound reaches the threshold.  The threshold is a lower bound of the
 // best ln P: every screened cell gives a lower bound beside its upper bound,
@@ -1401,9 +1400,8 @@ __device__ __forceinline__ bool evaluate_cell_warp(const FoldGeom& g,
 // = (order key of the gain rounded to FP32) << 32 | (2^32 - 1 - e), the
 // maximum over the curve's grid entries e (duration-major, e < 2^32 - 1), so
 // the largest rounded gain wins and ties go to the first entry.  key[g] must
-// be zero on entry and stays zero when no gain is finite.  blockIdx.x is the
-// curve (s_off == nullptr: one curve of n_t0 epochs); the blocks along y
-// share a curve's entries.
+// be zero on entry and stays zero when no gain is finite.  n_blocks blocks share
+// a curve's entries (k_gain_peak: blockIdx.x is the curve of a batch).
 template <typename T>
 __device__ __forceinline__ void gain_peak(const T* __restrict__ row, int64_t n, unsigned block,
                                           unsigned n_blocks, unsigned long long* __restrict__ key) {
@@ -1426,11 +1424,10 @@ __device__ __forceinline__ void gain_peak(const T* __restrict__ row, int64_t n, 
 }
 template <typename T>
 __global__ void k_gain_peak(const T* __restrict__ gain, const int64_t* __restrict__ s_off,
-                            int64_t n_t0, int n_D, unsigned long long* __restrict__ key) {
+                            int n_D, unsigned long long* __restrict__ key) {
     const int g = blockIdx.x;
-    const int64_t s0 = s_off ? s_off[g] : 0;
-    const int64_t ng = s_off ? s_off[g + 1] - s0 : n_t0;
-    gain_peak<T>(gain + s0 * n_D, ng * n_D, blockIdx.y, gridDim.y, key + g);
+    const int64_t s0 = s_off[g];
+    gain_peak<T>(gain + s0 * n_D, (s_off[g + 1] - s0) * n_D, blockIdx.y, gridDim.y, key + g);
 }
 
 // The tables of one curve's exact path that only read the inputs, in one
@@ -2085,8 +2082,8 @@ struct SCell {
 // slot centres (checked to be below 1e-3 slot).
 //
 // Per item: the filters, whose tables hold the events of this walk; the first
-// pass (FP32 compensated sums) of the cells they leave, with the bound of
-// cannot_win_f and a lower bound that raises the threshold; and the second
+// pass (FP32 compensated sums) of the cells they leave, with the bounds of
+// SlotPass1, the lower one raising the threshold; and the second
 // pass of the cells whose bound still reaches it, at the end or when 32 are
 // queued.
 struct SlotItem {
@@ -2636,10 +2633,10 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
         launched += 2;
     }
     if (fp64)
-        k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)gain, s_off_dev, 0, n_D,
+        k_gain_peak<double><<<peak_grid, 256, 0, st>>>((const double*)gain, s_off_dev, n_D,
                                                        fs.peak);
     else
-        k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)gain, s_off_dev, 0, n_D,
+        k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)gain, s_off_dev, n_D,
                                                       fs.peak);
     ++launched;
     e = launch_filter_tables(segs_dev, FoldSeg{}, n_seg, n_D, fb.n_tab_total, n_total / n_seg,
