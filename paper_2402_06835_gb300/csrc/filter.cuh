@@ -253,8 +253,9 @@ __device__ __forceinline__ int64_t filter_pair(const FoldSeg& sg, int n_D, int d
 }
 
 // L, S, gB and Z of every (duration, slot).  Grids of the exact paths: from
-// the screening records and epoch positions.  Slot path: an event in slot s
-// interpolates the records of s and s + 1, nothing else.
+// the screening records and epoch positions (the last epoch's interval is
+// invalid, so the slot that holds it only counts its gains).  Slot path: an
+// event in slot s interpolates the records of s and s + 1, nothing else.
 __global__ void k_filter_slots(const ScreenRec* __restrict__ screen,
                                const ulonglong2* __restrict__ vpair,
                                const int* __restrict__ bucket,
@@ -296,7 +297,11 @@ __global__ void k_filter_slots(const ScreenRec* __restrict__ screen,
                 }
             }
         }
-        write_slot(tab, o, so, any, false, odd, zA, zB, e, v, gA, gB, lmax);
+        // The last epoch may lie up to 1e-3 slot before its slot: positions past it
+        // on the interval that ends there have no event, and a group's walk may
+        // reach them while its first phase has not (only the gains count then).
+        const bool past = ((unsigned long long)fs.s + 1ull) << 40 > sg.ulast + 1ull;
+        write_slot(tab, o, so, any, past, odd, zA, zB, e, v, gA, gB, lmax);
         return;
     }
     if (!sg.screen) return;
