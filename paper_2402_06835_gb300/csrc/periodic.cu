@@ -2696,7 +2696,12 @@ static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int
             }
             if (nw == 2) NU_CELLS(2, (unsigned)items, st);
             else NU_CELLS(1, div_up(items, 4), st);
-            if (forked) check(cudaStreamWaitEvent(st, join, 0));
+            if (forked) {
+                const cudaError_t ej = cudaStreamWaitEvent(st, join, 0);
+                check(ej);
+                // not joined: the caller gives the scratch back in st's order
+                if (ej != cudaSuccess) cudaStreamSynchronize(side);
+            }
             if (fork) cudaEventDestroy(fork);
             if (join) cudaEventDestroy(join);
         }
@@ -2833,14 +2838,17 @@ static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, int64
 
 // Enqueue the fold of one light curve on st with its scratch at `scratch`
 // (laid out by single_layout).  The mixed-precision slot test reads one flag
-// back (one synchronisation of st).
+// back (one synchronisation of st).  fork: the block items of a call with a
+// list may run on a side stream (two events per call, and the stream with the
+// thread's first such call).
 static nu_status single_fold(const char* who, char* scratch, const SingleLayout& L,
                              const double* t0s_dev, int64_t n_t0, int n_D, const void* depth_dev,
                              const void* var_dev, const void* dlnl_dev, bool fp64,
                              const double* periods_dev, int64_t n_P, double phase_step,
                              double gap_factor, double t_ref, double t_last, int64_t n_bucket,
-                             cudaStream_t st, double* Q_dev, double* T0_dev, int32_t* D_idx_dev,
-                             double* depth_out_dev, double* sigma_out_dev, double* lnP_dev) {
+                             cudaStream_t st, bool fork, double* Q_dev, double* T0_dev,
+                             int32_t* D_idx_dev, double* depth_out_dev, double* sigma_out_dev,
+                             double* lnP_dev) {
     const double span_steps = (t_last - t_ref) / phase_step;
     const int64_t ngrid = n_t0 * (int64_t)n_D;
     const int64_t n_slots = n_bucket + 2;
@@ -3003,7 +3011,8 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
                                  J.vpair, J.bucket, J.rec, J.tab, st, &launched);
     if (J.items && nw != 8)
         J.list = FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K};
-    launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, thread_side_stream(), &e);
+    const cudaStream_t side = fork && J.list.block ? thread_side_stream() : nullptr;
+    launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, side, &e);
     count_launches(launched);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, (std::string(who) + ": launch").c_str());
@@ -3079,7 +3088,7 @@ extern "C" nu_status nu_periodic_search(const double* t0s_dev, int64_t n_t0,
     e = cudaMallocAsync((void**)&scratch, L.total, st);
     if (e != cudaSuccess) return cuda_fail(e, "nu_periodic_search: cudaMallocAsync");
     s = single_fold(who, scratch, L, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev, fp64,
-                    periods_dev, n_P, phase_step, gap_factor, t_ref, t_last, n_bucket, st,
+                    periods_dev, n_P, phase_step, gap_factor, t_ref, t_last, n_bucket, st, true,
                     Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
     e = cudaFreeAsync(scratch, st);
     if (s != NU_OK) return s;
@@ -3201,7 +3210,9 @@ extern "C" nu_status nu_rotation_alias_filter(const double* periods_dev, int64_t
 // nu_periodic_search_noalloc runs the same kernels as nu_periodic_search but
 // takes its scratch (epoch records, bucket table, slot table, flag) from the
 // file-scope device array below instead of the stream-ordered pool, for
-// callers that must not allocate device memory.  The array is part of the
+// callers that must not allocate device memory (it creates no stream and no
+// event either: the block items run before the others, on the call's stream).
+// The array is part of the
 // library image: every GPU that loads the library holds it until the process
 // exits.  Its address is looked up once per device (cudaGetSymbolAddress with
 // that device current) on the first call made on the device.
@@ -3297,5 +3308,5 @@ extern "C" nu_status nu_periodic_search_noalloc(const double* t0s_dev, int64_t n
                     L.total, (unsigned long long)NU_NOALLOC_SCRATCH_BYTES);
     return single_fold(who, (char*)base, L, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev,
                        fp64, periods_dev, n_P, phase_step, gap_factor, t_ref, t_last, n_bucket,
-                       st, Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+                       st, false, Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
 }
