@@ -183,6 +183,11 @@ __device__ __forceinline__ void write_slot(const FilterTab& tab, int64_t o, int6
                                            bool any, bool mixed, bool odd, float zA, float zB, float e, float v,
                                            float gA, float gB, float lmax) {
     const float tiny = 1e-30f;
+    if (!tab.S) {                       // the gains alone
+        const float g = fmaxf(lmax * 1.000001f, tiny);
+        tab.L[o] = !any ? 0.f : (odd || !(g < 1e30f) ? INFINITY : g);
+        return;
+    }
     float z0 = 0.f, dz = 0.f, vv = 0.f, a = 0.f, b = 0.f, l = 0.f, zmx = 0.f, zmn = 0.f;
     if (any) {
         l = fmaxf(lmax * 1.000001f, tiny);
@@ -268,9 +273,9 @@ __global__ void k_filter_slots(const ScreenRec* __restrict__ screen,
     FoldSeg sg;
     if (!filter_slot(segs, one, n_seg, n_D, o, fs, sg)) return;
     const int64_t so = filter_pair(sg, n_D, fs.d, fs.s);
-    if (fs.d == n_D - 1 && (n_D & 1))                // the other half of the last pair
+    if (tab.S && fs.d == n_D - 1 && (n_D & 1))       // the other half of the last pair
         tab.S[so + 1] = make_uint2(0u, 0u);
-    const float vm = __uint_as_float(tab.vmax[fs.seg * n_D + fs.d]);
+    const float vm = tab.S ? __uint_as_float(tab.vmax[fs.seg * n_D + fs.d]) : 0.f;
     const float rs = vm > 0.f ? 1.f / sqrtf(vm) : 0.f;
     bool any = false, none = false, odd = false;
     float zA = 0.f, zB = 0.f, e = 0.f, v = INFINITY, gA = -INFINITY, gB = -INFINITY;
@@ -398,7 +403,7 @@ __global__ void k_filter_groups(const FoldSeg* __restrict__ segs, FoldSeg one, i
             break;
         }
         l = fmaxf(l, tab.L[o + w]);
-        if (w < 4) {
+        if (w < 4 && tab.S) {
             const unsigned z = tab.Z[o + w];
             mx = fmaxf(mx, __half2float(__ushort_as_half((unsigned short)(z >> 16))));
             mn = fminf(mn, __half2float(__ushort_as_half((unsigned short)(z & 0xffffu))));
@@ -408,10 +413,13 @@ __global__ void k_filter_groups(const FoldSeg* __restrict__ segs, FoldSeg one, i
     }
     // (-mn and mx: both rounded up; the low half of a word holds the other
     // number as BF16)
-    const int64_t qo = filter_pair(sg, n_D, fs.d, (int64_t)(fs.s & 3) * (ns >> 2) + (fs.s >> 2));
-    tab.Q[qo] = make_uint2(pack_hi(mx, bf16_bits_ru(-mn), true),
-                           pack_hi(v, bf16_bits_ru(g), false));
-    if (fs.d == n_D - 1 && (n_D & 1)) tab.Q[qo + 1] = make_uint2(0u, 0u);
+    if (tab.S) {
+        const int64_t qo =
+            filter_pair(sg, n_D, fs.d, (int64_t)(fs.s & 3) * (ns >> 2) + (fs.s >> 2));
+        tab.Q[qo] = make_uint2(pack_hi(mx, bf16_bits_ru(-mn), true),
+                               pack_hi(v, bf16_bits_ru(g), false));
+        if (fs.d == n_D - 1 && (n_D & 1)) tab.Q[qo + 1] = make_uint2(0u, 0u);
+    }
     const int W = 2 * filter_words(n_D);
     const int gi = fs.d / W;
     __half* G = reinterpret_cast<__half*>(tab.G + sg.g_off) +
@@ -433,9 +441,9 @@ struct FilterView {
 };
 __device__ __forceinline__ FilterView filter_view(const FilterTab& tab, const FoldSeg& sg) {
     FilterView v;
-    v.S = tab.S + sg.pair_off;
-    v.Q = tab.Q + sg.pair_off;
-    v.gB = tab.gB + sg.tab_off;
+    v.S = tab.S ? tab.S + sg.pair_off : nullptr;
+    v.Q = tab.S ? tab.Q + sg.pair_off : nullptr;
+    v.gB = tab.S ? tab.gB + sg.tab_off : nullptr;
     v.L = tab.L + sg.tab_off;
     v.G = tab.G + sg.g_off;
     v.ns = (int)filter_slots(sg.n_slots);
@@ -453,12 +461,15 @@ struct FilterPeriod {
     int mode;
 };
 // (n_cells < 2^31: the filters count groups in 32 bits)
-__device__ __forceinline__ int filter_mode(bool tables, unsigned long long ustep, float K,
-                                           int64_t n_cells) {
-    if (!tables || ustep < (1ull << 32) || ustep >= (1ull << 60) || !(K < FILTER_K_MAX) ||
+__device__ __forceinline__ int filter_mode(const FilterTab& tab, unsigned long long ustep,
+                                           float K, int64_t n_cells) {
+    if (!tab.L || ustep < (1ull << 32) || ustep >= (1ull << 60) || !(K < FILTER_K_MAX) ||
         n_cells >= 0x7fff0000LL)
         return FILTER_NONE;
-    return K < NU_FILTER_K_QUAD ? FILTER_GAIN : (K < NU_FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL);
+    if (K < NU_FILTER_K_QUAD) return FILTER_GAIN;
+    // (without S and Q the cells one by one, by their gains; 19 440 epochs x 12
+    // durations x 3 000 periods, FP64: 1.69 ms, 4.7 in groups of eight)
+    return tab.S && K < NU_FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL;
 }
 
 __device__ __forceinline__ float filter_weight(unsigned long long u) {
@@ -632,13 +643,29 @@ __device__ __noinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q
     return pass;
 }
 
-// Bounds of four phases (Q) or one phase (S) of four durations from d0 (the
-// walk from u; the odd last pair reads its own row twice).  Two epochs a
+// Bounds of four phases (Q) or one phase (S, or L where there are no others) of
+// four durations from d0 (the walk from u; the odd last pair reads its own row
+// twice).  Two epochs a
 // round: a position past the end reads the empty last entry.
 __device__ __noinline__ float4 filter_sums(const FilterCtx& x, unsigned long long u, int d0) {
     const FilterPeriod fp = x.fp;
     const bool quad = fp.mode == FILTER_QUAD;
     const unsigned last = (unsigned)x.f.ns - 1u, n4 = (unsigned)x.f.ns >> 2;
+    if (!x.f.S) {
+        const float* __restrict__ r = x.f.L + (int64_t)d0 * x.f.ns;
+        float l[4] = {0.f, 0.f, 0.f, 0.f};
+        for (; u < fp.uend; u += fp.ustep) {
+            const unsigned o = min((unsigned)(u >> 40), last);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (d0 + i < x.n_D) l[i] += r[(int64_t)i * x.f.ns + o];
+        }
+        const float ch = 1.f + filter_slack(fp);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            l[i] = l[i] > 0.f ? fmaf(l[i], ch, 0.500001f) : -INFINITY;
+        return make_float4(l[0], l[1], l[2], l[3]);
+    }
     const uint4* __restrict__ p0 = reinterpret_cast<const uint4*>(quad ? x.f.Q : x.f.S) +
                                    (int64_t)(d0 >> 1) * x.f.ns;
     const uint4* __restrict__ p1 = p0 + (d0 + 2 < x.n_D ? x.f.ns : 0);
@@ -787,7 +814,7 @@ __device__ __noinline__ void filter_expand(FilterCtx& x, FilterQueues& qs, const
                 float ub = gain ? filter_one_gain(x.f, (int)d, u, x.fp, c)
                                 : filter_one(x.f, (int)d, u, x.fp, c);
                 keep = !(ub < filter_thr(x)) && ub != -INFINITY;
-                if (keep && x.fp.K > 5.5f && x.fp.K < 14.f) {
+                if (keep && x.f.S && x.fp.K > 5.5f && x.fp.K < 14.f) {
                     ub = gain ? filter_one(x.f, (int)d, u, x.fp, c)
                               : filter_one_gain(x.f, (int)d, u, x.fp, c);
                     keep = !(ub < filter_thr(x)) && ub != -INFINITY;
@@ -836,7 +863,7 @@ __device__ __noinline__ void filter_drain(FilterCtx& x, FilterQueues& q, bool al
                                           Screen& screen) {
     const int lane = threadIdx.x & 31;
     const bool gain = x.fp.mode == FILTER_GAIN;
-    const bool mid = gain && x.fp.K >= NU_FILTER_K_MID + 2.f;
+    const bool mid = gain && x.f.Q && x.fp.K >= NU_FILTER_K_MID + 2.f;
     const int ni = q.ni;
     const int round = mid ? 16 : (gain ? 4 : 8);
     const int n = all ? ni : ni & ~(round - 1);

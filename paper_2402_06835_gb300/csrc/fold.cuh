@@ -78,7 +78,9 @@ __host__ __device__ inline int filter_groups(int n_D) {
 }
 
 // Tables of all curves; rows of filter_slots(n_slots) per duration from
-// tab_off on (in rows' entries), G from g_off on (in words).
+// tab_off on (in rows' entries), G from g_off on (in words).  Where scratch is
+// short only L and G are there (S, Q, gB, Z and vmax null): the fold then bounds
+// by gains alone.  All null: no tables.
 struct FilterTab {
     uint2* S;
     float* gB;
@@ -92,20 +94,25 @@ struct FilterTab {
 struct FilterLayout {
     size_t S, gB, L, Z, Q, G, vmax, total;
 };
-inline FilterLayout filter_layout(int64_t entries, int64_t pairs, int64_t words, int64_t rows) {
+inline FilterLayout filter_layout(int64_t entries, int64_t pairs, int64_t words, int64_t rows,
+                                  bool gains_only = false) {
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t all = gains_only ? 0 : 1;
     FilterLayout F;
     F.S = 0;
-    F.Q = F.S + al((size_t)pairs * 8);
-    F.gB = F.Q + al((size_t)pairs * 8);
-    F.L = F.gB + al((size_t)entries * 4);
-    F.Z = F.L + al((size_t)entries * 4);
-    F.G = F.Z + al((size_t)entries * 4);
-    F.vmax = F.G + al((size_t)words * 4);
-    F.total = F.vmax + al((size_t)rows * 4);
+    F.Q = F.S + all * al((size_t)pairs * 8);
+    F.gB = F.Q + all * al((size_t)pairs * 8);
+    F.Z = F.gB + all * al((size_t)entries * 4);
+    F.vmax = F.Z + all * al((size_t)entries * 4);
+    F.L = F.vmax + all * al((size_t)rows * 4);
+    F.G = F.L + al((size_t)entries * 4);
+    F.total = F.G + al((size_t)words * 4);
     return F;
 }
-inline FilterTab filter_tab(char* p, const FilterLayout& F) {
+inline FilterTab filter_tab(char* p, const FilterLayout& F, bool gains_only = false) {
+    if (gains_only)
+        return FilterTab{nullptr, nullptr, (float*)(p + F.L), nullptr, nullptr,
+                         (unsigned*)(p + F.G), nullptr};
     return FilterTab{(uint2*)(p + F.S), (float*)(p + F.gB), (float*)(p + F.L),
                      (unsigned*)(p + F.Z), (uint2*)(p + F.Q), (unsigned*)(p + F.G),
                      (unsigned*)(p + F.vmax)};

@@ -1751,9 +1751,9 @@ __device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs
     f.uend = sp.uend;
     f.n_phi = pc->n_phi;
     f.K = ic.K + 2.f;
-    f.mode = on ? filter_mode(J.tab.S != nullptr && sp.delta <= 8ull * FILTER_MARGIN, sp.ustep,
-                              ic.K, f.n_phi * J.n_D)
-                : FILTER_NONE;
+    f.mode = on && sp.delta <= 8ull * FILTER_MARGIN
+                 ? filter_mode(J.tab, sp.ustep, ic.K, f.n_phi * J.n_D)
+                 : FILTER_NONE;
     it.x.fp = f;
     it.x.f = filter_view(J.tab, fs);
     it.x.n_D = J.n_D;
@@ -2243,7 +2243,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
         f.n_phi = sp.n_phi;
         const float K = slot_K(fs, sp);
         f.K = K + 2.f;
-        f.mode = filter_mode(J.tab.S != nullptr, sp.ustep, K, f.n_phi * n_D);
+        f.mode = filter_mode(J.tab, sp.ustep, K, f.n_phi * n_D);
         it.x.fp = f;
         it.x.f = filter_view(J.tab, fs);
         it.x.n_D = n_D;
@@ -2572,14 +2572,18 @@ static cudaError_t launch_filter_tables(const FoldSeg* segs, const FoldSeg& one,
                                         const FilterTab& tab, cudaStream_t st, int* launched) {
     if (n_entries == 0) return cudaSuccess;
     const int64_t rows = (int64_t)n_seg * n_D;
-    const cudaError_t e = cudaMemsetAsync(tab.vmax, 0, (size_t)rows * sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-    const unsigned gy = (unsigned)std::min<int64_t>(std::max<int64_t>(n_t0 / 512, 1), 64);
-    k_filter_vmax<<<dim3((unsigned)rows, gy), 256, 0, st>>>(screen, rec, segs, one, n_D, tab.vmax);
+    if (tab.S) {
+        const cudaError_t e = cudaMemsetAsync(tab.vmax, 0, (size_t)rows * sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+        const unsigned gy = (unsigned)std::min<int64_t>(std::max<int64_t>(n_t0 / 512, 1), 64);
+        k_filter_vmax<<<dim3((unsigned)rows, gy), 256, 0, st>>>(screen, rec, segs, one, n_D,
+                                                                tab.vmax);
+        ++*launched;
+    }
     k_filter_slots<<<div_up(n_entries, 128), 128, 0, st>>>(screen, vpair, bucket, rec, segs, one,
                                                            n_seg, n_D, n_entries, tab);
     k_filter_groups<<<div_up(n_entries, 256), 256, 0, st>>>(segs, one, n_seg, n_D, n_entries, tab);
-    *launched += 3;
+    *launched += 2;
     return cudaSuccess;
 }
 
@@ -2792,93 +2796,176 @@ int launch_slots_test(const double* t, const int64_t* s_off_dev, int n_seg, int6
 // ------------------------------------------------ single-curve host side
 namespace nu {
 
-// Scratch layout of the single-curve fold.  In mixed precision the regular
-// and the irregular path are two uses of one region (which of them runs is
-// known after the slot test).  level 2: everything; 1: without the filter
-// tables, the period table and the lists (every cell is screened, survivors
-// are evaluated in place); 0: also without what the screen of the mixed
-// irregular path needs (every cell is evaluated).
-struct SingleLayout {
-    ExactLayout el;
-    FilterLayout fl;
-    size_t exact, bucket, slot_of, flag, rec, srec, tab, ptab, cand, range, items, list, sbest, total;
-    unsigned long long cap;
-    int level;
+// One call of the single-curve fold.
+struct FoldCall {
+    const char* who;
+    const double* t0s;
+    int64_t n_t0;
+    int n_D;
+    const void *depth, *var, *dlnl;
+    bool fp64;
+    const double* periods;
+    int64_t n_P;
+    double phase_step, gap_factor, t_ref, t_last;
+    int64_t n_bucket;
+    cudaStream_t st;
+    bool fork;           // block items may run on a side stream (two events per pass
+                         // with a list, and the stream with a thread's first such call)
+    double *Q, *T0;
+    int32_t* D_idx;
+    double *dep, *sig, *lnP;
+
+    double span_steps() const { return (t_last - t_ref) / phase_step; }
+    int64_t n_slots() const { return n_bucket + 2; }      // slot records, NaN padded
+    double item_steps() const { return span_steps() * n_D; }
+    // the slot path needs a regular grid and a gap rule that only joins
+    // neighbouring slots (1 < gap_factor < 2)
+    bool may_use_slots() const {
+        return !fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span_steps() < 4.0e6;
+    }
+    // gap rules and spans that the screen does not cover: every cell is evaluated
+    bool may_screen() const { return gap_factor < 2.0 && span_steps() < 8.0e6; }
+    // Small calls: screening every cell costs less than the filters' tables and
+    // rounds, and a few survivors per block less than the launches that pack
+    // them.  Mixed / FP64, us with filters -> without: 4 000 epochs x 4 durations
+    // x 1 200 periods (19 M steps) 309 / 365 -> 208 / 276, 1 100 x 12 x 300 (4 M)
+    // 239 / 285 -> 158 / 174; 2 000 x 12 x 1 200 (29 M) 269 / 325 -> 272 / 352; one
+    // duration, 8 000 x 4 000 (32 M) 432 / 472 -> 299 / 429.
+    bool small() const { return item_steps() * (double)n_P < (n_D == 1 ? 4.0e7 : 2.4e7); }
+    // Warps per period of a pass of n: eight where the periods are few for their
+    // size, two (and eight for the long ones) from where they fill the GPU, one
+    // from 40 000.  FP64: 4 000 periods of 2 000 epochs x 4 durations 0.49 ms with
+    // eight, 0.31 with two, 0.34 with one; 1 200 of 8 000 x 4 0.40 / 0.49 / 0.66;
+    // 2 500 of 19 440 x 10 1.7 with eight, 2.0 with one.
+    int warps(int64_t n) const {
+        if (n >= NU_ONE_WARP_FROM) return 1;
+        return n >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + item_steps() / 32.0) ? 2 : 8;
+    }
 };
 
-static SingleLayout single_layout(int64_t n_t0, int n_D, int64_t n_bucket, int64_t n_P, bool fp64,
-                                  int level = 2) {
-    auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    SingleLayout L;
-    L.level = level;
-    L.el = exact_layout(n_t0, n_D, fp64, fp64 || level > 0);
-    const int64_t n_slots = n_bucket + 2;          // slot records, NaN padded
-    L.flag = 0;
-    L.slot_of = 256;
-    L.exact = L.slot_of + al((size_t)n_t0 * sizeof(int));
-    L.rec = L.exact;                               // the mixed regular path's
-    L.bucket = L.exact + L.el.total;               // the others'
-    L.srec = L.bucket + al((size_t)n_bucket * sizeof(int));
-    size_t end = L.srec + (fp64 ? al((size_t)n_slots * n_D * sizeof(ScreenRec)) : 0);
-    if (!fp64) end = std::max(end, L.rec + al((size_t)n_slots * n_D * sizeof(Node4<float>)));
-    const int64_t ns = filter_slots(n_slots);
-    L.fl = filter_layout(ns * n_D, ns * ((n_D + 1) / 2 * 2),
-                         ns * filter_groups(n_D) * filter_words(n_D), n_D);
-    L.cap = (unsigned long long)std::min<int64_t>(8 * n_P + 4096, 1ll << 30);
-    L.tab = end;
-    L.ptab = L.tab + L.fl.total;
-    L.cand = L.ptab + al((size_t)n_P * period_const_bytes());
-    L.range = L.cand + al((size_t)L.cap * sizeof(FoldCand));
-    L.items = L.range + al((size_t)n_P * sizeof(int2));
-    L.list = L.items + al((size_t)n_P * sizeof(ItemConst));
-    L.sbest = L.list + al((size_t)n_P * sizeof(unsigned));
-    L.total = level == 2 ? L.sbest + (fp64 ? 0 : al((size_t)n_P * sizeof(SlotBest))) : end;
+// What a fold keeps in scratch beside the records of its events.
+struct FoldPlan {
+    bool slots;          // the mixed regular path's records, else the exact paths'
+    bool screen;         // exact paths: the screen's records
+    int tables;          // filter tables: 2 all, 1 the gains', 0 none
+    int64_t pass;        // periods per pass, with their table and lists; 0: all in one
+                         // pass without (survivors are evaluated in place)
+};
+
+// The plans of a call, the best one first; the last needs the least.  Period
+// tables and lists take 290 bytes per period, so that a long grid of periods goes
+// through them in passes: 2^19 periods at most, and fewer where scratch is
+// short, as the filters are worth more than one pass (19 440 epochs x 10
+// durations x 20 000 periods, FP64: 2.9 ms in one pass, 4.2 in the passes that
+// 32 MiB hold, 23.6 in one without filters).
+constexpr int64_t PASS_MAX = 1ll << 19, PASS_MIN = 2048;
+static std::vector<FoldPlan> fold_plans(const FoldCall& C, bool slots) {
+    std::vector<FoldPlan> plans;
+    const bool screen = !slots && C.may_screen();
+    if (slots || screen) {
+        for (int tables = C.small() ? 0 : 2; tables >= 0; --tables) {
+            for (int64_t k = (C.n_P + PASS_MAX - 1) / PASS_MAX;; k += std::max<int64_t>(1, k / 4)) {
+                const int64_t pass = (C.n_P + k - 1) / k;
+                if (pass < PASS_MIN && pass < C.n_P) break;
+                plans.push_back(FoldPlan{slots, screen, tables, pass});
+                if (pass == 1) break;
+            }
+            plans.push_back(FoldPlan{slots, screen, tables, 0});
+        }
+    }
+    if (!slots && !(screen && C.fp64)) plans.push_back(FoldPlan{false, false, 0, 0});
+    return plans;
+}
+
+// Scratch layout of one plan.  The flags and the epochs' slots come first in
+// all of them: which records a mixed call fills is known after its slot test.
+struct SingleLayout {
+    FoldPlan plan;
+    ExactLayout el;
+    FilterLayout fl;
+    size_t flag, slot_of, records, bucket, srec, tab, ptab, cand, range, items, list, sbest, total;
+    unsigned long long cap;
+};
+static SingleLayout single_layout(const FoldCall& C, const FoldPlan& plan) {
+    SingleLayout L{};
+    L.plan = plan;
+    size_t end = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = end;
+        end += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const int64_t n_slots = C.n_slots();
+    L.flag = take(256);
+    L.slot_of = take((size_t)C.n_t0 * sizeof(int));
+    if (plan.slots) {
+        L.records = take((size_t)n_slots * C.n_D * sizeof(Node4<float>));
+    } else {
+        L.el = exact_layout(C.n_t0, C.n_D, C.fp64, plan.screen);
+        L.records = take(L.el.total);
+        L.bucket = take((size_t)C.n_bucket * sizeof(int));
+        if (C.fp64 && plan.screen) L.srec = take((size_t)n_slots * C.n_D * sizeof(ScreenRec));
+    }
+    if (plan.tables) {
+        const int64_t ns = filter_slots(n_slots);
+        L.fl = filter_layout(ns * C.n_D, ns * ((C.n_D + 1) / 2 * 2),
+                             ns * filter_groups(C.n_D) * filter_words(C.n_D), C.n_D,
+                             plan.tables == 1);
+        L.tab = take(L.fl.total);
+    }
+    if (plan.pass) {
+        L.ptab = take((size_t)plan.pass * (plan.slots ? sizeof(SlotPeriod) : sizeof(PeriodConst)));
+        L.list = take((size_t)plan.pass * sizeof(unsigned));
+        if (plan.slots) {
+            L.sbest = take((size_t)plan.pass * sizeof(SlotBest));
+        } else {
+            // (an item that finds the list full evaluates its cells in place)
+            L.cap = (unsigned long long)(4 * plan.pass + 1024);
+            L.cand = take((size_t)L.cap * sizeof(FoldCand));
+            L.range = take((size_t)plan.pass * sizeof(int2));
+            L.items = take((size_t)plan.pass * sizeof(ItemConst));
+        }
+    }
+    L.total = end;
     return L;
 }
 
-// Enqueue the fold of one light curve on st with its scratch at `scratch`
-// (laid out by single_layout).  The mixed-precision slot test reads one flag
-// back (one synchronisation of st).  fork: the block items of a call with a
-// list may run on a side stream (two events per call, and the stream with the
-// thread's first such call).
-static nu_status single_fold(const char* who, char* scratch, const SingleLayout& L,
-                             const double* t0s_dev, int64_t n_t0, int n_D, const void* depth_dev,
-                             const void* var_dev, const void* dlnl_dev, bool fp64,
-                             const double* periods_dev, int64_t n_P, double phase_step,
-                             double gap_factor, double t_ref, double t_last, int64_t n_bucket,
-                             cudaStream_t st, bool fork, double* Q_dev, double* T0_dev,
-                             int32_t* D_idx_dev, double* depth_out_dev, double* sigma_out_dev,
-                             double* lnP_dev) {
-    const double span_steps = (t_last - t_ref) / phase_step;
+// Enqueue the fold of one light curve with its scratch at `scratch`, laid out by
+// Le, or by Ls (if given) when the mixed precision's slot test finds a regular
+// grid; the test reads one flag back (one synchronisation of the stream).
+static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayout* Ls,
+                             const SingleLayout& Le) {
+    const int64_t n_t0 = C.n_t0, n_P = C.n_P, n_bucket = C.n_bucket, n_slots = C.n_slots();
+    const int n_D = C.n_D;
+    const bool fp64 = C.fp64;
+    const double phase_step = C.phase_step;
+    const cudaStream_t st = C.st;
     const int64_t ngrid = n_t0 * (int64_t)n_D;
-    const int64_t n_slots = n_bucket + 2;
-    int* slot_of = (int*)(scratch + L.slot_of);
-    int* flag = (int*)(scratch + L.flag);
+    int* slot_of = (int*)(scratch + Le.slot_of);
+    int* flag = (int*)(scratch + Le.flag);
     int launched = 0;
     // one block of flags: [0] slot test, [1..2] regular-grid test, then the
     // peak key and the candidate counter
     cudaError_t e = cudaMemsetAsync(flag, 0, 256, st);
     const unsigned peak_grid = (unsigned)std::min<int64_t>(div_up(ngrid, 2048), 608);
-    unsigned long long* peak = (unsigned long long*)(scratch + L.flag + 16);
-    // the slot path needs a regular grid and a gap rule that only joins
-    // neighbouring slots (1 < gap_factor < 2)
-    bool use_slots = !fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span_steps < 4.0e6;
+    unsigned long long* peak = (unsigned long long*)(scratch + Le.flag + 16);
+    bool use_slots = Ls != nullptr;
     if (use_slots) {
         int irregular = 0;
-        k_slots<<<div_up(n_t0, 256), 256, 0, st>>>(t0s_dev, n_t0, t_ref, 1.0 / phase_step,
+        k_slots<<<div_up(n_t0, 256), 256, 0, st>>>(C.t0s, n_t0, C.t_ref, 1.0 / phase_step,
                                                   slot_of, flag);
         // The tables of that path are filled before the test is read, so that
         // the host's next launch is the fold's (an irregular curve overwrites
         // them: 10 us on the GPU, hidden in part by the wait).
         const int64_t nrec = n_slots * n_D;
-        Node4<float>* rec = (Node4<float>*)(scratch + L.rec);
+        Node4<float>* rec = (Node4<float>*)(scratch + Ls->records);
         const unsigned b_rec = (unsigned)div_up(nrec, 256), b_peak = b_rec + peak_grid;
-        const unsigned b_all = b_peak + (L.level == 2 ? (unsigned)div_up(n_P, 256) : 0u);
-        k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, b_rec, (const float*)dlnl_dev, ngrid,
-                                           b_peak, peak, periods_dev, n_P, phase_step,
-                                           (SlotPeriod*)(scratch + L.ptab));
+        const unsigned b_all = b_peak + (unsigned)div_up(Ls->plan.pass, 256);
+        k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, b_rec, (const float*)C.dlnl, ngrid,
+                                           b_peak, peak, C.periods, Ls->plan.pass, phase_step,
+                                           (SlotPeriod*)(scratch + Ls->ptab));
         k_slot_fill<<<div_up(ngrid, 256), 256, 0, st>>>(
-            (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, slot_of,
+            (const float*)C.depth, (const float*)C.var, (const float*)C.dlnl, slot_of,
             n_t0, n_D, n_slots, rec);
         launched += 3;
         if (e == cudaSuccess)
@@ -2888,89 +2975,57 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
     }
     if (e != cudaSuccess) {
         count_launches(launched);
-        return cuda_fail(e, (std::string(who) + ": slot test").c_str());
+        return cuda_fail(e, (std::string(C.who) + ": slot test").c_str());
     }
+    const SingleLayout& L = use_slots ? *Ls : Le;
     FoldJob J{};
     J.n_seg = 1;
     J.n_D = n_D;
     J.dt = phase_step;
     J.inv_dt = 1.0 / phase_step;
-    J.gap_max = gap_factor * phase_step;
-    J.t = t0s_dev;
-    J.nodes = scratch + L.exact;
-    J.screen = (const ScreenRec*)(scratch + L.exact + L.el.off_screen);
-    J.vpair = (const ulonglong2*)(scratch + L.exact + L.el.off_vpos);
-    J.srec = fp64 ? (const ScreenRec*)(scratch + L.srec) : nullptr;
+    J.gap_max = C.gap_factor * phase_step;
+    J.t = C.t0s;
+    J.nodes = scratch + L.records;
+    J.screen = (const ScreenRec*)(scratch + L.records + L.el.off_screen);
+    J.vpair = (const ulonglong2*)(scratch + L.records + L.el.off_vpos);
+    J.srec = fp64 && L.plan.screen ? (const ScreenRec*)(scratch + L.srec) : nullptr;
     J.reg = (const unsigned*)(flag + 1);
-    J.peak = (const unsigned long long*)(scratch + L.flag + 16);
+    J.peak = peak;
     J.bucket = (const int*)(scratch + L.bucket);
-    J.rec = (const Node4<float>*)(scratch + L.rec);
-    J.periods = periods_dev;
-    J.n_P = n_P;
-    J.Q = Q_dev;
-    J.T0 = T0_dev;
-    J.Didx = D_idx_dev;
-    J.dep = depth_out_dev;
-    J.sig = sigma_out_dev;
-    J.lnp = lnP_dev;
+    J.rec = (const Node4<float>*)(scratch + L.records);
     FoldSeg& one = J.one;
     one.n_t0 = n_t0;
-    one.t_ref = t_ref;
-    one.t_last = t_last;
+    one.t_ref = C.t_ref;
+    one.t_last = C.t_last;
     one.n_bucket = n_bucket;
     one.n_slots = n_slots;
     one.use_slots = use_slots ? 1 : 0;
-    one.screen = !use_slots && gap_factor < 2.0 && span_steps < 8.0e6 && (fp64 || L.level > 0);
-    if (use_slots) one.ulast = slot_ulast(t_ref, t_last, phase_step);
-    else one.uspan = exact_uspan(t_ref, t_last, phase_step);
-    // Warps per period: eight where the periods are few for their size, two (and
-    // eight for the long ones) from where they fill the GPU, one from 40 000.
-    // FP64: 4 000 periods of 2 000 epochs x 4 durations 0.49 ms with eight, 0.31
-    // with two, 0.34 with one; 1 200 of 8 000 x 4 0.40 / 0.49 / 0.66; 2 500 of
-    // 19 440 x 10 1.7 with eight, 2.0 with one.
-    const double item_steps = span_steps * n_D;
-    const int nw = n_P >= NU_ONE_WARP_FROM
-                       ? 1
-                       : (n_P >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + item_steps / 32.0)
-                              ? 2 : 8);
-    // Small calls: screening every cell costs less than the filters' tables and
-    // rounds, and a few survivors per block less than the launches that pack
-    // them.  Mixed / FP64, us with filters -> without: 4 000 epochs x 4 durations
-    // x 1 200 periods (19 M steps) 309 / 365 -> 208 / 276, 1 100 x 12 x 300 (4 M)
-    // 239 / 285 -> 158 / 174; 2 000 x 12 x 1 200 (29 M) 269 / 325 -> 272 / 352; one
-    // duration, 8 000 x 4 000 (32 M) 432 / 472 -> 299 / 429.
-    const bool small = item_steps * (double)n_P < (n_D == 1 ? 4.0e7 : 2.4e7);
-    if (L.level == 2) {
+    one.screen = L.plan.screen ? 1 : 0;
+    if (use_slots) one.ulast = slot_ulast(C.t_ref, C.t_last, phase_step);
+    else one.uspan = exact_uspan(C.t_ref, C.t_last, phase_step);
+    const int64_t pass = L.plan.pass ? L.plan.pass : n_P;
+    if (L.plan.pass) {
         J.ptab = (const PeriodConst*)(scratch + L.ptab);
         J.stab = (const SlotPeriod*)(scratch + L.ptab);
-        if (!small) J.tab = filter_tab(scratch + L.tab, L.fl);
     }
-    if (L.level == 2 && !(small && (nw == 8 || use_slots))) {
-        J.cand = (FoldCand*)(scratch + L.cand);
-        J.counters = (unsigned*)(scratch + L.flag + 64);
-        J.n_cand = (unsigned long long*)(J.counters + 4);
-        J.cap = L.cap;
-        J.range = (int2*)(scratch + L.range);
-        J.items = (ItemConst*)(scratch + L.items);
-        J.sbest = fp64 ? nullptr : (SlotBest*)(scratch + L.sbest);
-    }
+    if (L.plan.tables) J.tab = filter_tab(scratch + L.tab, L.fl, L.plan.tables == 1);
     if (!use_slots) {
-        const double gap_max = gap_factor * phase_step;
-        ScreenRec* screen = (ScreenRec*)(scratch + L.exact + L.el.off_screen);
-        ulonglong2* vpair = (ulonglong2*)(scratch + L.exact + L.el.off_vpos);
-        ScreenRec* srec = fp64 ? (ScreenRec*)(scratch + L.srec) : nullptr;
+        const double gap_max = J.gap_max;
+        ScreenRec* screen = (ScreenRec*)J.screen;
+        ulonglong2* vpair = (ulonglong2*)J.vpair;
+        ScreenRec* srec = (ScreenRec*)J.srec;
         auto prep = [&](auto zero) {
             using T = decltype(zero);
-            FoldPrep<T> A{(const T*)depth_dev, (const T*)var_dev, (const T*)dlnl_dev, t0s_dev,
-                          n_t0, n_D, t_ref, phase_step, gap_max, n_bucket,
-                          (int*)(scratch + L.bucket), (Node8<T>*)(scratch + L.exact), n_slots,
-                          slot_of, (unsigned*)(flag + 1), srec, periods_dev, n_P,
+            FoldPrep<T> A{(const T*)C.depth, (const T*)C.var, (const T*)C.dlnl, C.t0s,
+                          n_t0, n_D, C.t_ref, phase_step, gap_max, n_bucket,
+                          (int*)(scratch + L.bucket), (Node8<T>*)(scratch + L.records), n_slots,
+                          slot_of, (unsigned*)(flag + 1), srec, C.periods, L.plan.pass,
                           J.ptab ? (PeriodConst*)(scratch + L.ptab) : nullptr, peak, {}};
             const unsigned blocks[PREP_N] = {
                 (unsigned)div_up(n_bucket, 256), one.screen ? peak_grid : 0u,
-                one.screen && J.ptab ? (unsigned)div_up(n_P, 256) : 0u,
-                one.screen && srec ? (unsigned)div_up(n_t0, 256) : 0u,
-                one.screen && srec ? (unsigned)div_up(n_slots * n_D, 256) : 0u,
+                J.ptab ? (unsigned)div_up(L.plan.pass, 256) : 0u,
+                srec ? (unsigned)div_up(n_t0, 256) : 0u,
+                srec ? (unsigned)div_up(n_slots * n_D, 256) : 0u,
                 (unsigned)div_up(ngrid, 256)};
             unsigned n = 0;
             for (int q = 0; q < PREP_N; ++q) A.end[q] = n += blocks[q];
@@ -2979,43 +3034,75 @@ static nu_status single_fold(const char* who, char* scratch, const SingleLayout&
         if (fp64) prep(0.0); else prep(0.0f);
         ++launched;
         if (!one.screen) {
-            // gap rules and spans the screen does not cover: every cell
-            const FoldGeom g{t0s_dev, n_t0, t_ref, t_last, phase_step, 1.0 / phase_step, gap_max,
-                             (const int*)(scratch + L.bucket), n_bucket};
+            const FoldGeom g{C.t0s, n_t0, C.t_ref, C.t_last, phase_step, 1.0 / phase_step,
+                             gap_max, (const int*)(scratch + L.bucket), n_bucket};
             if (fp64)
                 k_fold_exact<double, 8><<<(unsigned)n_P, 256, 0, st>>>(
-                    g, (const Node8<double>*)(scratch + L.exact), n_D, periods_dev, n_P, Q_dev,
-                    T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+                    g, (const Node8<double>*)J.nodes, n_D, C.periods, n_P, C.Q, C.T0, C.D_idx,
+                    C.dep, C.sig, C.lnP);
             else
                 k_fold_exact<float, 8><<<(unsigned)n_P, 256, 0, st>>>(
-                    g, (const Node8<float>*)(scratch + L.exact), n_D, periods_dev, n_P, Q_dev,
-                    T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+                    g, (const Node8<float>*)J.nodes, n_D, C.periods, n_P, C.Q, C.T0, C.D_idx,
+                    C.dep, C.sig, C.lnP);
             count_launches(launched + 1);
             e = cudaGetLastError();
-            if (e != cudaSuccess) return cuda_fail(e, (std::string(who) + ": launch").c_str());
+            if (e != cudaSuccess) return cuda_fail(e, (std::string(C.who) + ": launch").c_str());
             return NU_OK;
         }
         if (fp64) {
             k_screen<double><<<div_up(ngrid, 256), 256, 0, st>>>(
-                (const double*)depth_dev, (const double*)var_dev, (const double*)dlnl_dev,
-                t0s_dev, n_t0, n_D, gap_max, phase_step, screen, srec, n_slots, slot_of, vpair);
+                (const double*)C.depth, (const double*)C.var, (const double*)C.dlnl, C.t0s, n_t0,
+                n_D, gap_max, phase_step, screen, srec, n_slots, slot_of, vpair);
         } else {
             k_screen<float><<<div_up(ngrid, 256), 256, 0, st>>>(
-                (const float*)depth_dev, (const float*)var_dev, (const float*)dlnl_dev, t0s_dev,
-                n_t0, n_D, gap_max, phase_step, screen, nullptr, n_slots, nullptr, vpair);
+                (const float*)C.depth, (const float*)C.var, (const float*)C.dlnl, C.t0s, n_t0,
+                n_D, gap_max, phase_step, screen, nullptr, n_slots, nullptr, vpair);
         }
         ++launched;
     }
-    if (J.tab.S)
+    if (J.tab.L)
         e = launch_filter_tables(nullptr, one, 1, n_D, filter_slots(n_slots) * n_D, n_t0, J.screen,
                                  J.vpair, J.bucket, J.rec, J.tab, st, &launched);
-    if (J.items && nw != 8)
-        J.list = FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K};
-    const cudaStream_t side = fork && J.list.block ? thread_side_stream() : nullptr;
-    launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, side, &e);
+    for (int64_t p0 = 0; p0 < n_P && e == cudaSuccess; p0 += pass) {
+        const int64_t n = std::min(pass, n_P - p0);
+        J.periods = C.periods + p0;
+        J.n_P = n;
+        J.Q = C.Q + p0;
+        J.T0 = C.T0 + p0;
+        J.Didx = C.D_idx + p0;
+        J.dep = C.dep + p0;
+        J.sig = C.sig + p0;
+        J.lnp = C.lnP + p0;
+        if (p0 > 0) {
+            if (use_slots)
+                k_slot_periods<<<div_up(n, 256), 256, 0, st>>>(J.periods, n, phase_step,
+                                                               (SlotPeriod*)(scratch + L.ptab));
+            else
+                k_period_consts<<<div_up(n, 256), 256, 0, st>>>(J.periods, n, phase_step,
+                                                                (PeriodConst*)(scratch + L.ptab));
+            ++launched;
+        }
+        const int nw = C.warps(n);
+        if (L.plan.pass && !(C.small() && (nw == 8 || use_slots))) {
+            J.counters = (unsigned*)(scratch + L.flag + 64);
+            if (use_slots) {
+                J.sbest = (SlotBest*)(scratch + L.sbest);
+            } else {
+                J.cand = (FoldCand*)(scratch + L.cand);
+                J.n_cand = (unsigned long long*)(J.counters + 4);
+                J.cap = L.cap;
+                J.range = (int2*)(scratch + L.range);
+                J.items = (ItemConst*)(scratch + L.items);
+            }
+            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K}
+                             : FoldLists{};
+        }
+        const cudaStream_t side = C.fork && J.list.block ? thread_side_stream() : nullptr;
+        launched += launch_cells(J, fp64, !use_slots, use_slots, nw, st, side, &e);
+    }
     count_launches(launched);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, (std::string(who) + ": launch").c_str());
+    if (e != cudaSuccess) return cuda_fail(e, (std::string(C.who) + ": launch").c_str());
     return NU_OK;
 }
 
@@ -3080,16 +3167,26 @@ extern "C" nu_status nu_periodic_search(const double* t0s_dev, int64_t n_t0,
     if (!(t_last >= t_ref)) return fail(NU_EINVAL, "nu_periodic_search: t0s not sorted");
     const double span_steps = (t_last - t_ref) / phase_step;
     if (span_steps > 1.0e9) return fail(NU_EINVAL, "nu_periodic_search: phase grid too fine");
-    const int64_t n_bucket = (int64_t)span_steps + 2;
-    const bool fp64 = prec == NU_FP64;
-    const SingleLayout L = single_layout(n_t0, n_D, n_bucket, n_P, fp64);
+    const FoldCall C{who, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev, prec == NU_FP64,
+                     periods_dev, n_P, phase_step, gap_factor, t_ref, t_last,
+                     (int64_t)span_steps + 2, st, true, Q_dev, T0_dev, D_idx_dev, depth_out_dev,
+                     sigma_out_dev, lnP_dev};
+    // the best plan that there is memory for
     pool_keep_memory();
+    const std::vector<FoldPlan> pe = fold_plans(C, false);
+    const std::vector<FoldPlan> ps =
+        C.may_use_slots() ? fold_plans(C, true) : std::vector<FoldPlan>{};
     char* scratch = nullptr;
-    e = cudaMallocAsync((void**)&scratch, L.total, st);
+    SingleLayout Le, Ls{};
+    for (size_t i = 0; i < std::max(pe.size(), ps.size()); ++i) {
+        Le = single_layout(C, pe[std::min(i, pe.size() - 1)]);
+        if (!ps.empty()) Ls = single_layout(C, ps[std::min(i, ps.size() - 1)]);
+        e = cudaMallocAsync((void**)&scratch, std::max(Le.total, Ls.total), st);
+        if (e != cudaErrorMemoryAllocation) break;
+        cudaGetLastError();
+    }
     if (e != cudaSuccess) return cuda_fail(e, "nu_periodic_search: cudaMallocAsync");
-    s = single_fold(who, scratch, L, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev, fp64,
-                    periods_dev, n_P, phase_step, gap_factor, t_ref, t_last, n_bucket, st, true,
-                    Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+    s = single_fold(C, scratch, ps.empty() ? nullptr : &Ls, Le);
     e = cudaFreeAsync(scratch, st);
     if (s != NU_OK) return s;
     if (e != cudaSuccess) return cuda_fail(e, "nu_periodic_search: cudaFreeAsync");
@@ -3294,19 +3391,26 @@ extern "C" nu_status nu_periodic_search_noalloc(const double* t0s_dev, int64_t n
     const double span_steps = (t_last - t_ref) / phase_step;
     if (span_steps > 1.0e9)
         return fail(NU_EINVAL, "nu_periodic_search_noalloc: phase grid too fine");
-    const int64_t n_bucket = (int64_t)span_steps + 2;
-    const bool fp64 = prec == NU_FP64;
-    // (near the limit without the filters, and the mixed path of irregular
-    // grids without its screen)
-    SingleLayout L = single_layout(n_t0, n_D, n_bucket, n_P, fp64);
-    for (int level = 1; level >= (fp64 ? 1 : 0) && L.total > NU_NOALLOC_SCRATCH_BYTES; --level)
-        L = single_layout(n_t0, n_D, n_bucket, n_P, fp64, level);
-    if (L.total > NU_NOALLOC_SCRATCH_BYTES)
+    const FoldCall C{who, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev, prec == NU_FP64,
+                     periods_dev, n_P, phase_step, gap_factor, t_ref, t_last,
+                     (int64_t)span_steps + 2, st, false, Q_dev, T0_dev, D_idx_dev, depth_out_dev,
+                     sigma_out_dev, lnP_dev};
+    // the best plan that fits, of either kind of records
+    auto fit = [&](bool slots) {
+        SingleLayout L{};
+        for (const FoldPlan& plan : fold_plans(C, slots)) {
+            L = single_layout(C, plan);
+            if (L.total <= NU_NOALLOC_SCRATCH_BYTES) break;
+        }
+        return L;
+    };
+    const SingleLayout Le = fit(false);
+    const SingleLayout Ls = C.may_use_slots() ? fit(true) : SingleLayout{};
+    const size_t need = std::max(Le.total, Ls.total);
+    if (need > NU_NOALLOC_SCRATCH_BYTES)
         return fail(NU_EINVAL,
                     "nu_periodic_search_noalloc: this grid needs %zu bytes of scratch, more "
                     "than the fixed %llu bytes; use nu_periodic_search",
-                    L.total, (unsigned long long)NU_NOALLOC_SCRATCH_BYTES);
-    return single_fold(who, (char*)base, L, t0s_dev, n_t0, n_D, depth_dev, var_dev, dlnl_dev,
-                       fp64, periods_dev, n_P, phase_step, gap_factor, t_ref, t_last, n_bucket,
-                       st, false, Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev, lnP_dev);
+                    need, (unsigned long long)NU_NOALLOC_SCRATCH_BYTES);
+    return single_fold(C, (char*)base, C.may_use_slots() ? &Ls : nullptr, Le);
 }
