@@ -252,12 +252,20 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
                                    "long for the phase step", g);
         }
     }
+    // the fold's tables and lists, as far as there is memory for them
     FoldBatch fbat;
-    plan_fold_batch(plan.s_off, t_first, t_last, irregular, fp64, phase_step, gap_factor, n_D,
-                    fbat);
-    const size_t f_segs = (fbat.segs.size() * sizeof(FoldSeg) + 255) / 256 * 256;
-    const size_t foff = f_segs + fold_scratch(fbat, N, n_lc, n_D, n_P, fp64, nullptr, nullptr);
-    e = cudaMallocAsync((void**)&fold_mem, foff, st);
+    size_t f_segs = 0;
+    for (int level = 2; level >= 0; --level) {
+        plan_fold_batch(plan.s_off, t_first, t_last, irregular, fp64, phase_step, gap_factor, n_D,
+                        level, fbat);
+        f_segs = (fbat.segs.size() * sizeof(FoldSeg) + 255) / 256 * 256;
+        e = cudaMallocAsync((void**)&fold_mem,
+                            f_segs + fold_scratch(fbat, N, n_lc, n_D, n_P, fp64, nullptr, nullptr),
+                            st);
+        if (e != cudaErrorMemoryAllocation) break;
+        cudaGetLastError();
+        fold_mem = nullptr;
+    }
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(fold_mem, fbat.segs.data(), fbat.segs.size() * sizeof(FoldSeg),
                             cudaMemcpyHostToDevice, st);

@@ -152,6 +152,7 @@ struct FoldScratch {
     int2* range;            // per item: its candidates
     struct ItemConst* items;   // per item: constants of the screen
     SlotBest* sbest;        // per item of the slot path
+    int64_t pass;           // items per pass (the lists' room); 0: one pass without lists
 };
 
 // Host side of the batch fold: per-curve layout and launches.
@@ -162,14 +163,23 @@ struct FoldBatch {
     int64_t n_pair_total = 0;    // of those with durations in pairs
     int64_t n_g_total = 0;       // words of their G tables
     bool any_slots = false, any_exact = false;
+    // What the scratch holds beside the records: 2 filter tables, and lists for the
+    // items of a pass; 1 neither (every cell is screened, survivors evaluated in
+    // place); 0 nor the screen's records of the mixed irregular path (every cell
+    // is evaluated).
+    int level = 2;
 };
-// Bytes of the batch fold's scratch; with a base, *fs receives its pointers.
+// Bytes of the batch fold's scratch; with a base, *fs receives its pointers.  The
+// lists take 230 bytes per (curve, period) item, so that a large batch goes
+// through them in passes of 2^22 items (1 GB) at most.
+constexpr int64_t BATCH_PASS = 1ll << 22;
 size_t fold_scratch(const FoldBatch& fb, int64_t n_total, int n_lc, int n_D, int64_t n_P,
                     bool fp64, char* base, FoldScratch* fs);
 
 void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double>& t_first,
                      const std::vector<double>& t_last, const std::vector<int>& irregular,
-                     bool fp64, double dt, double gap_factor, int n_D, FoldBatch& fb);
+                     bool fp64, double dt, double gap_factor, int n_D, int level,
+                     FoldBatch& fb);
 
 // Enqueues the fold's preparation kernels; returns the first error of an
 // enqueued memset (the launches are checked by the caller) and the number of

@@ -2490,8 +2490,11 @@ __global__ void k_slots_batch(const double* __restrict__ t, const int64_t* __res
 
 void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double>& t_first,
                      const std::vector<double>& t_last, const std::vector<int>& irregular,
-                     bool fp64, double dt, double gap_factor, int n_D, FoldBatch& fb) {
+                     bool fp64, double dt, double gap_factor, int n_D, int level,
+                     FoldBatch& fb) {
     const int n_seg = (int)t_first.size();
+    fb = FoldBatch{};
+    fb.level = level;
     fb.segs.resize(n_seg);
     for (int g = 0; g < n_seg; ++g) {
         FoldSeg& f = fb.segs[g];
@@ -2506,12 +2509,13 @@ void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double
         f.n_slots = f.n_bucket + 2;
         f.use_slots = (!fp64 && gap_factor > 1.0 && gap_factor < 2.0 && span < 4.0e6 &&
                        !irregular[g]) ? 1 : 0;
-        f.screen = (!f.use_slots && gap_factor < 2.0 && span < 8.0e6) ? 1 : 0;
+        f.screen = (!f.use_slots && gap_factor < 2.0 && span < 8.0e6 && (fp64 || level > 0)) ? 1
+                                                                                             : 0;
         f.srec_off = fb.n_srec_total;
         fb.n_srec_total += fp64 && f.screen ? f.n_slots * n_D : 0;
         f.tab_off = fb.n_tab_total;
         f.g_off = fb.n_g_total;
-        if (f.screen || f.use_slots) {
+        if (level == 2 && (f.screen || f.use_slots)) {
             const int64_t ns = filter_slots(f.n_slots);
             f.pair_off = fb.n_pair_total;
             fb.n_pair_total += ns * ((n_D + 1) / 2 * 2);
@@ -2535,9 +2539,11 @@ size_t fold_scratch(const FoldBatch& fb, int64_t n_total, int n_lc, int n_D, int
         off += (bytes + 255) / 256 * 256;
         return p;
     };
-    const int64_t items = (int64_t)n_lc * n_P;
-    FoldScratch f;
-    f.nodes = take(fb.any_exact ? exact_layout(n_total, n_D, fp64).total : 0);
+    const bool lists = fb.level == 2;
+    const int64_t items = std::min<int64_t>((int64_t)n_lc * n_P, BATCH_PASS);
+    FoldScratch f{};
+    f.pass = lists ? items : 0;
+    f.nodes = take(fb.any_exact ? exact_layout(n_total, n_D, fp64, fp64 || fb.level > 0).total : 0);
     f.bucket = (int*)take((size_t)(fb.n_bucket_total + 1) * 4);
     f.rec = (Node4<float>*)take((size_t)(fb.n_rec_total + 1) * sizeof(Node4<float>));
     f.srec = (ScreenRec*)take((size_t)(fb.n_srec_total + 1) * sizeof(ScreenRec));
@@ -2545,20 +2551,24 @@ size_t fold_scratch(const FoldBatch& fb, int64_t n_total, int n_lc, int n_D, int
     f.reg = (unsigned*)take((size_t)n_lc * 2 * sizeof(unsigned));
     f.peak = (unsigned long long*)take((size_t)n_lc * sizeof(unsigned long long));
     f.ptab = (PeriodConst*)take((size_t)n_P * period_const_bytes());
-    const FilterLayout F = filter_layout(fb.n_tab_total, fb.n_pair_total, fb.n_g_total,
-                                          (int64_t)n_lc * n_D);
-    char* tab = take(F.total);
-    f.tab = base ? filter_tab(tab, F) : FilterTab{};
-    // one item leaves a few cells; an item that finds the list full evaluates
-    // its own
-    f.cap = fb.any_exact ? (unsigned long long)std::min<int64_t>(4 * items + 4096, 1ll << 30) : 0;
-    f.cand = (FoldCand*)take((size_t)f.cap * sizeof(FoldCand));
-    f.n_list = (unsigned*)take(32);
-    f.n_cand = (unsigned long long*)(f.n_list + 4);
-    f.list = (unsigned*)take((size_t)items * sizeof(unsigned));
-    f.range = (int2*)take(fb.any_exact ? (size_t)items * sizeof(int2) : 0);
-    f.items = (ItemConst*)take(fb.any_exact ? (size_t)items * sizeof(ItemConst) : 0);
-    f.sbest = (SlotBest*)take(fb.any_slots ? (size_t)items * sizeof(SlotBest) : 0);
+    if (lists) {
+        const FilterLayout F = filter_layout(fb.n_tab_total, fb.n_pair_total, fb.n_g_total,
+                                              (int64_t)n_lc * n_D);
+        char* tab = take(F.total);
+        if (base) f.tab = filter_tab(tab, F);
+        f.n_list = (unsigned*)take(32);
+        f.list = (unsigned*)take((size_t)items * sizeof(unsigned));
+        if (fb.any_exact) {
+            // one item leaves a few cells; an item that finds the list full
+            // evaluates its own
+            f.cap = (unsigned long long)(4 * items + 4096);
+            f.cand = (FoldCand*)take((size_t)f.cap * sizeof(FoldCand));
+            f.n_cand = (unsigned long long*)(f.n_list + 4);
+            f.range = (int2*)take((size_t)items * sizeof(int2));
+            f.items = (ItemConst*)take((size_t)items * sizeof(ItemConst));
+        }
+        if (fb.any_slots) f.sbest = (SlotBest*)take((size_t)items * sizeof(SlotBest));
+    }
     if (fs) *fs = f;
     return off;
 }
@@ -2595,7 +2605,7 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
     int launched = 0;
     *n_launched = 0;
     const int64_t ngrid = n_total * (int64_t)n_D;
-    const ExactLayout L = exact_layout(n_total, n_D, fp64);
+    const ExactLayout L = exact_layout(n_total, n_D, fp64, fp64 || fb.level > 0);
     ScreenRec* screen = (ScreenRec*)((char*)fs.nodes + L.off_screen);
     ulonglong2* vpair = (ulonglong2*)((char*)fs.nodes + L.off_vpos);
     cudaError_t e = cudaMemsetAsync(fs.peak, 0, (size_t)n_seg * sizeof(unsigned long long), st);
@@ -2623,10 +2633,13 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
             k_nodes_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
                 s_off_dev, n_D, gap_factor * dt, (Node8<float>*)fs.nodes);
+            ++launched;
+        }
+        if (!fp64 && fb.level > 0) {
             k_screen_batch<float><<<div_up(ngrid, 256), 256, 0, st>>>(
                 (const float*)depth, (const float*)var, (const float*)gain, t, segs_dev, n_seg,
                 s_off_dev, n_D, gap_factor * dt, dt, screen, vpair, nullptr, nullptr);
-            launched += 2;
+            ++launched;
         }
     }
     if (fb.any_slots) {
@@ -2643,8 +2656,10 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
         k_gain_peak<float><<<peak_grid, 256, 0, st>>>((const float*)gain, s_off_dev, n_D,
                                                       fs.peak);
     ++launched;
-    e = launch_filter_tables(segs_dev, FoldSeg{}, n_seg, n_D, fb.n_tab_total, n_total / n_seg,
-                             screen, vpair, fs.bucket, fs.rec, fs.tab, st, &launched);
+    if (fb.level == 2)
+        e = launch_filter_tables(segs_dev, FoldSeg{}, n_seg, n_D, fb.n_tab_total,
+                                 n_total / n_seg, screen, vpair, fs.bucket, fs.rec, fs.tab, st,
+                                 &launched);
     *n_launched = launched;
     return e;
 }
@@ -2733,7 +2748,7 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       double* sig, double* lnp, cudaStream_t st, cudaStream_t side,
                       cudaError_t* err) {
     int launched = 0;
-    const ExactLayout L = exact_layout(n_total, n_D, fp64);
+    const ExactLayout L = exact_layout(n_total, n_D, fp64, fp64 || fb.level > 0);
     FoldJob J{};
     J.segs = segs_dev;
     J.n_seg = n_seg;
@@ -2769,17 +2784,45 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
     J.sbest = fs.sbest;
     J.counters = fs.n_list;
     const int nw = warps == 8 ? 8 : warps & 3;
-    if ((warps & 4) && nw != 8 && (int64_t)n_seg * n_P < 0xffffffffLL)    // (32-bit list)
-        J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
+    if ((warps & 4) && nw != 8 && fs.list) J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
+    // The passes: whole curves, or parts of one curve's periods.
+    const int64_t pass = fs.pass ? fs.pass : (int64_t)n_seg * n_P;
+    int64_t segs_pass = std::min<int64_t>(std::max<int64_t>(pass / n_P, 1), n_seg);
+    segs_pass = div_up(n_seg, div_up(n_seg, segs_pass));
+    const int64_t per_pass = std::min(n_P, pass);
+    auto cells = [&](bool exact) {
+        for (int64_t g = 0; g < n_seg; g += segs_pass)
+            for (int64_t p = 0; p < n_P; p += per_pass) {
+                FoldJob K = J;
+                const int64_t o = g * n_P + p;
+                K.segs += g;
+                K.n_seg = (int)std::min<int64_t>(segs_pass, n_seg - g);
+                K.reg += 2 * g;
+                K.peak += g;
+                K.periods += p;
+                K.ptab += p;
+                K.stab += p;
+                K.n_P = std::min(per_pass, n_P - p);
+                K.Q += o;
+                K.T0 += o;
+                K.Didx += o;
+                K.dep += o;
+                K.sig += o;
+                K.lnp += o;
+                launched += launch_cells(K, fp64, exact, !exact, nw, st, side, err);
+            }
+    };
     // (the two paths' period tables share a buffer)
     if (fb.any_exact) {
         k_period_consts<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt, fs.ptab);
-        launched += 1 + launch_cells(J, fp64, true, false, nw, st, side, err);
+        ++launched;
+        cells(true);
     }
     if (fb.any_slots) {
         k_slot_periods<<<div_up(n_P, 256), 256, 0, st>>>(periods, n_P, dt,
                                                          reinterpret_cast<SlotPeriod*>(fs.ptab));
-        launched += 1 + launch_cells(J, fp64, false, true, nw, st, side, err);
+        ++launched;
+        cells(false);
     }
     return launched;
 }
