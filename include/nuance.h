@@ -326,9 +326,9 @@ uint64_t nu_periodic_search_noalloc_limit(void);
  *   outputs, [n_lc][n_P] each: Q, T0, D_idx, depth, sigma, lnP (as in
  *   nu_periodic_search); status_host (n_lc) per-curve factor status.
  * Synchronises the stream before returning (the statuses are host data).
- * The launch shapes of the fold and of the linear search are tuned the first
- * time a configuration (state size, k, precision, n_D) is seen in the process
- * and cached; the executable graph of a configuration (the same and n_lc,
+ * The launch shape of the linear search is tuned the first time a
+ * configuration (state size, k, precision, n_D) is seen in the process and
+ * cached; the executable graph of a configuration (the same and n_lc,
  * total samples, n_P) is kept and updated with the next call's parameters.
  * Errors: NU_EINVAL, NU_ENOMEM, NU_ECUDA. */
 nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,

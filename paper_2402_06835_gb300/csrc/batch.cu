@@ -10,12 +10,11 @@
 // happens before capture; the kernels are captured into one CUDA graph and
 // launched once.  The instantiated graph of a configuration is kept and, on
 // later calls, updated in place with the new call's parameters
-// (cudaGraphExecUpdate) instead of being instantiated again.  The launch
-// shapes of the fold (which items take a block, which a warp) and of the
-// linear search's window-start kernel (window starts per block, staged chunk)
-// are chosen by a small autotuner the first time a configuration is seen:
-// the candidates are timed on a slice of the batch and the fastest are
-// cached for the process.
+// (cudaGraphExecUpdate) instead of being instantiated again.  The fold's launch
+// shape follows from the batch's size; that of the linear search's window-start
+// kernel (window starts per block, staged chunk) is chosen by a small autotuner
+// the first time a configuration is seen: the candidates are timed on a slice
+// of the batch and the fastest is cached for the process.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -31,13 +30,6 @@
 namespace nu {
 
 // n_out periods spread evenly over the grid (the autotuner's slice)
-__global__ void k_sample_periods(const double* __restrict__ periods, int64_t n_P, int n_out,
-                                 double* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_out) return;
-    out[i] = periods[(int64_t)((double)i * (double)n_P / (double)n_out)];
-}
-
 __global__ void k_init_dstat(long long* dstat, const int64_t* __restrict__ s_off, int n_seg) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_seg) return;
@@ -59,25 +51,20 @@ struct TuneKey {
         return std::tie(nb, k, prec, n_D) < std::tie(o.nb, o.k, o.prec, o.n_D);
     }
 };
-struct TuneVal {
-    int warps;                      // fold: one of FOLD_SHAPES (0: not tuned)
-    WindowShape win;                // linear search
-};
 
 std::mutex g_tune_mu;
-std::map<TuneKey, TuneVal> g_tune;
+std::map<TuneKey, WindowShape> g_tune;
 
 // Instantiated graphs by configuration (device, state size, k, precision,
-// grid sizes, batch shape and tuned launch shapes).  A call takes its entry
+// grid sizes, batch shape and tuned launch shape).  A call takes its entry
 // out of the cache while it uses it, so two threads never launch one
 // executable graph at once.
 struct GraphKey {
-    int dev, nb, k, prec, n_D, n_lc, warps, tlo, ch;
+    int dev, nb, k, prec, n_D, n_lc, tlo, ch;
     int64_t N, n_P;
     bool operator<(const GraphKey& o) const {
-        return std::tie(dev, nb, k, prec, n_D, n_lc, warps, tlo, ch, N, n_P) <
-               std::tie(o.dev, o.nb, o.k, o.prec, o.n_D, o.n_lc, o.warps, o.tlo, o.ch, o.N,
-                        o.n_P);
+        return std::tie(dev, nb, k, prec, n_D, n_lc, tlo, ch, N, n_P) <
+               std::tie(o.dev, o.nb, o.k, o.prec, o.n_D, o.n_lc, o.tlo, o.ch, o.N, o.n_P);
     }
 };
 std::mutex g_graph_mu;
@@ -181,7 +168,6 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     const size_t o_ends = off;  off += al((size_t)n_lc * 2 * 8);
     const size_t o_irr = off;   off += al((size_t)n_lc * 4);
     const size_t o_Ds = off;    off += al((size_t)n_D * 8);
-    const size_t o_tune = off;  off += al(512 * 8);
     const bool win_lo = n_D <= 4096;            // window-start recursion of the box search
     const size_t o_wplan = off; off += win_lo ? al((size_t)n_lc * window_plan_ints(n_D) * 4) : 0;
     const size_t base_bytes = off;
@@ -285,7 +271,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     cudaStream_t side = thread_side_stream();
     cudaError_t enq_err = cudaSuccess;      // first failed enqueue of a memset
     WindowShape win_shape = default_window_shape(N);
-    auto enqueue = [&](int warps, int64_t nP_run, int n_run, cudaStream_t st) -> int {
+    auto enqueue = [&](int64_t nP_run, int n_run, cudaStream_t st) -> int {
         int l = 0;
         k_init_dstat<<<div_up(n_lc, 128), 128, 0, st>>>(fb.dstat, s_off_dev, n_lc);
         ++l;
@@ -310,7 +296,7 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
         l += lp;
         if (ep != cudaSuccess && enq_err == cudaSuccess) enq_err = ep;
         l += launch_fold_batch(fbat, fsegs, n_run, N, fp64, t_dev, fsc, n_D,
-                               phase_step, gap_factor, periods_dev, nP_run, warps,
+                               phase_step, gap_factor, periods_dev, nP_run,
                                Q_dev, T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev,
                                lnP_dev, st, side, &enq_err);
         count_launches(l - lf);      // launch_factor counted its own
@@ -318,106 +304,79 @@ extern "C" nu_status nu_batch_search(int n_lc, const int64_t* offsets_host,
     };
     // ------------------------------------------------------- autotuning
     const TuneKey key{nb, k, (int)prec, n_D};
-    TuneVal tv{0, win_shape};
-    {
+    bool tuned = !win_lo;
+    if (!tuned) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune.find(key);
-        if (it != g_tune.end()) tv = it->second;
+        if (it != g_tune.end()) {
+            win_shape = it->second;
+            tuned = true;
+        }
     }
-    if (tv.warps == 0) {
-        // time the fold on a slice (the first curves, periods spread over the
-        // whole grid) for each shape; the slice holds several times more
-        // (curve, period) items than the largest grid has blocks, so that it
-        // measures throughput rather than the latency of single items
+    if (!tuned) {
+        // window starts per block x samples per staged chunk, timed on the first
+        // curves
         const int n_run = n_lc < 64 ? n_lc : 64;
-        const int64_t nP_run = n_P < 512 ? n_P : 512;
-        double* tune_periods = (double*)(mem + o_tune);
-        k_sample_periods<<<2, 256, 0, st>>>(periods_dev, n_P, (int)nP_run, tune_periods);
-        count_launches(1);
-        ++launched;
-        float best_ms = 1e30f;
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
-        launched += enqueue(FOLD_SHAPES[0], nP_run, n_run, st);    // warm the caches
+        launched += enqueue(std::min<int64_t>(n_P, 512), n_run, st);       // warm the caches
         if (enq_err != cudaSuccess) {
             cudaEventDestroy(e0);
             cudaEventDestroy(e1);
             cleanup();
             return cuda_fail(enq_err, "nu_batch_search: memset");
         }
-        for (int c = 0; c < 5; ++c) {
+        const WindowShape wc[6] = {{32, 64}, {64, 64}, {64, 32}, {128, 64}, {128, 128},
+                                   {256, 64}};
+        const int64_t n_part = offsets_host[n_run];
+        float best_lin = 1e30f;
+        WindowShape best = win_shape;
+        for (int c = 0; c < 6; ++c) {
             cudaEventRecord(e0, st);
-            const int lt = launch_fold_batch(fbat, fsegs, n_run, N, fp64, t_dev, fsc,
-                                             n_D, phase_step, gap_factor, tune_periods,
-                                             nP_run, FOLD_SHAPES[c], Q_dev,
-                                             T0_dev, D_idx_dev, depth_out_dev, sigma_out_dev,
-                                             lnP_dev, st, side, &enq_err);
+            int lt;
+            if (fp64) {
+                FactorView<double> fv{fb.F, fb.kg, fb.invD, fb.G, fb.z0, fb.Zt};
+                lt = launch_window_batch(nb, true, t_dev, k, &fv, s_off_dev, n_run, n_part,
+                                         Ds_dev, n_D, (int*)(mem + o_wplan), wc[c], lin_d,
+                                         lin_v, lin_l, st);
+            } else {
+                FactorView<float> fv{fb.F32, fb.kg32, fb.invD32, fb.G32, fb.z032, fb.Zt32};
+                lt = launch_window_batch(nb, false, t_dev, k, &fv, s_off_dev, n_run, n_part,
+                                         Ds_dev, n_D, (int*)(mem + o_wplan), wc[c], lin_d,
+                                         lin_v, lin_l, st);
+            }
             count_launches(lt);
             launched += lt;
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best_ms) {
-                best_ms = ms;
-                tv.warps = FOLD_SHAPES[c];
-            }
-        }
-        // the linear search's window-start kernel on the same curves: window
-        // starts per block x samples per staged chunk
-        if (win_lo) {
-            const WindowShape wc[6] = {{32, 64}, {64, 64}, {64, 32}, {128, 64}, {128, 128},
-                                       {256, 64}};
-            const int64_t n_part = offsets_host[n_run];
-            float best_lin = 1e30f;
-            for (int c = 0; c < 6; ++c) {
-                cudaEventRecord(e0, st);
-                int lt;
-                if (fp64) {
-                    FactorView<double> fv{fb.F, fb.kg, fb.invD, fb.G, fb.z0, fb.Zt};
-                    lt = launch_window_batch(nb, true, t_dev, k, &fv, s_off_dev, n_run, n_part,
-                                             Ds_dev, n_D, (int*)(mem + o_wplan), wc[c], lin_d,
-                                             lin_v, lin_l, st);
-                } else {
-                    FactorView<float> fv{fb.F32, fb.kg32, fb.invD32, fb.G32, fb.z032, fb.Zt32};
-                    lt = launch_window_batch(nb, false, t_dev, k, &fv, s_off_dev, n_run, n_part,
-                                             Ds_dev, n_D, (int*)(mem + o_wplan), wc[c], lin_d,
-                                             lin_v, lin_l, st);
-                }
-                count_launches(lt);
-                launched += lt;
-                cudaEventRecord(e1, st);
-                cudaEventSynchronize(e1);
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                if (ms < best_lin) {
-                    best_lin = ms;
-                    tv.win = wc[c];
-                }
+            if (ms < best_lin) {
+                best_lin = ms;
+                best = wc[c];
             }
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
+        win_shape = best;
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune[key] = tv;
+        g_tune[key] = best;
     }
-    win_shape = tv.win;
     // ------------------------------------------------ capture and launch
     // capture on a private stream (the caller's may be the legacy default
     // stream, which cannot be captured), launch on the caller's stream
     // the executable graph of this configuration, when a previous call left
     // one, takes this call's parameters (buffers, outputs) by an update
     cudaGraph_t graph = nullptr;
-    const GraphKey gkey{dev, nb, k, (int)prec, n_D, n_lc, tv.warps,
-                        win_shape.tlo, win_shape.ch, N, n_P};
+    const GraphKey gkey{dev, nb, k, (int)prec, n_D, n_lc, win_shape.tlo, win_shape.ch, N, n_P};
     cudaGraphExec_t exec = take_graph(gkey);
     cudaStream_t cs = nullptr;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     int in_graph = 0;
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        in_graph = enqueue(tv.warps, n_P, n_lc, cs);
+        in_graph = enqueue(n_P, n_lc, cs);
         e = cudaStreamEndCapture(cs, &graph);
         if (e == cudaSuccess && enq_err != cudaSuccess) e = enq_err;
     }

@@ -450,7 +450,7 @@ __device__ __forceinline__ FilterView filter_view(const FilterTab& tab, const Fo
     return v;
 }
 
-enum { FILTER_NONE = 0, FILTER_GAIN = 1, FILTER_QUAD = 2, FILTER_CELL = 3 };
+enum { FILTER_NONE = 0, FILTER_GAIN = 1, FILTER_QUAD = 2, FILTER_CELL = 3, FILTER_LONE = 4 };
 
 // One period's walk: epochs at u0 + k ustep < uend, u0 = j uph for phase j, in
 // 2^-40 slots (2^32 <= ustep < 2^60, uend < 2^62: no position wraps).
@@ -469,7 +469,8 @@ __device__ __forceinline__ int filter_mode(const FilterTab& tab, unsigned long l
     if (K < NU_FILTER_K_QUAD) return FILTER_GAIN;
     // (without S and Q the cells one by one, by their gains; 19 440 epochs x 12
     // durations x 3 000 periods, FP64: 1.69 ms, 4.7 in groups of eight)
-    return tab.S && K < NU_FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL;
+    if (!tab.S) return FILTER_LONE;
+    return K < NU_FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL;
 }
 
 __device__ __forceinline__ float filter_weight(unsigned long long u) {
@@ -643,29 +644,13 @@ __device__ __noinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q
     return pass;
 }
 
-// Bounds of four phases (Q) or one phase (S, or L where there are no others) of
-// four durations from d0 (the walk from u; the odd last pair reads its own row
-// twice).  Two epochs a
+// Bounds of four phases (Q) or one phase (S) of four durations from d0 (the
+// walk from u; the odd last pair reads its own row twice).  Two epochs a
 // round: a position past the end reads the empty last entry.
 __device__ __noinline__ float4 filter_sums(const FilterCtx& x, unsigned long long u, int d0) {
     const FilterPeriod fp = x.fp;
     const bool quad = fp.mode == FILTER_QUAD;
     const unsigned last = (unsigned)x.f.ns - 1u, n4 = (unsigned)x.f.ns >> 2;
-    if (!x.f.S) {
-        const float* __restrict__ r = x.f.L + (int64_t)d0 * x.f.ns;
-        float l[4] = {0.f, 0.f, 0.f, 0.f};
-        for (; u < fp.uend; u += fp.ustep) {
-            const unsigned o = min((unsigned)(u >> 40), last);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (d0 + i < x.n_D) l[i] += r[(int64_t)i * x.f.ns + o];
-        }
-        const float ch = 1.f + filter_slack(fp);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            l[i] = l[i] > 0.f ? fmaf(l[i], ch, 0.500001f) : -INFINITY;
-        return make_float4(l[0], l[1], l[2], l[3]);
-    }
     const uint4* __restrict__ p0 = reinterpret_cast<const uint4*>(quad ? x.f.Q : x.f.S) +
                                    (int64_t)(d0 >> 1) * x.f.ns;
     const uint4* __restrict__ p1 = p0 + (d0 + 2 < x.n_D ? x.f.ns : 0);
@@ -728,6 +713,27 @@ __device__ __noinline__ float4 filter_sums(const FilterCtx& x, unsigned long lon
             v[i] = filter_bound(a[i], v[i], g[i], FILTER_BETA_A / (1.f - FILTER_TAU), xl, c);
     }
     return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// Bounds of one phase of four durations by their gains (the only tables).
+__device__ __noinline__ float4 filter_gain_sums(const FilterCtx& x, unsigned long long u, int d0) {
+    const unsigned last = (unsigned)x.f.ns - 1u;
+    const float* __restrict__ r = x.f.L + (int64_t)d0 * x.f.ns;
+    const float ch = 1.f + filter_slack(x.fp);
+    float l[4] = {0.f, 0.f, 0.f, 0.f};
+    for (; u < x.fp.uend; u += x.fp.ustep) {
+        const unsigned o = min((unsigned)(u >> 40), last);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (d0 + i < x.n_D) l[i] += r[(int64_t)i * x.f.ns + o];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) l[i] = l[i] > 0.f ? fmaf(l[i], ch, 0.500001f) : -INFINITY;
+    return make_float4(l[0], l[1], l[2], l[3]);
+}
+// The bounds of a group in the modes that take four durations.
+__device__ __forceinline__ float4 filter_four(const FilterCtx& x, unsigned long long u, int d0) {
+    return x.fp.mode == FILTER_LONE ? filter_gain_sums(x, u, d0) : filter_sums(x, u, d0);
 }
 
 // Q of one duration.
@@ -886,7 +892,7 @@ __device__ __noinline__ void filter_take(FilterCtx& x, FilterQueues& q, unsigned
                                          int d0, Screen& screen) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    if (x.fp.mode == FILTER_CELL) {
+    if (x.fp.mode >= FILTER_CELL) {
         for (unsigned any = __reduce_or_sync(FULL, pass); any; any &= any - 1u) {
             const int i = __ffs(any) - 1;
             filter_push_cells(q, (pass >> i) & 1u, g, (unsigned)(d0 + i), screen);
@@ -971,7 +977,7 @@ __device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool ac
     } else {
         const int d0 = gi * 4;
         if (act) {
-            const float4 u = filter_sums(x, ((unsigned long long)qi << filter_shift(x.fp.mode)) *
+            const float4 u = filter_four(x, ((unsigned long long)qi << filter_shift(x.fp.mode)) *
                                                 x.fp.uph, d0);
             const float ub[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
@@ -1033,7 +1039,7 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
             const int d0 = gi * 4;
             unsigned pass = 0u;
             if (i < g.n_it) {
-                const float4 u = filter_sums(x, ((unsigned long long)qi << sh) * x.fp.uph, d0);
+                const float4 u = filter_four(x, ((unsigned long long)qi << sh) * x.fp.uph, d0);
                 const float t = filter_thr(x);
                 pass = (!(u.x < t) && u.x != -INFINITY ? 1u : 0u) |
                        (!(u.y < t) && u.y != -INFINITY ? 2u : 0u) |
@@ -1045,7 +1051,7 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
             g.advance(qi, gi);
         }
     }
-    if (mode != FILTER_CELL) filter_drain(x, q, true, screen);
+    if (mode < FILTER_CELL) filter_drain(x, q, true, screen);
     filter_rest(q, screen);
 }
 

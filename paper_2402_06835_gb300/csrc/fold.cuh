@@ -190,16 +190,13 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
                              const void* gain, int n_D, double dt, double gap_factor,
                              const FoldScratch& fs, cudaStream_t st, int* n_launched);
 
-// Shapes of the batch fold the autotuner tries: warps per (curve, period) item,
-// + 4: items of long cells take a block of eight.
-constexpr int FOLD_SHAPES[5] = {1, 2, 1 + 4, 2 + 4, 8};
-// Enqueues the fold of the first n_seg curves (warps: one of FOLD_SHAPES); side:
-// a stream of the caller's for the block items; returns the number of kernels launched, and the first error of an enqueued memset
-// in *err.
+// Enqueues the fold of the first n_seg curves; side: a stream of the caller's for
+// the block items.  Returns the number of kernels launched, and the first error
+// of an enqueued memset in *err.
 int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       int64_t n_total, bool fp64, const double* t, const FoldScratch& fs,
                       int n_D, double dt, double gap_factor, const double* periods,
-                      int64_t n_P, int warps, double* Q, double* T0, int* Didx, double* dep,
+                      int64_t n_P, double* Q, double* T0, int* Didx, double* dep,
                       double* sig, double* lnp, cudaStream_t st, cudaStream_t side,
                       cudaError_t* err);
 

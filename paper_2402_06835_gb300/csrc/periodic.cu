@@ -2664,6 +2664,16 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
     return e;
 }
 
+// Warps per item of n, each of `steps` slots x durations: eight where the items are
+// few for their size, two (and eight for the long ones) from where they fill the
+// GPU, one from 40 000.  One curve, FP64: 4 000 periods of 2 000 epochs x 4
+// durations 0.49 ms with eight, 0.31 with two, 0.34 with one; 1 200 of 8 000 x 4
+// 0.40 / 0.49 / 0.66; 2 500 of 19 440 x 10 1.7 with eight, 2.0 with one.
+static int fold_warps(int64_t n, double steps) {
+    if (n >= NU_ONE_WARP_FROM) return 1;
+    return n >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + steps / 32.0) ? 2 : 8;
+}
+
 // The cell kernels of one job: the exact paths' items, then the slot path's.
 // nw = 1 or 2 warps per item; with a list, its items run in eight-warp blocks on
 // the side stream meanwhile.  nw = 8: every item in such a block.
@@ -2744,7 +2754,7 @@ static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int
 int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                       int64_t n_total, bool fp64, const double* t, const FoldScratch& fs,
                       int n_D, double dt, double gap_factor, const double* periods,
-                      int64_t n_P, int warps, double* Q, double* T0, int* Didx, double* dep,
+                      int64_t n_P, double* Q, double* T0, int* Didx, double* dep,
                       double* sig, double* lnp, cudaStream_t st, cudaStream_t side,
                       cudaError_t* err) {
     int launched = 0;
@@ -2783,8 +2793,10 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
     J.items = fs.items;
     J.sbest = fs.sbest;
     J.counters = fs.n_list;
-    const int nw = warps == 8 ? 8 : warps & 3;
-    if ((warps & 4) && nw != 8 && fs.list) J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
+    int64_t slots = 0;
+    for (int g = 0; g < n_seg; ++g) slots += fb.segs[g].n_bucket;
+    const int nw = fold_warps((int64_t)n_seg * n_P, (double)slots / n_seg * n_D);
+    if (nw != 8 && fs.list) J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
     // The passes: whole curves, or parts of one curve's periods.
     const int64_t pass = fs.pass ? fs.pass : (int64_t)n_seg * n_P;
     int64_t segs_pass = std::min<int64_t>(std::max<int64_t>(pass / n_P, 1), n_seg);
@@ -2875,15 +2887,7 @@ struct FoldCall {
     // 239 / 285 -> 158 / 174; 2 000 x 12 x 1 200 (29 M) 269 / 325 -> 272 / 352; one
     // duration, 8 000 x 4 000 (32 M) 432 / 472 -> 299 / 429.
     bool small() const { return item_steps() * (double)n_P < (n_D == 1 ? 4.0e7 : 2.4e7); }
-    // Warps per period of a pass of n: eight where the periods are few for their
-    // size, two (and eight for the long ones) from where they fill the GPU, one
-    // from 40 000.  FP64: 4 000 periods of 2 000 epochs x 4 durations 0.49 ms with
-    // eight, 0.31 with two, 0.34 with one; 1 200 of 8 000 x 4 0.40 / 0.49 / 0.66;
-    // 2 500 of 19 440 x 10 1.7 with eight, 2.0 with one.
-    int warps(int64_t n) const {
-        if (n >= NU_ONE_WARP_FROM) return 1;
-        return n >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + item_steps() / 32.0) ? 2 : 8;
-    }
+    int warps(int64_t n) const { return fold_warps(n, item_steps()); }
 };
 
 // What a fold keeps in scratch beside the records of its events.
