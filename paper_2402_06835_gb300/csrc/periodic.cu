@@ -1709,7 +1709,8 @@ struct CellScreen {
 
 // Shared state of an item, by one warp (an invalid period is written here).
 __device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs, int64_t seg,
-                                             int64_t p, int64_t o, bool f32, CellItem& it) {
+                                             int64_t p, int64_t o, bool f32, int nw,
+                                             CellItem& it) {
     if ((threadIdx.x & 31) != 0) return;
     const double P = J.periods[p];
     const FoldGeom g = job_geom(J, fs);
@@ -1752,7 +1753,7 @@ __device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs
     f.n_phi = pc->n_phi;
     f.K = ic.K + 2.f;
     f.mode = on && sp.delta <= 8ull * FILTER_MARGIN
-                 ? filter_mode(J.tab, sp.ustep, ic.K, f.n_phi * J.n_D)
+                 ? filter_mode(J.tab, sp.ustep, ic.K, f.n_phi * J.n_D, nw)
                  : FILTER_NONE;
     it.x.fp = f;
     it.x.f = filter_view(J.tab, fs);
@@ -1781,7 +1782,7 @@ __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int
         q.f.ni = q.f.nq = q.f.nc = q.nb = 0;
         tbs[w] = Best{-INFINITY, LLONG_MAX, NAN, NAN};
     }
-    if (w == 0) cell_item_setup(J, fs, seg, p, o, sizeof(T) == 4, it);
+    if (w == 0) cell_item_setup(J, fs, seg, p, o, sizeof(T) == 4, nw, it);
     item_sync<nw>();
     if (it.item < 0) return;
     CellScreen<T> screen{it, q, (const Node8<T>*)J.nodes + fs.s_off * n_D, tbs[w]};
@@ -2243,7 +2244,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
         f.n_phi = sp.n_phi;
         const float K = slot_K(fs, sp);
         f.K = K + 2.f;
-        f.mode = filter_mode(J.tab, sp.ustep, K, f.n_phi * n_D);
+        f.mode = filter_mode(J.tab, sp.ustep, K, f.n_phi * n_D, nw);
         it.x.fp = f;
         it.x.f = filter_view(J.tab, fs);
         it.x.n_D = n_D;
