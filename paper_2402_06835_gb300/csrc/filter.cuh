@@ -741,11 +741,6 @@ __device__ __noinline__ float4 filter_gain_sums(const FilterCtx& x, unsigned lon
     for (int i = 0; i < 4; ++i) l[i] = l[i] > 0.f ? fmaf(l[i], ch, 0.500001f) : -INFINITY;
     return make_float4(l[0], l[1], l[2], l[3]);
 }
-// The bounds of a group in the modes that take four durations.
-__device__ __forceinline__ float4 filter_four(const FilterCtx& x, unsigned long long u, int d0) {
-    return x.fp.mode == FILTER_LONE ? filter_gain_sums(x, u, d0) : filter_sums(x, u, d0);
-}
-
 // Q of one duration.
 __device__ __forceinline__ float filter_one_quad(const FilterView& f, int d, unsigned long long u,
                                                  const FilterPeriod& fp, float c) {
@@ -830,7 +825,7 @@ __device__ __noinline__ void filter_expand(FilterCtx& x, FilterQueues& qs, const
                 float ub = gain ? filter_one_gain(x.f, (int)d, u, x.fp, c)
                                 : filter_one(x.f, (int)d, u, x.fp, c);
                 keep = !(ub < filter_thr(x)) && ub != -INFINITY;
-                if (keep && x.f.S && x.fp.K > 5.5f && x.fp.K < 14.f) {
+                if (keep && x.fp.K > 5.5f && x.fp.K < 14.f && x.f.S) {
                     ub = gain ? filter_one(x.f, (int)d, u, x.fp, c)
                               : filter_one_gain(x.f, (int)d, u, x.fp, c);
                     keep = !(ub < filter_thr(x)) && ub != -INFINITY;
@@ -902,7 +897,7 @@ __device__ __noinline__ void filter_take(FilterCtx& x, FilterQueues& q, unsigned
                                          int d0, Screen& screen) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    if (x.fp.mode >= FILTER_CELL) {
+    if (x.fp.mode == FILTER_CELL) {
         for (unsigned any = __reduce_or_sync(FULL, pass); any; any &= any - 1u) {
             const int i = __ffs(any) - 1;
             filter_push_cells(q, (pass >> i) & 1u, g, (unsigned)(d0 + i), screen);
@@ -987,7 +982,7 @@ __device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool ac
     } else {
         const int d0 = gi * 4;
         if (act) {
-            const float4 u = filter_four(x, ((unsigned long long)qi << filter_shift(x.fp.mode)) *
+            const float4 u = filter_sums(x, ((unsigned long long)qi << filter_shift(x.fp.mode)) *
                                                 x.fp.uph, d0);
             const float ub[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
@@ -1002,6 +997,50 @@ __device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool ac
     filter_seed(x, q, b, qi, bd, screen);
 }
 
+// The cells of a period by their gains, four durations a lane (FILTER_LONE; apart
+// from the other modes, whose walks it would slow down by 2-4 %).
+template <class Screen>
+__device__ __noinline__ void filter_lone(FilterCtx& x, int wid, int nw, FilterQueues& q,
+                                         Screen& screen) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned n_phi = (unsigned)x.fp.n_phi;
+    const unsigned n_it = n_phi * (unsigned)((x.n_D + 3) / 4);
+    bool first = true;
+    for (unsigned base = (unsigned)wid * 32u; base < n_it; base += (unsigned)nw * 32u) {
+        const unsigned i = base + (unsigned)lane;
+        const int gi = (int)(i / n_phi), d0 = 4 * gi;
+        const unsigned j = i - (unsigned)gi * n_phi;
+        float ub[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        if (i < n_it) {
+            const float4 u = filter_gain_sums(x, (unsigned long long)j * x.fp.uph, d0);
+            ub[0] = u.x;
+            ub[1] = u.y;
+            ub[2] = u.z;
+            ub[3] = u.w;
+        }
+        if (first) {
+            float b = 0.f;
+            int bd = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (d0 + k < x.n_D && ub[k] > b && ub[k] < INFINITY) {
+                    b = ub[k];
+                    bd = k;
+                }
+            filter_seed(x, q, b, j, d0 + bd, screen);
+            first = false;
+        }
+        const float t = filter_thr(x);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool keep = d0 + k < x.n_D && !(ub[k] < t) && ub[k] != -INFINITY;
+            if (__any_sync(FULL, keep)) filter_push_cells(q, keep, j, (unsigned)(d0 + k), screen);
+        }
+    }
+    filter_rest(q, screen);
+}
+
 // Runs the filters over every cell of a period.  The item's warps (wid of
 // nw) share the work.  Cells below the threshold are dropped, the others go
 // through the screen.
@@ -1011,6 +1050,10 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int n_D = x.n_D, mode = x.fp.mode;
+    if (mode == FILTER_LONE) {
+        filter_lone(x, wid, nw, q, screen);
+        return;
+    }
     const int sh = filter_shift(mode);
     FilterGroups g;
     g.W = mode == FILTER_GAIN ? 2 * filter_words(n_D) : 4;
@@ -1049,7 +1092,7 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
             const int d0 = gi * 4;
             unsigned pass = 0u;
             if (i < g.n_it) {
-                const float4 u = filter_four(x, ((unsigned long long)qi << sh) * x.fp.uph, d0);
+                const float4 u = filter_sums(x, ((unsigned long long)qi << sh) * x.fp.uph, d0);
                 const float t = filter_thr(x);
                 pass = (!(u.x < t) && u.x != -INFINITY ? 1u : 0u) |
                        (!(u.y < t) && u.y != -INFINITY ? 2u : 0u) |
@@ -1061,7 +1104,7 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
             g.advance(qi, gi);
         }
     }
-    if (mode < FILTER_CELL) filter_drain(x, q, true, screen);
+    if (mode != FILTER_CELL) filter_drain(x, q, true, screen);
     filter_rest(q, screen);
 }
 
