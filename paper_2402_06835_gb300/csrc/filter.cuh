@@ -176,6 +176,22 @@ __device__ __forceinline__ float portion_g(const Portion& p, float beta) {
            2e-6f * (fabsf(p.l0) + fabsf(p.l1) + ym * ym);
 }
 
+// Whether the interval between two slot records is outside what is bounded.
+__device__ __forceinline__ bool slot_odd(const Node4<float>& a, const Node4<float>& b) {
+    return !(a.s >= 1e-12f && a.s <= 1e12f) || !(b.s >= 1e-12f && b.s <= 1e12f) ||
+           !(a.s <= 3.f * b.s) || !(b.s <= 3.f * a.s) || !(fabsf(a.d) <= 1e8f * a.s) ||
+           !(fabsf(b.d) <= 1e8f * b.s) || !(fabsf(a.l) <= 1e20f) || !(fabsf(b.l) <= 1e20f);
+}
+// L of a slot: its largest gain lmax with room for rounding, +inf where it is not
+// bounded.
+__device__ __forceinline__ float bounded_gain(float lmax, bool odd) {
+    const float l = fmaxf(lmax * 1.000001f, 1e-30f);
+    return odd || !(l < 1e30f) ? INFINITY : l;
+}
+__device__ __forceinline__ float slot_gain(const Node4<float>& a, const Node4<float>& b) {
+    return bounded_gain(fmaxf(a.l, b.l), slot_odd(a, b));
+}
+
 // Writes the entries of one slot.  ok: every event of the slot is on a valid
 // interval (chord from zA to zB, within e; the smallest v; the largest gA,
 // gB); maybe: some are, some are not (their gains lmax count); odd: not bounded.
@@ -184,8 +200,7 @@ __device__ __forceinline__ void write_slot(const FilterTab& tab, int64_t o, int6
                                            float gA, float gB, float lmax) {
     const float tiny = 1e-30f;
     if (!tab.S) {                       // the gains alone
-        const float g = fmaxf(lmax * 1.000001f, tiny);
-        tab.L[o] = !any ? 0.f : (odd || !(g < 1e30f) ? INFINITY : g);
+        tab.L[o] = any ? bounded_gain(lmax, odd) : 0.f;
         return;
     }
     float z0 = 0.f, dz = 0.f, vv = 0.f, a = 0.f, b = 0.f, l = 0.f, zmx = 0.f, zmn = 0.f;
@@ -286,10 +301,7 @@ __global__ void k_filter_slots(const ScreenRec* __restrict__ screen,
             const Node4<float> a = r[0], b = r[1];
             if (!isnan(a.s) && !isnan(b.s)) {
                 any = true;
-                odd = !(a.s >= 1e-12f && a.s <= 1e12f) || !(b.s >= 1e-12f && b.s <= 1e12f) ||
-                      !(a.s <= 3.f * b.s) || !(b.s <= 3.f * a.s) || !(fabsf(a.d) <= 1e8f * a.s) ||
-                      !(fabsf(b.d) <= 1e8f * b.s) || !(fabsf(a.l) <= 1e20f) ||
-                      !(fabsf(b.l) <= 1e20f);
+                odd = slot_odd(a, b);
                 if (!odd) {
                     const Portion p = portion(a.d, a.s, a.l, b.d, b.s, b.l, rs);
                     zA = p.h0;
@@ -445,7 +457,7 @@ __device__ __forceinline__ FilterView filter_view(const FilterTab& tab, const Fo
     v.Q = tab.S ? tab.Q + sg.pair_off : nullptr;
     v.gB = tab.S ? tab.gB + sg.tab_off : nullptr;
     v.L = tab.L + sg.tab_off;
-    v.G = tab.G + sg.g_off;
+    v.G = tab.G ? tab.G + sg.g_off : nullptr;
     v.ns = (int)filter_slots(sg.n_slots);
     return v;
 }
@@ -476,6 +488,7 @@ __device__ __forceinline__ int filter_mode(const FilterTab& tab, unsigned long l
     if (!tab.L || ustep < (1ull << 32) || ustep >= (1ull << 60) || !(K < FILTER_K_MAX) ||
         n_cells >= 0x7fff0000LL)
         return FILTER_NONE;
+    if (!tab.G) return FILTER_LONE;
     if (K < NU_FILTER_K_QUAD) return FILTER_GAIN;
     // (without S and Q the cells one by one, by their gains; 19 440 epochs x 12
     // durations x 3 000 periods, FP64: 1.69 ms, 4.7 in groups of eight)
@@ -773,7 +786,9 @@ __device__ __forceinline__ void filter_shift_queue(uint2* q, int len, int n) {
 // The functions below are not inlined: they run on the few groups and cells
 // that pass, and inlining them into the walks' loop spills its registers.  A
 // screen is a functor: screen(cnt) takes the first cnt <= 32 cells of the
-// queue, one per lane.
+// queue, one per lane.  Screen::lone: the kernel of calls that have the gains'
+// tables alone (in the other kernels the walk for them costs the other walks up to
+// 8 %: 420 curves of 1 700-3 700 x 7 durations x 1 000 periods, FP64, 37.7 -> 34.8 ms).
 template <class Screen>
 __device__ __noinline__ void filter_push_cells(FilterQueues& q, bool keep, unsigned j, unsigned d,
                                                Screen& screen) {
@@ -825,7 +840,7 @@ __device__ __noinline__ void filter_expand(FilterCtx& x, FilterQueues& qs, const
                 float ub = gain ? filter_one_gain(x.f, (int)d, u, x.fp, c)
                                 : filter_one(x.f, (int)d, u, x.fp, c);
                 keep = !(ub < filter_thr(x)) && ub != -INFINITY;
-                if (keep && x.fp.K > 5.5f && x.fp.K < 14.f && x.f.S) {
+                if (!Screen::lone && keep && x.fp.K > 5.5f && x.fp.K < 14.f) {
                     ub = gain ? filter_one(x.f, (int)d, u, x.fp, c)
                               : filter_one_gain(x.f, (int)d, u, x.fp, c);
                     keep = !(ub < filter_thr(x)) && ub != -INFINITY;
@@ -874,7 +889,7 @@ __device__ __noinline__ void filter_drain(FilterCtx& x, FilterQueues& q, bool al
                                           Screen& screen) {
     const int lane = threadIdx.x & 31;
     const bool gain = x.fp.mode == FILTER_GAIN;
-    const bool mid = gain && x.f.Q && x.fp.K >= NU_FILTER_K_MID + 2.f;
+    const bool mid = !Screen::lone && gain && x.fp.K >= NU_FILTER_K_MID + 2.f;
     const int ni = q.ni;
     const int round = mid ? 16 : (gain ? 4 : 8);
     const int n = all ? ni : ni & ~(round - 1);
@@ -997,8 +1012,7 @@ __device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool ac
     filter_seed(x, q, b, qi, bd, screen);
 }
 
-// The cells of a period by their gains, four durations a lane (FILTER_LONE; apart
-// from the other modes, whose walks it would slow down by 2-4 %).
+// The cells of a period by their gains, four durations a lane (FILTER_LONE).
 template <class Screen>
 __device__ __noinline__ void filter_lone(FilterCtx& x, int wid, int nw, FilterQueues& q,
                                          Screen& screen) {
@@ -1050,9 +1064,11 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int n_D = x.n_D, mode = x.fp.mode;
-    if (mode == FILTER_LONE) {
-        filter_lone(x, wid, nw, q, screen);
-        return;
+    if constexpr (Screen::lone) {
+        if (mode == FILTER_LONE) {
+            filter_lone(x, wid, nw, q, screen);
+            return;
+        }
     }
     const int sh = filter_shift(mode);
     FilterGroups g;

@@ -79,8 +79,8 @@ __host__ __device__ inline int filter_groups(int n_D) {
 
 // Tables of all curves; rows of filter_slots(n_slots) per duration from
 // tab_off on (in rows' entries), G from g_off on (in words).  Where scratch is
-// short only L and G are there (S, Q, gB, Z and vmax null): the fold then bounds
-// by gains alone.  All null: no tables.
+// short only L and G are there (S, Q, gB, Z and vmax null), in small calls of the
+// slot path L alone: the fold then bounds by gains.  All null: no tables.
 struct FilterTab {
     uint2* S;
     float* gB;

@@ -130,24 +130,34 @@ __global__ void k_slots(const double* __restrict__ t0s, int64_t n_t0, double t_r
     if (bad) atomicExch(irregular, 1);
 }
 
+__device__ __forceinline__ Node4<float> slot_record(const float* __restrict__ depth,
+                                                    const float* __restrict__ var,
+                                                    const float* __restrict__ gain,
+                                                    int64_t gid) {
+    const float d = depth[gid], v = var[gid], l = gain[gid];
+    const bool ok = isfinite(d) && isfinite(v) && isfinite(l) && v > 0.f;
+    return Node4<float>{d, ok ? sqrtf(v) : NAN, l, 0.f};
+}
+
 // Slot records (mixed path): node values placed at their slot, NaN sigma in
 // empty slots.  One thread per (duration, epoch); slots were cleared to NaN.
+// L (if given): the filters' gain table, rows of ns, cleared to 0: the largest
+// gain on the interval that starts at the slot.
 __global__ void k_slot_fill(const float* __restrict__ depth, const float* __restrict__ var,
                             const float* __restrict__ gain, const int* __restrict__ slot_of,
                             int64_t n_t0, int n_D, int64_t n_slots,
-                            Node4<float>* __restrict__ rec) {
+                            Node4<float>* __restrict__ rec, float* __restrict__ L, int64_t ns) {
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (gid >= n_t0 * (int64_t)n_D) return;
     const int64_t d = gid / n_t0, i = gid - d * n_t0;
     const int s = slot_of[i];
     if (s < 0 || s >= n_slots) return;
-    const float dd = depth[gid], v = var[gid], l = gain[gid];
-    Node4<float> r;
-    r.d = dd;
-    r.l = l;
-    r.s = (isfinite(dd) && isfinite(v) && isfinite(l) && v > 0.f) ? sqrtf(v) : NAN;
-    r.ig = 0.f;
+    const Node4<float> r = slot_record(depth, var, gain, gid);
     rec[d * n_slots + s] = r;
+    if (L && i + 1 < n_t0 && slot_of[i + 1] == s + 1) {
+        const Node4<float> q = slot_record(depth, var, gain, gid + 1);
+        if (!isnan(r.s) && !isnan(q.s)) L[d * ns + s] = slot_gain(r, q);
+    }
 }
 
 __global__ void k_fill_nan(Node4<float>* rec, int64_t n) {
@@ -1454,17 +1464,18 @@ template <typename T> struct FoldPrep {
     unsigned long long* peak;
     unsigned end[PREP_N];
 };
-// The same on the slot path: blocks [0, b_rec) clear the slot records, [b_rec,
+// The same on the slot path: blocks [0, b_rec) clear the slot records and L, [b_rec,
 // b_peak) find the largest gain, the rest fill the period table.
 __global__ void __launch_bounds__(256)
-k_slot_prep(Node4<float>* __restrict__ rec, int64_t n_rec, unsigned b_rec,
-            const float* __restrict__ gain, int64_t n, unsigned b_peak,
+k_slot_prep(Node4<float>* __restrict__ rec, int64_t n_rec, float* __restrict__ L, int64_t n_L,
+            unsigned b_rec, const float* __restrict__ gain, int64_t n, unsigned b_peak,
             unsigned long long* __restrict__ peak, const double* __restrict__ periods,
             int64_t n_P, double dt, SlotPeriod* __restrict__ stab) {
     const unsigned b = blockIdx.x;
     if (b < b_rec) {
         const int64_t i = b * (int64_t)blockDim.x + threadIdx.x;
         if (i < n_rec) rec[i] = Node4<float>{NAN, NAN, NAN, 0.f};
+        if (i < n_L) L[i] = 0.f;
     } else if (b < b_peak) {
         gain_peak<float>(gain, n, b - b_rec, b_peak - b_rec, peak);
     } else {
@@ -1522,12 +1533,6 @@ __device__ __forceinline__ void item_sync() {
 #ifndef NU_FOLD_WARPS
 #define NU_FOLD_WARPS 32           // resident warps per SM (64 registers)
 #endif
-#ifndef NU_WARP_ITEMS_FROM
-#define NU_WARP_ITEMS_FROM 6000    // periods from which two warps fold one (single curve)
-#endif
-#ifndef NU_ONE_WARP_FROM
-#define NU_ONE_WARP_FROM 40000     // and one warp
-#endif
 #ifndef NU_HEAVY_K
 #define NU_HEAVY_K 22.f            // epochs per cell of an item that takes a block then
 #endif
@@ -1582,8 +1587,9 @@ struct CellItem {          // per-item shared state of the exact paths
 };
 
 // The screen of the exact paths (filter.cuh) and what follows it.
-template <typename T>
+template <typename T, bool LONE>
 struct CellScreen {
+    static constexpr bool lone = LONE;
     CellItem& it;
     CellQueues& q;
     const Node8<T>* nodes;
@@ -1767,7 +1773,7 @@ __device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs
 }
 
 // One item of the exact paths by the nw warps that share it (w: this one).
-template <typename T, int nw>
+template <typename T, int nw, bool LONE>
 __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int w, CellItem& it,
                                                 CellQueues& q, Best* tbs) {
     const unsigned FULL = 0xffffffffu;
@@ -1785,7 +1791,7 @@ __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int
     if (w == 0) cell_item_setup(J, fs, seg, p, o, sizeof(T) == 4, nw, it);
     item_sync<nw>();
     if (it.item < 0) return;
-    CellScreen<T> screen{it, q, (const Node8<T>*)J.nodes + fs.s_off * n_D, tbs[w]};
+    CellScreen<T, LONE> screen{it, q, (const Node8<T>*)J.nodes + fs.s_off * n_D, tbs[w]};
     if (it.x.fp.mode != FILTER_NONE) {
         // peak seed: the cells about the curve's largest single-event gain
         const unsigned long long pk = J.peak[seg];
@@ -1866,7 +1872,7 @@ __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int
 }
 
 // Exact paths (FP64 epochs; T: the type of the events).
-template <typename T, int NW>
+template <typename T, int NW, bool LONE>
 __global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
 k_fold_cells(const __grid_constant__ FoldJob J) {
     constexpr int W = fold_threads(NW) / 32;
@@ -1878,10 +1884,10 @@ k_fold_cells(const __grid_constant__ FoldJob J) {
     if (NW == 8) {
         __shared__ unsigned sh_k;
         for (int k = 0; next_item(J, k, &sh_k, item); ++k)
-            fold_cells_item<T, NW>(J, item, wid, sh_i[0], sh_q[wid], sh_tb);
+            fold_cells_item<T, NW, LONE>(J, item, wid, sh_i[0], sh_q[wid], sh_tb);
     } else if (warp_item<NW>(J, item)) {
-        fold_cells_item<T, NW>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid],
-                               sh_tb + wid / NW * NW);
+        fold_cells_item<T, NW, LONE>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid],
+                                     sh_tb + wid / NW * NW);
     }
 }
 
@@ -2101,7 +2107,9 @@ struct SlotQueues {
     int bd[32];                        // -1: none
 };
 
+template <bool LONE>
 struct SlotScreen {
+    static constexpr bool lone = LONE;
     SlotItem& it;
     SlotQueues& q;
     const Node4<float>* rec;
@@ -2219,7 +2227,7 @@ __global__ void k_slot_items(const __grid_constant__ FoldJob J) {
 }
 
 // One item of the slot path by the nw warps that share it.
-template <int nw>
+template <int nw, bool LONE>
 __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int w, SlotItem& it,
                                                 SlotQueues& q) {
     const unsigned FULL = 0xffffffffu;
@@ -2258,7 +2266,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
         }
         return;
     }
-    SlotScreen screen{it, q, J.rec + fs.rec_off, fs.n_slots, fs.ulast};
+    SlotScreen<LONE> screen{it, q, J.rec + fs.rec_off, fs.n_slots, fs.ulast};
     if (it.x.fp.mode != FILTER_NONE) {
         const unsigned long long pk = J.peak[seg];
         if (pk != 0 && w == 0) {
@@ -2324,7 +2332,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
     }
 }
 
-template <int NW>
+template <int NW, bool LONE>
 __global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
 k_fold_slot_cells(const __grid_constant__ FoldJob J) {
     constexpr int W = fold_threads(NW) / 32;
@@ -2335,9 +2343,9 @@ k_fold_slot_cells(const __grid_constant__ FoldJob J) {
     if (NW == 8) {
         __shared__ unsigned sh_k;
         for (int k = 0; next_item(J, k, &sh_k, item); ++k)
-            fold_slots_item<NW>(J, item, wid, sh_i[0], sh_q[wid]);
+            fold_slots_item<NW, LONE>(J, item, wid, sh_i[0], sh_q[wid]);
     } else if (warp_item<NW>(J, item)) {
-        fold_slots_item<NW>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid]);
+        fold_slots_item<NW, LONE>(J, item, wid % NW, sh_i[wid / NW], sh_q[wid]);
     }
 }
 
@@ -2671,8 +2679,8 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
 // durations 0.49 ms with eight, 0.31 with two, 0.34 with one; 1 200 of 8 000 x 4
 // 0.40 / 0.49 / 0.66; 2 500 of 19 440 x 10 1.7 with eight, 2.0 with one.
 static int fold_warps(int64_t n, double steps) {
-    if (n >= NU_ONE_WARP_FROM) return 1;
-    return n >= std::min<double>(NU_WARP_ITEMS_FROM, 1000.0 + steps / 32.0) ? 2 : 8;
+    if (n >= 40000) return 1;
+    return n >= std::min(6000.0, 1000.0 + steps / 32.0) ? 2 : 8;
 }
 
 // The cell kernels of one job: the exact paths' items, then the slot path's.
@@ -2690,12 +2698,20 @@ static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int
     };
     if (nw == 2 && items > 0x7fffffffLL) nw = 1;          // the grid's limit
     const int g8 = (int)std::min<int64_t>(items, (int64_t)n_sm * (NU_FOLD_WARPS / 8));
+    // (the gains' tables alone: kernels of their own)
+    const bool lone = J.tab.L && !J.tab.S;
+#define NU_CELLS_AS(NW_, LONE_, GRID_, ST_)                                                \
+    do {                                                                                   \
+        const dim3 g_(GRID_), b_(fold_threads(NW_));                                       \
+        if (path == 1) k_fold_slot_cells<NW_, LONE_><<<g_, b_, 0, ST_>>>(J);               \
+        else if (fp64) k_fold_cells<double, NW_, LONE_><<<g_, b_, 0, ST_>>>(J);            \
+        else k_fold_cells<float, NW_, LONE_><<<g_, b_, 0, ST_>>>(J);                       \
+        ++launched;                                                                        \
+    } while (0)
 #define NU_CELLS(NW_, GRID_, ST_)                                                          \
     do {                                                                                   \
-        if (path == 1) k_fold_slot_cells<NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J);    \
-        else if (fp64) k_fold_cells<double, NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J); \
-        else k_fold_cells<float, NW_><<<GRID_, fold_threads(NW_), 0, ST_>>>(J);            \
-        ++launched;                                                                        \
+        if (lone) NU_CELLS_AS(NW_, true, GRID_, ST_);                                      \
+        else NU_CELLS_AS(NW_, false, GRID_, ST_);                                          \
     } while (0)
     for (int path = 0; path < 2; ++path) {
         if (!(path == 0 ? exact : slots)) continue;
@@ -2749,6 +2765,7 @@ static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int
         }
     }
 #undef NU_CELLS
+#undef NU_CELLS_AS
     return launched;
 }
 
@@ -2883,11 +2900,19 @@ struct FoldCall {
     bool may_screen() const { return gap_factor < 2.0 && span_steps() < 8.0e6; }
     // Small calls: screening every cell costs less than the filters' tables and
     // rounds, and a few survivors per block less than the launches that pack
-    // them.  Mixed / FP64, us with filters -> without: 4 000 epochs x 4 durations
-    // x 1 200 periods (19 M steps) 309 / 365 -> 208 / 276, 1 100 x 12 x 300 (4 M)
-    // 239 / 285 -> 158 / 174; 2 000 x 12 x 1 200 (29 M) 269 / 325 -> 272 / 352; one
-    // duration, 8 000 x 4 000 (32 M) 432 / 472 -> 299 / 429.
-    bool small() const { return item_steps() * (double)n_P < (n_D == 1 ? 4.0e7 : 2.4e7); }
+    // them.  FP64, us with filters -> without: 4 000 epochs x 4 durations x 1 200
+    // periods (19 M steps) 365 -> 276, 1 100 x 12 x 300 (4 M) 285 -> 174; 2 000 x 12
+    // x 1 200 (29 M) 325 -> 352; one duration, 8 000 x 4 000 (32 M) 472 -> 429.
+    // On the slot path they bound by the gains that the records hold, which are
+    // written with them (slots: 2 000 x 4 x 2 000, 17 M, 223 -> 186 us against
+    // every cell; 1 100 x 4 x 12 000, 54 M, 344 -> 250 against all tables; items of
+    // more steps go to the tables sooner: 4 000 x 20 x 1 000, 88 M, 330 with, 360
+    // without).
+    bool small(bool slots) const {
+        const double work = item_steps() * (double)n_P;
+        if (slots) return work < (item_steps() < 4.0e4 ? 6.0e7 : 2.4e7);
+        return work < (n_D == 1 ? 4.0e7 : 2.4e7);
+    }
     int warps(int64_t n) const { return fold_warps(n, item_steps()); }
 };
 
@@ -2895,11 +2920,13 @@ struct FoldCall {
 struct FoldPlan {
     bool slots;          // the mixed regular path's records, else the exact paths'
     bool screen;         // exact paths: the screen's records
-    int tables;          // filter tables: 2 all, 1 the gains', 0 none
+    int tables;          // filter tables: 2 all, 1 the gains', 0 none; TABLES_SLOT: the
+                         // slot path's L, written with its records
     int64_t pass;        // periods per pass, with their table and lists; 0: all in one
                          // pass without (survivors are evaluated in place)
 };
 
+constexpr int TABLES_SLOT = 3;
 // The plans of a call, the best one first; the last needs the least.  Period
 // tables and lists take 290 bytes per period, so that a long grid of periods goes
 // through them in passes: 2^19 periods at most, and fewer where scratch is
@@ -2911,7 +2938,8 @@ static std::vector<FoldPlan> fold_plans(const FoldCall& C, bool slots) {
     std::vector<FoldPlan> plans;
     const bool screen = !slots && C.may_screen();
     if (slots || screen) {
-        for (int tables = C.small() ? 0 : 2; tables >= 0; --tables) {
+        for (int tables = !C.small(slots) ? 2 : (slots ? TABLES_SLOT : 0); tables >= 0;
+             tables = tables == TABLES_SLOT ? 0 : tables - 1) {
             for (int64_t k = (C.n_P + PASS_MAX - 1) / PASS_MAX;; k += std::max<int64_t>(1, k / 4)) {
                 const int64_t pass = (C.n_P + k - 1) / k;
                 if (pass < PASS_MIN && pass < C.n_P) break;
@@ -2954,8 +2982,10 @@ static SingleLayout single_layout(const FoldCall& C, const FoldPlan& plan) {
         L.bucket = take((size_t)C.n_bucket * sizeof(int));
         if (C.fp64 && plan.screen) L.srec = take((size_t)n_slots * C.n_D * sizeof(ScreenRec));
     }
-    if (plan.tables) {
-        const int64_t ns = filter_slots(n_slots);
+    const int64_t ns = filter_slots(n_slots);
+    if (plan.tables == TABLES_SLOT) {
+        L.tab = take((size_t)ns * C.n_D * sizeof(float));
+    } else if (plan.tables) {
         L.fl = filter_layout(ns * C.n_D, ns * ((C.n_D + 1) / 2 * 2),
                              ns * filter_groups(C.n_D) * filter_words(C.n_D), C.n_D,
                              plan.tables == 1);
@@ -3007,14 +3037,17 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
         // them: 10 us on the GPU, hidden in part by the wait).
         const int64_t nrec = n_slots * n_D;
         Node4<float>* rec = (Node4<float>*)(scratch + Ls->records);
-        const unsigned b_rec = (unsigned)div_up(nrec, 256), b_peak = b_rec + peak_grid;
+        const int64_t ns = filter_slots(n_slots);
+        float* Lg = Ls->plan.tables == TABLES_SLOT ? (float*)(scratch + Ls->tab) : nullptr;
+        const int64_t n_L = Lg ? ns * n_D : 0;
+        const unsigned b_rec = (unsigned)div_up(std::max(nrec, n_L), 256), b_peak = b_rec + peak_grid;
         const unsigned b_all = b_peak + (unsigned)div_up(Ls->plan.pass, 256);
-        k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, b_rec, (const float*)C.dlnl, ngrid,
+        k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, Lg, n_L, b_rec, (const float*)C.dlnl, ngrid,
                                            b_peak, peak, C.periods, Ls->plan.pass, phase_step,
                                            (SlotPeriod*)(scratch + Ls->ptab));
         k_slot_fill<<<div_up(ngrid, 256), 256, 0, st>>>(
             (const float*)C.depth, (const float*)C.var, (const float*)C.dlnl, slot_of,
-            n_t0, n_D, n_slots, rec);
+            n_t0, n_D, n_slots, rec, Lg, ns);
         launched += 3;
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&irregular, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -3056,7 +3089,8 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
         J.ptab = (const PeriodConst*)(scratch + L.ptab);
         J.stab = (const SlotPeriod*)(scratch + L.ptab);
     }
-    if (L.plan.tables) J.tab = filter_tab(scratch + L.tab, L.fl, L.plan.tables == 1);
+    if (L.plan.tables == TABLES_SLOT) J.tab.L = (float*)(scratch + L.tab);
+    else if (L.plan.tables) J.tab = filter_tab(scratch + L.tab, L.fl, L.plan.tables == 1);
     if (!use_slots) {
         const double gap_max = J.gap_max;
         ScreenRec* screen = (ScreenRec*)J.screen;
@@ -3108,7 +3142,7 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
         }
         ++launched;
     }
-    if (J.tab.L)
+    if (J.tab.G)
         e = launch_filter_tables(nullptr, one, 1, n_D, filter_slots(n_slots) * n_D, n_t0, J.screen,
                                  J.vpair, J.bucket, J.rec, J.tab, st, &launched);
     for (int64_t p0 = 0; p0 < n_P && e == cudaSuccess; p0 += pass) {
@@ -3131,7 +3165,7 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
             ++launched;
         }
         const int nw = C.warps(n);
-        if (L.plan.pass && !(C.small() && (nw == 8 || use_slots))) {
+        if (L.plan.pass && !(C.small(use_slots) && (nw == 8 || use_slots))) {
             J.counters = (unsigned*)(scratch + L.flag + 64);
             if (use_slots) {
                 J.sbest = (SlotBest*)(scratch + L.sbest);

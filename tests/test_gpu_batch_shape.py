@@ -30,8 +30,8 @@ def _kernels(path, call):
     return names
 
 
-@pytest.mark.parametrize("precision, block", [("fp64", "k_fold_cells<double, 8>"),
-                                              ("mixed", "k_fold_slot_cells<8>")])
+@pytest.mark.parametrize("precision, block", [("fp64", "k_fold_cells<double, 8"),
+                                              ("mixed", "k_fold_slot_cells<8")])
 @pytest.mark.parametrize("n_D", [1, 4, 9])
 def test_long_cells_take_blocks_after_a_batch_of_short_ones(precision, block, n_D, tmp_path):
     dt = synth.CADENCE_DAYS

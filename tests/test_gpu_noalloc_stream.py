@@ -38,8 +38,8 @@ def _streams(path, call):
 def test_noalloc_uses_one_stream(precision, tmp_path):
     t, depth, var, dlnl, dt = _grid(1203, 12, 23, "regular")
     span = t[-1] - t[0]
-    periods = np.concatenate([np.linspace(span / 70, span / 15, 800),
-                              np.linspace(0.9 * span, span / 15, 2700)])
+    periods = np.concatenate([np.linspace(span / 70, span / 15, 1500),
+                              np.linspace(0.9 * span, span / 15, 4500)])
     out = {}
 
     def run(fn):
