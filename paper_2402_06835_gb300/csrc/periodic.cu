@@ -1243,7 +1243,11 @@ struct FoldLists {
     unsigned* block;       // item indices, appended by the preparation kernels
     unsigned* n;           // [0] their number, [1] taken
     float heavy_k;
+    unsigned max;          // with more of them the warps keep them (list_max)
 };
+__device__ __forceinline__ bool list_taken(const FoldLists& l) {
+    return l.block && l.n[0] <= l.max;
+}
 __device__ __forceinline__ void list_item(const FoldLists& l, bool heavy, unsigned o) {
     const int lane = threadIdx.x & 31;
     const unsigned m = __ballot_sync(0xffffffffu, heavy);
@@ -1553,7 +1557,7 @@ __device__ __forceinline__ bool next_item(const FoldJob& J, int k_th, unsigned* 
     if (threadIdx.x == 0) *sh = atomicAdd(J.list.n + 1, 1u);
     __syncthreads();
     const unsigned k = *sh;
-    if (k >= J.list.n[0]) return false;
+    if (k >= J.list.n[0] || !list_taken(J.list)) return false;
     item = J.list.block[k];
     return true;
 }
@@ -1759,7 +1763,7 @@ __device__ __noinline__ void cell_item_setup(const FoldJob& J, const FoldSeg& fs
     f.n_phi = pc->n_phi;
     f.K = ic.K + 2.f;
     f.mode = on && sp.delta <= 8ull * FILTER_MARGIN
-                 ? filter_mode(J.tab, sp.ustep, ic.K, f.n_phi * J.n_D, nw)
+                 ? filter_mode(J.tab, sp.ustep, ic.K, f.n_phi * J.n_D, nw, sp.slots)
                  : FILTER_NONE;
     it.x.fp = f;
     it.x.f = filter_view(J.tab, fs);
@@ -1782,7 +1786,7 @@ __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int
     const int64_t p = o - seg * J.n_P;
     const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
     if (fs.use_slots) return;
-    if (nw < 8 && J.items && item_heavy(J, J.items[o])) return;
+    if (nw < 8 && J.items && item_heavy(J, J.items[o]) && list_taken(J.list)) return;
     const int n_D = J.n_D;
     if (lane == 0) {
         q.f.ni = q.f.nq = q.f.nc = q.nb = 0;
@@ -2236,7 +2240,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
     const int64_t p = o - seg * J.n_P;
     const FoldSeg& fs = J.segs ? J.segs[seg] : J.one;
     if (!fs.use_slots) return;
-    if (nw < 8 && J.list.block && !(slot_K(fs, J.stab[p]) < J.list.heavy_k)) return;
+    if (nw < 8 && list_taken(J.list) && !(slot_K(fs, J.stab[p]) < J.list.heavy_k)) return;
     const int n_D = J.n_D;
     if (lane == 0) q.f.ni = q.f.nq = q.f.nc = q.n = 0;
     q.bd[lane] = -1;
@@ -2252,7 +2256,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
         f.n_phi = sp.n_phi;
         const float K = slot_K(fs, sp);
         f.K = K + 2.f;
-        f.mode = filter_mode(J.tab, sp.ustep, K, f.n_phi * n_D, nw);
+        f.mode = filter_mode(J.tab, sp.ustep, K, f.n_phi * n_D, nw, true);
         it.x.fp = f;
         it.x.f = filter_view(J.tab, fs);
         it.x.n_D = n_D;
@@ -2675,12 +2679,26 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
 
 // Warps per item of n, each of `steps` slots x durations: eight where the items are
 // few for their size, two (and eight for the long ones) from where they fill the
-// GPU, one from 40 000.  One curve, FP64: 4 000 periods of 2 000 epochs x 4
-// durations 0.49 ms with eight, 0.31 with two, 0.34 with one; 1 200 of 8 000 x 4
-// 0.40 / 0.49 / 0.66; 2 500 of 19 440 x 10 1.7 with eight, 2.0 with one.
+// GPU, one from 6 000 to 40 000 by size.  One curve, FP64, us with eight / two / one:
+// 2 000 periods of 2 000 epochs x 4 durations 307 / 281 / 358, 10 000 of them 717 /
+// 471 / 400; 2 000 of 8 000 x 4 475 / 531 / 637; 10 000 of 19 440 x 10 2 148 / 1 792 /
+// 2 052.  100 curves of 2 000 x 8, 1 000 periods: two 8.4 ms, one 7.2.
 static int fold_warps(int64_t n, double steps) {
-    if (n >= 40000) return 1;
+    if (n >= std::min(40000.0, 6000.0 + steps / 6.0)) return 1;
     return n >= std::min(6000.0, 1000.0 + steps / 32.0) ? 2 : 8;
+}
+
+// How many of the n items may take blocks of eight: more fill the GPU either way,
+// and one or two warps idle less at the ends of an item's rounds.  Beside two
+// warps, periods uniform in frequency, with blocks / without: 10 000 of 19 440 x 10,
+// mixed 3.28 / 2.50 ms, FP64 3.48 / 3.06; 14 curves of 12 000-18 000 x 7 durations x
+// 969, mixed, 4.69 / 4.14 (one duration has few cells a period: 10 000 of 100 000 x
+// 1, FP64, 3.93 / 4.44).  Beside one warp: 404 curves of 4 600-7 000 x 3 x 3 340, 23 %
+// of the items long, FP64, 95.6 / 91.5; 438 of 8 000-20 000 x 10 x 4 000, 4 % long,
+// mixed, 240 / 244.
+static unsigned list_max(int nw, int n_D, int64_t n) {
+    if (nw == 1) return (unsigned)std::min<int64_t>(n / 10, 0xffffffffll);
+    return n_D > 1 ? 5000u : ~0u;
 }
 
 // The cell kernels of one job: the exact paths' items, then the slot path's.
@@ -2814,7 +2832,6 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
     int64_t slots = 0;
     for (int g = 0; g < n_seg; ++g) slots += fb.segs[g].n_bucket;
     const int nw = fold_warps((int64_t)n_seg * n_P, (double)slots / n_seg * n_D);
-    if (nw != 8 && fs.list) J.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K};
     // The passes: whole curves, or parts of one curve's periods.
     const int64_t pass = fs.pass ? fs.pass : (int64_t)n_seg * n_P;
     int64_t segs_pass = std::min<int64_t>(std::max<int64_t>(pass / n_P, 1), n_seg);
@@ -2833,6 +2850,9 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                 K.ptab += p;
                 K.stab += p;
                 K.n_P = std::min(per_pass, n_P - p);
+                if (nw != 8 && fs.list)
+                    K.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K,
+                                       list_max(nw, n_D, K.n_seg * K.n_P)};
                 K.Q += o;
                 K.T0 += o;
                 K.Didx += o;
@@ -3176,7 +3196,8 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
                 J.range = (int2*)(scratch + L.range);
                 J.items = (ItemConst*)(scratch + L.items);
             }
-            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K}
+            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K,
+                                         list_max(nw, n_D, n)}
                              : FoldLists{};
         }
         const cudaStream_t side = C.fork && J.list.block ? thread_side_stream() : nullptr;

@@ -32,3 +32,26 @@ def test_periods_about_the_line(kind, precision, n_D):
                     precision, dt)
         for k in KEYS:
             np.testing.assert_array_equal(got[k], np.tile(few[k], copies), err_msg=k)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("kind", ["regular", "drift"])
+@pytest.mark.parametrize("n_P, long", [(4990, 1.0), (5800, 1.0), (5800, 0.3), (41000, 0.05),
+                                       (41000, 1.0)])
+def test_many_long_items(kind, precision, n_P, long):
+    """Items of 22 or more epochs per cell take blocks beside the warps of the
+    others up to 5 000 of them (a tenth of the items, beside one warp each), and
+    warps beyond."""
+    t, depth, var, dlnl, dt = _grid(6500, 20, 71, kind)
+    span = t[-1] - t[0]
+    n = 60
+    n_long = int(round(long * n))
+    base = np.concatenate([span / np.linspace(24, 90, n_long),
+                           span / np.linspace(3, 18, n - n_long)])
+    few = [_fold(api.nu_periodic_search, t, depth, var, dlnl, base[lo:lo + 30], precision, dt)
+           for lo in (0, 30)]
+    copies = -(-n_P // n)
+    got = _fold(api.nu_periodic_search, t, depth, var, dlnl, np.tile(base, copies), precision, dt)
+    for k in KEYS:
+        want = np.concatenate([f[k] for f in few])
+        np.testing.assert_array_equal(got[k], np.tile(want, copies), err_msg=k)
