@@ -31,11 +31,13 @@
 // slot apart at every epoch):
 //   Q    over four slots: the largest and smallest Delta v, the smallest v, the
 //        largest gB (four phases of one duration);
-//   G    over eight slots: the largest L as FP16 rounded up (eight phases of up
-//        to eight durations in one load).
+//   G    over eight slots: the largest L (eight phases of up to eight durations).
 // S and Q are packed as the high halves of two words whose low halves hold
 // another BF16 number: the word itself is read as the FP32 value of the high
 // half, and its rounding direction is chosen with the low half in place.
+// G and L are FP32, and so are all sums (G as FP16 with FP16 sums: 1 to 4 % faster
+// on the folds of 10 to 20 durations, but 2^-11 of the sum looser per event, and
+// a gain above 65 504 passed everything).
 // Q and G are stored by slot modulo 4 and 8, so that the lanes of a warp, on
 // consecutive groups of phases, read consecutive entries.
 //
@@ -432,13 +434,12 @@ __global__ void k_filter_groups(const FoldSeg* __restrict__ segs, FoldSeg one, i
                                pack_hi(v, bf16_bits_ru(g), false));
         if (fs.d == n_D - 1 && (n_D & 1)) tab.Q[qo + 1] = make_uint2(0u, 0u);
     }
-    const int W = 2 * filter_words(n_D);
-    const int gi = fs.d / W;
-    __half* G = reinterpret_cast<__half*>(tab.G + sg.g_off) +
-                ((int64_t)gi * ns + (int64_t)(fs.s & 7) * (ns >> 3) + (fs.s >> 3)) * W;
-    G[fs.d - gi * W] = __float2half_ru(l);
+    const int gi = fs.d >> 3, W = filter_width(n_D, gi), c = fs.d & 7;
+    float* G = tab.G + sg.g_off + (int64_t)gi * 8 * ns +
+               ((int64_t)(fs.s & 7) * (ns >> 3) + (fs.s >> 3)) * W;
+    G[c] = l;
     if (fs.d == n_D - 1)
-        for (int c = fs.d - gi * W + 1; c < W; ++c) G[c] = __float2half(0.f);
+        for (int q = c + 1; q < W; ++q) G[q] = 0.f;
 }
 
 // ------------------------------------------------------------------ walks
@@ -448,7 +449,7 @@ struct FilterView {
     const float* gB;
     const float* L;
     const uint2* Q;
-    const unsigned* G;
+    const float* G;
     int ns;
 };
 __device__ __forceinline__ FilterView filter_view(const FilterTab& tab, const FoldSeg& sg) {
@@ -519,22 +520,21 @@ __device__ __forceinline__ float filter_bound(float sd, float v, float g, float 
     return fmaf(g, 1.f + c, 0.500001f) + eff * sd * sd * r * 1.00001f;
 }
 
-// Gain sums of two groups of eight phases, each of 2 NW durations (rows r0, r1,
-// walks from u0, u1; the rest of a stays 0).  Two epochs of both a round, four
-// loads in flight: the walks are short (two to five epochs), so that a round
-// is mostly the latency of its loads.  Positions past the end, of either walk,
-// add terms >= 0 (the empty last entry, or an event the cell does not have).
-template <int NW> struct FilterWords;
-template <> struct FilterWords<1> { typedef unsigned T; };
-template <> struct FilterWords<2> { typedef uint2 T; };
-template <> struct FilterWords<4> { typedef uint4 T; };
-template <int NW>
-__device__ __forceinline__ void filter_gain(const unsigned* __restrict__ g0,
-                                            const unsigned* __restrict__ g1, unsigned ns,
+// Gain sums of two groups of eight phases, of W durations each (rows r0, r1, walks
+// from u0, u1).  64 bytes in flight a lane, two epochs of both groups or one:
+// the walks are short (two to five epochs), so that a round is mostly the latency
+// of its loads.  Positions past the end, of either walk, add terms >= 0 (the empty
+// last entry, or an event the cell does not have).
+template <int W> struct __align__(W >= 4 ? 16 : 4 * W) FilterEntry {
+    float l[W];
+};
+template <int W>
+__device__ __forceinline__ void filter_gain(const float* __restrict__ g0,
+                                            const float* __restrict__ g1, unsigned ns,
                                             unsigned long long u0, unsigned long long u1,
                                             unsigned long long ustep, unsigned long long uend,
-                                            __half2 (&a)[4], __half2 (&b)[4]) {
-    typedef typename FilterWords<NW>::T V;
+                                            float (&a)[8], float (&b)[8]) {
+    typedef FilterEntry<W> V;
     const V* __restrict__ r0 = reinterpret_cast<const V*>(g0);
     const V* __restrict__ r1 = reinterpret_cast<const V*>(g1);
     const unsigned n8 = ns >> 3, last = ns - 1u;
@@ -542,18 +542,23 @@ __device__ __forceinline__ void filter_gain(const unsigned* __restrict__ g0,
         const unsigned s = min((unsigned)(x >> 40), last);
         return (s & 7u) * n8 + (s >> 3);
     };
-    auto add = [&](__half2 (&c)[4], const V& v) {
-        const unsigned* w = reinterpret_cast<const unsigned*>(&v);
+    auto add = [&](float (&c)[8], const V& v) {
 #pragma unroll
-        for (int i = 0; i < NW; ++i) c[i] = __hadd2(c[i], *reinterpret_cast<const __half2*>(w + i));
+        for (int i = 0; i < W; ++i) c[i] += v.l[i];
     };
-    for (; min(u0, u1) < uend; u0 += 2ull * ustep, u1 += 2ull * ustep) {
+    constexpr int E = W == 8 ? 1 : 2;
+    for (; min(u0, u1) < uend; u0 += E * ustep, u1 += E * ustep) {
         const V x0 = r0[at(u0)], x1 = r1[at(u1)];
-        const V y0 = r0[at(u0 + ustep)], y1 = r1[at(u1 + ustep)];
-        add(a, x0);
-        add(b, x1);
-        add(a, y0);
-        add(b, y1);
+        if (E == 2) {
+            const V y0 = r0[at(u0 + ustep)], y1 = r1[at(u1 + ustep)];
+            add(a, x0);
+            add(b, x1);
+            add(a, y0);
+            add(b, y1);
+        } else {
+            add(a, x0);
+            add(b, x1);
+        }
     }
 }
 
@@ -634,43 +639,51 @@ __device__ __forceinline__ float filter_slack(const FilterPeriod& fp) {
     return (fp.K + 8.f) * 1.1920929e-7f;
 }
 
-// Gain sums of the groups (q0, g0) and (q1, g1): eight durations' FP16 numbers
-// each.
+// Gain sums of the groups (q0, g0) and (q1, g1).
 struct FilterGains {
-    __half2 a[4], b[4];
+    float a[8], b[8];
 };
+template <int W>
 __device__ __forceinline__ void filter_gains(const FilterCtx& x, unsigned q0, int g0, unsigned q1,
                                              int g1, FilterGains& s) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) s.a[i] = s.b[i] = __half2half2(__float2half(0.f));
-    const int NW = filter_words(x.n_D);
+    for (int i = 0; i < 8; ++i) s.a[i] = s.b[i] = 0.f;
     const unsigned ns = (unsigned)x.f.ns;
     const unsigned long long uph8 = x.fp.uph << 3;
-    const unsigned long long u0 = q0 * uph8, u1 = q1 * uph8;
-    const unsigned* r0 = x.f.G + (int64_t)g0 * (int)ns * NW;
-    const unsigned* r1 = x.f.G + (int64_t)g1 * (int)ns * NW;
-    if (NW == 4) filter_gain<4>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
-    else if (NW == 2) filter_gain<2>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
-    else filter_gain<1>(r0, r1, ns, u0, u1, x.fp.ustep, x.fp.uend, s.a, s.b);
+    filter_gain<W>(x.f.G + (int64_t)g0 * 8 * (int)ns, x.f.G + (int64_t)g1 * 8 * (int)ns, ns,
+                   q0 * uph8, q1 * uph8, x.fp.ustep, x.fp.uend, s.a, s.b);
 }
 // Which of them reach the threshold: bit i is duration i of the first group,
 // bit 16 + i of the second.
-__device__ __noinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q0, int g0,
-                                                  unsigned q1, int g1) {
+template <int W>
+__device__ __forceinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q0, int g0,
+                                                     unsigned q1, int g1) {
     FilterGains s;
-    filter_gains(x, q0, g0, q1, g1, s);
-    // FP16 sums of K terms: 2^-11 of the sum per addition; a sum of 0, no event,
-    // is below the smallest FP16 number
-    const float inv_ch = 0.999999f - (x.fp.K + 4.f) * 5.4e-4f;
-    const float t = fmaxf((filter_thr(x) - 0.500002f) * inv_ch, 5.9604645e-08f);
-    const __half2 t2 = __half2half2(__float2half_rd(t));
+    filter_gains<W>(x, q0, g0, q1, g1, s);
+    // (a sum of 0, no event, is below every entry)
+    const float t = fmaxf((filter_thr(x) - 0.500002f) * (1.f - filter_slack(x.fp)), 5e-31f);
     unsigned pass = 0u;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const unsigned m = __hge2_mask(s.a[i], t2), n = __hge2_mask(s.b[i], t2);
-        pass |= ((m & 1u) | ((m >> 15) & 2u) | ((n & 1u) << 16) | ((n & 0x10000u) << 1)) << (2 * i);
-    }
+    for (int i = 0; i < W; ++i)
+        pass |= (s.a[i] >= t ? 1u << i : 0u) | (s.b[i] >= t ? 0x10000u << i : 0u);
     return pass;
+}
+__device__ __noinline__ unsigned filter_gain_pass(const FilterCtx& x, unsigned q0, int g0,
+                                                  unsigned q1, int g1) {
+    const int w = filter_width(x.n_D, g0);
+    if (w == filter_width(x.n_D, g1)) {
+        if (w == 8) return filter_gain_pass<8>(x, q0, g0, q1, g1);
+        if (w == 4) return filter_gain_pass<4>(x, q0, g0, q1, g1);
+        if (w == 2) return filter_gain_pass<2>(x, q0, g0, q1, g1);
+        return filter_gain_pass<1>(x, q0, g0, q1, g1);
+    }
+    // (the second of the pair is in the last, narrower group)
+    const int w1 = filter_width(x.n_D, g1);
+    const unsigned p0 = filter_gain_pass<8>(x, q0, g0, q0, g0);
+    const unsigned p1 = w1 == 4 ? filter_gain_pass<4>(x, q1, g1, q1, g1)
+                                : (w1 == 2 ? filter_gain_pass<2>(x, q1, g1, q1, g1)
+                                           : filter_gain_pass<1>(x, q1, g1, q1, g1));
+    return (p0 & 0xffffu) | (p1 << 16);
 }
 
 // Bounds of four phases (Q) or one phase (S) of four durations from d0 (the
@@ -988,16 +1001,20 @@ __device__ __noinline__ void filter_first(FilterCtx& x, FilterQueues& q, bool ac
     int bd = 0;
     const int n_D = x.n_D;
     if (x.fp.mode == FILTER_GAIN) {
-        const int d0 = gi * 2 * filter_words(n_D);
+        const int d0 = gi * 8;
         if (act) {
             FilterGains s;
-            filter_gains(x, qi, gi, qi, gi, s);
+            const int w = filter_width(n_D, gi);
+            if (w == 8) filter_gains<8>(x, qi, gi, qi, gi, s);
+            else if (w == 4) filter_gains<4>(x, qi, gi, qi, gi, s);
+            else if (w == 2) filter_gains<2>(x, qi, gi, qi, gi, s);
+            else filter_gains<1>(x, qi, gi, qi, gi, s);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float lo = __low2float(s.a[i]), hi = __high2float(s.a[i]);
-                if (lo > b && lo < INFINITY) { b = lo; bd = 2 * i; }
-                if (hi > b && hi < INFINITY) { b = hi; bd = 2 * i + 1; }
-            }
+            for (int i = 0; i < 8; ++i)
+                if (s.a[i] > b && s.a[i] < INFINITY) {
+                    b = s.a[i];
+                    bd = i;
+                }
         }
         bd += d0;
     } else {
@@ -1078,7 +1095,7 @@ __device__ __forceinline__ void filter_cells(FilterCtx& x, int wid, int nw, Filt
     }
     const int sh = filter_shift(mode);
     FilterGroups g;
-    g.W = mode == FILTER_GAIN ? 2 * filter_words(n_D) : 4;
+    g.W = mode == FILTER_GAIN ? 8 : 4;
     g.nq = (unsigned)((x.fp.n_phi + (1 << sh) - 1) >> sh);
     g.n_it = g.nq * (unsigned)((n_D + g.W - 1) / g.W);
     g.stride = (unsigned)nw * 32u;

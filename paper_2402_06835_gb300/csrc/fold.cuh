@@ -70,11 +70,15 @@ struct FoldSeg {
 
 // ---- filter tables (see filter.cuh) and the lists of the cell kernels
 __host__ __device__ inline int64_t filter_slots(int64_t n_slots) { return (n_slots + 7) / 8 * 8; }
-// FP16 words of one G entry: 8, 4 or 2 durations per load
-__host__ __device__ inline int filter_words(int n_D) { return n_D >= 5 ? 4 : (n_D >= 3 ? 2 : 1); }
-__host__ __device__ inline int filter_groups(int n_D) {
-    const int w = 2 * filter_words(n_D);
-    return (n_D + w - 1) / w;
+// Durations of G's group gi (eight, the last group one, two, four or eight), and
+// the numbers of all groups per slot.
+__host__ __device__ inline int filter_width(int n_D, int gi) {
+    const int r = n_D - 8 * gi;
+    return r >= 5 ? 8 : (r >= 3 ? 4 : r);
+}
+__host__ __device__ inline int filter_cols(int n_D) {
+    const int last = (n_D - 1) / 8;
+    return 8 * last + filter_width(n_D, last);
 }
 
 // Tables of all curves; rows of filter_slots(n_slots) per duration from
@@ -87,7 +91,7 @@ struct FilterTab {
     float* L;
     unsigned* Z;      // per slot (largest, smallest) Delta v as FP16 (source of Q)
     uint2* Q;
-    unsigned* G;
+    float* G;
     unsigned* vmax;   // per (curve, duration): max 1/s^2 (float bits)
 };
 
@@ -112,9 +116,9 @@ inline FilterLayout filter_layout(int64_t entries, int64_t pairs, int64_t words,
 inline FilterTab filter_tab(char* p, const FilterLayout& F, bool gains_only = false) {
     if (gains_only)
         return FilterTab{nullptr, nullptr, (float*)(p + F.L), nullptr, nullptr,
-                         (unsigned*)(p + F.G), nullptr};
+                         (float*)(p + F.G), nullptr};
     return FilterTab{(uint2*)(p + F.S), (float*)(p + F.gB), (float*)(p + F.L),
-                     (unsigned*)(p + F.Z), (uint2*)(p + F.Q), (unsigned*)(p + F.G),
+                     (unsigned*)(p + F.Z), (uint2*)(p + F.Q), (float*)(p + F.G),
                      (unsigned*)(p + F.vmax)};
 }
 

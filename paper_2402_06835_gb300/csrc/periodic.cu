@@ -2533,7 +2533,7 @@ void plan_fold_batch(const std::vector<int64_t>& s_off, const std::vector<double
             f.pair_off = fb.n_pair_total;
             fb.n_pair_total += ns * ((n_D + 1) / 2 * 2);
             fb.n_tab_total += ns * n_D;
-            fb.n_g_total += ns * filter_groups(n_D) * filter_words(n_D);
+            fb.n_g_total += ns * filter_cols(n_D);
         }
         f.bucket_off = fb.n_bucket_total;
         fb.n_bucket_total += f.use_slots ? 0 : f.n_bucket;
@@ -3007,7 +3007,7 @@ static SingleLayout single_layout(const FoldCall& C, const FoldPlan& plan) {
         L.tab = take((size_t)ns * C.n_D * sizeof(float));
     } else if (plan.tables) {
         L.fl = filter_layout(ns * C.n_D, ns * ((C.n_D + 1) / 2 * 2),
-                             ns * filter_groups(C.n_D) * filter_words(C.n_D), C.n_D,
+                             ns * filter_cols(C.n_D), C.n_D,
                              plan.tables == 1);
         L.tab = take(L.fl.total);
     }
