@@ -481,17 +481,19 @@ struct FilterPeriod {
 // 19 440 x 10 linear, FP64, 1.63 -> 1.33.  Two or eight warps: 6 / 9 / 14 cells
 // 2.10 / 1.88 / 1.99 ms on 3 500 of 19 440 x 10 uniform in frequency; one warp: 9 /
 // 20 / 45 cells 86.1 / 81.6 / 90.0 ms on 1 000 curves of 2 880 x 4 000 periods.
-// Where the screen searches the epochs' positions (!placed) it costs more: 2 026
-// periods uniform in frequency of 6 000 x 13, mixed, 7 / 9 cells 1.15 / 1.22 ms;
-// 12 586 of 3 200 x 11, FP64, 0 / 7 cells 1.63 / 1.74; one warp, 60 000 periods of
-// 9 000 x 1, FP64, 7 / 20 cells 4.07 / 4.76.
-__device__ __forceinline__ int filter_rounds(int nw, bool placed) {
-    return !placed ? 6 : (nw == 1 ? 20 : 9);
+// Where the screen searches the epochs' positions (!placed) it costs more, and only
+// long walks are worth it.  All / none up to 9 cells: 20 000 periods of 19 440 x 10,
+// FP64 (K to 135), 3.61 / 3.76 ms; 1 630 of 17 000 x 11, mixed (K 89), 1.36 / 1.44; but
+// 2 026 uniform in frequency of 6 000 x 13, mixed (K 38), 1.22 / 1.15, and 12 586 of
+// 3 200 x 11, FP64 (K 23), 1.74 / 1.63; one warp, 60 000 of 9 000 x 1, FP64 (K 13 to
+// 43), 20 / 7 cells 4.76 / 4.07.
+__device__ __forceinline__ int filter_rounds(int nw, bool placed, float K) {
+    return !placed && K < 40.f ? 4 : (nw == 1 ? 20 : 9);
 }
 // (n_cells < 2^31: the filters count groups in 32 bits)
 __device__ __forceinline__ int filter_mode(const FilterTab& tab, unsigned long long ustep,
                                            float K, int64_t n_cells, int nw, bool placed) {
-    if (n_cells <= filter_rounds(nw, placed) * 32 * nw) return FILTER_NONE;
+    if (n_cells <= filter_rounds(nw, placed, K) * 32 * nw) return FILTER_NONE;
     if (!tab.L || ustep < (1ull << 32) || ustep >= (1ull << 60) || !(K < FILTER_K_MAX) ||
         n_cells >= 0x7fff0000LL)
         return FILTER_NONE;
