@@ -258,9 +258,11 @@ nu_status nu_rotation_alias_filter(const double* periods_dev, int64_t n_P, doubl
  *   depth_dev, var_dev, dlnl_dev, snr_dev  (n_cand) FP64 outputs
  * A candidate with P or T0 not finite, D_idx outside [0, n_D), 2 D > P
  * (windows would overlap), no sample in any window, or a template in the
- * span of X gets NaN in all four outputs.  Always FP64.  One warp per
- * candidate, its lanes over 32 segments of the samples; gaps between windows
- * advance in blocks of 32 samples.  Enqueued on `stream`; no synchronisation.
+ * span of X gets NaN in all four outputs.  Always FP64.  Eight, two or one
+ * warps per candidate, the fewer the more candidates the call has, their lanes
+ * over 32 segments of the samples per warp (so that a candidate's last bits can
+ * depend on how many share its call); gaps between windows advance in blocks of
+ * 32 samples.  Enqueued on `stream`; no synchronisation.
  * Errors: NU_EINVAL (null pointer, n_cand < 1, n_D < 1, a duration not finite
  * and > 0, bad template or template parameters), NU_ENOMEM, NU_ECUDA. */
 nu_status nu_periodic_refine(const nu_factor* f, const double* P_dev, const double* T0_dev,
@@ -279,7 +281,8 @@ nu_status nu_periodic_refine(const nu_factor* f, const double* P_dev, const doub
  * tables) lives in a fixed array of NU_NOALLOC_SCRATCH_LIMIT bytes inside the
  * library, which every GPU that loads the library holds until the process
  * exits; grids that need more return NU_EINVAL (nu_periodic_search handles
- * them).  This call makes no cudaMalloc/cudaFree or other allocating call.
+ * them).  This call makes no cudaMalloc/cudaFree or other allocating call and
+ * creates no stream or event; many periods go through the array in passes.
  *   - phase_step must be > 0 (the median-spacing default would need a host
  *     buffer).
  *   - The array of the device that `stream` belongs to is used; that device

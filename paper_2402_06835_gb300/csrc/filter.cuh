@@ -57,16 +57,10 @@ namespace nu {
 #define FILTER_BETA_A 0.465f    // x_max <= 1/13.3
 #define FILTER_BETA_B 0.38f     // x_max <= 1/3.2
 #define FILTER_TAU 0.125f
-#ifndef NU_FILTER_K_QUAD
-#define NU_FILTER_K_QUAD 5.5f   // epochs per cell from which Q bounds better than G
-#endif
-#ifndef NU_FILTER_K_CELL
-#define NU_FILTER_K_CELL 22.0f  // and S better than Q
-#endif
+#define FILTER_K_QUAD 5.5f   // epochs per cell from which Q bounds better than G
+#define FILTER_K_CELL 22.0f  // and S better than Q
 #define FILTER_K_A 16.5f        // and beta A is allowed (with a margin for holes)
-#ifndef NU_FILTER_K_MID
-#define NU_FILTER_K_MID 3.8f    // groups that G passes are bounded by Q next
-#endif
+#define FILTER_K_MID 3.8f    // groups that G passes are bounded by Q next
 #define FILTER_K_MAX 4000.0f    // FP32 sums: K 2^-24 stays below the tables' slack
 // margin of the tables in walk units (2^-40 slot); a period's band half-width
 // delta (16 times the walk's error) must not exceed 16 times this
@@ -498,11 +492,11 @@ __device__ __forceinline__ int filter_mode(const FilterTab& tab, unsigned long l
         n_cells >= 0x7fff0000LL)
         return FILTER_NONE;
     if (!tab.G) return FILTER_LONE;
-    if (K < NU_FILTER_K_QUAD) return FILTER_GAIN;
+    if (K < FILTER_K_QUAD) return FILTER_GAIN;
     // (without S and Q the cells one by one, by their gains; 19 440 epochs x 12
     // durations x 3 000 periods, FP64: 1.69 ms, 4.7 in groups of eight)
     if (!tab.S) return FILTER_LONE;
-    return K < NU_FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL;
+    return K < FILTER_K_CELL ? FILTER_QUAD : FILTER_CELL;
 }
 
 __device__ __forceinline__ float filter_weight(unsigned long long u) {
@@ -910,7 +904,7 @@ __device__ __noinline__ void filter_drain(FilterCtx& x, FilterQueues& q, bool al
                                           Screen& screen) {
     const int lane = threadIdx.x & 31;
     const bool gain = x.fp.mode == FILTER_GAIN;
-    const bool mid = !Screen::lone && gain && x.fp.K >= NU_FILTER_K_MID + 2.f;
+    const bool mid = !Screen::lone && gain && x.fp.K >= FILTER_K_MID + 2.f;
     const int ni = q.ni;
     const int round = mid ? 16 : (gain ? 4 : 8);
     const int n = all ? ni : ni & ~(round - 1);

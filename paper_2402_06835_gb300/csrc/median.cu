@@ -1,10 +1,10 @@
 // Median spacing of a sorted grid of epochs, and the grid's ends, on the device.
 //
 // The default phase step is the median of t[i+1] - t[i].  Copying the epochs to
-// the host and sorting the differences there cost 1.1 ms for 19 440 epochs, a
-// third of the fold that follows.  Here one block selects the middle element
-// (or the two middle ones) by radix, eight bits of an order-preserving key per
-// pass, and 32 bytes come back.
+// the host and sorting the differences there took 112 us of a mixed fold's 281 at
+// 16 000 epochs and 232 of 431 at 30 000.  Here one block selects the middle
+// element (or the two middle ones) by radix, eight bits of an order-preserving key
+// per pass, and 32 bytes come back: 35 and 79 us with the wait for them.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -32,24 +32,16 @@ __global__ void k_diff_keys(const double* __restrict__ t, int64_t m,
     if (i < m) key[i] = diff_key(t[i + 1] - t[i]);
 }
 
-// Short grids: the keys stay in the selecting block's shared memory, computed by
-// that block (48 FP64 subtractions a warp at most).
-constexpr int64_t MEDIAN_SHARED = 5120;
-
 // out = {element (m - 1) / 2, element m / 2 of the sorted differences, t[0], t[m]}.
-// keys: those of k_diff_keys, or nullptr: in shared memory (m <= MEDIAN_SHARED).
+// key: those of k_diff_keys.
 __global__ void __launch_bounds__(1024)
-k_median(const double* __restrict__ t, int64_t m, const unsigned long long* __restrict__ keys,
+k_median(const double* __restrict__ t, int64_t m, const unsigned long long* __restrict__ key,
          double* __restrict__ out) {
     __shared__ unsigned hist[256];
-    __shared__ unsigned long long sh_key[MEDIAN_SHARED];
     __shared__ unsigned long long sh_prefix, sh_next;
     __shared__ unsigned sh_rank, sh_left;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const unsigned long long* key = keys ? keys : sh_key;
-    if (!keys)
-        for (int64_t i = threadIdx.x; i < m; i += blockDim.x) sh_key[i] = diff_key(t[i + 1] - t[i]);
     if (threadIdx.x == 0) {
         sh_prefix = 0ull;
         sh_rank = (unsigned)((m - 1) / 2);      // (m < 2^31)
@@ -158,13 +150,12 @@ cudaError_t median_spacing(const double* t_dev, int64_t n, cudaStream_t st, doub
     if (m > 0 && n <= MEDIAN_HOST) return median_on_host(t_dev, n, st, step, t_first, t_last);
     char* mem = nullptr;
     pool_keep_memory();
-    const bool shared = m <= MEDIAN_SHARED;
-    cudaError_t e = cudaMallocAsync((void**)&mem, (shared ? 0 : (size_t)m * 8) + 256, st);
+    cudaError_t e = cudaMallocAsync((void**)&mem, (size_t)m * 8 + 256, st);
     if (e != cudaSuccess) return e;
-    unsigned long long* key = shared ? nullptr : (unsigned long long*)(mem + 256);
-    if (!shared) k_diff_keys<<<div_up(m, 256), 256, 0, st>>>(t_dev, m, key);
+    unsigned long long* key = (unsigned long long*)(mem + 256);
+    if (m > 0) k_diff_keys<<<div_up(m, 256), 256, 0, st>>>(t_dev, m, key);
     k_median<<<1, 1024, 0, st>>>(t_dev, m, key, (double*)mem);
-    count_launches(shared ? 1 : 2);
+    count_launches(m > 0 ? 2 : 1);
     double h[4];
     e = cudaGetLastError();
     if (e == cudaSuccess)

@@ -1,9 +1,9 @@
 // nu_periodic_search: Sect. 2.3-2.4 on the products of the linear search.
 //
-// For each trial period P every (duration d, phase j) cell gathers its single events at epochs T_k = T_ref + (j/n_phi + k) P,
-// linearly interpolated in time between the bracketing grid epochs, and
-// combines them with Eq. result using the biased estimates of
-// Eq. sigma_delta:
+// For each trial period P every (duration d, phase j) cell gathers its single
+// events at epochs T_k = T_ref + (j/n_phi + k) P, linearly interpolated in time
+// between the bracketing grid epochs, and combines them with Eq. result using the
+// biased estimates of Eq. sigma_delta:
 //   pass 1:  S_inv = sum 1/s_k^2,  S_d = sum Delta_k / s_k^2,  S_L = sum gain_k
 //            sigma^2 = 1/S_inv,    Delta = sigma^2 S_d
 //   pass 2:  pen = sum [ln s_k^2 - ln(sigma^2 + s_k^2) + (Delta_k - Delta)^2/(s_k^2 + sigma^2)]
@@ -633,8 +633,9 @@ __device__ __forceinline__ void cell_pass2(const FoldGeom& g, const Node8<T>* __
 // first pass of one cell, the cells whose bound can still beat the block's
 // best are compacted into a shared queue, and the queue's second passes run
 // densely (a warp instruction costs the same however many lanes are active).
-template <typename T, int KC, int MAXT = 256>
-__device__ __forceinline__ void fold_exact_one(const FoldGeom& g, const Node8<T>* __restrict__ nodes,
+template <typename T, int MAXT = 256>
+__device__ __forceinline__ void fold_exact_one(const FoldGeom& g,
+                                               const Node8<T>* __restrict__ nodes,
                                                int n_D, double P, int64_t p,
                                                double* __restrict__ Q_out,
                                                double* __restrict__ T0_out,
@@ -725,7 +726,7 @@ __device__ __forceinline__ int64_t period_slot(int64_t b, const double* __restri
     return okey(periods[n_P - 1]) < okey(periods[0]) ? n_P - 1 - b : b;
 }
 
-template <typename T, int KC>
+template <typename T>
 __global__ void __launch_bounds__(256)
 k_fold_exact(FoldGeom g, const Node8<T>* __restrict__ nodes, int n_D,
              const double* __restrict__ periods, int64_t n_P, double* __restrict__ Q_out,
@@ -734,7 +735,7 @@ k_fold_exact(FoldGeom g, const Node8<T>* __restrict__ nodes, int n_D,
              double* __restrict__ lnp_out) {
     if ((int64_t)blockIdx.x >= n_P) return;
     const int64_t p = period_slot(blockIdx.x, periods, n_P);
-    fold_exact_one<T, KC>(g, nodes, n_D, periods[p], p, Q_out, T0_out, Didx_out, dep_out,
+    fold_exact_one<T>(g, nodes, n_D, periods[p], p, Q_out, T0_out, Didx_out, dep_out,
                           sig_out, lnp_out);
 }
 
@@ -1534,12 +1535,8 @@ template <int NW>
 __device__ __forceinline__ void item_sync() {
     if (NW == 1) __syncwarp(); else __syncthreads();
 }
-#ifndef NU_FOLD_WARPS
-#define NU_FOLD_WARPS 32           // resident warps per SM (64 registers)
-#endif
-#ifndef NU_HEAVY_K
-#define NU_HEAVY_K 22.f            // epochs per cell of an item that takes a block then
-#endif
+constexpr int FOLD_WARPS = 32;     // resident warps per SM (64 registers)
+constexpr float HEAVY_K = 22.f;    // epochs per cell of an item that takes a block
 // Work item i of the job in the order of the fold (short periods first).
 __device__ __forceinline__ bool ordered_item(const FoldJob& J, int64_t i, int64_t& item) {
     if (i >= (int64_t)J.n_seg * J.n_P) return false;
@@ -1877,7 +1874,7 @@ __device__ __forceinline__ void fold_cells_item(const FoldJob& J, int64_t o, int
 
 // Exact paths (FP64 epochs; T: the type of the events).
 template <typename T, int NW, bool LONE>
-__global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
+__global__ void __launch_bounds__(fold_threads(NW), FOLD_WARPS * 32 / fold_threads(NW))
 k_fold_cells(const __grid_constant__ FoldJob J) {
     constexpr int W = fold_threads(NW) / 32;
     __shared__ CellQueues sh_q[W];
@@ -2147,8 +2144,6 @@ struct SlotScreen {
         }
         filter_raise(it.x, fkey(screen_threshold<float>(lnp, it.x.fp.K)));
     }
-    // (inlined: the lanes leave pass2 one by one, and a caller's shuffle after a
-    // call that returns like that has been seen to miss the late ones)
     __device__ __forceinline__ void flush(int cnt) {
         const int lane = threadIdx.x & 31;
         if (lane < cnt) pass2(q.c[lane]);
@@ -2337,7 +2332,7 @@ __device__ __forceinline__ void fold_slots_item(const FoldJob& J, int64_t o, int
 }
 
 template <int NW, bool LONE>
-__global__ void __launch_bounds__(fold_threads(NW), NU_FOLD_WARPS * 32 / fold_threads(NW))
+__global__ void __launch_bounds__(fold_threads(NW), FOLD_WARPS * 32 / fold_threads(NW))
 k_fold_slot_cells(const __grid_constant__ FoldJob J) {
     constexpr int W = fold_threads(NW) / 32;
     __shared__ SlotQueues sh_q[W];
@@ -2715,7 +2710,7 @@ static int launch_cells(const FoldJob& J, bool fp64, bool exact, bool slots, int
         if (e != cudaSuccess && *err == cudaSuccess) *err = e;
     };
     if (nw == 2 && items > 0x7fffffffLL) nw = 1;          // the grid's limit
-    const int g8 = (int)std::min<int64_t>(items, (int64_t)n_sm * (NU_FOLD_WARPS / 8));
+    const int g8 = (int)std::min<int64_t>(items, (int64_t)n_sm * (FOLD_WARPS / 8));
     // (the gains' tables alone: kernels of their own)
     const bool lone = J.tab.L && !J.tab.S;
 #define NU_CELLS_AS(NW_, LONE_, GRID_, ST_)                                                \
@@ -2851,7 +2846,7 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                 K.stab += p;
                 K.n_P = std::min(per_pass, n_P - p);
                 if (nw != 8 && fs.list)
-                    K.list = FoldLists{fs.list, fs.n_list, NU_HEAVY_K,
+                    K.list = FoldLists{fs.list, fs.n_list, HEAVY_K,
                                        list_max(nw, n_D, K.n_seg * K.n_P)};
                 K.Q += o;
                 K.T0 += o;
@@ -3060,7 +3055,8 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
         const int64_t ns = filter_slots(n_slots);
         float* Lg = Ls->plan.tables == TABLES_SLOT ? (float*)(scratch + Ls->tab) : nullptr;
         const int64_t n_L = Lg ? ns * n_D : 0;
-        const unsigned b_rec = (unsigned)div_up(std::max(nrec, n_L), 256), b_peak = b_rec + peak_grid;
+        const unsigned b_rec = (unsigned)div_up(std::max(nrec, n_L), 256);
+        const unsigned b_peak = b_rec + peak_grid;
         const unsigned b_all = b_peak + (unsigned)div_up(Ls->plan.pass, 256);
         k_slot_prep<<<b_all, 256, 0, st>>>(rec, nrec, Lg, n_L, b_rec, (const float*)C.dlnl, ngrid,
                                            b_peak, peak, C.periods, Ls->plan.pass, phase_step,
@@ -3139,11 +3135,11 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
             const FoldGeom g{C.t0s, n_t0, C.t_ref, C.t_last, phase_step, 1.0 / phase_step,
                              gap_max, (const int*)(scratch + L.bucket), n_bucket};
             if (fp64)
-                k_fold_exact<double, 8><<<(unsigned)n_P, 256, 0, st>>>(
+                k_fold_exact<double><<<(unsigned)n_P, 256, 0, st>>>(
                     g, (const Node8<double>*)J.nodes, n_D, C.periods, n_P, C.Q, C.T0, C.D_idx,
                     C.dep, C.sig, C.lnP);
             else
-                k_fold_exact<float, 8><<<(unsigned)n_P, 256, 0, st>>>(
+                k_fold_exact<float><<<(unsigned)n_P, 256, 0, st>>>(
                     g, (const Node8<float>*)J.nodes, n_D, C.periods, n_P, C.Q, C.T0, C.D_idx,
                     C.dep, C.sig, C.lnP);
             count_launches(launched + 1);
@@ -3196,7 +3192,7 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
                 J.range = (int2*)(scratch + L.range);
                 J.items = (ItemConst*)(scratch + L.items);
             }
-            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, NU_HEAVY_K,
+            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, HEAVY_K,
                                          list_max(nw, n_D, n)}
                              : FoldLists{};
         }

@@ -64,7 +64,7 @@ k_refine_blocks(const double* __restrict__ F, const double* __restrict__ kg,
                 double* __restrict__ Mq) {
     constexpr int J = Dims<NB>::J;
     constexpr int JJ = Dims<NB>::JJ;
-    // J lanes per block (8 or 32 / J rounded down: J = 6 uses 30 lanes of a warp)
+    // J lanes per block, 32 / J blocks per warp (J = 6: 30 of its lanes)
     constexpr int PER = 32 / J;
     const int lane = threadIdx.x & 31, c = lane % J, base = lane - c;
     const int64_t b = (blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5)) * PER +
@@ -426,19 +426,24 @@ k_refine(const double* __restrict__ t, int64_t n, int k, FactorView<double> fv,
     out_snr[cid] = dep / sqrt(var);
 }
 
-// Warps per candidate: as many as leave every warp an FP64 pipe of its own
-// (608 sub-partitions: 76 x 8, 304 x 2); beyond, more warps only take turns and
-// add segments to walk.
-static int refine_warps(int64_t n_cand) { return n_cand <= 76 ? 8 : (n_cand <= 304 ? 2 : 1); }
+// Warps per candidate: eight or two where every warp then still has an FP64 pipe of
+// its own (four per SM: up to 76 and 304 candidates on 152 SMs), else one; beyond,
+// more warps only take turns and add segments to walk.
+static int refine_warps(int64_t n_cand) {
+    int dev = 0, n_sm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t pipes = 4 * (int64_t)n_sm;
+    return 8 * n_cand <= pipes ? 8 : (2 * n_cand <= pipes ? 2 : 1);
+}
 
 template <int NB>
 static void launch_refine(const nu_factor* f, const double* Phi, const double* Mq,
-                          int64_t n_blk, double* Pseg, const double* P, const double* T0,
+                          int64_t n_blk, double* Pseg, int W, const double* P, const double* T0,
                           const int* Didx, int64_t n_cand, const double* Ds, int n_D, int tmpl,
                           const TmplArgs& ta, double* d, double* v, double* l, double* snr,
                           cudaStream_t st) {
     const FactorView<double> fv{f->F, f->kg, f->invD, f->G, f->z0, f->Zt};
-    const int W = refine_warps(n_cand);
     // segments of nbs blocks cover every sample: n_segs * nbs * RB >= n
     const int n_segs = RS * W;
     const int64_t blocks_all = (f->n + RB - 1) / RB;
@@ -491,7 +496,9 @@ extern "C" nu_status nu_periodic_refine(const nu_factor* f, const double* P_dev,
     cudaStream_t st = (cudaStream_t)stream;
     const int J = 2 * f->nb, JJ = J * (J + 1) / 2;
     const int64_t n_blk = (f->n - 1) / RB;
-    const size_t bytes = (n_D + n_blk * (int64_t)(J * J + JJ) + RS * refine_warps(n_cand) * J * J) * sizeof(double);
+    const int W = refine_warps(n_cand);
+    const size_t bytes =
+        (n_D + n_blk * (int64_t)(J * J + JJ) + RS * W * J * J) * sizeof(double);
     pool_keep_memory();
     double* mem = nullptr;
     cudaError_t e = cudaMallocAsync(&mem, bytes, st);
@@ -511,10 +518,10 @@ extern "C" nu_status nu_periodic_refine(const nu_factor* f, const double* P_dev,
         }
     }
     switch (f->nb) {
-        case 1: launch_refine<1>(f, Phi, Mq, n_blk, Pseg, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
-        case 2: launch_refine<2>(f, Phi, Mq, n_blk, Pseg, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
-        case 3: launch_refine<3>(f, Phi, Mq, n_blk, Pseg, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
-        default: launch_refine<4>(f, Phi, Mq, n_blk, Pseg, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
+        case 1: launch_refine<1>(f, Phi, Mq, n_blk, Pseg, W, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
+        case 2: launch_refine<2>(f, Phi, Mq, n_blk, Pseg, W, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
+        case 3: launch_refine<3>(f, Phi, Mq, n_blk, Pseg, W, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
+        default: launch_refine<4>(f, Phi, Mq, n_blk, Pseg, W, P_dev, T0_dev, D_idx_dev, n_cand, Ds_dev, n_D, tmpl, ta, depth_dev, var_dev, dlnl_dev, snr_dev, st); break;
     }
     count_launches(n_blk > 0 ? 3 : 2);
     e = cudaGetLastError();
