@@ -1536,7 +1536,6 @@ __device__ __forceinline__ void item_sync() {
     if (NW == 1) __syncwarp(); else __syncthreads();
 }
 constexpr int FOLD_WARPS = 32;     // resident warps per SM (64 registers)
-constexpr float HEAVY_K = 22.f;    // epochs per cell of an item that takes a block
 // Work item i of the job in the order of the fold (short periods first).
 __device__ __forceinline__ bool ordered_item(const FoldJob& J, int64_t i, int64_t& item) {
     if (i >= (int64_t)J.n_seg * J.n_P) return false;
@@ -2683,6 +2682,12 @@ static int fold_warps(int64_t n, double steps) {
     return n >= std::min(6000.0, 1000.0 + steps / 32.0) ? 2 : 8;
 }
 
+// Epochs per cell of one of n items that takes a block of eight warps.  Beside two
+// warps, 45 / 22: 20 000 periods of 19 440 x 16, mixed, 3.00 / 3.10 ms, x 10, FP64,
+// 2.81 / 2.87, barycentric 3.63 / 3.75; but 9 900 of 29 600 x 13, mixed and
+// barycentric, 3.67 / 3.42.  Beside one warp: 100 000 of 136 080 x 20, mixed, 98.3 /
+// 95.9 ms; 438 curves of 8 000-20 000 x 10 x 4 000, 244.7 / 241.9.
+static float heavy_k(int nw, int64_t n) { return nw == 2 && n >= 15000 ? 45.f : 22.f; }
 // How many of the n items may take blocks of eight: more fill the GPU either way,
 // and one or two warps idle less at the ends of an item's rounds.  Beside two
 // warps, periods uniform in frequency, with blocks / without: 10 000 of 19 440 x 10,
@@ -2846,7 +2851,7 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                 K.stab += p;
                 K.n_P = std::min(per_pass, n_P - p);
                 if (nw != 8 && fs.list)
-                    K.list = FoldLists{fs.list, fs.n_list, HEAVY_K,
+                    K.list = FoldLists{fs.list, fs.n_list, heavy_k(nw, K.n_seg * K.n_P),
                                        list_max(nw, n_D, K.n_seg * K.n_P)};
                 K.Q += o;
                 K.T0 += o;
@@ -3192,7 +3197,7 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
                 J.range = (int2*)(scratch + L.range);
                 J.items = (ItemConst*)(scratch + L.items);
             }
-            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, HEAVY_K,
+            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, heavy_k(nw, n),
                                          list_max(nw, n_D, n)}
                              : FoldLists{};
         }
