@@ -2673,21 +2673,22 @@ cudaError_t launch_fold_prep(const FoldBatch& fb, const FoldSeg* segs_dev,
 
 // Warps per item of n, each of `steps` slots x durations: eight where the items are
 // few for their size, two (and eight for the long ones) from where they fill the
-// GPU, one from 6 000 to 40 000 by size.  One curve, FP64, us with eight / two / one:
-// 2 000 periods of 2 000 epochs x 4 durations 307 / 281 / 358, 10 000 of them 717 /
-// 471 / 400; 2 000 of 8 000 x 4 475 / 531 / 637; 10 000 of 19 440 x 10 2 148 / 1 792 /
-// 2 052.  100 curves of 2 000 x 8, 1 000 periods: two 8.4 ms, one 7.2.
-static int fold_warps(int64_t n, double steps) {
-    if (n >= std::min(40000.0, 6000.0 + steps / 6.0)) return 1;
+// GPU, one from 6 000 up by size, at the latest from 18 000 periods of one curve or
+// 40 000 items of a batch.  One curve, FP64, us with eight / two / one: 2 000 periods
+// of 2 000 epochs x 4 durations 307 / 281 / 358, 10 000 of them 717 / 471 / 400; 2 000
+// of 8 000 x 4 475 / 531 / 637; 10 000 of 19 440 x 10 2 148 / 1 792 / 2 052, 18 000 two
+// 2 630, one 2 400, 18 000 uniform in frequency 4 350, 5 170, 26 000 5 900, 5 970.  100
+// curves of 2 000 x 8, 1 000 periods: two 8.4 ms, one 7.2; 64 of 18 000 x 10, 500
+// periods, 15.4, 16.3.
+static int fold_warps(int64_t n, double steps, bool batch) {
+    if (n >= std::min(batch ? 40000.0 : 18000.0, 6000.0 + steps / 6.0)) return 1;
     return n >= std::min(6000.0, 1000.0 + steps / 32.0) ? 2 : 8;
 }
 
-// Epochs per cell of one of n items that takes a block of eight warps.  Beside two
-// warps, 45 / 22: 20 000 periods of 19 440 x 16, mixed, 3.00 / 3.10 ms, x 10, FP64,
-// 2.81 / 2.87, barycentric 3.63 / 3.75; but 9 900 of 29 600 x 13, mixed and
-// barycentric, 3.67 / 3.42.  Beside one warp: 100 000 of 136 080 x 20, mixed, 98.3 /
-// 95.9 ms; 438 curves of 8 000-20 000 x 10 x 4 000, 244.7 / 241.9.
-static float heavy_k(int nw, int64_t n) { return nw == 2 && n >= 15000 ? 45.f : 22.f; }
+// Epochs per cell of an item that takes a block of eight warps (45 beside one warp:
+// 100 000 periods of 136 080 x 20, mixed, 95.9 -> 98.3 ms; 438 curves of 8 000-20 000 x
+// 10 x 4 000, 241.9 -> 244.7).
+constexpr float HEAVY_K = 22.f;
 // How many of the n items may take blocks of eight: more fill the GPU either way,
 // and one or two warps idle less at the ends of an item's rounds.  Beside two
 // warps, periods uniform in frequency, with blocks / without: 10 000 of 19 440 x 10,
@@ -2831,7 +2832,7 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
     J.counters = fs.n_list;
     int64_t slots = 0;
     for (int g = 0; g < n_seg; ++g) slots += fb.segs[g].n_bucket;
-    const int nw = fold_warps((int64_t)n_seg * n_P, (double)slots / n_seg * n_D);
+    const int nw = fold_warps((int64_t)n_seg * n_P, (double)slots / n_seg * n_D, true);
     // The passes: whole curves, or parts of one curve's periods.
     const int64_t pass = fs.pass ? fs.pass : (int64_t)n_seg * n_P;
     int64_t segs_pass = std::min<int64_t>(std::max<int64_t>(pass / n_P, 1), n_seg);
@@ -2851,7 +2852,7 @@ int launch_fold_batch(const FoldBatch& fb, const FoldSeg* segs_dev, int n_seg,
                 K.stab += p;
                 K.n_P = std::min(per_pass, n_P - p);
                 if (nw != 8 && fs.list)
-                    K.list = FoldLists{fs.list, fs.n_list, heavy_k(nw, K.n_seg * K.n_P),
+                    K.list = FoldLists{fs.list, fs.n_list, HEAVY_K,
                                        list_max(nw, n_D, K.n_seg * K.n_P)};
                 K.Q += o;
                 K.T0 += o;
@@ -2933,7 +2934,7 @@ struct FoldCall {
         if (slots) return work < (item_steps() < 4.0e4 ? 6.0e7 : 2.4e7);
         return work < (n_D == 1 ? 4.0e7 : 2.4e7);
     }
-    int warps(int64_t n) const { return fold_warps(n, item_steps()); }
+    int warps(int64_t n) const { return fold_warps(n, item_steps(), false); }
 };
 
 // What a fold keeps in scratch beside the records of its events.
@@ -3197,7 +3198,7 @@ static nu_status single_fold(const FoldCall& C, char* scratch, const SingleLayou
                 J.range = (int2*)(scratch + L.range);
                 J.items = (ItemConst*)(scratch + L.items);
             }
-            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, heavy_k(nw, n),
+            J.list = nw != 8 ? FoldLists{(unsigned*)(scratch + L.list), J.counters, HEAVY_K,
                                          list_max(nw, n_D, n)}
                              : FoldLists{};
         }
