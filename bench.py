@@ -48,11 +48,11 @@ METRIC = "linear-search (t0,D) fits/s + period trials/s, %HBM roofline, mixed vs
 MEASURED_FP64_TFLOPS = 1.197   # DFMA microbenchmark on this machine's GB300 (2 DFMA/clk/SM)
 N_SMSP = 152 * 4               # SM sub-partitions (one warp instruction issued per clock each)
 # Per call of the fold (FP64 on the sector, mixed on the 16-duration sector), summed
-# over its cell and evaluation kernels in one-pass ncu launch lists (summarised under
-# profiles/): DRAM bytes read (what is written back meanwhile is the L2 flush's
-# own), warp instructions.
-FOLD_NCU = {("sector_19440", "fp64"): {"traffic": 44758144, "inst": 1586653231},
-            ("sector_19440_16d", "mixed"): {"traffic": 28111360, "inst": 1961906828}}
+# over its cell and evaluation kernels, each captured by itself in one pass of ncu
+# (summarised under profiles/): DRAM bytes read (what is written back meanwhile is the
+# L2 flush's own), warp instructions.
+FOLD_NCU = {("sector_19440", "fp64"): {"traffic": 62752768, "inst": 1478929660},
+            ("sector_19440_16d", "mixed"): {"traffic": 27993856, "inst": 1907287426}}
 FLUSH_BYTES = 512 << 20        # > 129 MB L2
 ORACLE_TEMPLATES = 256         # bounded oracle sample per step (both CPU legs)
 ORACLE_PERIODS = 8
